@@ -311,37 +311,40 @@ int setup_plane(ch_env* env, PlaneArgs<R>* a, size_t* smem) {
     if ((size_t)6 * (g.mz / S) * g.nxh * csz > 160 * 1024) continue;
     feasible[nf++] = S;
   }
-  // three passes through a global scratch array: planes of 256 x 256 modes,
-  // whose padded z-slab fits no portable cluster in either precision (the
-  // traffic costs less than serialising 16-CTA clusters, of which the device
-  // holds few), and the FP64 planes of 64 x 64 and 128 x 128 modes; only in
-  // the precision the handle steps in (the other plane keeps a cluster, for
-  // ch_nonlinear, where one fits)
+  // a 16-CTA cluster (non-portable opt-in) only where no portable size fits
+  if (!nf && g.mz % 16 == 0 && (g.mz / 16) % 2 == 0 && (size_t)6 * (g.mz / 16) * g.nxh * csz <= 160 * 1024)
+    feasible[nf++] = 16;
+  // Three passes through a global scratch array where the padded lengths are
+  // built (plane_pass.cu), in the precision the handle steps in; the other
+  // plane keeps a cluster, for ch_nonlinear, where one fits.  Planes of
+  // 256 x 256 modes fit no portable cluster.
   const bool stepping = (sizeof(R) == 8) == (env->prm.precision == 0);
-  if (stepping && two_pass_chosen(g.mx, g.mz, g.nxh, sizeof(R) == 8)) {
-    a->two_pass = 1;
+  const bool large = g.mx == 384 && g.mz == 384;
+  if (stepping && passes_built(g.mx, g.mz) && (nf || large)) {
+    a->passes = 1;
     a->S = 1;
     a->Lz = g.mz;
     a->NP = 0;
     *smem = 0;
+    // reported: the cluster that would hold the plane; 0 where none does, and
+    // for FP64 planes of 64 x 64 and 128 x 128 modes (the value is part of the ABI)
+    const bool fp64_square = sizeof(R) == 8 && g.mx == g.mz && (g.mx == 96 || g.mx == 192);
+    a->cluster = large || fp64_square ? 0 : feasible[nf - 1];
+    for (int k = 0; k < nf && a->cluster; ++k)
+      if ((long)g.ny * env->B * feasible[k] >= nsm) { a->cluster = feasible[k]; break; }
     C* y = nullptr;
     RC(dalloc(env, &y, (size_t)env->B * g.ny * 6 * g.mz * g.nxh));
     a->y = y;
-    if (!fft_plan(g.mx, &a->px) || !fft_plan(g.mz, &a->pz)) return CH_ERR_UNSUPPORTED;
     auto cast2 = [](const std::vector<double2>& v) {
       std::vector<C> o(v.size());
       for (size_t i = 0; i < v.size(); ++i) o[i] = mk((R)v[i].x, (R)v[i].y);
       return o;
     };
     RC(dupload(env, &a->tw_x, cast2(twiddles(g.mx))));
-    RC(dupload(env, &a->tw_z, cast2(twiddles(g.mz))));
     RC(dupload(env, &a->tw_mz, cast2(twiddles(g.mz))));
     a->scale = (R)(1.0 / ((double)g.mx * g.mz));
     return CH_OK;
   }
-  // a 16-CTA cluster (non-portable opt-in) only where no portable size fits
-  if (!nf && g.mz % 16 == 0 && (g.mz / 16) % 2 == 0 && (size_t)6 * (g.mz / 16) * g.nxh * csz <= 160 * 1024)
-    feasible[nf++] = 16;
   if (!nf) return CH_ERR_UNSUPPORTED;
   int S = feasible[nf - 1];
   for (int k = 0; k < nf; ++k)
@@ -371,6 +374,7 @@ int setup_plane(ch_env* env, PlaneArgs<R>* a, size_t* smem) {
     a->S = 1;
     a->Lz = g.mz;
   }
+  a->cluster = a->S;
   if (!fft_plan(g.mx, &a->px) || !fft_plan(a->Lz, &a->pz)) return CH_ERR_UNSUPPORTED;
   if (a->S > 8) {
     int clusters = 0;
@@ -747,7 +751,7 @@ int run_stage(ch_env* env, int k, double theta) {
 // passes, the implicit half two in its wide form
 static void set_launch_count(ch_env* env) {
   const ch_params_t* p = &env->prm;
-  const bool passes = p->precision == 1 ? env->plane_f.two_pass : env->plane.two_pass;
+  const bool passes = p->precision == 1 ? env->plane_f.passes : env->plane.passes;
   const int stage = 1 + (passes ? 3 : 1) + stage_post_launches(env->g, p->top_bc, env->post_batched);
   env->launches_per_step = (p->control == 0 ? 2 : p->control == 1 ? 1 : 5) + p->steps_per_action * (3 * stage + 1) + 3;
 }
@@ -1002,9 +1006,8 @@ size_t env_footprint(const ch_params_t* p) {
   // the scratch of the three-pass nonlinear term, where it runs in passes
   // (complex values of the plane's precision)
   const size_t mx = 3 * (size_t)p->nx / 2, mz = 3 * (size_t)p->nz / 2;
-  const size_t two_pass = two_pass_chosen((int)mx, (int)mz, (int)nxh, p->precision == 0)
-                              ? B * ny * 6 * mz * nxh * (p->precision == 0 ? 16 : 8) : 0;
-  return state + tables + two_pass + ((size_t)4 << 20);  // plus twiddles and rounding slack
+  const size_t passes = passes_built((int)mx, (int)mz) ? B * ny * 6 * mz * nxh * (p->precision == 0 ? 16 : 8) : 0;
+  return state + tables + passes + ((size_t)4 << 20);  // plus twiddles and rounding slack
 }
 }  // namespace chdns
 
@@ -1250,8 +1253,7 @@ int env_info(const ch_env_t* env, ch_info_t* info) {
   info->tau_ref = env->tau_ref;
   info->state_bytes = ch_state_bytes(&env->prm);
   info->device_bytes = env->device_bytes;
-  info->plane_cluster = env->prm.precision == 1 ? (env->plane_f.two_pass ? 0 : env->plane_f.S)
-                                               : (env->plane.two_pass ? 0 : env->plane.S);
+  info->plane_cluster = env->prm.precision == 1 ? env->plane_f.cluster : env->plane.cluster;
   info->launches_per_step = env->launches_per_step;
   info->post_batched = env->post_batched ? 1 : 0;
   info->ppc_pre = env->ppc_pre;

@@ -480,10 +480,11 @@ struct PlaneArgs {
   // planes of 16 x 16 modes in batches that fill the GPU: one plane per team
   // of threads, line transforms in registers (plane_small.cu)
   int team16;
-  // planes that fit no cluster's shared memory: three passes through global
-  // memory (z inverse, x transforms and products, z forward)
-  int two_pass;
+  // three passes through global memory (z inverse, x transforms and products,
+  // z forward; plane_pass.cuh)
+  int passes;
   C* y;                // [B][ny][6][mz][nxh] scratch: z-transformed columns, then H in fields 0..2
+  int cluster;         // ch_info_t.plane_cluster
 };
 
 // Per-mode tau tables (device), mode index fastest so that threads owning

@@ -15,11 +15,10 @@ cudaError_t plane_max_clusters(const PlaneArgs<R>& a, size_t smem, int* clusters
 bool plane16_shape(int mx, int mz, int nxh, int nz);
 template <typename R>
 cudaError_t launch_plane16(const PlaneArgs<R>& a, int B, cudaStream_t st);
-// nonlinear term in three passes through global memory (plane2.cu), FP64
-bool two_pass_shape_ok(int mx, int mz, int nxh);
-bool two_pass_chosen(int mx, int mz, int nxh, bool fp64);
+// nonlinear term in three passes through global memory (plane_pass.cu)
+bool passes_built(int mx, int mz);
 template <typename R>
-cudaError_t launch_plane_two_pass(const PlaneArgs<R>& a, int B, cudaStream_t st);
+cudaError_t launch_plane_passes(const PlaneArgs<R>& a, int B, cudaStream_t st);
 
 struct PencilBufs {
   double2 *V, *G;               // [B][ny][P]

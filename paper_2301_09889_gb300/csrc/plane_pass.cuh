@@ -1,0 +1,266 @@
+// Dealiased nonlinear term H = u x omega (3/2 rule; paper Sec. 3.1
+// pseudo-spectral method) in three passes through a global scratch array
+// y[B][ny][6][mz][nxh] that stays in L2 for all but the largest planes:
+//   1. z inverse: the kept kz rows of a (node, field, kx) column -> mz rows;
+//   2. x pass: two physical z rows of a field packed into one complex line,
+//      inverse transform, the three products, forward transform, unpacked over
+//      fields 0..2 of the same rows;
+//   3. z forward: mz rows of H -> the rows |kz| < nz/2, scaled by 1/(mx mz).
+// Every line goes through two register DFTs and one exchange in shared memory
+// (fft_reg.cuh): no index arithmetic or barrier inside a transform, and the
+// padding third of every line costs no operation.
+//
+// What bounds it: FP64 planes by the FP64 pipe.  On GB300 a warp-wide FP64
+// operation holds its sub-partition's pipe for 64 cycles (76 with all four
+// sub-partitions busy: 1.06 TFLOP/s per GPU), whatever its active lanes, so
+// the passes are shaped for the fewest operations with every lane at work:
+// tiles whose task counts are multiples of a warp, small CTAs that even out
+// over the SMs.  FP32 planes by L2 and instruction issue.
+#pragma once
+
+#include "common.cuh"
+#include "fft_reg.cuh"
+#include "internal.h"
+
+namespace chdns {
+
+// z passes: CTAs of W warps on 8 W adjacent columns
+constexpr int kZCols = 8;
+template <typename R> constexpr int z_warps() { return sizeof(R) == 4 ? 2 : 1; }
+
+// x pass: row pairs per CTA (multiples of 8 fill every warp of every phase;
+// fewer where six fields of M points outgrow shared memory) and threads
+template <typename R> constexpr int x_pairs(int m) {
+  return (sizeof(R) == 4 ? m <= 192 : m <= 144) ? 8 : (sizeof(R) == 4 || m <= 192) ? 4 : 2;
+}
+template <typename R> constexpr int x_threads(int m) { return m <= 24 ? 96 : 192; }
+// odd row stride: the transposing accesses of the exchange meet no bank twice
+__host__ __device__ constexpr int x_stride(int m) { return line_a(m) | 1; }
+
+template <typename R, int MZ, int W>
+__global__ void __launch_bounds__(32 * W) zpass_inverse_kernel(PlaneArgs<R> a) {
+  using C = typename cpx<R>::T;
+  constexpr int A = line_a(MZ), B = line_b(MZ), CT = kZCols * W, NT = 32 * W;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* T = reinterpret_cast<C*>(smem_raw);  // [B][A][CT]
+  const int b = blockIdx.y, nxh = a.nxh;
+  if (a.active && !a.active[b]) return;
+  const int cols = a.ny * 6 * nxh, c0 = blockIdx.x * CT;  // column (j, f, i), i fastest
+  pdl_wait_then_release();  // the node values come from stage_pre
+  for (int w = threadIdx.x; w < B * CT; w += NT) {
+    const int c = w % CT, kb = w / CT, g = c0 + c;
+    if (g >= cols) continue;
+    const int i = g % nxh, jf = g / nxh, f = jf % 6, j = jf / 6;
+    const C* src = a.q + (((size_t)b * 6 + f) * a.ny + j) * a.P + i;
+    C x[A];
+#pragma unroll
+    for (int p = 0; p < A / 3; ++p) x[p] = src[(size_t)(B * p + kb) * nxh];
+#pragma unroll
+    for (int p = 2 * A / 3; p < A; ++p) {
+      const int row = B * p + kb - MZ / 3;  // kz = B p + kb - MZ; the row of -nz/2 stays zero
+      x[p] = (p == 2 * A / 3 && kb == 0) ? czero<C>() : src[(size_t)row * nxh];
+    }
+    dft_reg<+1, true, A, R>(x);
+#pragma unroll
+    for (int p = 0; p < A; ++p) T[(kb * A + p) * CT + c] = x[p];
+  }
+  __syncthreads();
+  C* yb = a.y + (size_t)b * a.ny * 6 * MZ * nxh;
+  for (int w = threadIdx.x; w < A * CT; w += NT) {
+    const int c = w % CT, ka = w / CT, g = c0 + c;
+    if (g >= cols) continue;
+    C x[B];
+    x[0] = T[ka * CT + c];
+#pragma unroll
+    for (int s = 1; s < B; ++s) x[s] = cmul(T[(s * A + ka) * CT + c], a.tw_mz[s * ka]);
+    small_dft_ct<+1, B, C, R>(x);
+    C* dst = yb + (size_t)(g / nxh) * MZ * nxh + g % nxh;
+#pragma unroll
+    for (int s = 0; s < B; ++s) dst[(size_t)(ka + A * s) * nxh] = x[s];
+  }
+}
+
+template <typename R, int MX, int NPR, int NT>
+__global__ void __launch_bounds__(NT) xpass_kernel(PlaneArgs<R> a) {
+  using C = typename cpx<R>::T;
+  constexpr int A = line_a(MX), B = line_b(MX), A1 = x_stride(MX), LS = B * A1, NXH = MX / 3;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* X = reinterpret_cast<C*>(smem_raw);  // [6][NPR][B][A1]
+  const int b = blockIdx.y, hz = a.mz / 2;
+  if (a.active && !a.active[b]) return;
+  const int npairs = a.ny * hz, g0 = blockIdx.x * NPR;  // row pair (j, m), m fastest
+  pdl_wait_then_release();
+  C* yb = a.y + (size_t)b * a.ny * 6 * a.mz * NXH;
+  auto rows = [&](int g, int f) { return yb + ((size_t)(g / hz * 6 + f) * a.mz + 2 * (g % hz)) * NXH; };
+  // every read of this CTA's rows happens before the first barrier; the rows
+  // of H are written over fields 0..2 of the same rows at the end
+  for (int w = threadIdx.x; w < 6 * NPR * B; w += NT) {
+    const int kb = w % B, line = w / B, g = g0 + line % NPR;
+    if (g >= npairs) continue;
+    const C* r1 = rows(g, line / NPR);
+    const C* r2 = r1 + NXH;
+    C x[A];
+#pragma unroll
+    for (int p = 0; p < A / 3; ++p) {
+      const C u = r1[B * p + kb], v = r2[B * p + kb];
+      x[p] = (p == 0 && kb == 0) ? mk(u.x, v.x) : mk(u.x - v.y, u.y + v.x);
+    }
+#pragma unroll
+    for (int p = 2 * A / 3; p < A; ++p) {
+      const int k = MX - (B * p + kb);  // Hermitian half; k = nxh (the Nyquist mode) stays zero
+      if (p == 2 * A / 3 && kb == 0) {
+        x[p] = czero<C>();
+      } else {
+        const C u = r1[k], v = r2[k];
+        x[p] = mk(u.x + v.y, v.x - u.y);
+      }
+    }
+    dft_reg<+1, true, A, R>(x);
+#pragma unroll
+    for (int p = 0; p < A; ++p) X[line * LS + kb * A1 + p] = x[p];
+  }
+  __syncthreads();
+  // second half of the inverse lines, products and first half of the forward
+  // lines at the points ka + A kb of one row pair (real parts: first row,
+  // imaginary parts: second row); each thread reads and writes its own slots
+  for (int w = threadIdx.x; w < NPR * A; w += NT) {
+    const int ka = w % A, pp = w / A;
+    if (g0 + pp >= npairs) continue;
+    C t[B];
+#pragma unroll
+    for (int s = 1; s < B; ++s) t[s] = a.tw_x[s * ka];
+    C* slot = X + pp * LS + ka;
+    constexpr int FS = NPR * LS;
+    C v[6][B];
+#pragma unroll
+    for (int f = 0; f < 6; ++f) {
+      v[f][0] = slot[f * FS];
+#pragma unroll
+      for (int s = 1; s < B; ++s) v[f][s] = cmul(slot[f * FS + s * A1], t[s]);
+      small_dft_ct<+1, B, C, R>(v[f]);
+    }
+    C h[3][B];
+#pragma unroll
+    for (int s = 0; s < B; ++s) {
+      const C u = v[0][s], vv = v[1][s], ww = v[2][s], ox = v[3][s], oy = v[4][s], oz = v[5][s];
+      h[0][s] = mk(vv.x * oz.x - ww.x * oy.x, vv.y * oz.y - ww.y * oy.y);
+      h[1][s] = mk(ww.x * ox.x - u.x * oz.x, ww.y * ox.y - u.y * oz.y);
+      h[2][s] = mk(u.x * oy.x - vv.x * ox.x, u.y * oy.y - vv.y * ox.y);
+    }
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      small_dft_ct<-1, B, C, R>(h[f]);
+      slot[f * FS] = h[f][0];
+#pragma unroll
+      for (int s = 1; s < B; ++s) slot[f * FS + s * A1] = cmul(h[f][s], cconj(t[s]));
+    }
+  }
+  __syncthreads();
+  for (int w = threadIdx.x; w < 3 * NPR * B; w += NT) {
+    const int s = w % B, line = w / B;
+    C* slot = X + line * LS + s * A1;
+    C x[A];
+#pragma unroll
+    for (int p = 0; p < A; ++p) x[p] = slot[p];
+    dft_reg<-1, false, A, R>(x);
+#pragma unroll
+    for (int p = 0; p < A; ++p)
+      if (p < A / 3 || p >= 2 * A / 3) slot[p] = x[p];  // k = B p + s
+  }
+  __syncthreads();
+  for (int w = threadIdx.x; w < 3 * NPR * NXH; w += NT) {
+    const int i = w % NXH, line = w / NXH, g = g0 + line % NPR;
+    if (g >= npairs) continue;
+    const int im = i == 0 ? 0 : MX - i;
+    const C zk = X[line * LS + (i % B) * A1 + i / B];
+    const C zm = X[line * LS + (im % B) * A1 + im / B];
+    C* dst = rows(g, line / NPR);
+    dst[i] = mk((zk.x + zm.x) * (R)0.5, (zk.y - zm.y) * (R)0.5);
+    dst[NXH + i] = mk((zk.y + zm.y) * (R)0.5, (zm.x - zk.x) * (R)0.5);
+  }
+}
+
+template <typename R, int MZ, int W>
+__global__ void __launch_bounds__(32 * W) zpass_forward_kernel(PlaneArgs<R> a) {
+  using C = typename cpx<R>::T;
+  constexpr int A = line_a(MZ), B = line_b(MZ), CT = kZCols * W, NT = 32 * W;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* T = reinterpret_cast<C*>(smem_raw);  // [B][A][CT]
+  const int b = blockIdx.y, nxh = a.nxh;
+  if (a.active && !a.active[b]) return;
+  const int cols = a.ny * 3 * nxh, c0 = blockIdx.x * CT;  // column (j, f, i), i fastest
+  pdl_wait_then_release();
+  const C* yb = a.y + (size_t)b * a.ny * 6 * MZ * nxh;
+  for (int w = threadIdx.x; w < A * CT; w += NT) {
+    const int c = w % CT, ka = w / CT, g = c0 + c;
+    if (g >= cols) continue;
+    const int jf = g / nxh;
+    const C* src = yb + (size_t)(jf / 3 * 6 + jf % 3) * MZ * nxh + g % nxh;
+    C x[B];
+#pragma unroll
+    for (int s = 0; s < B; ++s) x[s] = src[(size_t)(ka + A * s) * nxh];
+    small_dft_ct<-1, B, C, R>(x);
+    T[ka * CT + c] = x[0];
+#pragma unroll
+    for (int s = 1; s < B; ++s) T[(s * A + ka) * CT + c] = cmul(x[s], cconj(a.tw_mz[s * ka]));
+  }
+  __syncthreads();
+  for (int w = threadIdx.x; w < B * CT; w += NT) {
+    const int c = w % CT, s = w / CT, g = c0 + c;
+    if (g >= cols) continue;
+    const int i = g % nxh, jf = g / nxh, f = jf % 3, j = jf / 3;
+    C x[A];
+#pragma unroll
+    for (int p = 0; p < A; ++p) x[p] = T[(s * A + p) * CT + c];
+    dft_reg<-1, false, A, R>(x);
+    C* dst = a.h + (((size_t)b * 3 + f) * a.ny + j) * a.P + i;
+#pragma unroll
+    for (int p = 0; p < A / 3; ++p) dst[(size_t)(B * p + s) * nxh] = a.scale * x[p];
+#pragma unroll
+    for (int p = 2 * A / 3; p < A; ++p) {
+      const int row = B * p + s - MZ / 3;
+      dst[(size_t)row * nxh] = (p == 2 * A / 3 && s == 0) ? czero<C>() : a.scale * x[p];
+    }
+  }
+}
+
+template <typename R, int MZ>
+cudaError_t zpass_inverse_m(const PlaneArgs<R>& a, int B, cudaStream_t st) {
+  constexpr int W = z_warps<R>(), CT = kZCols * W;
+  constexpr size_t smem = (size_t)MZ * CT * sizeof(typename cpx<R>::T);
+  static SmemLimit lim;
+  const cudaError_t e = raise_smem_limit(zpass_inverse_kernel<R, MZ, W>, &lim, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl_if<sizeof(R) == 4>(zpass_inverse_kernel<R, MZ, W>, dim3((a.ny * 6 * a.nxh + CT - 1) / CT, B),
+                                       dim3(32 * W), smem, st, a);
+}
+template <typename R, int MZ>
+cudaError_t zpass_forward_m(const PlaneArgs<R>& a, int B, cudaStream_t st) {
+  constexpr int W = z_warps<R>(), CT = kZCols * W;
+  constexpr size_t smem = (size_t)MZ * CT * sizeof(typename cpx<R>::T);
+  static SmemLimit lim;
+  const cudaError_t e = raise_smem_limit(zpass_forward_kernel<R, MZ, W>, &lim, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl_if<sizeof(R) == 4>(zpass_forward_kernel<R, MZ, W>, dim3((a.ny * 3 * a.nxh + CT - 1) / CT, B),
+                                       dim3(32 * W), smem, st, a);
+}
+template <typename R, int MX>
+cudaError_t xpass_m(const PlaneArgs<R>& a, int B, cudaStream_t st) {
+  constexpr int NPR = x_pairs<R>(MX), NT = x_threads<R>(MX);
+  constexpr size_t smem = (size_t)6 * NPR * line_b(MX) * x_stride(MX) * sizeof(typename cpx<R>::T);
+  static SmemLimit lim;
+  const cudaError_t e = raise_smem_limit(xpass_kernel<R, MX, NPR, NT>, &lim, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl_if<sizeof(R) == 4>(xpass_kernel<R, MX, NPR, NT>, dim3((a.ny * (a.mz / 2) + NPR - 1) / NPR, B),
+                                       dim3(NT), smem, st, a);
+}
+
+}  // namespace chdns
+
+// explicit instantiations of the three passes for one padded length
+#define CH_PASS_INSTANTIATE(R, M)                                                      \
+  namespace chdns {                                                                    \
+  template cudaError_t zpass_inverse_m<R, M>(const PlaneArgs<R>&, int, cudaStream_t);  \
+  template cudaError_t zpass_forward_m<R, M>(const PlaneArgs<R>&, int, cudaStream_t);  \
+  template cudaError_t xpass_m<R, M>(const PlaneArgs<R>&, int, cudaStream_t);          \
+  }
