@@ -412,22 +412,27 @@ int build_tables(ch_env* env) {
     for (int n = 0; n < ny; ++n) cheb[(size_t)j * ny + n] = std::cos(M_PI * (double)((j * n) % (2 * N)) / N);
 
   // tau tables, mode index fastest: [stage][parity][e, h, b, Q][Mh][P]
-  std::vector<double> helm((size_t)3 * 2 * 4 * Mh * P, 0.0), helm_isq((size_t)3 * 2 * P, 0.0);
-  std::vector<double> pois((size_t)2 * 4 * Mh * P, 0.0), pois_isq((size_t)2 * P, 0.0);
+  // (e, h, b, Q: the scan solves of the no-slip top)
+  const bool top = p.top_bc == 1;
+  std::vector<double> helm(top ? 0 : (size_t)3 * 2 * 4 * Mh * P, 0.0), helm_isq((size_t)3 * 2 * P, 0.0);
+  std::vector<double> pois(top ? 0 : (size_t)2 * 4 * Mh * P, 0.0), pois_isq((size_t)2 * P, 0.0);
   std::vector<double> vh((size_t)3 * 2 * Mh * P, 0.0), vh_idv((size_t)3 * 2 * P, 0.0);
   std::vector<double> u1((size_t)3 * Mh, 0.0), u1_iflux(3, 0.0);
   // free-slip top: sum Q, sum n^2 Q per parity; A, B of vh per parity
   std::vector<double> helm_top((size_t)3 * 2 * 2 * P, 0.0), vh_top((size_t)3 * 2 * 2 * P, 0.0);
-  const bool top = p.top_bc == 1;
-  // no-slip top: the folded tables of the per-thread solves, [..][eA, eB, eC, h, b, W (, E1)][Mh][P];
-  // e1 > 0 adds E1 = e1 e (the Helmholtz tables, e1 = 1 + alpha/beta of the stage)
-  std::vector<double> helm_f(top ? 0 : (size_t)3 * 2 * 7 * Mh * P, 0.0);
-  std::vector<double> pois_f(top ? 0 : (size_t)2 * 6 * Mh * P, 0.0);
+  std::vector<double> mean_top((size_t)3 * 4, 0.0);
+  // the folded tables of the per-thread solves, [..][eA, eB, eC, h, b, W (, E1 (, W2))][Mh][P];
+  // e1 > 0 adds E1 = e1 e (the Helmholtz tables, e1 = 1 + alpha/beta of the
+  // stage) and under a free-slip top the weights W2 of sum n^2 P
+  const int htabs = top ? 8 : 7;
+  std::vector<double> helm_f((size_t)3 * 2 * htabs * Mh * P, 0.0);
+  std::vector<double> pois_f((size_t)2 * 6 * Mh * P, 0.0);
   auto put_f = [&](std::vector<double>& tab, size_t base, const Factor& F, int M, int pp, int sig, double e1) {
-    double w = 1.0;  // W_{M-1}
+    double w = 1.0, w2 = 0.0;  // W_{M-1}
     for (int i = M - 1; i >= 1; --i) {
       const int n = 2 * i + sig;
       if (i < M - 1) w = 1.0 + F.b[i + 1] * w;
+      w2 = (double)n * n + (i < M - 1 ? F.b[i + 1] * w2 : 0.0);
       tab[base + ((size_t)0 * Mh + i) * P + pp] = F.e[i] * cA(n);
       tab[base + ((size_t)1 * Mh + i) * P + pp] = F.e[i] * cB(n, N);
       tab[base + ((size_t)2 * Mh + i) * P + pp] = F.e[i] * cC(n, N);
@@ -435,6 +440,7 @@ int build_tables(ch_env* env) {
       tab[base + ((size_t)4 * Mh + i) * P + pp] = F.b[i];
       tab[base + ((size_t)5 * Mh + i) * P + pp] = w;
       if (e1 > 0.0) tab[base + ((size_t)6 * Mh + i) * P + pp] = e1 * F.e[i];
+      if (e1 > 0.0 && top) tab[base + ((size_t)7 * Mh + i) * P + pp] = w2;
     }
   };
   auto put = [&](std::vector<double>& tab, size_t base, const Factor& F, int M, int pp) {
@@ -451,8 +457,8 @@ int build_tables(ch_env* env) {
     for (int sig = 0; sig < 2; ++sig) {
       const int M = (N - sig) / 2 + 1;
       const Factor Fp = host_factor(N, sig, k2);
-      put(pois, (size_t)sig * 4 * Mh * P, Fp, M, pp);
-      if (!top) put_f(pois_f, (size_t)sig * 6 * Mh * P, Fp, M, pp, sig, 0.0);
+      if (!top) put(pois, (size_t)sig * 4 * Mh * P, Fp, M, pp);
+      put_f(pois_f, (size_t)sig * 6 * Mh * P, Fp, M, pp, sig, 0.0);
       pois_isq[(size_t)sig * P + pp] = Fp.isq;
       for (int k = 0; k < 3; ++k) {
         const double ibdn = 1.0 / (rk_beta(k) * p.dt * env->nu);
@@ -463,8 +469,8 @@ int build_tables(ch_env* env) {
         // it in the elimination factor e and the kernels leave it out
         Factor Fs = Fh;
         for (double& e : Fs.e) e *= -ibdn;
-        put(helm, slot * 4 * Mh * P, Fs, M, pp);
-        if (!top) put_f(helm_f, slot * 7 * Mh * P, Fs, M, pp, sig, 1.0 + rk_alpha(k) / rk_beta(k));
+        if (!top) put(helm, slot * 4 * Mh * P, Fs, M, pp);
+        put_f(helm_f, slot * htabs * Mh * P, Fs, M, pp, sig, 1.0 + rk_alpha(k) / rk_beta(k));
         helm_isq[slot * P + pp] = Fh.isq;
         {
           double sq = 0.0, sq2 = 0.0;
@@ -513,6 +519,13 @@ int build_tables(ch_env* env) {
       flux += 2.0 / (1.0 - (double)n * n) * v;
     }
     u1_iflux[k] = top ? 0.0 : 1.0 / flux;
+    for (int i = 0; i < M; ++i) {
+      const double n = 2 * i, w = 2.0 / (1.0 - n * n), u = u1[(size_t)k * Mh + i];
+      mean_top[4 * k + 0] += w * F.Q[i];
+      mean_top[4 * k + 1] += u;
+      mean_top[4 * k + 2] += n * n * u;
+      mean_top[4 * k + 3] += w * u;
+    }
   }
   // tau row constants per n
   std::vector<double> rowc((size_t)3 * ny, 0.0);
@@ -544,10 +557,18 @@ int build_tables(ch_env* env) {
   RC(dupload(env, &env->tab.tau.helm_isq, helm_isq));
   RC(dupload(env, &env->tab.tau.pois, pois));
   RC(dupload(env, &env->tab.tau.pois_isq, pois_isq));
-  if (!top) {
-    RC(dupload(env, &env->tab.tau.helm_f, helm_f));
-    RC(dupload(env, &env->tab.tau.pois_f, pois_f));
+  RC(dupload(env, &env->tab.tau.helm_f, helm_f));
+  RC(dupload(env, &env->tab.tau.pois_f, pois_f));
+  {
+    std::vector<double> n2(ny), wint(ny, 0.0);
+    for (int n = 0; n < ny; ++n) {
+      n2[n] = (double)n * n;
+      if (n % 2 == 0) wint[n] = 2.0 / (1.0 - (double)n * n);
+    }
+    RC(dupload(env, &env->tab.tau.n2, n2));
+    RC(dupload(env, &env->tab.tau.wint, wint));
   }
+  RC(dupload(env, &env->tab.tau.mean_top, mean_top));
   RC(dupload(env, &env->tab.tau.vh, vh));
   RC(dupload(env, &env->tab.tau.vh_idv, vh_idv));
   RC(dupload(env, &env->tab.tau.u1, u1));
@@ -737,7 +758,7 @@ int run_stage(ch_env* env, int k, double theta) {
   }
   const StageCoef sc = stage_coef(env, k, theta);
   if (mixed)
-    LAUNCH(2, launch_stage_post<float>(g, B, env->pb, env->tab, reinterpret_cast<const float2*>(env->pb.R), sc,
+    LAUNCH(2, launch_stage_post<float>(g, B, env->pb, env->tab, reinterpret_cast<float2*>(env->pb.R), sc,
                                        env->ppc_post, env->post_batched, st));
   else
     LAUNCH(2, launch_stage_post<double>(g, B, env->pb, env->tab, env->pb.R, sc, env->ppc_post, env->post_batched,
@@ -752,7 +773,7 @@ int run_stage(ch_env* env, int k, double theta) {
 static void set_launch_count(ch_env* env) {
   const ch_params_t* p = &env->prm;
   const bool passes = p->precision == 1 ? env->plane_f.passes : env->plane.passes;
-  const int stage = 1 + (passes ? 3 : 1) + stage_post_launches(env->g, p->top_bc, env->post_batched);
+  const int stage = 1 + (passes ? 3 : 1) + stage_post_launches(p->top_bc, env->post_batched);
   env->launches_per_step = (p->control == 0 ? 2 : p->control == 1 ? 1 : 5) + p->steps_per_action * (3 * stage + 1) + 3;
 }
 
@@ -826,12 +847,11 @@ bool tiles_valid(const ch_env* env, int smem_max, int ppc_pre, int ppc_post, int
   const size_t node = env->prm.precision == 1 ? sizeof(float2) : sizeof(double2);
   auto pow2 = [](int v, int hi) { return v >= 1 && v <= hi && (v & (v - 1)) == 0; };
   if (!pow2(ppc_pre, 8) || stage_pre_smem(g, ppc_pre, node) > (size_t)smem_max) return false;
-  const int top = env->prm.top_bc;
-  if (post_batched == 1) return pow2(ppc_post, 16) && stage_post_batched_smem(g, ppc_post, top, node) <= (size_t)smem_max;
+  if (post_batched == 1) return pow2(ppc_post, 16);
   if (post_batched != 0) return false;
   // the per-tile form runs 8 ppc threads and any tile width up to 8 (widths
   // that are not powers of two fill the resident CTA slots more evenly)
-  return ppc_post >= 1 && ppc_post <= 8 && stage_post_smem(g, env->tab.tau.Mh, ppc_post, top) <= (size_t)smem_max;
+  return ppc_post >= 1 && ppc_post <= 8 && stage_post_smem(g, env->tab.tau.Mh, ppc_post) <= (size_t)smem_max;
 }
 
 int drop_graphs(ch_env* env) {
@@ -900,7 +920,7 @@ int autotune_tiles(ch_env* env, int smem_max) {
   };
   auto post = [&](int ppc, bool batched) {
     const cudaError_t e =
-        mixed ? launch_stage_post<float>(g, B, pb, env->tab, reinterpret_cast<const float2*>(pb.R), sc, ppc, batched, st)
+        mixed ? launch_stage_post<float>(g, B, pb, env->tab, reinterpret_cast<float2*>(pb.R), sc, ppc, batched, st)
               : launch_stage_post<double>(g, B, pb, env->tab, pb.R, sc, ppc, batched, st);
     return e == cudaSuccess ? CH_OK : CH_ERR_CUDA;
   };
@@ -908,6 +928,7 @@ int autotune_tiles(ch_env* env, int smem_max) {
   float best = 0.f;
   bool have = false;
   for (int ppc : {8, 4, 2}) {
+    if (!stage_pre_tiled(g)) break;  // register transforms: one shape
     if (!tiles_valid(env, smem_max, ppc, env->ppc_post, env->post_batched ? 1 : 0)) continue;
     float ms = 0.f;
     RC(time_launches(st, kReps, [&] { return pre(ppc); }, &ms));
@@ -921,16 +942,14 @@ int autotune_tiles(ch_env* env, int smem_max) {
   // widths of the form the size rule chose: the per-tile and batched forms of
   // the no-slip solves sum in different orders (four-lane scans against one
   // thread per system), so timing never switches between them
-  const int form = env->post_batched ? 1 : 0;
-  const std::pair<int, int> cands[] = {{0, 8}, {0, 7}, {0, 6}, {0, 5}, {0, 4}, {0, 3}, {0, 2}, {0, 1}, {1, 16}, {1, 8}};
-  for (const auto& c : cands) {
-    if (c.first != form || !tiles_valid(env, smem_max, env->ppc_pre, c.second, c.first)) continue;
+  for (int ppc = 8; ppc >= 1; --ppc) {
+    if (env->post_batched || env->prm.top_bc) break;  // the two-launch form has one shape
+    if (!tiles_valid(env, smem_max, env->ppc_pre, ppc, 0)) continue;
     float ms = 0.f;
-    RC(time_launches(st, kReps, [&] { return post(c.second, c.first == 1); }, &ms));
+    RC(time_launches(st, kReps, [&] { return post(ppc, false); }, &ms));
     if (!have || ms < best) {
       best = ms;
-      env->post_batched = c.first == 1;
-      env->ppc_post = c.second;
+      env->ppc_post = ppc;
       have = true;
     }
   }
@@ -999,8 +1018,9 @@ size_t env_footprint(const ch_params_t* p) {
   const size_t nxh = p->nx / 2, P = nxh * p->nz, ny = p->ny, Mh = (ny - 1) / 2 + 1;
   const size_t state = B * (4 * ny * P * 16 + 4 * ny * 8 + 9 * ny * P * 16 + 3 * P * 16 + 8 +
                             (size_t)p->nz * p->nx * 8 + (2 * (size_t)p->nz * p->nx + 2) * 8);
-  const size_t folded = p->top_bc == 0 ? (3 * 2 * 7 * Mh * P + 2 * 6 * Mh * P) * 8 : 0;
-  const size_t tables = (3 * 2 * 4 * Mh * P + 3 * 2 * P + 2 * 4 * Mh * P + 2 * P + 3 * 2 * Mh * P + 3 * 2 * P +
+  const size_t folded = (3 * 2 * (p->top_bc ? 8 : 7) * Mh * P + 2 * 6 * Mh * P) * 8;
+  const size_t scan = p->top_bc ? 0 : (3 * 2 * 4 + 2 * 4) * Mh * P;
+  const size_t tables = (scan + 3 * 2 * P + 2 * P + 3 * 2 * Mh * P + 3 * 2 * P +
                          3 * Mh + 3 + 3 * ny + ny + 2 * 3 * 2 * 2 * P) * 8 + ny * ny * 12 + (nxh + p->nz) * 8 +
                         folded;
   // the scratch of the three-pass nonlinear term, where it runs in passes
@@ -1101,21 +1121,19 @@ int env_create(const ch_params_t* p, ch_env_t** out) {
     env->ppc_post = 8;
     while (env->ppc_post > 1 && ((size_t)B * P + env->ppc_post - 1) / env->ppc_post < (size_t)nsm)
       env->ppc_post /= 2;
-    while (env->ppc_post > 1 && stage_post_smem(g, env->tab.tau.Mh, env->ppc_post, p->top_bc) > (size_t)smem_max)
+    while (env->ppc_post > 1 && stage_post_smem(g, env->tab.tau.Mh, env->ppc_post) > (size_t)smem_max)
       env->ppc_post /= 2;
     env->ppc_pre = 8;
     while (env->ppc_pre > 1 && stage_pre_smem(g, env->ppc_pre, sizeof(double2)) > (size_t)smem_max) env->ppc_pre /= 2;
-    if (stage_post_smem(g, env->tab.tau.Mh, env->ppc_post, p->top_bc) > (size_t)smem_max) return fail(CH_ERR_UNSUPPORTED);
+    if (stage_post_smem(g, env->tab.tau.Mh, env->ppc_post) > (size_t)smem_max) return fail(CH_ERR_UNSUPPORTED);
     // The batched form of stage_post runs four threads per mode, each with
     // the same work; it pays once the batch supplies at least two such warps
     // per SM sub-partition (B P / 8 >= 2 x 4 x SMs).
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return fail(CH_ERR_CUDA);
-    const size_t node = p->precision == 1 ? sizeof(float2) : sizeof(double2);
-    if ((size_t)B * P >= (size_t)64 * sms && stage_post_batched_smem(g, 8, p->top_bc, node) <= (size_t)smem_max) {
+    if ((size_t)B * P >= (size_t)64 * sms) {
       env->post_batched = true;
-      env->ppc_post = 16;  // 64 threads; 8 when the tile would leave fewer than 3 CTAs per SM
-      if (stage_post_batched_smem(g, 16, p->top_bc, node) > (size_t)76 * 1024) env->ppc_post = 8;
+      env->ppc_post = 16;
     }
     if (p->autotune && (rc = autotune_tiles(env, smem_max))) return fail(rc);
   }

@@ -499,30 +499,22 @@ struct TauTables {
   const double* u1;        // [3][Mh]           mean response to unit forcing (even parity)
   const double* u1_iflux;  // [3]               1 / int u1 dy
   const double* rowc;      // [3][ny]           tau row constants cA_n, cB_n, cC_n
-  // no-slip top (top_bc = 0): the same factorisations with the row constants
-  // folded in, eA = e cA_n, eB = e cB_n, eC = e cC_n, then h, b, the wall
-  // weights W (W_{M-1} = 1, W_i = 1 + b_{i+1} W_{i+1}: sum_i P_i = sum_i W_i a_i)
-  // and, for the stage's Helmholtz operator, E1 = (1 + alpha/beta) e
-  const double* helm_f;    // [3][2][7][Mh][P]  eA, eB, eC, h, b, W, E1 per stage, parity
+  // the same factorisations with the row constants folded in, eA = e cA_n,
+  // eB = e cB_n, eC = e cC_n, then h, b, the wall weights W (W_{M-1} = 1,
+  // W_i = 1 + b_{i+1} W_{i+1}: sum_i P_i = sum_i W_i a_i) and, for the stage's
+  // Helmholtz operator, E1 = (1 + alpha/beta) e and under a free-slip top W2
+  // (W2_{M-1} = n^2, W2_i = n_i^2 + b_{i+1} W2_{i+1}: sum n^2 P = sum W2_i a_i)
+  const double* helm_f;    // [3][2][7 or 8][Mh][P] eA, eB, eC, h, b, W, E1 (, W2) per stage, parity
   const double* pois_f;    // [2][6][Mh][P]     eA, eB, eC, h, b, W
+  const double* n2;        // [ny] n^2
+  const double* wint;      // [ny] int T_n dy = 2 / (1 - n^2) of the even n, 0 of the odd
   // free-slip top (top_bc = 1): the wall rows couple the parities
   const double* helm_top;  // [3][2][2][P]      sum Q, sum n^2 Q of the stage's factorisation, per parity
   const double* vh_top;    // [3][2][2][P]      A = sum n^2 (n^2 - 1) / 3 vh_n, B = sum n^2 vh_n, per parity
+  const double* mean_top;  // [3][4]            mean mode: int Q_e; sum, sum n^2 and int of u1
   int Mh;
   int top_bc;              // 0 no-slip upper wall; 1 free slip (u1 then holds the affine forcing response)
 };
-
-// Shared memory of the batched implicit half before its exchange slots: the
-// tile of H, [3][ny][ppc] complex in the node precision, then for FP32 nodes
-// the staged previous right-hand sides [2][ny][ppc] (FP32 pairs), for FP64
-// nodes six more complex values per mode (scratch of the fast analysis);
-// 16-byte aligned.
-constexpr bool kPostStageHV = true, kPostStageHG = true;
-__host__ __device__ inline size_t stage_post_batched_tile_bytes(int ny, int ppc, size_t node_bytes) {
-  const size_t staged = (size_t)kPostStageHV + (size_t)kPostStageHG;
-  const size_t b = node_bytes == 8 ? (3 + staged) * ny * ppc * 8 : ((size_t)3 * ny + 6) * ppc * 16;
-  return (b + 15) & ~(size_t)15;
-}
 
 struct StageCoef {
   double alpha, beta, gamma, zeta, dt, nu, theta, flux;

@@ -46,19 +46,20 @@ struct DevTables {
 
 // fused wall-normal halves of a stage (stage.cu); ppc = modes per CTA
 size_t stage_pre_smem(const Grid& g, int ppc, size_t node_bytes);  // node_bytes: one complex node value
-size_t stage_post_smem(const Grid& g, int Mh, int ppc, int top);
-size_t stage_post_batched_smem(const Grid& g, int ppc, int top, size_t node_bytes);
-// kernels one launch_stage_post issues (the batched form above 65 nodes: two)
-int stage_post_launches(const Grid& g, int top, bool batched);
+size_t stage_post_smem(const Grid& g, int Mh, int ppc);
+// the explicit half works on tiles of ppc modes (false: register cosine transforms)
+bool stage_pre_tiled(const Grid& g);
+// kernels one launch_stage_post issues
+int stage_post_launches(int top, bool batched);
 template <typename RN>
 cudaError_t launch_stage_pre(const Grid& g, int B, const PencilBufs& pb, const DevTables& t,
                              typename cpx<RN>::T* q, int ppc, cudaStream_t st);
-// batched: one thread per (mode, class, component) and only H staged in shared
-// memory (for batches that supply many modes); otherwise one thread per
-// (mode, class, component, equation) on a shared-memory tile
+// batched (and every handle under a free-slip top): the analysis of H over its
+// nodal values h in place, then one thread per (mode, class, component,
+// equation); otherwise four lanes per system on a shared-memory tile of ppc modes
 template <typename RN>
 cudaError_t launch_stage_post(const Grid& g, int B, const PencilBufs& pb, const DevTables& t,
-                              const typename cpx<RN>::T* h, const StageCoef& sc, int ppc, bool batched,
+                              typename cpx<RN>::T* h, const StageCoef& sc, int ppc, bool batched,
                               cudaStream_t st);
 cudaError_t launch_wall_shear(const Grid& g, int B, const double* UM, double nu, double* acc,
                               const int* active, cudaStream_t st);

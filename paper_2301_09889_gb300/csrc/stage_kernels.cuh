@@ -57,756 +57,6 @@ struct TabSm {
   __device__ double Q(int i) const { return base[(3 * Mh + i) * ppc]; }
 };
 
-// folded tau tables of one (mode, parity) of a no-slip solve: element (f, i)
-// at base[(f * Mh + i) * ppc], f = eA, eB, eC, h, b, W, and for the stage's
-// Helmholtz operator E1 = (1 + alpha/beta) e
-struct TabF {
-  const double* base;
-  int Mh, ppc;
-  __device__ double eA(int i) const { return base[(0 * Mh + i) * ppc]; }
-  __device__ double eB(int i) const { return base[(1 * Mh + i) * ppc]; }
-  __device__ double eC(int i) const { return base[(2 * Mh + i) * ppc]; }
-  __device__ double h(int i) const { return base[(3 * Mh + i) * ppc]; }
-  __device__ double b(int i) const { return base[(4 * Mh + i) * ppc]; }
-  __device__ double W(int i) const { return base[(5 * Mh + i) * ppc]; }
-  __device__ double E1(int i) const { return base[(6 * Mh + i) * ppc]; }  // Helmholtz tables only
-};
-// a right-hand side value r and the operand x of a diagonal term E1_j x_j
-struct RhsX {
-  double r, x;
-};
-
-// ---------------------------------------------------------------------------
-// Chebyshev-tau Dirichlet solve (D^2 - lam) f = r of one parity of one real
-// component.  For n >= 2 the tau rows are equivalent to the quasi-tridiagonal
-// rows
-//   -lam cA_n f_{n-2} + (1 + lam cB_n) f_n - lam cC_n f_{n+2}
-//       = cA_n r_{n-2} - cB_n r_n + cC_n r_{n+2},
-//   cA_n = c_{n-2}/(4n(n-1)), cB_n = [n <= N-2]/(2(n^2-1)), cC_n = [n+2 <= N-2]/(4n(n+1)),
-// obtained by integrating D^2 f = r + lam f twice; the two highest rows of r
-// are dropped (tau).  With parity index i the rows i >= 1 are tridiagonal and
-// the wall row sum_i f_i = s closes the system.  Bottom-up elimination gives
-// f_i = a_i + b_i f_{i-1}; every f_i is then affine in f_0, which the wall row
-// fixes.  The lam-dependent factors e = 1/den, h = U/den, b = -L/den, Q = prod b
-// and 1/sum Q are precomputed per mode and stage.  rowc = [cA | cB | cC].
-// ---------------------------------------------------------------------------
-template <int MH, class Tab>
-__device__ __forceinline__ void tau_seq(int N, int ny, int sig, const double (&r)[MH], double (&f)[MH],
-                                        const Tab& T, double isq, double s, const double* __restrict__ rowc) {
-  const int M = (N - sig) / 2 + 1;
-  double anext = 0.0;
-#pragma unroll
-  for (int i = MH - 1; i >= 1; --i) {
-    if (i < M) {
-      const int n = 2 * i + sig;
-      double R = fma_rn(-rowc[ny + n], r[i], mul_rn(rowc[n], r[i - 1]));
-      if (i + 1 < MH && i + 1 < M) R = fma_rn(rowc[2 * ny + n], r[i + 1 < MH ? i + 1 : i], R);
-      const double a = fma_rn(-T.h(i), anext, mul_rn(T.e(i), R));
-      f[i] = a;
-      anext = a;
-    }
-  }
-  double Pp = 0.0, sum = 0.0;
-#pragma unroll
-  for (int i = 1; i < MH; ++i) {
-    if (i < M) {
-      Pp = fma_rn(T.b(i), Pp, f[i]);
-      f[i] = Pp;
-      sum += Pp;
-    }
-  }
-  const double f0 = mul_rn(isq, s - sum);
-  f[0] = f0;
-#pragma unroll
-  for (int i = 1; i < MH; ++i)
-    if (i < M) f[i] = fma_rn(T.Q(i), f0, f[i]);
-}
-
-// symmetry class of a solve compiled for one class (a constant) or for both
-template <int V>
-__device__ __forceinline__ constexpr int class_of(std::integral_constant<int, V>) { return V; }
-__device__ __forceinline__ int class_of(int v) { return v; }
-
-// ---------------------------------------------------------------------------
-// Free-slip top (open channel, top_bc = 1; paper Sec. 3.1).  The tau rows
-// n >= 2 are those of the no-slip channel, so elimination still leaves each
-// parity affine in its lowest coefficient, f = P + x Q (P_0 = 0, Q_0 = 1, Q
-// the precomputed products of b); only the wall rows change, and they couple
-// the two parities, which live in the two class threads of a mode:
-//   omega_y, W:  f(-1) = S_e - S_o,  Df(+1) = S2_e + S2_o
-//                (S = sum over the parity of f_n, S2 = sum of n^2 f_n);
-//   U:           the same two rows and the flow rate, with the response to
-//                the unknown forcing (even parity);
-//   v:           v(+-1) stay Dirichlet per parity; phi = P + c vh per parity,
-//                and D^2 v(+1) = A_e + A_o, Dv(-1) = -B_e + B_o
-//                (A = sum n^2 (n^2 - 1) / 3 v_n, B = sum n^2 v_n) fix c_e, c_o.
-// With the shifted unknowns f' = f + cc f_old every row's value is cc times
-// that row applied to the old field.  Each thread of a pair publishes the
-// sums of its parity; after a barrier both solve the same closure, summing
-// in parity order, so both find the same coefficients.
-// ---------------------------------------------------------------------------
-
-// The affine family of one parity: f_i = P_i (i >= 1), f_0 = 0, with
-// sp = sum P and sp2 = sum n^2 P (the same elimination as tau_seq).
-template <int MH, class Tab>
-__device__ __forceinline__ void tau_affine(int N, int ny, int sig, const double (&r)[MH], double (&f)[MH],
-                                           const Tab& T, const double* __restrict__ rowc, double& sp, double& sp2) {
-  const int M = (N - sig) / 2 + 1;
-  double anext = 0.0;
-#pragma unroll
-  for (int i = MH - 1; i >= 1; --i) {
-    if (i < M) {
-      const int n = 2 * i + sig;
-      double R = fma_rn(-rowc[ny + n], r[i], mul_rn(rowc[n], r[i - 1]));
-      if (i + 1 < MH && i + 1 < M) R = fma_rn(rowc[2 * ny + n], r[i + 1 < MH ? i + 1 : i], R);
-      const double a = fma_rn(-T.h(i), anext, mul_rn(T.e(i), R));
-      f[i] = a;
-      anext = a;
-    }
-  }
-  double Pp = 0.0;
-  sp = 0.0;
-  sp2 = 0.0;
-#pragma unroll
-  for (int i = 1; i < MH; ++i) {
-    if (i < M) {
-      const double n = 2 * i + sig;
-      Pp = fma_rn(T.b(i), Pp, f[i]);
-      f[i] = Pp;
-      sp += Pp;
-      sp2 = fma_rn(n * n, Pp, sp2);
-    }
-  }
-  f[0] = 0.0;
-}
-
-// f = P + x Q
-template <int MH, class Arr, class Tab>
-__device__ __forceinline__ void tau_close(int N, int sig, Arr& f, const Tab& T, double x) {
-  const int M = (N - sig) / 2 + 1;
-  f[0] = x;
-#pragma unroll
-  for (int i = 1; i < MH; ++i)
-    if (i < M) f[i] = fma_rn(T.Q(i), x, f[i]);
-}
-
-// a11 x1 + a12 x2 = b1, a21 x1 + a22 x2 = b2 (Cramer's rule)
-__device__ __forceinline__ void solve2(double a11, double a12, double a21, double a22, double b1, double b2,
-                                       double* x1, double* x2) {
-  const double id = 1.0 / fma_rn(a11, a22, -mul_rn(a12, a21));
-  *x1 = mul_rn(fma_rn(b1, a22, -mul_rn(a12, b2)), id);
-  *x2 = mul_rn(fma_rn(a11, b2, -mul_rn(a21, b1)), id);
-}
-
-// Dirichlet bottom and Neumann top rows over the two parities of omega_y or W.
-// se, so: {sum P, sum n^2 P, sum f_old, sum n^2 f_old} of the even and odd
-// parity; q*: the table sums sum Q and sum n^2 Q.
-__device__ __forceinline__ void close_neumann_top(const double* se, const double* so, double qe, double qo,
-                                                  double q2e, double q2o, double cc, double* xe, double* xo) {
-  solve2(qe, -qo, q2e, q2o, fma_rn(cc, se[2] - so[2], -(se[0] - so[0])), fma_rn(cc, se[3] + so[3], -(se[1] + so[1])),
-         xe, xo);
-}
-
-// Influence coefficients of v: se, so = {A_p, B_p, A_old, B_old}; a*, b*: A
-// and B of the homogeneous solutions vh of the two parities.
-__device__ __forceinline__ void close_free_slip_v(const double* se, const double* so, double ae, double ao,
-                                                  double be, double bo, double cc, double* ce, double* co) {
-  solve2(ae, ao, -be, bo, fma_rn(cc, se[2] + so[2], -(se[0] + so[0])), fma_rn(cc, so[3] - se[3], -(so[1] - se[1])),
-         ce, co);
-}
-
-// Mean U at constant flow rate: unknowns (x_e, x_o, forcing).  se = {sum P,
-// sum n^2 P, sum U_old, sum n^2 U_old, int P, int U_old}, so = the first four
-// of the odd parity; q*: sum Q, sum n^2 Q; wq: int Q_e; u*: sum, sum n^2 and
-// int of the forcing response (even).  int = sum of 2 / (1 - n^2) x_n.
-__device__ __forceinline__ void close_free_slip_mean(const double* se, const double* so, double qe, double qo,
-                                                     double q2e, double q2o, double wq, double us, double u2,
-                                                     double uw, double cc, double flux, double* xe, double* xo,
-                                                     double* fc) {
-  const double a11 = qe, a12 = -qo, a13 = us;
-  const double a21 = q2e, a22 = q2o, a23 = u2;
-  const double a31 = wq, a32 = 0.0, a33 = uw;
-  const double b1 = fma_rn(cc, se[2] - so[2], -(se[0] - so[0]));
-  const double b2 = fma_rn(cc, se[3] + so[3], -(se[1] + so[1]));
-  const double b3 = fma_rn(cc, se[5], flux) - se[4];
-  // 2 x 2 minors (x y - z w, fused on the first product)
-  auto det2 = [](double x, double y, double z, double w) { return fma_rn(x, y, -mul_rn(z, w)); };
-  const double m1 = det2(a22, a33, a23, a32), m2 = det2(a21, a33, a23, a31), m3 = det2(a21, a32, a22, a31);
-  const double id = 1.0 / fma_rn(a13, m3, fma_rn(a11, m1, -mul_rn(a12, m2)));
-  *xe = mul_rn(fma_rn(a13, det2(b2, a32, a22, b3), fma_rn(b1, m1, -mul_rn(a12, det2(b2, a33, a23, b3)))), id);
-  *xo = mul_rn(fma_rn(a13, det2(a21, b3, b2, a31), fma_rn(a11, det2(b2, a33, a23, b3), -mul_rn(b1, m2))), id);
-  *fc = mul_rn(fma_rn(b1, m3, fma_rn(a11, det2(a22, b3, b2, a32), -mul_rn(a12, det2(a21, b3, b2, a31)))), id);
-}
-
-// Right-hand side of the v equation of parity sv and component r, one walk
-// from n = N down to 0 carrying Dv, D^2 v, t = i kx H_x + i kz H_z and Dt;
-// also stores h_v for the next stage.  Iteration i runs the other-parity step
-// at 2i + sv + 1 (Dv, t) and then the own step at 2i + sv, so the register
-// index i is fixed at compile time and the code is the same for both
-// parities (threads of the two classes share warps).  The other-parity step
-// at n = 0 (sv = 1) has no consumer and is not run.  The terms of v (Dv, D^2 v,
-// phi) are FP64; the nonlinear-term part (t, Dt, h_v and dt (gamma h_v +
-// zeta h_v')) runs in the node precision RN, FP32 in the mixed path, where
-// H itself is FP32-accurate.  h_v' is read through HVr and the new h_v
-// written through HVw (the same column, or a shared-memory copy and global).
-template <int MH, typename RN>
-__device__ __forceinline__ void v_walk(int N, int ny, int ppc, int sv, const CompS& Vc, const CompT<RN>& HVr,
-                                       const CompT<RN>& HVw,
-                                       const typename cpx<RN>::T* Hx, const typename cpx<RN>::T* Hy,
-                                       const typename cpx<RN>::T* Hz, int r, double sgn, double kx, double kz,
-                                       double k2, double cc, const StageCoef& sc, double (&rhs)[MH]) {
-  using CN = typename cpx<RN>::T;
-  const int ra = 1 - r;
-  auto comp = [](const CN z, int qd) { return qd == 0 ? z.x : z.y; };
-  const double dsv = 2.0 * sv;
-  const RN dsvn = (RN)(2 * sv);
-  const RN sgnn = (RN)sgn, kxn = (RN)kx, kzn = (RN)kz, k2n = (RN)k2;
-  const RN dtn = (RN)sc.dt, gan = (RN)sc.gamma, zen = (RN)sc.zeta;
-  double dv = 0.0, d2v = 0.0;
-  RN tt = 0, dtt = 0;
-#pragma unroll
-  for (int i = MH - 1; i >= 0; --i) {
-    const int no = 2 * i + sv + 1;
-    if (no <= N) {
-      const double vn1 = (no + 1 <= N) ? Vc[no + 1] : 0.0;
-      dv = fma_rn((double)(4 * i + 4) + dsv, vn1, dv);  // 2 (no + 1)
-      tt = mul_rn(sgnn, fma_rn(kxn, comp(Hx[no * ppc], ra), mul_rn(kzn, comp(Hz[no * ppc], ra))));
-    }
-    const int n = 2 * i + sv;
-    if (n <= N) {
-      const double fac = (double)(4 * i + 2) + dsv;  // 2 (n + 1)
-      const RN facn = (RN)(4 * i + 2) + dsvn;
-      const double t1 = fma_rn(fac, dv, d2v);
-      const RN t2 = fma_rn(facn, (n + 1 <= N) ? tt : (RN)0, dtt);
-      d2v = (n == 0) ? 0.5 * t1 : t1;
-      dtt = (n == 0) ? (RN)0.5 * t2 : t2;
-      const double phi = fma_rn(-k2, Vc[n], d2v);
-      const RN hv = fma_rn(-k2n, comp(Hy[n * ppc], r), -dtt);
-      const RN hp = HVr[n];
-      HVw[n] = hv;
-      const RN q = mul_rn(dtn, fma_rn(gan, hv, mul_rn(zen, hp)));
-      rhs[i] = fma_rn(1.0 + cc, phi, (double)q);
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// The implicit solves of the no-slip channel with one register array per
-// thread.  tau_fused is tau_seq with the right-hand side produced on the fly:
-// rhs(i) is called once per coefficient, for i = M-1 down to 0, and row i of
-// the elimination runs as soon as r_{i-1} exists, so no array of right-hand
-// sides is held.  A solve may read its right-hand side from f itself (the
-// second solve of v): f[i] is read at step i and written at step i - 1.
-// The wall value s is asked for after the last call of rhs, so the sums that
-// rhs accumulates are complete.  The row arithmetic is tau_seq's.  f is a
-// per-thread array of MH doubles: registers (RegArr), or a column of shared
-// memory (SmemArr) where MH doubles per thread exceed the register file.
-// ---------------------------------------------------------------------------
-template <int MH, class V = double>
-struct RegArr {
-  V v[MH];
-  __device__ __forceinline__ V& operator[](int i) { return v[i]; }
-};
-struct SmemArr {
-  double* p;
-  int stride;
-  __device__ __forceinline__ double& operator[](int i) const { return p[i * stride]; }
-};
-
-template <int MH, class Arr, class Tab, class Rhs, class Wall>
-__device__ __forceinline__ void tau_fused(int N, int ny, int sig, Rhs&& rhs, Arr& f, const Tab& T, double isq,
-                                          Wall&& wall, const double* __restrict__ rowc) {
-  using V = std::decay_t<decltype(f[0])>;  // double, or a Pair of components
-  const int M = (N - sig) / 2 + 1;
-  V r1{}, r2{}, anext{};  // r_{i+1}, r_{i+2}, a_{i+2}
-#pragma unroll
-  for (int i = MH - 1; i >= 0; --i) {
-    V r0{};
-    if (i < M) r0 = rhs(i);
-    const int j = i + 1;  // row j needs r_{j-1} = r0, r_j = r1, r_{j+1} = r2
-    if (j < MH && j < M) {
-      const int n = 2 * j + sig;
-      V R = fma_rn(-rowc[ny + n], r1, mul_rn(rowc[n], r0));
-      if (j + 1 < M) R = fma_rn(rowc[2 * ny + n], r2, R);
-      const V a = fma_rn(-T.h(j), anext, mul_rn(T.e(j), R));
-      f[j] = a;
-      anext = a;
-    }
-    r2 = r1;
-    r1 = r0;
-  }
-  V Pp{}, sum{};
-#pragma unroll
-  for (int i = 1; i < MH; ++i) {
-    if (i < M) {
-      Pp = fma_rn(T.b(i), Pp, f[i]);
-      f[i] = Pp;
-      sum = sum + Pp;
-    }
-  }
-  const V f0 = mul_rn(isq, wall() - sum);
-  f[0] = f0;
-#pragma unroll
-  for (int i = 1; i < MH; ++i)
-    if (i < M) f[i] = fma_rn(T.Q(i), f0, f[i]);
-}
-
-// tau_fused on the folded tables (no-slip top).  Row j of the elimination
-// is a_j = eA_j r_{j-1} - eB_j r_j + eC_j r_{j+1} - h_j a_{j+1}: the same
-// rows with the factor e taken into the row constants.  The wall row needs
-// sum_i P_i, the sum of the particular solution P_i = a_i + b_i P_{i-1}
-// (P_0 = 0); it equals sum_i W_i a_i and is accumulated during the
-// elimination.  f_0 = (s - sum_i P_i) / sum_i Q_i then follows at once, and the
-// back substitution f_i = a_i + b_i f_{i-1} gives the solution in one pass
-// (f_i = P_i + Q_i f_0, Q_i the products of b).  With DIAG, rhs(i) returns
-// RhsX{r_i, x_i} and row j takes the extra term E1_j x_j.
-template <int MH, bool DIAG = false, class Arr, class Rhs, class Wall>
-__device__ __forceinline__ void tau_fold(int N, int sig, Rhs&& rhs, Arr& f, const TabF& T, double isq,
-                                         Wall&& wall) {
-  const int M = (N - sig) / 2 + 1;
-  double r1 = 0.0, r2 = 0.0, x1 = 0.0, anext = 0.0, sum = 0.0;  // r_{i+1}, r_{i+2}, x_{i+1}, a_{i+2}
-#pragma unroll
-  for (int i = MH - 1; i >= 0; --i) {
-    double r0 = 0.0, x0 = 0.0;
-    if (i < M) {
-      if constexpr (DIAG) {
-        const RhsX v = rhs(i);
-        r0 = v.r;
-        x0 = v.x;
-      } else {
-        r0 = rhs(i);
-      }
-    }
-    const int j = i + 1;  // row j needs r_{j-1} = r0, r_j = r1, r_{j+1} = r2 (and x_j = x1)
-    if (j < MH && j < M) {
-      double R = fma_rn(-T.eB(j), r1, mul_rn(T.eA(j), r0));
-      if (j + 1 < M) R = fma_rn(T.eC(j), r2, R);
-      if constexpr (DIAG) R = fma_rn(T.E1(j), x1, R);
-      const double a = fma_rn(-T.h(j), anext, R);
-      f[j] = a;
-      anext = a;
-      sum = fma_rn(T.W(j), a, sum);
-    }
-    r2 = r1;
-    r1 = r0;
-    x1 = x0;
-  }
-  double fp = mul_rn(isq, wall() - sum);
-  f[0] = fp;
-#pragma unroll
-  for (int i = 1; i < MH; ++i)
-    if (i < M) {
-      fp = fma_rn(T.b(i), fp, f[i]);
-      f[i] = fp;
-    }
-}
-
-// omega_y of parity sq: (D^2 - lam) g' = -((1 + cc) g + dt (gamma h_g + zeta
-// h_g'))/(beta dt nu), the factor -1/(beta dt nu) folded into the table's e;
-// wall row sum g' = cc sum g; g <- g' - cc g.  h_g = sgn (-kx H_z + kz H_x) of
-// the other component, in the node precision; h_g' is read through HGr and
-// the new h_g written through HGw.
-template <int MH, typename RN, class Arr, class GV, class HR, class HW, class Tab>
-__device__ __forceinline__ void omega_solve(Arr& f, int N, int ny, int ppc, int sq, const GV& Gc, const HR& HGr,
-                                            const HW& HGw, const typename cpx<RN>::T* Hx,
-                                            const typename cpx<RN>::T* Hz, int r, double sgn, double kx, double kz,
-                                            double cc, const StageCoef& sc, const Tab& T, double isq) {
-  using CN = typename cpx<RN>::T;
-  const int ra = 1 - r;
-  auto comp = [](const CN z, int qd) { return qd == 0 ? z.x : z.y; };
-  const RN sgnn = (RN)sgn, kxn = (RN)kx, kzn = (RN)kz;
-  const RN dtn = (RN)sc.dt, gan = (RN)sc.gamma, zen = (RN)sc.zeta;
-  const int M = (N - sq) / 2 + 1;
-  double sum = 0.0;
-  tau_fold<MH>(
-      N, sq,
-      [&](int i) {
-        const int n = 2 * i + sq;
-        const double gn = Gc[n];
-        const RN hg = mul_rn(sgnn, fma_rn(-kxn, comp(Hz[n * ppc], ra), mul_rn(kzn, comp(Hx[n * ppc], ra))));
-        const RN hp = HGr[n];
-        HGw[n] = hg;
-        const RN q = mul_rn(dtn, fma_rn(gan, hg, mul_rn(zen, hp)));
-        sum += gn;
-        return fma_rn(1.0 + cc, gn, (double)q);
-      },
-      f, T, isq, [&] { return mul_rn(cc, sum); });
-#pragma unroll
-  for (int i = 0; i < MH; ++i)
-    if (i < M) {
-      const int n = 2 * i + sq;
-      Gc[n] = fma_rn(-cc, Gc[n], f[i]);
-    }
-}
-
-// v of parity sv.  The phi solve's right-hand side is (1 + cc)(D^2 v - k^2 v)
-// + q; its tau rows apply to it the stencil r -> cA r_{n-2} - cB r_n +
-// cC r_{n+2}, which integrates D^2 twice, so the stencil of D^2 v is v_n
-// itself (n >= 2).  Row j therefore takes (1 + cc) e v_n through E1 plus the
-// stencil of u = -(1 + cc) k^2 v + q, and no D^2 v is formed; only the FP32
-// walk of t and Dt (from n = N down) remains for q.  The wall sums S0 = sum v,
-// S2 = sum n^2 v of the old field are taken on the way down.  Then the Dirichlet solve of
-// (D^2 - k^2) v_p = phi with v_p(+-1) = cc v(+-1) + (wall velocity), reading
-// phi from the same array, and the influence correction c_I vh that fixes
-// Dv at the wall: v <- v_p + c_I vh - cc v.
-template <int MH, typename RN, class Arr, class VV, class HR, class HW, class Tab, class TabP, class VH>
-__device__ __forceinline__ void v_solve(Arr& f, int N, int ny, int ppc, int sv, const VV& Vc, const HR& HVr,
-                                        const HW& HVw,
-                                        const typename cpx<RN>::T* Hx, const typename cpx<RN>::T* Hy,
-                                        const typename cpx<RN>::T* Hz, int r, double sgn, double kx, double kz,
-                                        double k2, double cc, const StageCoef& sc, const Tab& Th, double isq_h,
-                                        const TabP& Tp, double isq_p, const VH& vh, double idv, double vw) {
-  using CN = typename cpx<RN>::T;
-  const int ra = 1 - r;
-  auto comp = [](const CN z, int qd) { return qd == 0 ? z.x : z.y; };
-  const RN dsvn = (RN)(2 * sv);
-  const RN sgnn = (RN)sgn, kxn = (RN)kx, kzn = (RN)kz, k2n = (RN)k2;
-  const RN dtn = (RN)sc.dt, gan = (RN)sc.gamma, zen = (RN)sc.zeta;
-  const int M = (N - sv) / 2 + 1;
-  const double ck2 = -(1.0 + cc) * k2;
-  double S0 = 0.0, S2 = 0.0;
-  RN tt = 0, dtt = 0;
-  tau_fold<MH, true>(
-      N, sv,
-      [&](int i) {
-        const int no = 2 * i + sv + 1;
-        if (no <= N) tt = mul_rn(sgnn, fma_rn(kxn, comp(Hx[no * ppc], ra), mul_rn(kzn, comp(Hz[no * ppc], ra))));
-        const int n = 2 * i + sv;
-        const RN facn = (RN)(4 * i + 2) + dsvn;  // 2 (n + 1)
-        const RN t2 = fma_rn(facn, (n + 1 <= N) ? tt : (RN)0, dtt);
-        dtt = (n == 0) ? (RN)0.5 * t2 : t2;
-        const double vn = Vc[n];
-        S0 += vn;
-        S2 = fma_rn((double)n * n, vn, S2);
-        const RN hv = fma_rn(-k2n, comp(Hy[n * ppc], r), -dtt);
-        const RN hp = HVr[n];
-        HVw[n] = hv;
-        const RN q = mul_rn(dtn, fma_rn(gan, hv, mul_rn(zen, hp)));
-        return RhsX{fma_rn(ck2, vn, (double)q), vn};
-      },
-      f, Th, isq_h, [] { return 0.0; });
-  const double s = fma_rn(cc, S0, ((sv == 0) ? 0.5 : -0.5) * vw);
-  tau_fold<MH>(N, sv, [&](int i) { return f[i]; }, f, Tp, isq_p, [&] { return s; });
-  double dp = 0.0;
-#pragma unroll
-  for (int i = 0; i < MH; ++i)
-    if (i < M) {
-      const double n = 2 * i + sv;
-      dp = fma_rn(n * n, f[i], dp);
-    }
-  const double cI = mul_rn(fma_rn(cc, S2, -dp), idv);
-#pragma unroll
-  for (int i = 0; i < MH; ++i)
-    if (i < M) {
-      const int n = 2 * i + sv;
-      Vc[n] = fma_rn(-cc, Vc[n], fma_rn(cI, vh(i), f[i]));
-    }
-}
-
-// ---------------------------------------------------------------------------
-// The affine families of the free-slip top with the right-hand sides produced
-// on the fly, as in tau_fused.  tau_affine_fused leaves f_i = P_i (i >= 1),
-// f_0 = 0, with sp = sum P and sp2 = sum n^2 P; tau_close then adds x Q.
-// The wall sums of the old field are taken on the way down.
-// ---------------------------------------------------------------------------
-template <int MH, class Arr, class Tab, class Rhs>
-__device__ __forceinline__ void tau_affine_fused(int N, int ny, int sig, Rhs&& rhs, Arr& f, const Tab& T,
-                                                 const double* __restrict__ rowc, double& sp, double& sp2) {
-  const int M = (N - sig) / 2 + 1;
-  double r1 = 0.0, r2 = 0.0, anext = 0.0;
-#pragma unroll
-  for (int i = MH - 1; i >= 0; --i) {
-    double r0 = 0.0;
-    if (i < M) r0 = rhs(i);
-    const int j = i + 1;
-    if (j < MH && j < M) {
-      const int n = 2 * j + sig;
-      double R = fma_rn(-rowc[ny + n], r1, mul_rn(rowc[n], r0));
-      if (j + 1 < M) R = fma_rn(rowc[2 * ny + n], r2, R);
-      const double a = fma_rn(-T.h(j), anext, mul_rn(T.e(j), R));
-      f[j] = a;
-      anext = a;
-    }
-    r2 = r1;
-    r1 = r0;
-  }
-  double Pp = 0.0;
-  sp = 0.0;
-  sp2 = 0.0;
-#pragma unroll
-  for (int i = 1; i < MH; ++i) {
-    if (i < M) {
-      const double n = 2 * i + sig;
-      Pp = fma_rn(T.b(i), Pp, f[i]);
-      f[i] = Pp;
-      sp += Pp;
-      sp2 = fma_rn(n * n, Pp, sp2);
-    }
-  }
-  f[0] = 0.0;
-}
-
-// omega_y of parity sq under the free-slip top: the affine family and
-// out = {sum P, sum n^2 P, sum g, sum n^2 g} for the closure
-template <int MH, typename RN, class Arr, class GV, class HR, class HW, class Tab>
-__device__ __forceinline__ void omega_open_affine(Arr& f, int N, int ny, int ppc, int sq, const GV& Gc,
-                                                  const HR& HGr, const HW& HGw, const typename cpx<RN>::T* Hx,
-                                                  const typename cpx<RN>::T* Hz, int r, double sgn, double kx,
-                                                  double kz, double cc, const StageCoef& sc, const Tab& T,
-                                                  const double* __restrict__ rowc, double* out) {
-  using CN = typename cpx<RN>::T;
-  const int ra = 1 - r;
-  auto comp = [](const CN z, int qd) { return qd == 0 ? z.x : z.y; };
-  const RN sgnn = (RN)sgn, kxn = (RN)kx, kzn = (RN)kz;
-  const RN dtn = (RN)sc.dt, gan = (RN)sc.gamma, zen = (RN)sc.zeta;
-  double so = 0.0, so2 = 0.0, sp, sp2;
-  tau_affine_fused<MH>(
-      N, ny, sq,
-      [&](int i) {
-        const int n = 2 * i + sq;
-        const double gn = Gc[n];
-        const RN hg = mul_rn(sgnn, fma_rn(-kxn, comp(Hz[n * ppc], ra), mul_rn(kzn, comp(Hx[n * ppc], ra))));
-        const RN hp = HGr[n];
-        HGw[n] = hg;
-        const RN q = mul_rn(dtn, fma_rn(gan, hg, mul_rn(zen, hp)));
-        so += gn;
-        so2 = fma_rn((double)n * n, gn, so2);
-        return fma_rn(1.0 + cc, gn, (double)q);
-      },
-      f, T, rowc, sp, sp2);
-  out[0] = sp;
-  out[1] = sp2;
-  out[2] = so;
-  out[3] = so2;
-}
-
-// mean flow of parity s under the free-slip top (U: e = 0, W: e = 1): the
-// affine family and out = {sum P, sum n^2 P, sum X, sum n^2 X, int P, int X}
-// (int x = sum 2 / (1 - n^2) x_n, even parity only)
-template <int MH, typename RN, class Arr, class Tab>
-__device__ __forceinline__ void mean_open_affine(Arr& f, int N, int ny, int ppc, int s, double* X, double* XP,
-                                                 const typename cpx<RN>::T* Hm, double cc, const StageCoef& sc,
-                                                 const Tab& T, const double* __restrict__ rowc, double* out) {
-  const int M = (N - s) / 2 + 1;
-  double so = 0.0, so2 = 0.0, wo = 0.0, sp, sp2;
-  tau_affine_fused<MH>(
-      N, ny, s,
-      [&](int i) {
-        const int n = 2 * i + s;
-        const double xn = X[n];
-        const double hv = (double)Hm[n * ppc].x;
-        const double hp = XP[n];
-        XP[n] = hv;
-        so += xn;
-        so2 = fma_rn((double)n * n, xn, so2);
-        if (s == 0) wo = fma_rn(2.0 / (1.0 - (double)n * n), xn, wo);
-        return fma_rn(1.0 + cc, xn, mul_rn(sc.dt, fma_rn(sc.gamma, hv, mul_rn(sc.zeta, hp))));
-      },
-      f, T, rowc, sp, sp2);
-  double wp = 0.0;
-  if (s == 0) {
-#pragma unroll
-    for (int i = 0; i < MH; ++i)
-      if (i < M) wp = fma_rn(2.0 / (1.0 - 4.0 * (double)i * i), f[i], wp);
-  }
-  out[0] = sp;
-  out[1] = sp2;
-  out[2] = so;
-  out[3] = so2;
-  out[4] = wp;
-  out[5] = wo;
-}
-
-// v of parity sv under the free-slip top: phi and v_p with the Dirichlet rows
-// of the no-slip channel (f = v_p on return), then out = {A_p, B_p, A_old,
-// B_old} of the free-slip rows (A = sum n^2 (n^2 - 1) / 3 v_n, B = sum n^2
-// v_n); vw is the wall velocity of this component
-template <int MH, typename RN, class Arr, class VV, class HR, class HW, class Tab, class TabP>
-__device__ __forceinline__ void v_open_part(Arr& f, int N, int ny, int ppc, int sv, const VV& Vc, const HR& HVr,
-                                            const HW& HVw, const typename cpx<RN>::T* Hx,
-                                            const typename cpx<RN>::T* Hy, const typename cpx<RN>::T* Hz, int r,
-                                            double sgn, double kx, double kz, double k2, double cc,
-                                            const StageCoef& sc, const Tab& Th, double isq_h, const TabP& Tp,
-                                            double isq_p, double vw, const double* __restrict__ rowc, double* out) {
-  using CN = typename cpx<RN>::T;
-  const int ra = 1 - r;
-  auto comp = [](const CN z, int qd) { return qd == 0 ? z.x : z.y; };
-  const double dsv = 2.0 * sv;
-  const RN dsvn = (RN)(2 * sv);
-  const RN sgnn = (RN)sgn, kxn = (RN)kx, kzn = (RN)kz, k2n = (RN)k2;
-  const RN dtn = (RN)sc.dt, gan = (RN)sc.gamma, zen = (RN)sc.zeta;
-  const int M = (N - sv) / 2 + 1;
-  double dv = 0.0, d2v = 0.0, S0 = 0.0, Bo = 0.0, Ao = 0.0;
-  RN tt = 0, dtt = 0;
-  tau_fused<MH>(
-      N, ny, sv,
-      [&](int i) {
-        const int no = 2 * i + sv + 1;
-        if (no <= N) {
-          const double vn1 = (no + 1 <= N) ? Vc[no + 1] : 0.0;
-          dv = fma_rn((double)(4 * i + 4) + dsv, vn1, dv);  // 2 (no + 1)
-          tt = mul_rn(sgnn, fma_rn(kxn, comp(Hx[no * ppc], ra), mul_rn(kzn, comp(Hz[no * ppc], ra))));
-        }
-        const int n = 2 * i + sv;
-        const double fac = (double)(4 * i + 2) + dsv;  // 2 (n + 1)
-        const RN facn = (RN)(4 * i + 2) + dsvn;
-        const double t1 = fma_rn(fac, dv, d2v);
-        const RN t2 = fma_rn(facn, (n + 1 <= N) ? tt : (RN)0, dtt);
-        d2v = (n == 0) ? 0.5 * t1 : t1;
-        dtt = (n == 0) ? (RN)0.5 * t2 : t2;
-        const double vn = Vc[n];
-        const double nn = (double)n * n;
-        S0 += vn;
-        Bo = fma_rn(nn, vn, Bo);
-        Ao = fma_rn(nn * (nn - 1.0) / 3.0, vn, Ao);
-        const double phi = fma_rn(-k2, vn, d2v);
-        const RN hv = fma_rn(-k2n, comp(Hy[n * ppc], r), -dtt);
-        const RN hp = HVr[n];
-        HVw[n] = hv;
-        const RN q = mul_rn(dtn, fma_rn(gan, hv, mul_rn(zen, hp)));
-        return fma_rn(1.0 + cc, phi, (double)q);
-      },
-      f, Th, isq_h, [] { return 0.0; }, rowc);
-  const double s = fma_rn(cc, S0, ((sv == 0) ? 0.5 : -0.5) * vw);
-  tau_fused<MH>(N, ny, sv, [&](int i) { return f[i]; }, f, Tp, isq_p, [&] { return s; }, rowc);
-  double Ap = 0.0, Bp = 0.0;
-#pragma unroll
-  for (int i = 0; i < MH; ++i)
-    if (i < M) {
-      const double n = 2 * i + sv;
-      Bp = fma_rn(n * n, f[i], Bp);
-      Ap = fma_rn(n * n * (n * n - 1.0) / 3.0, f[i], Ap);
-    }
-  out[0] = Ap;
-  out[1] = Bp;
-  out[2] = Ao;
-  out[3] = Bo;
-}
-
-// mean flow of parity s: U (e = 0, at constant flow rate through the
-// response u1 to a unit forcing) or W (e = 1); X the coefficients, XP the
-// previous plane means of H_x or H_z (FP64), Hm the new plane mean.
-template <int MH, typename RN, class Arr, class Tab>
-__device__ __forceinline__ void mean_solve(Arr& f, int N, int ny, int ppc, int s, int e, double* X, double* XP,
-                                           const typename cpx<RN>::T* Hm, double cc, const StageCoef& sc,
-                                           const Tab& T, double isq,
-                                           const double* __restrict__ u1, double u1_iflux) {
-  const int M = (N - s) / 2 + 1;
-  double sum = 0.0, flux_old = 0.0;
-  tau_fold<MH>(
-      N, s,
-      [&](int i) {
-        const int n = 2 * i + s;
-        const double xn = X[n];
-        const double hv = (double)Hm[n * ppc].x;
-        const double hp = XP[n];
-        XP[n] = hv;
-        sum += xn;
-        if (s == 0) flux_old = fma_rn(2.0 / (1.0 - (double)n * n), xn, flux_old);
-        return fma_rn(1.0 + cc, xn, mul_rn(sc.dt, fma_rn(sc.gamma, hv, mul_rn(sc.zeta, hp))));
-      },
-      f, T, isq, [&] { return mul_rn(cc, sum); });
-  double fc = 0.0;
-  if (e == 0 && s == 0) {
-    double flux = 0.0;
-#pragma unroll
-    for (int i = 0; i < MH; ++i)
-      if (i < M) flux = fma_rn(2.0 / (1.0 - 4.0 * (double)i * i), f[i], flux);
-    fc = mul_rn(fma_rn(cc, flux_old, sc.flux) - flux, u1_iflux);
-  }
-#pragma unroll
-  for (int i = 0; i < MH; ++i) {
-    if (i < M) {
-      const int n = 2 * i + s;
-      double v = fma_rn(-cc, X[n], f[i]);
-      if (e == 0 && s == 0) v = fma_rn(fc, u1[i], v);
-      X[n] = v;
-    }
-  }
-}
-
-
-// One (mode p, class, component r) thread's implicit solves under the no-slip
-// top: the mean flow (p = 0), else omega_y of parity 1 - c and v of parity c.
-// H_x, H_y, H_z: Chebyshev coefficients of the mode, element n at n * hs;
-// HGr, HVr: the previous nonlinear right-hand sides (node precision); the new
-// ones go to the pencil buffers.  Each solve keeps its array of MH doubles in
-// registers (col = nullptr) or in the thread's column of shared memory,
-// col[i * cs].
-template <int MH, typename RN, bool SMEM, class Cls>
-__device__ __forceinline__ void post_solve_noslip(double* col, int cs, Cls cls, const Grid& g, const PencilBufs& pb,
-                                                  const DevTables& t, const StageCoef& sc, int b, int p, int r,
-                                                  const typename cpx<RN>::T* Hx, const typename cpx<RN>::T* Hy,
-                                                  const typename cpx<RN>::T* Hz, int hs, const CompT<RN>& HGr,
-                                                  const CompT<RN>& HVr) {
-  const int c = class_of(cls);
-  const int P = g.P, ny = g.ny, N = g.N, Mh = t.tau.Mh;
-  const double cc = sc.alpha / sc.beta;
-  auto comp = [](auto z, int qq) { return qq == 0 ? z.x : z.y; };
-  auto helm = [&](int sig) { return TabF{t.tau.helm_f + (size_t)(sc.k * 2 + sig) * 7 * Mh * P + p, Mh, P}; };
-  auto helm_isq = [&](int sig) { return t.tau.helm_isq[(size_t)(sc.k * 2 + sig) * P + p]; };
-  if (p == 0) {
-    // mean mode: U (r = 0) at constant flow rate and W (r = 1), parity c
-    const int e = r;
-    auto run = [&](auto& f) {
-      mean_solve<MH, RN>(f, N, ny, hs, c, e, (e == 0 ? pb.UM : pb.WM) + (size_t)b * ny,
-                       (e == 0 ? pb.HXP : pb.HZP) + (size_t)b * ny, (e == 0) ? Hx : Hz, cc, sc, helm(c),
-                       helm_isq(c), t.tau.u1 + (size_t)sc.k * Mh, t.tau.u1_iflux[sc.k]);
-    };
-    if constexpr (SMEM) {
-      SmemArr f{col, cs};
-      run(f);
-    } else {
-      RegArr<MH> f;
-      run(f);
-    }
-    return;
-  }
-  const int row = p / g.nxh, ix = p % g.nxh;
-  const double kx = t.kx[ix], kz = t.kz[row], k2 = kx * kx + kz * kz;
-  const double sgn = (r == 0) ? -1.0 : 1.0;
-  const size_t base = 2 * ((size_t)b * ny * P + p) + r;  // component r of element n at base + 2 P n
-  {
-    // wall-normal vorticity, parity 1 - c; previous right-hand sides are
-    // stored in the node precision
-    const int sq = 1 - c;
-    const CompS Gc{reinterpret_cast<double*>(pb.G) + base, 2 * P};
-    const CompT<RN> HGc{reinterpret_cast<RN*>(pb.HGP) + base, 2 * P};
-    auto run = [&](auto& f) {
-      omega_solve<MH, RN>(f, N, ny, hs, sq, Gc, HGr, HGc, Hx, Hz, r, sgn, kx, kz, cc, sc, helm(sq), helm_isq(sq));
-    };
-    if constexpr (SMEM) {
-      SmemArr f{col, cs};
-      run(f);
-    } else {
-      RegArr<MH> f;
-      run(f);
-    }
-  }
-  {
-    // wall-normal velocity, parity c
-    const int sv = c;
-    const CompS Vc{reinterpret_cast<double*>(pb.V) + base, 2 * P};
-    const CompT<RN> HVc{reinterpret_cast<RN*>(pb.HVP) + base, 2 * P};
-    const size_t vo = (size_t)b * P + p;
-    const double vw = fma_rn(sc.theta, comp(pb.vw_new[vo], r) - comp(pb.vw_old[vo], r), comp(pb.vw_old[vo], r));
-    const TabF TP{t.tau.pois_f + (size_t)sv * 6 * Mh * P + p, Mh, P};
-    const double* vh = t.tau.vh + (size_t)(sc.k * 2 + sv) * Mh * P + p;
-    auto run = [&](auto& f) {
-      v_solve<MH, RN>(f, N, ny, hs, sv, Vc, HVr, HVc, Hx, Hy, Hz, r, sgn, kx, kz, k2, cc, sc, helm(sv),
-                      helm_isq(sv), TP, t.tau.pois_isq[(size_t)sv * P + p], [&](int i) { return vh[(size_t)i * P]; },
-                      t.tau.vh_idv[(size_t)(sc.k * 2 + sv) * P + p], vw);
-    };
-    if constexpr (SMEM) {
-      SmemArr f{col, cs};
-      run(f);
-    } else {
-      RegArr<MH> f;
-      run(f);
-    }
-  }
-}
-
 // cos(pi j n / N) table in the node precision
 template <typename RN>
 __device__ __forceinline__ const RN* cheb_table(const DevTables& t);
@@ -1020,11 +270,6 @@ __global__ void __launch_bounds__(128) stage_pre_kernel(Grid g, int B, PencilBuf
   if (pb.active && !pb.active[b]) return;
   const int tid = threadIdx.x, nt = blockDim.x;
   pdl_wait_then_release();  // v, omega_y come from the previous stage
-  // FP64 nodes on a grid whose N the FFT plan covers: fast synthesis
-  constexpr int NF = 2 * (MH - 1);
-  constexpr bool kFastOk = std::is_same<RN, double>::value && ct_plan_ok(NF);
-  const bool fast = kFastOk && N == NF;
-
   for (int w = tid; w < ny * ppc; w += nt) {
     const int pl = w % ppc, n = w / ppc;
     const int p = p0 + pl;
@@ -1058,7 +303,7 @@ __global__ void __launch_bounds__(128) stage_pre_kernel(Grid g, int B, PencilBuf
     RN mid[6] = {0, 0, 0, 0, 0, 0};
     auto W = [&](int f, int n, RN x) {
       out[f * fs + n * 2 * ppc] = x;
-      if (!fast && (n & 1) == 0) mid[f] = (n & 2) ? mid[f] - x : mid[f] + x;
+      if ((n & 1) == 0) mid[f] = (n & 2) ? mid[f] - x : mid[f] + x;
     };
     // inclusive prefix over the 4-lane group of this lane's block total;
     // returns the exclusive offset
@@ -1174,7 +419,7 @@ __global__ void __launch_bounds__(128) stage_pre_kernel(Grid g, int B, PencilBuf
 #pragma unroll
       for (int o = 1; o < LC; o <<= 1) mid[f] = mid[f] + __shfl_xor_sync(0xffffffffu, mid[f], o, LC);
     // this chain wrote the even coefficients of fields 0, 2, 4 (c = 1) or 1, 3, 5 (c = 0)
-    if (on && lc == 0 && !fast && (N & 1) == 0 && p < P) {
+    if (on && lc == 0 && (N & 1) == 0 && p < P) {
       RN* qr = reinterpret_cast<RN*>(q);
 #pragma unroll
       for (int f = 0; f < 6; ++f)
@@ -1182,71 +427,6 @@ __global__ void __launch_bounds__(128) stage_pre_kernel(Grid g, int B, PencilBuf
     }
   }
   __syncthreads();
-
-  if constexpr (kFastOk) {
-    if (fast) {
-      const int nl = 6 * ppc;
-      const int LS = ny * ppc;
-      double2* X = sC;                   // [6][ny][ppc] coefficients, then y, then Z
-      double2* sHalf = sC + 6 * ny * ppc;  // [6 ppc] (x_0 + x_N) / 2
-      double2* sF1 = sHalf + nl;           // [6 ppc] F_1
-      const double* cheb = t.cheb;       // cheb[ny + m] = cos(pi m / N)
-      for (int l = tid; l < nl; l += nt) {
-        const double2* x = X + (l / ppc) * LS + (l % ppc);
-        double2 s1 = mk(0.0, 0.0);
-        for (int n = 0; n <= N; ++n) s1 = s1 + cheb[ny + n] * x[n * ppc];
-        sF1[l] = s1;
-        sHalf[l] = 0.5 * (x[0] + x[N * ppc]);
-      }
-      __syncthreads();
-      for (int w = tid; w < nl * (N / 2); w += nt) {
-        const int l = w % nl, n = w / nl;
-        double2* x = X + (l / ppc) * LS + (l % ppc);
-        if (n == 0) {
-          x[0] = sHalf[l];  // y_0; y_{N/2} = x_{N/2} stays
-          continue;
-        }
-        const double2 xa = x[n * ppc], xb = x[(N - n) * ppc];
-        const double sn = cheb[ny + N / 2 - n];  // sin(pi n / N)
-        const double2 sm = 0.5 * (xa + xb), d = xa - xb;
-        x[n * ppc] = sm - sn * d;
-        x[(N - n) * ppc] = sm + sn * d;
-      }
-      __syncthreads();
-      lines_dif<NF, 0>(X, t.tw_cheb, nl, ppc, LS);
-      // even outputs, and the odd-output differences -i (Z_k - Z_{N-k}) / 2
-      // stored in Z_k's own slot (slots of Z_{N-k}, k < N/2, are only read)
-      for (int w = tid; w < nl * (NF / 2 + 1); w += nt) {
-        const int l = w % nl, k = w / nl;
-        const int f = l / ppc, pl = l % ppc, p = p0 + pl;
-        double2* Z = X + f * LS + pl;
-        const int ik = dif_pos<NF>(k) * ppc;
-        const double2 zk = Z[ik];
-        const double2 zn = Z[dif_pos<NF>((NF - k) % NF) * ppc];
-        if (p < P) q[((size_t)(b * 6 + f) * ny + 2 * k) * P + p] = 0.5 * (zk + zn) + sHalf[l];
-        if (k >= 1 && k < NF / 2) {
-          const double2 dd = zk - zn;
-          Z[ik] = mk(0.5 * dd.y, -0.5 * dd.x);
-        }
-      }
-      __syncthreads();
-      // odd outputs: prefix sums from F_1
-      for (int l = tid; l < nl; l += nt) {
-        const int f = l / ppc, pl = l % ppc, p = p0 + pl;
-        if (p >= P) continue;
-        const double2* Z = X + f * LS + pl;
-        double2* dst = q + ((size_t)(b * 6 + f) * ny) * P + p;
-        double2 fo = sF1[l];
-        dst[P] = fo;
-#pragma unroll 4
-        for (int k = 1; k < NF / 2; ++k) {
-          fo = fo + Z[dif_pos<NF>(k) * ppc];
-          dst[(size_t)(2 * k + 1) * P] = fo;
-        }
-      }
-      return;
-    }
-  }
 
   // synthesis of the six fields at the nodes.  Thread (mode pl, group g of
   // nt / ppc) evaluates the node pairs j = g, g + ng, ... of all six fields of
@@ -1327,13 +507,11 @@ __global__ void __launch_bounds__(128) stage_pre_kernel(Grid g, int B, PencilBuf
 // 1-c, e = 1 v on parity c.  The mean mode solves U at constant flow rate
 // (e = 0) and W (e = 1) on parity c, real component only.
 // ---------------------------------------------------------------------------
-// Lanes per system of the per-tile form: four under the no-slip top (the
-// scan solves of stage_scan.cuh), one under the free-slip top.
-template <int TOP>
-constexpr int post_tile_lanes() { return TOP == 0 ? 4 : 1; }
+// Lanes per system of the per-tile form (the scan solves of stage_scan.cuh)
+constexpr int kPostTileLanes = 4;
 
-template <typename RN, int MH, int TOP>
-__global__ void __launch_bounds__(64 * post_tile_lanes<TOP>()) stage_post_kernel(Grid g, int B, PencilBufs pb, DevTables t,
+template <typename RN, int MH>
+__global__ void __launch_bounds__(64 * kPostTileLanes) stage_post_kernel(Grid g, int B, PencilBufs pb, DevTables t,
                                                         const typename cpx<RN>::T* __restrict__ hn, StageCoef sc,
                                                         int ppc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1411,7 +589,7 @@ __global__ void __launch_bounds__(64 * post_tile_lanes<TOP>()) stage_post_kernel
     // of the three fields of its mode: every pair f_j, f_{N-j} it loads feeds
     // all of its outputs, and the outputs are independent accumulation chains.
     // n and g share their parity, so the folding sign is fixed per thread.
-    constexpr int GA = 8 * post_tile_lanes<TOP>();
+    constexpr int GA = 8 * kPostTileLanes;
     constexpr int KN = (2 * MH + GA - 1) / GA;  // n values per thread
     const int pl = tid % ppc, gq = tid / ppc;  // blockDim = GA ppc
     const RN* cheb = cheb_table<RN>(t);
@@ -1463,65 +641,16 @@ __global__ void __launch_bounds__(64 * post_tile_lanes<TOP>()) stage_post_kernel
     __syncthreads();
   }
 
-  if constexpr (TOP == 0) {
-    // ---- implicit solves, system (mode pl, class c, component r, equation
-    // e) on the four lanes q of a group
-    const int q = tid & 3, sys = tid >> 2;
-    const int pl = sys % ppc;
-    const int combo = sys / ppc;
-    const int p = p0 + pl;
-    const int c = combo & 1, r = (combo >> 1) & 1, e = combo >> 2;
-    const int row = p / g.nxh, ix = p % g.nxh;
-    // a whole group is live or idle together
-    if (p < P && row != g.nz / 2 && (p != 0 || r == 0)) {
-      const double cc = sc.alpha / sc.beta;
-      const double* rowc = t.tau.rowc;
-      const CN* Hx = reinterpret_cast<const CN*>(sH) + pl;
-      const CN* Hy = Hx + ny * ppc;
-      const CN* Hz = Hy + ny * ppc;
-      auto helm = [&](int sig) { return TabSm{sh + sig * 4 * Mh * ppc + pl, Mh, ppc}; };
-      auto comp = [](auto z, int qd) { return qd == 0 ? z.x : z.y; };
-      if (p == 0) {
-        mean_scan<MH, RN>(N, ny, ppc, c, e, (e == 0 ? pb.UM : pb.WM) + (size_t)b * ny,
-                          (e == 0 ? pb.HXP : pb.HZP) + (size_t)b * ny, (e == 0) ? Hx : Hz, cc, sc, helm(c),
-                          ss[(0 * 2 + c) * ppc + pl], rowc, t.tau.u1 + (size_t)sc.k * Mh, t.tau.u1_iflux[sc.k], q);
-      } else {
-        const double kx = t.kx[ix], kz = t.kz[row], k2 = kx * kx + kz * kz;
-        const double sgn = (r == 0) ? -1.0 : 1.0;
-        if (e == 0) {
-          // wall-normal vorticity, parity 1 - c
-          const int sq = 1 - c;
-          const CompS Gc{reinterpret_cast<double*>(sG) + 2 * pl + r, 2 * ppc};
-          const CompT<RN> HGc{reinterpret_cast<RN*>(sHG) + 2 * pl + r, 2 * ppc};
-          omega_scan<MH, RN>(N, ny, ppc, sq, Gc, HGc, Hx, Hz, r, sgn, kx, kz, cc, sc, helm(sq),
-                             ss[(0 * 2 + sq) * ppc + pl], rowc, q);
-        } else {
-          // wall-normal velocity, parity c
-          const int sv = c;
-          const CompS Vc{reinterpret_cast<double*>(sV) + 2 * pl + r, 2 * ppc};
-          const CompT<RN> HVc{reinterpret_cast<RN*>(sHV) + 2 * pl + r, 2 * ppc};
-          const size_t vo = (size_t)b * P + p;
-          const double vw =
-              fma_rn(sc.theta, comp(pb.vw_new[vo], r) - comp(pb.vw_old[vo], r), comp(pb.vw_old[vo], r));
-          const TabSm TP{sp + sv * 4 * Mh * ppc + pl, Mh, ppc};
-          v_scan<MH, RN>(N, ny, ppc, sv, Vc, HVc, Hx, Hy, Hz, r, sgn, kx, kz, k2, cc, sc, helm(sv),
-                         ss[(0 * 2 + sv) * ppc + pl], TP, ss[(1 * 2 + sv) * ppc + pl], svh + sv * Mh * ppc + pl,
-                         ppc, ss[(2 * 2 + sv) * ppc + pl], vw, rowc, q);
-        }
-      }
-    }
-  } else {
-    // ---- implicit solves under a free-slip top: each thread forms the
-    // affine family of its parity and publishes its sums; the closure follows
-    // the barrier.  Thread (mode, class c, component r, equation e) as above;
-    // its partner of the other parity is class 1 - c.
-    double* xch = reinterpret_cast<double*>(ss + 6 * ppc) + 12 * ppc;  // [8 ppc threads][6]
-    const int pl = tid % ppc;
-    const int combo = tid / ppc;
-    const int p = p0 + pl;
-    const int c = combo & 1, r = (combo >> 1) & 1, e = combo >> 2;
-    const int row = p / g.nxh, ix = p % g.nxh;
-    const bool live = p < P && combo < 8 && row != g.nz / 2 && !(p == 0 && r == 1);
+  // ---- implicit solves, system (mode pl, class c, component r, equation
+  // e) on the four lanes q of a group
+  const int q = tid & 3, sys = tid >> 2;
+  const int pl = sys % ppc;
+  const int combo = sys / ppc;
+  const int p = p0 + pl;
+  const int c = combo & 1, r = (combo >> 1) & 1, e = combo >> 2;
+  const int row = p / g.nxh, ix = p % g.nxh;
+  // a whole group is live or idle together
+  if (p < P && row != g.nz / 2 && (p != 0 || r == 0)) {
     const double cc = sc.alpha / sc.beta;
     const double* rowc = t.tau.rowc;
     const CN* Hx = reinterpret_cast<const CN*>(sH) + pl;
@@ -1529,101 +658,32 @@ __global__ void __launch_bounds__(64 * post_tile_lanes<TOP>()) stage_post_kernel
     const CN* Hz = Hy + ny * ppc;
     auto helm = [&](int sig) { return TabSm{sh + sig * 4 * Mh * ppc + pl, Mh, ppc}; };
     auto comp = [](auto z, int qd) { return qd == 0 ? z.x : z.y; };
-    const int pc = min(p, P - 1);
-    // table sums of both parities: sum Q, sum n^2 Q of this stage; A, B of vh
-    auto qs = [&](int sig, int w) { return t.tau.helm_top[((size_t)(sc.k * 2 + sig) * 2 + w) * P + pc]; };
-    auto vs = [&](int sig, int w) { return t.tau.vh_top[((size_t)(sc.k * 2 + sig) * 2 + w) * P + pc]; };
-    double* mine = xch + tid * 6;
-    const double* other = xch + ((combo ^ 1) * ppc + pl) * 6;
-    RegArr<MH> f;
-    int sig = 0;
-    if (live) {
-      if (p == 0) {
-        // mean mode: U (e = 0) at constant flow rate, W (e = 1), parity c
-        sig = c;
-        mean_open_affine<MH, RN>(f, N, ny, ppc, sig, (e == 0 ? pb.UM : pb.WM) + (size_t)b * ny,
-                                 (e == 0 ? pb.HXP : pb.HZP) + (size_t)b * ny, (e == 0) ? Hx : Hz, cc, sc, helm(sig),
-                                 rowc, mine);
-      } else if (e == 0) {
+    if (p == 0) {
+      mean_scan<MH, RN>(N, ny, ppc, c, e, (e == 0 ? pb.UM : pb.WM) + (size_t)b * ny,
+                        (e == 0 ? pb.HXP : pb.HZP) + (size_t)b * ny, (e == 0) ? Hx : Hz, cc, sc, helm(c),
+                        ss[(0 * 2 + c) * ppc + pl], rowc, t.tau.u1 + (size_t)sc.k * Mh, t.tau.u1_iflux[sc.k], q);
+    } else {
+      const double kx = t.kx[ix], kz = t.kz[row], k2 = kx * kx + kz * kz;
+      const double sgn = (r == 0) ? -1.0 : 1.0;
+      if (e == 0) {
         // wall-normal vorticity, parity 1 - c
-        sig = 1 - c;
+        const int sq = 1 - c;
         const CompS Gc{reinterpret_cast<double*>(sG) + 2 * pl + r, 2 * ppc};
         const CompT<RN> HGc{reinterpret_cast<RN*>(sHG) + 2 * pl + r, 2 * ppc};
-        omega_open_affine<MH, RN>(f, N, ny, ppc, sig, Gc, HGc, HGc, Hx, Hz, r, (r == 0) ? -1.0 : 1.0, t.kx[ix],
-                                  t.kz[row], cc, sc, helm(sig), rowc, mine);
+        omega_scan<MH, RN>(N, ny, ppc, sq, Gc, HGc, Hx, Hz, r, sgn, kx, kz, cc, sc, helm(sq),
+                           ss[(0 * 2 + sq) * ppc + pl], rowc, q);
       } else {
-        // wall-normal velocity, parity c: phi_p and v_p as in the no-slip
-        // channel (Dirichlet rows of both), then the sums of the free-slip rows
-        sig = c;
-        const double kx = t.kx[ix], kz = t.kz[row], k2 = kx * kx + kz * kz;
+        // wall-normal velocity, parity c
+        const int sv = c;
         const CompS Vc{reinterpret_cast<double*>(sV) + 2 * pl + r, 2 * ppc};
         const CompT<RN> HVc{reinterpret_cast<RN*>(sHV) + 2 * pl + r, 2 * ppc};
         const size_t vo = (size_t)b * P + p;
         const double vw =
             fma_rn(sc.theta, comp(pb.vw_new[vo], r) - comp(pb.vw_old[vo], r), comp(pb.vw_old[vo], r));
-        const TabSm TP{sp + sig * 4 * Mh * ppc + pl, Mh, ppc};
-        v_open_part<MH, RN>(f, N, ny, ppc, sig, Vc, HVc, HVc, Hx, Hy, Hz, r, (r == 0) ? -1.0 : 1.0, kx, kz, k2, cc,
-                            sc, helm(sig), ss[(0 * 2 + sig) * ppc + pl], TP, ss[(1 * 2 + sig) * ppc + pl], vw, rowc,
-                            mine);
-      }
-    }
-    __syncthreads();
-    if (live) {
-      const double* se = sig == 0 ? mine : other;
-      const double* so = sig == 0 ? other : mine;
-      const int M = (N - sig) / 2 + 1;
-      if (p == 0) {
-        double* X = (e == 0 ? pb.UM : pb.WM) + (size_t)b * ny;
-        double xe, xo, fc = 0.0;
-        if (e == 1) {
-          close_neumann_top(se, so, qs(0, 0), qs(1, 0), qs(0, 1), qs(1, 1), cc, &xe, &xo);
-        } else {
-          // forcing response (even parity) and int Q_e
-          const double* u1 = t.tau.u1 + (size_t)sc.k * Mh;
-          const TabSm He = helm(0);
-          double us = 0.0, u2 = 0.0, uw = 0.0, wq = 0.0;
-          for (int i = 0; i < N / 2 + 1; ++i) {
-            const double n = 2 * i, w = 2.0 / (1.0 - n * n);
-            us += u1[i];
-            u2 = fma_rn(n * n, u1[i], u2);
-            uw = fma_rn(w, u1[i], uw);
-            wq = fma_rn(w, i == 0 ? 1.0 : He.Q(i), wq);
-          }
-          close_free_slip_mean(se, so, qs(0, 0), qs(1, 0), qs(0, 1), qs(1, 1), wq, us, u2, uw, cc, sc.flux, &xe,
-                               &xo, &fc);
-        }
-        tau_close<MH>(N, sig, f, helm(sig), sig == 0 ? xe : xo);
-#pragma unroll
-        for (int i = 0; i < MH; ++i)
-          if (i < M) {
-            const int n = 2 * i + sig;
-            double v = fma_rn(-cc, X[n], f[i]);
-            if (e == 0 && sig == 0) v = fma_rn(fc, t.tau.u1[(size_t)sc.k * Mh + i], v);
-            X[n] = v;
-          }
-      } else if (e == 0) {
-        const CompS Gc{reinterpret_cast<double*>(sG) + 2 * pl + r, 2 * ppc};
-        double xe, xo;
-        close_neumann_top(se, so, qs(0, 0), qs(1, 0), qs(0, 1), qs(1, 1), cc, &xe, &xo);
-        tau_close<MH>(N, sig, f, helm(sig), sig == 0 ? xe : xo);
-#pragma unroll
-        for (int i = 0; i < MH; ++i)
-          if (i < M) {
-            const int n = 2 * i + sig;
-            Gc[n] = fma_rn(-cc, Gc[n], f[i]);
-          }
-      } else {
-        const CompS Vc{reinterpret_cast<double*>(sV) + 2 * pl + r, 2 * ppc};
-        double ce, co;
-        close_free_slip_v(se, so, vs(0, 0), vs(1, 0), vs(0, 1), vs(1, 1), cc, &ce, &co);
-        const double cI = sig == 0 ? ce : co;
-        const double* vh = svh + sig * Mh * ppc + pl;
-#pragma unroll
-        for (int i = 0; i < MH; ++i)
-          if (i < M) {
-            const int n = 2 * i + sig;
-            Vc[n] = fma_rn(-cc, Vc[n], fma_rn(cI, vh[i * ppc], f[i]));
-          }
+        const TabSm TP{sp + sv * 4 * Mh * ppc + pl, Mh, ppc};
+        v_scan<MH, RN>(N, ny, ppc, sv, Vc, HVc, Hx, Hy, Hz, r, sgn, kx, kz, k2, cc, sc, helm(sv),
+                       ss[(0 * 2 + sv) * ppc + pl], TP, ss[(1 * 2 + sv) * ppc + pl], svh + sv * Mh * ppc + pl,
+                       ppc, ss[(2 * 2 + sv) * ppc + pl], vw, rowc, q);
       }
     }
   }
@@ -1643,270 +703,10 @@ __global__ void __launch_bounds__(64 * post_tile_lanes<TOP>()) stage_post_kernel
 }
 
 // ---------------------------------------------------------------------------
-// stage_post, batched form.  The same arithmetic as stage_post_kernel, mapped
-// for many modes: one thread per (mode, class c, component r) solves both
-// equations of its class (omega_y on parity 1-c, then v on parity c), so every
-// warp carries the same FP64 work, and only the Chebyshev coefficients of H
-// are staged in shared memory (3 ny complex per mode, against 7 ny complex
-// plus the tau tables in the per-tile form), which lets four times as many
-// modes be resident per SM.  The state, the previous right-hand sides and the
-// tau tables are read and written in place in global memory by the thread
-// that owns them; lanes (mode, r) make these accesses contiguous.  The
-// analysis runs field by field with four threads per mode (n = q + 4k); each
-// coefficient is accumulated in the same order as in the per-tile form.
-// ---------------------------------------------------------------------------
-// Five CTAs per SM with up to 65 nodes: the register budget (168) holds the
-// solves' one array of coefficients, and the shared tile (41.6 KB at 65
-// nodes in FP32, 44.6 KB with the free-slip exchange slots) allows five.
-template <int MH, int TOP>
-constexpr int post_batched_min_ctas() { return MH <= 33 ? 5 : 1; }
-
-template <typename RN, int MH, int TOP>
-__global__ void __launch_bounds__(64, post_batched_min_ctas<MH, TOP>()) stage_post_batched_kernel(Grid g, int B, PencilBufs pb, DevTables t,
-                                                                const typename cpx<RN>::T* __restrict__ hn,
-                                                                StageCoef sc, int ppc) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  using CN = typename cpx<RN>::T;
-  const int P = g.P, ny = g.ny, N = g.N;
-  const int Mh = t.tau.Mh;
-  double2* sH = reinterpret_cast<double2*>(smem_raw);  // [3][ny][ppc] coefficients
-  CN* sN = reinterpret_cast<CN*>(smem_raw);             // [3][ny][ppc] nodal values, same bytes
-  const int p0 = blockIdx.x * ppc;
-  const int b = blockIdx.y;
-  if (pb.active && !pb.active[b]) return;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  // FP32 nodes: the previous right-hand sides (FP32 pairs) are staged in shared
-  // memory behind the node tile, issued before the wait for H; the new ones go
-  // straight to global memory.  Both tiles arrive by asynchronous copies.
-  constexpr bool kStageHV = sizeof(RN) == 4 && kPostStageHV, kStageHG = sizeof(RN) == 4 && kPostStageHG;
-  CN* sHVt = sN + 3 * ny * ppc;
-  CN* sHGt = sHVt + (kStageHV ? ny * ppc : 0);
-  if (kStageHV || kStageHG) {
-    for (int w = tid; w < ny * ppc; w += nt) {
-      const int pl = w % ppc, n = w / ppc;
-      const size_t o = ((size_t)b * ny + n) * P + min(p0 + pl, P - 1);
-      if (kStageHV) cp_async_elem(sHVt + w, reinterpret_cast<const CN*>(pb.HVP) + o);
-      if (kStageHG) cp_async_elem(sHGt + w, reinterpret_cast<const CN*>(pb.HGP) + o);
-    }
-  }
-  pdl_wait_then_release();  // H comes from the preceding kernel
-  for (int w = tid; w < 3 * ny * ppc; w += nt) {
-    const int pl = w % ppc, fn = w / ppc;  // fn = f * ny + n
-    const int p = min(p0 + pl, P - 1);
-    cp_async_elem(sN + w, hn + ((size_t)b * 3 * ny + fn) * P + p);
-  }
-  cp_async_wait_all();
-  __syncthreads();
-  // thread (mode pl, class c, component r).  Under the no-slip top each warp
-  // holds one class (16 or more modes per CTA); under the free-slip top the
-  // two classes of a (mode, component) are neighbouring lanes, whose parity
-  // closures exchange their sums by shuffles.
-  const int r = TOP ? (tid >> 1) & 1 : tid & 1;
-  const int pl = TOP ? tid >> 2 : (tid >> 1) % ppc;
-  const int c = TOP ? tid & 1 : tid / (2 * ppc);
-
-  // ---- Chebyshev analysis of H_z, H_y, H_x, coefficients in the node
-  // precision over the nodal values of the same field (a barrier between
-  // reading and writing each field).
-  constexpr int NF = 2 * (MH - 1);
-  bool analysed = false;
-  if constexpr (std::is_same<RN, double>::value && ct_plan_ok(NF)) {
-    if (N == NF) {
-      analysis_fft<NF>(sH, ppc, ny, P, p0, sH + 3 * ny * ppc, t.cheb, t.tw_cheb,
-                       pb.R + (size_t)b * 3 * ny * P + p0);
-      analysed = true;
-    }
-  }
-  if (!analysed) {
-    constexpr int KN = (2 * MH + 3) / 4;  // n values per thread
-    const int qd = r + 2 * c;             // n = qd + 4k, parity of n = r
-    const RN* cheb = cheb_table<RN>(t);
-    const RN sg = r ? (RN)-1.0 : (RN)1.0;
-    for (int f = 2; f >= 0; --f) {
-      CN acc[KN];
-      analysis_sums<RN, KN>(sN + (size_t)f * ny * ppc + pl, ppc, N, ny, cheb, qd, 4, sg, acc);
-      __syncthreads();
-#pragma unroll
-      for (int k = 0; k < KN; ++k) {
-        const int n = qd + 4 * k;
-        if (n <= N) sN[((size_t)f * ny + n) * ppc + pl] = acc[k];
-      }
-    }
-    __syncthreads();
-  }
-
-  if constexpr (TOP == 0) {
-    // ---- implicit solves (no barrier below)
-    const int p = p0 + pl;
-    if (p >= P) return;
-    if (p / g.nxh == g.nz / 2) return;  // Nyquist row stays zero
-    const CN* Hx = sN + pl;
-    const CN* Hy = Hx + ny * ppc;
-    const CN* Hz = Hy + ny * ppc;
-    const size_t base = 2 * ((size_t)b * ny * P + p) + r;  // component r of element n at base + 2 P n
-    const CompT<RN> HGr = kStageHG ? CompT<RN>{reinterpret_cast<RN*>(sHGt) + 2 * pl + r, 2 * ppc}
-                                   : CompT<RN>{reinterpret_cast<RN*>(pb.HGP) + base, 2 * P};
-    const CompT<RN> HVr = kStageHV ? CompT<RN>{reinterpret_cast<RN*>(sHVt) + 2 * pl + r, 2 * ppc}
-                                   : CompT<RN>{reinterpret_cast<RN*>(pb.HVP) + base, 2 * P};
-    // The class c is uniform over each warp for tiles of 16 or more modes, so
-    // for up to 65 nodes (MH <= 33) the solve is compiled once per class: every
-    // parity-dependent factor (2 (n + 1), n^2, the row bounds) becomes a
-    // constant.  Larger buckets keep one run-time class (their unrolled code
-    // would double).  The arithmetic is the same either way: the factors are
-    // exact small integers and every fused operation is pinned.
-    auto solve = [&](auto cls) {
-      post_solve_noslip<MH, RN, false>(nullptr, 0, cls, g, pb, t, sc, b, p, r, Hx, Hy, Hz, ppc, HGr, HVr);
-    };
-    if constexpr (MH <= 33) {
-      if (c == 0) solve(std::integral_constant<int, 0>{});
-      else solve(std::integral_constant<int, 1>{});
-    } else {
-      solve(c);
-    }
-  } else {
-    // ---- implicit solves under a free-slip top, in two closures (omega_y or
-    // the mean flow, then v), each closed by the pair of class threads
-    // (c, 1 - c) of a (mode, component), neighbouring lanes that exchange
-    // their sums by shuffles; every lane of the warp takes part in both
-    // exchanges
-    const int p = p0 + pl;
-    const int pc = min(p, P - 1);
-    const int row = pc / g.nxh, ix = pc % g.nxh;
-    const bool live = p < P && row != g.nz / 2;
-    const bool mean = p == 0;
-    const double cc = sc.alpha / sc.beta;
-    const double* rowc = t.tau.rowc;
-    const CN* Hx = sN + pl;
-    const CN* Hy = Hx + ny * ppc;
-    const CN* Hz = Hy + ny * ppc;
-    auto comp = [](auto z, int qq) { return qq == 0 ? z.x : z.y; };
-    auto helm = [&](int sig) { return TabSm{t.tau.helm + (size_t)(sc.k * 2 + sig) * 4 * Mh * P + pc, Mh, P}; };
-    auto helm_isq = [&](int sig) { return t.tau.helm_isq[(size_t)(sc.k * 2 + sig) * P + pc]; };
-    auto qs = [&](int sig, int w) { return t.tau.helm_top[((size_t)(sc.k * 2 + sig) * 2 + w) * P + pc]; };
-    auto vs = [&](int sig, int w) { return t.tau.vh_top[((size_t)(sc.k * 2 + sig) * 2 + w) * P + pc]; };
-    const size_t base = 2 * ((size_t)b * ny * P + pc) + r;  // component r of element n at base + 2 P n
-    const double sgn = (r == 0) ? -1.0 : 1.0;
-    RegArr<MH> f;
-    // first closure: the mean mode (U for r = 0, W for r = 1) on parity c, or
-    // omega_y on parity 1 - c
-    {
-      const int sig = mean ? c : 1 - c;
-      const int M = (N - sig) / 2 + 1;
-      double mine[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-      if (live) {
-        if (mean) {
-          mean_open_affine<MH, RN>(f, N, ny, ppc, sig, (r == 0 ? pb.UM : pb.WM) + (size_t)b * ny,
-                                   (r == 0 ? pb.HXP : pb.HZP) + (size_t)b * ny, (r == 0) ? Hx : Hz, cc, sc, helm(sig),
-                                   rowc, mine);
-        } else {
-          const CompS Gc{reinterpret_cast<double*>(pb.G) + base, 2 * P};
-          const CompT<RN> HGc{reinterpret_cast<RN*>(pb.HGP) + base, 2 * P};
-          const CompT<RN> HGr = kStageHG ? CompT<RN>{reinterpret_cast<RN*>(sHGt) + 2 * pl + r, 2 * ppc} : HGc;
-          omega_open_affine<MH, RN>(f, N, ny, ppc, sig, Gc, HGr, HGc, Hx, Hz, r, sgn, t.kx[ix], t.kz[row], cc, sc,
-                                    helm(sig), rowc, mine);
-        }
-      }
-      // the mate (other class, same mode and component) is the neighbouring lane
-      double se[6], so[6];
-#pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        const double other = __shfl_xor_sync(0xffffffffu, mine[k], 1);
-        se[k] = sig == 0 ? mine[k] : other;
-        so[k] = sig == 0 ? other : mine[k];
-      }
-      if (live) {
-        double xe, xo, fc = 0.0;
-        if (mean && r == 0) {
-          const double* u1 = t.tau.u1 + (size_t)sc.k * Mh;
-          const TabSm He = helm(0);
-          double us = 0.0, u2 = 0.0, uw = 0.0, wq = 0.0;
-          for (int i = 0; i < N / 2 + 1; ++i) {
-            const double n = 2 * i, w = 2.0 / (1.0 - n * n);
-            us += u1[i];
-            u2 = fma_rn(n * n, u1[i], u2);
-            uw = fma_rn(w, u1[i], uw);
-            wq = fma_rn(w, i == 0 ? 1.0 : He.Q(i), wq);
-          }
-          close_free_slip_mean(se, so, qs(0, 0), qs(1, 0), qs(0, 1), qs(1, 1), wq, us, u2, uw, cc, sc.flux, &xe,
-                               &xo, &fc);
-        } else {
-          close_neumann_top(se, so, qs(0, 0), qs(1, 0), qs(0, 1), qs(1, 1), cc, &xe, &xo);
-        }
-        tau_close<MH>(N, sig, f, helm(sig), sig == 0 ? xe : xo);
-        if (mean) {
-          double* X = (r == 0 ? pb.UM : pb.WM) + (size_t)b * ny;
-#pragma unroll
-          for (int i = 0; i < MH; ++i)
-            if (i < M) {
-              const int n = 2 * i + sig;
-              double v = fma_rn(-cc, X[n], f[i]);
-              if (r == 0 && sig == 0) v = fma_rn(fc, t.tau.u1[(size_t)sc.k * Mh + i], v);
-              X[n] = v;
-            }
-        } else {
-          const CompS Gc{reinterpret_cast<double*>(pb.G) + base, 2 * P};
-#pragma unroll
-          for (int i = 0; i < MH; ++i)
-            if (i < M) {
-              const int n = 2 * i + sig;
-              Gc[n] = fma_rn(-cc, Gc[n], f[i]);
-            }
-        }
-      }
-    }
-    // second closure: v on parity c (every mode but the mean)
-    {
-      const int sig = c;
-      const int M = (N - sig) / 2 + 1;
-      double mine[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-      const bool on = live && !mean;
-      const CompS Vc{reinterpret_cast<double*>(pb.V) + base, 2 * P};
-      if (on) {
-        const double kx = t.kx[ix], kz = t.kz[row], k2 = kx * kx + kz * kz;
-        const CompT<RN> HVc{reinterpret_cast<RN*>(pb.HVP) + base, 2 * P};
-        const CompT<RN> HVr = kStageHV ? CompT<RN>{reinterpret_cast<RN*>(sHVt) + 2 * pl + r, 2 * ppc} : HVc;
-        const size_t vo = (size_t)b * P + pc;
-        const double vw =
-            fma_rn(sc.theta, comp(pb.vw_new[vo], r) - comp(pb.vw_old[vo], r), comp(pb.vw_old[vo], r));
-        const TabSm TP{t.tau.pois + (size_t)sig * 4 * Mh * P + pc, Mh, P};
-        v_open_part<MH, RN>(f, N, ny, ppc, sig, Vc, HVr, HVc, Hx, Hy, Hz, r, sgn, kx, kz, k2, cc, sc, helm(sig),
-                            helm_isq(sig), TP, t.tau.pois_isq[(size_t)sig * P + pc], vw, rowc, mine);
-      }
-      double se[6], so[6];
-#pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        const double other = __shfl_xor_sync(0xffffffffu, mine[k], 1);
-        se[k] = sig == 0 ? mine[k] : other;
-        so[k] = sig == 0 ? other : mine[k];
-      }
-      if (on) {
-        double ce, co;
-        close_free_slip_v(se, so, vs(0, 0), vs(1, 0), vs(0, 1), vs(1, 1), cc, &ce, &co);
-        const double cI = sig == 0 ? ce : co;
-        const double* vh = t.tau.vh + (size_t)(sc.k * 2 + sig) * Mh * P + pc;
-#pragma unroll
-        for (int i = 0; i < MH; ++i)
-          if (i < M) {
-            const int n = 2 * i + sig;
-            Vc[n] = fma_rn(-cc, Vc[n], fma_rn(cI, vh[(size_t)i * P], f[i]));
-          }
-      }
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// The implicit half for more than 65 nodes (no-slip top), in two launches.
-// One parity of one unknown then holds up to 101 coefficients, more than a
-// thread's registers next to the rest of the solve, and the node tile of H
-// (3 ny ppc values) would leave one or two CTAs per SM.  So:
-//   stage_post_analysis_kernel: the Chebyshev analysis of H, a tile of modes
-//     at a time, written over the nodal values in place (a CTA reads all the
-//     nodes of its modes before it writes their coefficients);
-//   stage_post_wide_kernel: one thread per (mode, class, component) as in the
-//     batched form, reading the coefficients of H from global memory and
-//     keeping its array of coefficients in a column of shared memory.
-// The per-output arithmetic of both halves is that of the batched form.
+// Chebyshev analysis of H by direct sums, for the orders without a register
+// cosine transform: a tile of modes at a time, coefficients over the nodal
+// values in place (a CTA reads all the nodes of its modes before it writes
+// their coefficients).
 // ---------------------------------------------------------------------------
 template <typename RN, int MH>
 __global__ void __launch_bounds__(256) stage_post_analysis_kernel(Grid g, int B, PencilBufs pb, DevTables t,
@@ -1920,20 +720,6 @@ __global__ void __launch_bounds__(256) stage_post_analysis_kernel(Grid g, int B,
   const int tid = threadIdx.x, nt = blockDim.x;
   pdl_wait_then_release();  // H comes from the nonlinear term
   CN* hb = hn + (size_t)b * 3 * ny * P;
-  constexpr int NF = 2 * (MH - 1);
-  if constexpr (std::is_same<RN, double>::value && ct_plan_ok(NF)) {
-    if (N == NF) {
-      // FFT form over the three fields of the tile, coefficients straight to hn
-      double2* X = reinterpret_cast<double2*>(smem_raw);  // [3][ny][ppc]
-      for (int w = tid; w < 3 * ny * ppc; w += nt) {
-        const int pl = w % ppc, fn = w / ppc;
-        X[w] = hb[(size_t)fn * P + min(p0 + pl, P - 1)];
-      }
-      __syncthreads();
-      analysis_fft<NF>(X, ppc, ny, P, p0, X + 3 * ny * ppc, t.cheb, t.tw_cheb, hb + p0);
-      return;
-    }
-  }
   // direct sums, one field at a time: thread (mode pl, group gq of 8) forms
   // the coefficients n = gq + 8 k
   constexpr int KN = (2 * MH + 7) / 8;
@@ -1963,38 +749,6 @@ __global__ void __launch_bounds__(256) stage_post_analysis_kernel(Grid g, int B,
   }
 }
 
-template <typename RN, int MH>
-__global__ void __launch_bounds__(64) stage_post_wide_kernel(Grid g, int B, PencilBufs pb, DevTables t,
-                                                             const typename cpx<RN>::T* __restrict__ hc,
-                                                             StageCoef sc, int ppc) {
-  extern __shared__ __align__(16) double sarr[];  // [MH][blockDim.x]
-  using CN = typename cpx<RN>::T;
-  const int P = g.P, ny = g.ny;
-  const int p0 = blockIdx.x * ppc;
-  const int b = blockIdx.y;
-  if (pb.active && !pb.active[b]) return;
-  pdl_wait_then_release();  // the coefficients of H come from the analysis
-  const int tid = threadIdx.x;
-  const int r = tid & 1, pl = (tid >> 1) % ppc, c = tid / (2 * ppc);
-  const int p = p0 + pl;
-  if (p >= P) return;  // no barrier in this kernel
-  if (p / g.nxh == g.nz / 2) return;  // Nyquist row stays zero
-  const CN* Hx = hc + (size_t)b * 3 * ny * P + p;
-  const CN* Hy = Hx + (size_t)ny * P;
-  const CN* Hz = Hy + (size_t)ny * P;
-  const size_t base = 2 * ((size_t)b * ny * P + p) + r;
-  const CompT<RN> HGr{reinterpret_cast<RN*>(pb.HGP) + base, 2 * P};
-  const CompT<RN> HVr{reinterpret_cast<RN*>(pb.HVP) + base, 2 * P};
-  post_solve_noslip<MH, RN, true>(sarr + tid, (int)blockDim.x, c, g, pb, t, sc, b, p, r, Hx, Hy, Hz, P, HGr, HVr);
-}
-
-// modes per CTA of the analysis half: 32 with direct sums (256 threads), 8
-// with the FP64 FFT form (three fields of the tile in shared memory)
-template <typename RN, int MH>
-constexpr int post_analysis_ppc() {
-  return (std::is_same<RN, double>::value && ct_plan_ok(2 * (MH - 1))) ? 8 : 32;
-}
-
 // ---------------------------------------------------------------------------
 // per-MH launchers, instantiated in the stage_mh*.cu translation units
 // ---------------------------------------------------------------------------
@@ -2008,46 +762,27 @@ cudaError_t pre_mh(const Grid& g, int B, const PencilBufs& pb, const DevTables& 
                                         st, g, B, pb, t, q, ppc);
 }
 
-template <typename RN, int MH, int TOP>
+template <typename RN, int MH>
 cudaError_t post_mh(const Grid& g, int B, const PencilBufs& pb, const DevTables& t,
                            const typename cpx<RN>::T* h, const StageCoef& sc, int ppc, size_t smem,
                            cudaStream_t st) {
   static SmemLimit lim;
-  const cudaError_t e = raise_smem_limit(stage_post_kernel<RN, MH, TOP>, &lim, smem);
+  const cudaError_t e = raise_smem_limit(stage_post_kernel<RN, MH>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(RN) == 4>(stage_post_kernel<RN, MH, TOP>, dim3((g.P + ppc - 1) / ppc, B),
-                                        dim3(8 * post_tile_lanes<TOP>() * ppc), smem, st, g, B, pb, t, h, sc, ppc);
+  return launch_pdl_if<sizeof(RN) == 4>(stage_post_kernel<RN, MH>, dim3((g.P + ppc - 1) / ppc, B),
+                                        dim3(8 * kPostTileLanes * ppc), smem, st, g, B, pb, t, h, sc, ppc);
 }
 
-template <typename RN, int MH, int TOP>
-cudaError_t post_batched_mh(const Grid& g, int B, const PencilBufs& pb, const DevTables& t,
-                                   const typename cpx<RN>::T* h, const StageCoef& sc, int ppc, size_t smem,
-                                   cudaStream_t st) {
-  using CN = typename cpx<RN>::T;
-  if constexpr (TOP == 0 && MH > 33) {
-    // two launches; the analysis replaces the nodal values of H, which no
-    // later kernel of the stage reads, by their coefficients
-    constexpr int apc = post_analysis_ppc<RN, MH>();
-    const size_t sa = std::is_same<RN, double>::value && apc == 8
-                          ? ((size_t)3 * g.ny + 6) * apc * sizeof(double2)
-                          : (size_t)g.ny * apc * sizeof(CN);
-    const int na = apc == 8 ? 128 : 8 * apc;
-    static SmemLimit lim_a, lim_w;
-    cudaError_t e = raise_smem_limit(stage_post_analysis_kernel<RN, MH>, &lim_a, sa);
-    if (e != cudaSuccess) return e;
-    if ((e = raise_smem_limit(stage_post_wide_kernel<RN, MH>, &lim_w, smem)) != cudaSuccess) return e;
-    e = launch_pdl_if<sizeof(RN) == 4>(stage_post_analysis_kernel<RN, MH>, dim3((g.P + apc - 1) / apc, B), dim3(na),
-                                       sa, st, g, B, pb, t, const_cast<CN*>(h), apc);
-    if (e != cudaSuccess) return e;
-    return launch_pdl_if<sizeof(RN) == 4>(stage_post_wide_kernel<RN, MH>, dim3((g.P + ppc - 1) / ppc, B),
-                                          dim3(4 * ppc), smem, st, g, B, pb, t, h, sc, ppc);
-  } else {
-    static SmemLimit lim;
-    const cudaError_t e = raise_smem_limit(stage_post_batched_kernel<RN, MH, TOP>, &lim, smem);
-    if (e != cudaSuccess) return e;
-    return launch_pdl_if<sizeof(RN) == 4>(stage_post_batched_kernel<RN, MH, TOP>, dim3((g.P + ppc - 1) / ppc, B),
-                                          dim3(4 * ppc), smem, st, g, B, pb, t, h, sc, ppc);
-  }
+template <typename RN, int MH>
+cudaError_t analysis_mh(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, typename cpx<RN>::T* h,
+                        cudaStream_t st) {
+  constexpr int ppc = 32;  // 8 threads per mode
+  const size_t smem = (size_t)g.ny * ppc * sizeof(typename cpx<RN>::T);
+  static SmemLimit lim;
+  const cudaError_t e = raise_smem_limit(stage_post_analysis_kernel<RN, MH>, &lim, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl_if<sizeof(RN) == 4>(stage_post_analysis_kernel<RN, MH>, dim3((g.P + ppc - 1) / ppc, B),
+                                        dim3(8 * ppc), smem, st, g, B, pb, t, h, ppc);
 }
 
 }  // namespace chdns
@@ -2061,25 +796,15 @@ cudaError_t post_batched_mh(const Grid& g, int B, const PencilBufs& pb, const De
   template cudaError_t pre_mh<float, MH>(const Grid&, int, const PencilBufs&, const DevTables&, float2*, int,    \
                                          size_t, cudaStream_t);                                                \
   }
-#define CH_STAGE_POST_TOP(MH, TOP)                                                                             \
+#define CH_STAGE_POST(MH)                                                                                      \
   namespace chdns {                                                                                            \
-  template cudaError_t post_mh<double, MH, TOP>(const Grid&, int, const PencilBufs&, const DevTables&,          \
-                                                const double2*, const StageCoef&, int, size_t, cudaStream_t);  \
-  template cudaError_t post_mh<float, MH, TOP>(const Grid&, int, const PencilBufs&, const DevTables&,           \
-                                               const float2*, const StageCoef&, int, size_t, cudaStream_t);    \
+  template cudaError_t post_mh<double, MH>(const Grid&, int, const PencilBufs&, const DevTables&, const double2*, \
+                                           const StageCoef&, int, size_t, cudaStream_t);                       \
+  template cudaError_t post_mh<float, MH>(const Grid&, int, const PencilBufs&, const DevTables&, const float2*,  \
+                                          const StageCoef&, int, size_t, cudaStream_t);                        \
+  template cudaError_t analysis_mh<double, MH>(const Grid&, int, const PencilBufs&, const DevTables&, double2*,  \
+                                               cudaStream_t);                                                  \
+  template cudaError_t analysis_mh<float, MH>(const Grid&, int, const PencilBufs&, const DevTables&, float2*,    \
+                                              cudaStream_t);                                                   \
   }
-#define CH_STAGE_POST_BATCHED_TOP(MH, TOP)                                                                     \
-  namespace chdns {                                                                                            \
-  template cudaError_t post_batched_mh<double, MH, TOP>(const Grid&, int, const PencilBufs&, const DevTables&,  \
-                                                        const double2*, const StageCoef&, int, size_t,         \
-                                                        cudaStream_t);                                         \
-  template cudaError_t post_batched_mh<float, MH, TOP>(const Grid&, int, const PencilBufs&, const DevTables&,   \
-                                                       const float2*, const StageCoef&, int, size_t,           \
-                                                       cudaStream_t);                                          \
-  }
-// no-slip upper wall (TOP = 0) for every bucket; the free-slip top (TOP = 1)
-// is instantiated for MH <= 33 (ny <= 65) in translation units of its own
-#define CH_STAGE_POST(MH) CH_STAGE_POST_TOP(MH, 0)
-#define CH_STAGE_POST_BATCHED(MH) CH_STAGE_POST_BATCHED_TOP(MH, 0)
-#define CH_STAGE_INSTANTIATE(MH) CH_STAGE_PRE(MH) CH_STAGE_POST(MH) CH_STAGE_POST_BATCHED(MH)
-#define CH_STAGE_INSTANTIATE_OPEN(MH) CH_STAGE_POST_TOP(MH, 1) CH_STAGE_POST_BATCHED_TOP(MH, 1)
+#define CH_STAGE_INSTANTIATE(MH) CH_STAGE_PRE(MH) CH_STAGE_POST(MH)

@@ -1,6 +1,7 @@
-// Per-MH launchers of the fused stage kernels.  MH bounds the per-thread
-// register arrays (unknowns of one parity); each bucket is compiled in its own
-// translation unit (stage_mh*.cu) so that the instantiations build in parallel.
+// Per-MH and per-order launchers of the stage kernels.  MH bounds the
+// per-thread register arrays (unknowns of one parity); each bucket and each
+// group of Chebyshev orders is compiled in its own translation unit
+// (stage_mh*.cu, stage_dct_*.cu) so that the instantiations build in parallel.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -13,12 +14,21 @@ namespace chdns {
 template <typename RN, int MH>
 cudaError_t pre_mh(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, typename cpx<RN>::T* q, int ppc,
                    size_t smem, cudaStream_t st);
-template <typename RN, int MH, int TOP>
+template <typename RN, int MH>
 cudaError_t post_mh(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, const typename cpx<RN>::T* h,
                     const StageCoef& sc, int ppc, size_t smem, cudaStream_t st);
-template <typename RN, int MH, int TOP>
-cudaError_t post_batched_mh(const Grid& g, int B, const PencilBufs& pb, const DevTables& t,
-                            const typename cpx<RN>::T* h, const StageCoef& sc, int ppc, size_t smem,
-                            cudaStream_t st);
+template <typename RN, int MH>
+cudaError_t analysis_mh(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, typename cpx<RN>::T* h,
+                        cudaStream_t st);
+// register cosine transforms (stage_dct.cuh)
+template <typename RN, int N>
+cudaError_t pre_dct_n(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, typename cpx<RN>::T* q,
+                      cudaStream_t st);
+template <typename RN, int N>
+cudaError_t analysis_dct_n(const Grid& g, int B, const PencilBufs& pb, typename cpx<RN>::T* h, cudaStream_t st);
+// implicit solves of handles with many modes (stage_solve.cu)
+template <typename RN>
+cudaError_t launch_stage_solve(const Grid& g, int B, const PencilBufs& pb, const DevTables& t,
+                               const typename cpx<RN>::T* h, const StageCoef& sc, cudaStream_t st);
 
 }  // namespace chdns
