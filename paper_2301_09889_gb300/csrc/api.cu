@@ -560,11 +560,13 @@ int build_tables(ch_env* env) {
   RC(dupload(env, &env->tab.tau.helm_f, helm_f));
   RC(dupload(env, &env->tab.tau.pois_f, pois_f));
   {
-    std::vector<double> n2(ny), wint(ny, 0.0);
+    std::vector<double> n1(ny), n2(ny), wint(ny, 0.0);
     for (int n = 0; n < ny; ++n) {
+      n1[n] = 2.0 * (n + 1);
       n2[n] = (double)n * n;
       if (n % 2 == 0) wint[n] = 2.0 / (1.0 - (double)n * n);
     }
+    RC(dupload(env, &env->tab.tau.n1, n1));
     RC(dupload(env, &env->tab.tau.n2, n2));
     RC(dupload(env, &env->tab.tau.wint, wint));
   }
@@ -733,6 +735,9 @@ StageCoef stage_coef(const ch_env* env, int k, double theta) {
   sc.nu = env->nu;
   sc.theta = theta;
   sc.flux = 2.0;
+  sc.cc = sc.alpha / sc.beta;
+  sc.dgaf = (float)(sc.dt * sc.gamma);
+  sc.dzef = (float)(sc.dt * sc.zeta);
   sc.k = k;
   return sc;
 }
@@ -1126,12 +1131,10 @@ int env_create(const ch_params_t* p, ch_env_t** out) {
     env->ppc_pre = 8;
     while (env->ppc_pre > 1 && stage_pre_smem(g, env->ppc_pre, sizeof(double2)) > (size_t)smem_max) env->ppc_pre /= 2;
     if (stage_post_smem(g, env->tab.tau.Mh, env->ppc_post) > (size_t)smem_max) return fail(CH_ERR_UNSUPPORTED);
-    // The batched form of stage_post runs four threads per mode, each with
-    // the same work; it pays once the batch supplies at least two such warps
-    // per SM sub-partition (B P / 8 >= 2 x 4 x SMs).
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return fail(CH_ERR_CUDA);
-    if ((size_t)B * P >= (size_t)64 * sms) {
+    // The two-launch form runs eight threads per mode; from 256 modes on it
+    // beats the four-lane scans (64x65x64 FP64: 226 against 338 us per RK step,
+    // 32x65x32 FP64: 192 against 197, 128x129x128 mixed: 463 against 1330).
+    if ((size_t)B * P >= (size_t)256) {
       env->post_batched = true;
       env->ppc_post = 16;
     }

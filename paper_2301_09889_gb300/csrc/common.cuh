@@ -61,6 +61,18 @@ __host__ __device__ __forceinline__ float mul_rn(float a, float b) {
 #endif
 }
 
+// float -> double by integer operations on the encoding: the conversion
+// instruction occupies the FP64 pipe like an FP64 operation (17 of 19 cycles
+// per warp and SM), and the implicit solves are bound by that pipe.  Exact for
+// zeros, normal numbers, infinities and NaN; subnormal floats become zero.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+  unsigned hi = (a >> 3) + (a >= 0x7f800000u ? 0x70000000u : 0x38000000u), lo = u << 29;
+  if (a < 0x00800000u) hi = lo = 0u;
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)lo);
+}
+__device__ __forceinline__ double widen(double f) { return f; }
+
 #define CH_CPX_OPS(C, R)                                                                   \
   __host__ __device__ __forceinline__ C operator+(C a, C b) { return mk(a.x + b.x, a.y + b.y); } \
   __host__ __device__ __forceinline__ C operator-(C a, C b) { return mk(a.x - b.x, a.y - b.y); } \
@@ -507,6 +519,7 @@ struct TauTables {
   const double* helm_f;    // [3][2][7 or 8][Mh][P] eA, eB, eC, h, b, W, E1 (, W2) per stage, parity
   const double* pois_f;    // [2][6][Mh][P]     eA, eB, eC, h, b, W
   const double* n2;        // [ny] n^2
+  const double* n1;        // [ny] 2 (n + 1)
   const double* wint;      // [ny] int T_n dy = 2 / (1 - n^2) of the even n, 0 of the odd
   // free-slip top (top_bc = 1): the wall rows couple the parities
   const double* helm_top;  // [3][2][2][P]      sum Q, sum n^2 Q of the stage's factorisation, per parity
@@ -518,6 +531,8 @@ struct TauTables {
 
 struct StageCoef {
   double alpha, beta, gamma, zeta, dt, nu, theta, flux;
+  double cc;                  // alpha / beta
+  float dgaf, dzef;           // dt gamma, dt zeta in FP32
   int k;
 };
 

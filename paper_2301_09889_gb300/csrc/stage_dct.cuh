@@ -53,14 +53,32 @@ template <typename RN, int N, int NF>
 __global__ void __launch_bounds__(64 * NF, ctas_of(pre_dct_regs<RN, N>(), 64 * NF)) stage_pre_dct_kernel(Grid g, PencilBufs pb, DevTables t,
                                                                     typename cpx<RN>::T* __restrict__ q) {
   constexpr int H = N / 2;
+  // FP32 lines: v and omega_y of the tile are rounded to FP32 once, into shared
+  // memory (a conversion costs as much as an FP64 operation, and every line
+  // reads two of the columns); FP64 lines read them in place
+  constexpr bool kTile = sizeof(RN) == 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int P = g.P, ny = N + 1;
   const int lane = threadIdx.x & 31, fl = threadIdx.x / 64, half = (threadIdx.x / 32) & 1, f = blockIdx.z * NF + fl;
+  RN* tile = reinterpret_cast<RN*>(smem_raw);  // [v, omega_y][ny][32], until the partial sums take its place
   RN* part = reinterpret_cast<RN*>(smem_raw) + fl * (N + 1) * 32;  // [E_0 .. E_H, O_0 .. O_{H-1}][32]
   const int p = blockIdx.x * 16 + (lane >> 1), r = lane & 1;
   const int b = blockIdx.y;
   if (pb.active && !pb.active[b]) return;
   pdl_wait_then_release();  // v, omega_y come from the previous stage
+  if constexpr (kTile) {
+    const size_t c0 = 2 * ((size_t)b * ny * P + blockIdx.x * 16) + lane;
+#pragma unroll 4
+    for (int n = threadIdx.x / 32; n < 2 * ny; n += 2 * NF) {
+      const int m = n < ny ? n : n - ny;
+      const double* src = reinterpret_cast<const double*>(n < ny ? pb.V : pb.G) + 2 * (size_t)P * m + c0;
+      // the columns of mode 0 hold W and U instead of omega_y
+      if (p == 0 && n >= ny) src = (r == 0 ? pb.WM : pb.UM) + (size_t)b * ny + m;
+      tile[n * 32 + lane] = p < P ? (RN)*src : (RN)0;
+    }
+    __syncthreads();
+  }
+  RN x[H + 1];
   if (p < P) {
     const int row = p / g.nxh, ix = p % g.nxh;
     const bool mean = p == 0, gen = !mean && row != g.nz / 2;
@@ -87,10 +105,12 @@ __global__ void __launch_bounds__(64 * NF, ctas_of(pre_dct_regs<RN, N>(), 64 * N
       if (f == 5) { cD = -ik2 * kx; cS = ik2 * kz; cV = sg * kx; }
     }
     const bool liveS = gen || (mean && !own && r == 0);
-    auto V = [&](int n) { return gen ? (RN)Vp[(size_t)n * ss] : (RN)0; };
-    auto S = [&](int n) { return liveS ? (RN)Sp[(size_t)n * ss] : (RN)0; };
+    const RN* Vt = tile + (lane ^ 1);
+    const RN* St = tile + (f == 1 ? 0 : ny * 32) + (own ? lane : !mean ? lane ^ 1 : f == 0 || f == 5 ? 1 : 0);
+    auto V = [&](int n) { return !gen ? (RN)0 : kTile ? Vt[n * 32] : (RN)Vp[(size_t)n * ss]; };
+    auto S = [&](int n) { return !liveS ? (RN)0 : kTile ? St[n * 32] : (RN)Sp[(size_t)n * ss]; };
     // coefficients of one parity, n = 2 i + par, from the top down
-    auto coefs = [&](auto& x, int par, int count) {
+    auto coefs = [&](int par, int count) {
       if (own) {
 #pragma unroll
         for (int i = count - 1; i >= 0; --i) x[i] = S(2 * i + par);
@@ -118,19 +138,21 @@ __global__ void __launch_bounds__(64 * NF, ctas_of(pre_dct_regs<RN, N>(), 64 * N
         }
       }
     };
-    if (half == 0) {
-      RN e[H + 1];
-      coefs(e, 0, H + 1);
-      dct1<H, RN>(e);
+    if (half == 0) coefs(0, H + 1);
+    else coefs(1, H);
+  }
+  if constexpr (kTile) __syncthreads();
+  if (half == 0) {
+    dct1<H, RN>(x);
 #pragma unroll
-      for (int j = 0; j <= H; ++j) part[j * 32 + lane] = e[j];
-    } else {
-      RN o[H];
-      coefs(o, 1, H);
-      dct2<H, RN>(o);
+    for (int j = 0; j <= H; ++j) part[j * 32 + lane] = x[j];
+  } else {
+    RN o[H];
 #pragma unroll
-      for (int j = 0; j < H; ++j) part[(H + 1 + j) * 32 + lane] = o[j];
-    }
+    for (int j = 0; j < H; ++j) o[j] = x[j];
+    dct2<H, RN>(o);
+#pragma unroll
+    for (int j = 0; j < H; ++j) part[(H + 1 + j) * 32 + lane] = o[j];
   }
   __syncthreads();
   if (p >= P) return;

@@ -81,9 +81,11 @@ struct Blk {
 // Chebyshev-tau Dirichlet solve (tau_seq's rows) over a four-lane group.  On
 // entry f[k] holds r at i = i_of(q, k) (0 outside 0 .. M - 1); on return the
 // solution f_i, with the wall row sum_i f_i = wall.
-template <int MH, class Tab>
+// With DIAG, row j also takes diag[k] (a term whose stencil is its own value).
+template <int MH, bool DIAG = false, class Tab>
 __device__ __forceinline__ void tau_scan(int N, int ny, int sig, double (&f)[Blk<MH>::K], const Tab& T, double isq,
-                                         double wall, const double* __restrict__ rowc, int q) {
+                                         double wall, const double* __restrict__ rowc, int q,
+                                         const double* diag = nullptr) {
   constexpr int K = Blk<MH>::K;
   const int M = (N - sig) / 2 + 1;
   // neighbours across the block edges: r at hi + 1 (bottom of the lane above)
@@ -105,6 +107,7 @@ __device__ __forceinline__ void tau_scan(int N, int ny, int sig, double (&f)[Blk
       const int n = 2 * j + sig;
       double R = fma_rn(-rowc[ny + n], rj, mul_rn(rowc[n], rlo));
       if (j + 1 < M) R = fma_rn(rowc[2 * ny + n], r_up, R);
+      if (DIAG) R = R + diag[k];
       const double al = mul_rn(T.e(j), R);
       const double be = -T.h(j);
       f[k] = al;
@@ -300,7 +303,9 @@ __device__ __forceinline__ void v_scan(int N, int ny, int ppc, int sv, const VV&
   }
 }
 
-// mean flow of parity s over a four-lane group (mean_solve)
+// mean flow of parity s over a four-lane group, solved for its increment
+// d = X^k - X^{k-1} (see stage_solve.cuh): right-hand side dt (...), and
+// (1 + c) beta dt nu X on the diagonal for (1 + c) D^2 X
 template <int MH, typename RN, class Tab>
 __device__ __forceinline__ void mean_scan(int N, int ny, int ppc, int s, int e, double* X, double* XP,
                                           const typename cpx<RN>::T* Hm, double cc, const StageCoef& sc,
@@ -308,12 +313,13 @@ __device__ __forceinline__ void mean_scan(int N, int ny, int ppc, int s, int e, 
                                           const double* __restrict__ u1, double u1_iflux, int q) {
   constexpr int K = Blk<MH>::K;
   const int M = (N - s) / 2 + 1;
-  double f[K];
+  double f[K], dg[K];
+  const double cb = (1.0 + cc) * sc.beta * sc.dt * sc.nu;
   double sum = 0.0, flux_old = 0.0;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     const int i = Blk<MH>::i_of(q, k);
-    f[k] = 0.0;
+    f[k] = dg[k] = 0.0;
     if (i >= 0 && i < M) {
       const int n = 2 * i + s;
       const double xn = X[n];
@@ -322,11 +328,12 @@ __device__ __forceinline__ void mean_scan(int N, int ny, int ppc, int s, int e, 
       XP[n] = hv;
       sum += xn;
       if (s == 0) flux_old = fma_rn(2.0 / (1.0 - (double)n * n), xn, flux_old);
-      f[k] = fma_rn(1.0 + cc, xn, mul_rn(sc.dt, fma_rn(sc.gamma, hv, mul_rn(sc.zeta, hp))));
+      f[k] = mul_rn(sc.dt, fma_rn(sc.gamma, hv, mul_rn(sc.zeta, hp)));
+      dg[k] = mul_rn(cb, xn);
     }
   }
   flux_old = scan4::lane_sum(flux_old);
-  tau_scan<MH>(N, ny, s, f, T, isq, mul_rn(cc, scan4::lane_sum(sum)), rowc, q);
+  tau_scan<MH, true>(N, ny, s, f, T, isq, -scan4::lane_sum(sum), rowc, q, dg);
   double fc = 0.0;
   if (e == 0 && s == 0) {
     double flux = 0.0;
@@ -335,14 +342,14 @@ __device__ __forceinline__ void mean_scan(int N, int ny, int ppc, int s, int e, 
       const int i = Blk<MH>::i_of(q, k);
       if (i >= 0 && i < M) flux = fma_rn(2.0 / (1.0 - 4.0 * (double)i * i), f[k], flux);
     }
-    fc = mul_rn(fma_rn(cc, flux_old, sc.flux) - scan4::lane_sum(flux), u1_iflux);
+    fc = mul_rn(sc.flux - flux_old - scan4::lane_sum(flux), u1_iflux);
   }
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     const int i = Blk<MH>::i_of(q, k);
     if (i >= 0 && i < M) {
       const int n = 2 * i + s;
-      double v = fma_rn(-cc, X[n], f[k]);
+      double v = X[n] + f[k];
       if (e == 0 && s == 0) v = fma_rn(fc, u1[i], v);
       X[n] = v;
     }

@@ -23,6 +23,12 @@
 // v_n itself (it integrates D^2 twice): row j takes E1_j v_j, E1 = (1 + c) e,
 // and the stencil of u = -(1 + c) k^2 v + dt (...), and no D^2 v is formed.
 //
+// The mean flow is solved for its increment d = X^k - X^{k-1} instead of
+// X' = X^k + c X^{k-1}: (D^2 - lam) d = -dt (...)/(beta dt nu) - (1 + c) D^2 X.
+// lam is large for the mean mode, so the solve of X' would return nearly
+// (1 + c) X through a system of condition ~ (N/2)^2; the increment's error is
+// smaller by |d| / |X|, and X carries most of the observation.
+//
 // No-slip walls: sum f' = c sum f_old per parity for omega_y, U, W; v' the
 // same plus the wall velocity, and the influence correction c_I vh that fixes
 // Dv.  Free-slip top (TOP = 1): the rows Df(+1) and f(-1) (omega_y, W), these
@@ -49,6 +55,52 @@ namespace chdns {
 template <int TOP> constexpr int solve_tabs() { return TOP ? 8 : 7; }  // eA, eB, eC, h, b, W, E1 (, W2)
 constexpr int kPoisTabs = 6;                                           // eA, eB, eC, h, b, W
 
+// dt gamma and dt zeta in the node precision
+template <typename RN>
+struct Coef3 {
+  RN dga, dze;
+};
+template <typename RN>
+__device__ __forceinline__ Coef3<RN> node_coef(const StageCoef& sc) {
+  if constexpr (sizeof(RN) == 4) return Coef3<RN>{sc.dgaf, sc.dzef};
+  else return Coef3<RN>{sc.dt * sc.gamma, sc.dt * sc.zeta};
+}
+
+// Rows i = M-1 .. 0 (down) or i0 .. M-1 (up) in order, the loads of a row D
+// rows ahead of its step.
+// The steady part is one basic block of D loads and D steps.
+template <int D, class Load, class Step>
+__device__ __forceinline__ void sweep_down(int top, int last, Load&& load, Step&& step) {
+  decltype(load(0)) ring[D];
+#pragma unroll
+  for (int k = 0; k < D; ++k) ring[k] = load(max(top - k, last));
+  int i = top;
+#pragma unroll 1
+  for (; i - 2 * D + 1 >= last; i -= D) {
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      const auto cur = ring[k];
+      ring[k] = load(i - k - D);
+      step(i - k, cur);
+    }
+  }
+  // fewer than 2 D rows left, the first D of them loaded
+  decltype(load(0)) rest[D > 1 ? D - 1 : 1];
+#pragma unroll
+  for (int k = 0; k < D - 1; ++k) rest[k] = load(max(i - k - D, last));
+#pragma unroll
+  for (int k = 0; k < D; ++k)
+    if (i - k >= last) step(i - k, ring[k]);
+#pragma unroll
+  for (int k = 0; k < D - 1; ++k)
+    if (i - k - D >= last) step(i - k - D, rest[k]);
+}
+template <int D, class Load, class Step>
+__device__ __forceinline__ void sweep_up(int first, int M, Load&& load, Step&& step) {
+  sweep_down<D>(M - 1, first, [&](int i) { return load(M - 1 + first - i); },
+                [&](int i, const auto& v) { step(M - 1 + first - i, v); });
+}
+
 // one row's table entries
 struct TabRow {
   double eA, eB, eC, h, W;
@@ -57,120 +109,195 @@ __device__ __forceinline__ TabRow tab_row(const double* __restrict__ T, size_t M
   return TabRow{__ldg(T + o), __ldg(T + MP + o), __ldg(T + 2 * MP + o), __ldg(T + 3 * MP + o), __ldg(T + 5 * MP + o)};
 }
 
-// Solve omega_y of parity sig of one (mode, component), or the mean flow in
-// the lanes of mode 0 (component 0: U at constant flow rate, 1: W).
+// what a thread's sweep down leaves for the closure
+struct Wall {
+  double sum = 0.0, sum2 = 0.0;  // sum P, sum n^2 P of the particular solution
+  double S0 = 0.0, S2 = 0.0;     // sum x, sum n^2 x of the old field
+  double wp = 0.0, wx = 0.0;     // int P, int x (mean flow, even parity)
+};
+
+struct Bw {
+  double b, w;
+};
+
+// omega_y of parity sig of one (mode, component): down
+template <typename RN, int TOP, int D>
+__device__ __forceinline__ Wall omega_down(double* f, const Grid& g, const PencilBufs& pb, const DevTables& t,
+                                           const StageCoef& sc, int b, int p, int r, int sig, const double* __restrict__ T,
+                                           const RN* __restrict__ hc) {
+  constexpr int NT = 64;
+  const size_t P = g.P, MP = (size_t)t.tau.Mh * P;
+  const int ny = g.ny, M = (g.N - sig) / 2 + 1, row = p / g.nxh, ix = p % g.nxh;
+  const double cc1 = 1.0 + sc.cc;
+  const double* __restrict__ n2 = t.tau.n2;
+  // element n of a component column: base + 2 P n
+  const size_t hP = 2 * P, base = 2 * ((size_t)b * ny * P + p) + r;
+  const double* G = reinterpret_cast<const double*>(pb.G) + base;
+  RN* HG = reinterpret_cast<RN*>(pb.HGP) + base;
+  const RN* hx = hc + 2 * ((size_t)b * 3 * ny * P + p) + 1 - r;
+  const RN* hz = hx + 2 * (size_t)ny * hP;
+  const RN sgn = r == 0 ? (RN)-1 : (RN)1, kx = sgn * (RN)t.kx[ix], kz = sgn * (RN)t.kz[row];
+  const Coef3<RN> nc = node_coef<RN>(sc);
+  struct In {
+    double x;
+    RN hx, hz, hp;
+    TabRow tb;
+    double W2;
+  };
+  Wall w;
+  double r1 = 0.0, r2 = 0.0, an = 0.0;
+  sweep_down<D>(
+      M - 1, 0,
+      [&](int i) {
+        In v;
+        const size_t n = 2 * i + sig, o = (size_t)min(i + 1, M - 1) * P;  // row i + 1 of the elimination
+        v.x = G[n * hP];
+        v.hx = __ldg(hx + n * hP);
+        v.hz = __ldg(hz + n * hP);
+        v.hp = HG[n * hP];
+        v.tb = tab_row(T, MP, o);
+        if (TOP) v.W2 = __ldg(T + 7 * MP + o);
+        return v;
+      },
+      [&](int i, const In& v) {
+        const size_t n = 2 * i + sig;
+        const RN hg = kz * v.hx - kx * v.hz;
+        HG[n * hP] = hg;
+        w.S0 += v.x;
+        if (TOP) w.S2 = fma(__ldg(n2 + n), v.x, w.S2);
+        const double r0 = fma(cc1, v.x, widen(nc.dga * hg + nc.dze * v.hp));
+        if (i + 1 < M) {
+          const double a = fma(-v.tb.h, an, fma(v.tb.eC, r2, fma(-v.tb.eB, r1, v.tb.eA * r0)));
+          f[(i + 1) * NT] = a;
+          w.sum = fma(v.tb.W, a, w.sum);
+          if (TOP) w.sum2 = fma(v.W2, a, w.sum2);
+          an = a;
+        }
+        r2 = r1;
+        r1 = r0;
+      });
+  return w;
+}
+
+// The mean flow (component 0: U, 1: W) of parity sig, in the lanes of mode 0:
+// down, for the increment.  X: coefficients, XP: previous plane means of H,
+// hm: its new ones (2 P apart).
 template <typename RN, int TOP>
+__device__ __forceinline__ Wall mean_down(double* f, const DevTables& t, const StageCoef& sc, int N, size_t P, int sig,
+                                       const double* __restrict__ T, const double* X, double* XP,
+                                       const RN* __restrict__ hm) {
+  constexpr int NT = 64;
+  const size_t MP = (size_t)t.tau.Mh * P;
+  const int M = (N - sig) / 2 + 1;
+  const double bdn = sc.beta * sc.dt * sc.nu;
+  Wall w;
+  double r1 = 0.0, r2 = 0.0, an = 0.0, x1 = 0.0;
+  struct In {
+    double x, hp, n2, wi;
+    RN h;
+    TabRow tb;
+    double E1, W2;
+  };
+  sweep_down<4>(
+      M - 1, 0,
+      [&](int i) {
+        In v;
+        const int n = 2 * i + sig;
+        const size_t o = (size_t)min(i + 1, M - 1) * P;
+        v.x = X[n];
+        v.hp = XP[n];
+        v.h = __ldg(hm + 2 * P * n);
+        v.wi = __ldg(t.tau.wint + n);
+        v.tb = tab_row(T, MP, o);
+        v.E1 = __ldg(T + 6 * MP + o);
+        if (TOP) {
+          v.n2 = __ldg(t.tau.n2 + n);
+          v.W2 = __ldg(T + 7 * MP + o);
+        }
+        return v;
+      },
+      [&](int i, const In& v) {
+        const double h = widen(v.h);
+        XP[2 * i + sig] = h;
+        w.S0 += v.x;
+        if (TOP) w.S2 = fma(v.n2, v.x, w.S2);
+        w.wx = fma(v.wi, v.x, w.wx);
+        const double r0 = sc.dt * fma(sc.gamma, h, sc.zeta * v.hp);
+        if (i + 1 < M) {
+          const double a = fma(v.E1, bdn * x1, fma(-v.tb.h, an, fma(v.tb.eC, r2, fma(-v.tb.eB, r1, v.tb.eA * r0))));
+          f[(i + 1) * NT] = a;
+          w.sum = fma(v.tb.W, a, w.sum);
+          if (TOP) w.sum2 = fma(v.W2, a, w.sum2);
+          an = a;
+        }
+        r2 = r1;
+        r1 = r0;
+        x1 = v.x;
+      });
+  if (TOP && sig == 0) {
+    double fp = 0.0;
+    sweep_up<4>(
+        1, M, [&](int i) { return Bw{__ldg(T + 4 * MP + (size_t)i * P), __ldg(t.tau.wint + 2 * i)}; },
+        [&](int i, const Bw& v) {
+          fp = fma(v.b, fp, f[i * NT]);
+          w.wp = fma(v.w, fp, w.wp);
+        });
+  }
+  return w;
+}
+
+// up: X <- X + d (+ the response u1 to the forcing of U)
+template <int TOP>
+__device__ __forceinline__ void mean_up(double* f, const DevTables& t, const StageCoef& sc, int N, size_t P, int sig,
+                                     bool forced, const double* __restrict__ T, double* X, double f0, double fc,
+                                     double wx) {
+  constexpr int NT = 64;
+  const size_t MP = (size_t)t.tau.Mh * P;
+  const int M = (N - sig) / 2 + 1;
+  double fp = f0, flux = t.tau.wint[0] * f0;
+  f[0] = f0;
+  sweep_up<4>(
+      1, M, [&](int i) { return Bw{__ldg(T + 4 * MP + (size_t)i * P), __ldg(t.tau.wint + 2 * i)}; },
+      [&](int i, const Bw& v) {
+        fp = fma(v.b, fp, f[i * NT]);
+        f[i * NT] = fp;
+        flux = fma(v.w, fp, flux);
+      });
+  if (TOP == 0) fc = (sc.flux - wx - flux) * t.tau.u1_iflux[sc.k];
+  if (!forced || sig != 0) fc = 0.0;
+  const double* u1 = t.tau.u1 + (size_t)sc.k * t.tau.Mh;
+  sweep_up<4>(
+      0, M, [&](int i) { return Bw{X[2 * i + sig], __ldg(u1 + i)}; },
+      [&](int i, const Bw& v) { X[2 * i + sig] = fma(fc, v.w, v.b + f[i * NT]); });
+}
+
+// Solve omega_y of parity sig of one (mode, component), or (MEAN) the mean flow
+// (component 0: U at constant flow rate, 1: W).
+template <typename RN, int TOP, int D, bool MEAN>
 __device__ __forceinline__ void solve_omega(double* f, double* xch, const Grid& g, const PencilBufs& pb,
                                             const DevTables& t, const StageCoef& sc, int b, int p, int r, int sig,
                                             bool live, const RN* __restrict__ hc) {
   constexpr int NT = 64;
   const size_t P = g.P, MP = (size_t)t.tau.Mh * P;
-  const int ny = g.ny, N = g.N, M = (N - sig) / 2 + 1, row = p / g.nxh, ix = p % g.nxh;
-  const bool mean = p == 0;
-  const double cc = sc.alpha / sc.beta;
+  const int ny = g.ny, M = (g.N - sig) / 2 + 1;
   const double* __restrict__ T = t.tau.helm_f + (size_t)(sc.k * 2 + sig) * solve_tabs<TOP>() * MP + p;
-  const double* __restrict__ n2 = t.tau.n2;
-  // column: value n at xp[n xs]; H: comp of two fields at ha[2 P n], hb[2 P n]
-  const size_t hP = 2 * P, base = 2 * ((size_t)b * ny * P + p) + r;
-  double* xp = mean ? (r == 0 ? pb.UM : pb.WM) + (size_t)b * ny : reinterpret_cast<double*>(pb.G) + base;
-  const size_t xs = mean ? 1 : hP;
-  double* XP = (r == 0 ? pb.HXP : pb.HZP) + (size_t)b * ny;
-  RN* HG = reinterpret_cast<RN*>(pb.HGP) + base;
-  const RN* H0 = hc + 2 * ((size_t)b * 3 * ny * P + p);
-  const RN* hx = mean ? H0 + (r == 0 ? 0 : 2 * (size_t)ny * hP) : H0 + 1 - r;
-  const RN* hz = H0 + 2 * (size_t)ny * hP + 1 - r;
-  const RN sgn = r == 0 ? (RN)-1 : (RN)1, kx = (RN)t.kx[ix], kz = (RN)t.kz[row];
-  const RN dtn = (RN)sc.dt, gan = (RN)sc.gamma, zen = (RN)sc.zeta;
-  double S0 = 0.0, S2 = 0.0, flux_old = 0.0, sum = 0.0, sum2 = 0.0, f0 = 0.0, fc = 0.0;
+  double* X = (r == 0 ? pb.UM : pb.WM) + (size_t)b * ny;
+  Wall w;
   if (live) {
-    struct In {
-      double x;
-      RN hx, hz, hp;
-      TabRow tb;
-      double W2;
-    };
-    auto load = [&](int i) {
-      In v;
-      const size_t n = 2 * i + sig;
-      v.x = xp[n * xs];
-      v.hx = __ldg(hx + n * hP);
-      v.hz = __ldg(hz + n * hP);
-      v.hp = HG[n * hP];
-      if (i + 1 < M) {
-        v.tb = tab_row(T, MP, (size_t)(i + 1) * P);
-        if (TOP) v.W2 = __ldg(T + 7 * MP + (size_t)(i + 1) * P);
-      }
-      return v;
-    };
-    double r1 = 0.0, r2 = 0.0, an = 0.0;
-    auto step = [&](int i, const In& v) {
-      const size_t n = 2 * i + sig;
-      double q;
-      if (mean) {
-        const double h = (double)v.hx, hp = XP[n];
-        XP[n] = h;
-        q = sc.dt * fma(sc.gamma, h, sc.zeta * hp);
-        if (sig == 0) flux_old = fma(t.tau.wint[n], v.x, flux_old);
-      } else {
-        const RN hg = sgn * (kz * v.hx - kx * v.hz);
-        HG[n * hP] = hg;
-        q = (double)(dtn * (gan * hg + zen * v.hp));
-      }
-      S0 += v.x;
-      if (TOP) S2 = fma(__ldg(n2 + n), v.x, S2);
-      const double r0 = fma(1.0 + cc, v.x, q);
-      if (i + 1 < M) {
-        const double a = fma(-v.tb.h, an, fma(v.tb.eC, r2, fma(-v.tb.eB, r1, v.tb.eA * r0)));
-        f[(i + 1) * NT] = a;
-        sum = fma(v.tb.W, a, sum);
-        if (TOP) sum2 = fma(v.W2, a, sum2);
-        an = a;
-      }
-      r2 = r1;
-      r1 = r0;
-    };
-    In u = load(M - 1), v = load(M - 2);
-    int i = M - 1;
-    for (; i >= 3; i -= 2) {
-      const In u1 = load(i - 2);
-      step(i, u);
-      const In v1 = load(i - 3);
-      step(i - 1, v);
-      u = u1;
-      v = v1;
-    }
-    // two or three rows left: i, i - 1 (and 0)
-    if (i == 2) {
-      const In w = load(0);
-      step(2, u);
-      step(1, v);
-      step(0, w);
+    if constexpr (MEAN) {
+      const RN* hm = hc + 2 * (size_t)b * 3 * ny * P + (r == 0 ? 0 : 2 * (size_t)ny * 2 * P);
+      w = mean_down<RN, TOP>(f, t, sc, g.N, P, sig, T, X, (r == 0 ? pb.HXP : pb.HZP) + (size_t)b * ny, hm);
     } else {
-      step(1, u);
-      step(0, v);
+      w = omega_down<RN, TOP, D>(f, g, pb, t, sc, b, p, r, sig, T, hc);
     }
   }
+  const double cx = MEAN ? -1.0 : sc.cc;  // the wall rows of X' take c X, those of d take -X
+  double f0, fc = 0.0;
   if (TOP == 0) {
-    f0 = t.tau.helm_isq[(size_t)(sc.k * 2 + sig) * P + p] * (cc * S0 - sum);
-    if (mean && r == 0 && sig == 0) {
-      double flux = 0.0, fp = f0;
-      for (int i = 0; i < M; ++i) {
-        if (i > 0) fp = fma(__ldg(T + 4 * MP + (size_t)i * P), fp, f[i * NT]);
-        flux = fma(t.tau.wint[2 * i], fp, flux);
-      }
-      fc = (fma(cc, flux_old, sc.flux) - flux) * t.tau.u1_iflux[sc.k];
-    }
+    f0 = t.tau.helm_isq[(size_t)(sc.k * 2 + sig) * P + p] * (cx * w.S0 - w.sum);
   } else {
-    double wp = 0.0;
-    if (live && mean && sig == 0) {
-      double fp = 0.0;
-      for (int i = 1; i < M; ++i) {
-        fp = fma(__ldg(T + 4 * MP + (size_t)i * P), fp, f[i * NT]);
-        wp = fma(t.tau.wint[2 * i], fp, wp);
-      }
-    }
     const int me = threadIdx.x, mate = me ^ 32;
-    const double mine[6] = {sum, sum2, S0, S2, wp, flux_old};
+    const double mine[6] = {w.sum, w.sum2, w.S0, w.S2, w.wp, w.wx};
 #pragma unroll
     for (int k = 0; k < 6; ++k) xch[k * NT + me] = mine[k];
     __syncthreads();
@@ -184,51 +311,45 @@ __device__ __forceinline__ void solve_omega(double* f, double* xch, const Grid& 
     }
     auto qs = [&](int s, int w) { return t.tau.helm_top[((size_t)(sc.k * 2 + s) * 2 + w) * P + p]; };
     double xe, xo;
-    if (mean && r == 0) {
+    if (MEAN && r == 0) {
       const double* m = t.tau.mean_top + 4 * sc.k;  // int Q_e; sum, sum n^2 and int of the forcing response
-      close_free_slip_mean(se, so, qs(0, 0), qs(1, 0), qs(0, 1), qs(1, 1), m[0], m[1], m[2], m[3], cc, sc.flux, &xe, &xo,
+      close_free_slip_mean(se, so, qs(0, 0), qs(1, 0), qs(0, 1), qs(1, 1), m[0], m[1], m[2], m[3], cx, sc.flux, &xe, &xo,
                            &fc);
-      if (sig != 0) fc = 0.0;
     } else {
-      close_neumann_top(se, so, qs(0, 0), qs(1, 0), qs(0, 1), qs(1, 1), cc, &xe, &xo);
+      close_neumann_top(se, so, qs(0, 0), qs(1, 0), qs(0, 1), qs(1, 1), cx, &xe, &xo);
     }
     f0 = sig == 0 ? xe : xo;
   }
-  // up: f_i = a_i + b_i f_{i-1}; x <- f - c x (+ the forced response of U)
-  const double* __restrict__ u1 = t.tau.u1 + (size_t)sc.k * t.tau.Mh;
-  auto out = [&](int i, double fi, double x) {
-    double y = fma(-cc, x, fi);
-    if (mean && r == 0 && sig == 0) y = fma(fc, u1[i], y);
-    xp[(size_t)(2 * i + sig) * xs] = y;
-  };
-  double fp = f0;
-  out(0, fp, xp[(size_t)sig * xs]);
-  for (int i = 1; i < M; i += 4) {
-    double bb[4], x[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (i + k < M) {
-        bb[k] = __ldg(T + 4 * MP + (size_t)(i + k) * P);
-        x[k] = xp[(size_t)(2 * (i + k) + sig) * xs];
-      }
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (i + k < M) {
-        fp = fma(bb[k], fp, f[(i + k) * NT]);
-        out(i + k, fp, x[k]);
-      }
+  if constexpr (MEAN) {
+    mean_up<TOP>(f, t, sc, g.N, P, sig, r == 0, T, X, f0, fc, w.wx);
+    return;
   }
+  // up: f_i = a_i + b_i f_{i-1}; g <- f - c g
+  const size_t hP = 2 * P;
+  double* G = reinterpret_cast<double*>(pb.G) + 2 * ((size_t)b * ny * P + p) + r + (size_t)sig * hP;
+  const double cc = sc.cc;
+  double fp = f0;
+  G[0] = fma(-cc, G[0], fp);
+  struct Up {
+    double b, x;
+  };
+  sweep_up<2 * D>(
+      1, M, [&](int i) { return Up{__ldg(T + 4 * MP + (size_t)i * P), G[(size_t)i * 2 * hP]}; },
+      [&](int i, const Up& u) {
+        fp = fma(u.b, fp, f[i * NT]);
+        G[(size_t)i * 2 * hP] = fma(-cc, u.x, fp);
+      });
 }
 
 // Solve v of parity sig of one (mode, component).
-template <typename RN, int TOP>
+template <typename RN, int TOP, int D>
 __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, const PencilBufs& pb, const DevTables& t,
                                         const StageCoef& sc, int b, int p, int r, int sig, bool live,
                                         const RN* __restrict__ hc) {
   constexpr int NT = 64;
   const size_t P = g.P, MP = (size_t)t.tau.Mh * P;
   const int ny = g.ny, N = g.N, M = (N - sig) / 2 + 1, row = p / g.nxh, ix = p % g.nxh;
-  const double cc = sc.alpha / sc.beta;
+  const double cc = sc.cc;
   const double* __restrict__ T = t.tau.helm_f + (size_t)(sc.k * 2 + sig) * solve_tabs<TOP>() * MP + p;
   const double* __restrict__ TP = t.tau.pois_f + (size_t)sig * kPoisTabs * MP + p;
   const double* __restrict__ n2 = t.tau.n2;
@@ -240,13 +361,13 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
   const RN* hy = H0 + (size_t)ny * hP + r;
   const RN* hz = H0 + 2 * (size_t)ny * hP + 1 - r;
   const double kxd = t.kx[ix], kzd = t.kz[row], k2 = fma(kxd, kxd, kzd * kzd), ck2 = -(1.0 + cc) * k2;
-  const RN sgn = r == 0 ? (RN)-1 : (RN)1, kx = (RN)kxd, kz = (RN)kzd, k2n = (RN)k2;
-  const RN dtn = (RN)sc.dt, gan = (RN)sc.gamma, zen = (RN)sc.zeta;
+  const RN sgn = r == 0 ? (RN)-1 : (RN)1, kx = sgn * (RN)kxd, kz = sgn * (RN)kzd, k2n = (RN)k2;
+  const Coef3<RN> nc = node_coef<RN>(sc);
   double Aw = 0.0, Bw = 0.0;
   if (live) {
     struct In {
       double x;
-      RN hx, hy, hz, hp;
+      RN hx, hy, hz, hp, fac;
       TabRow tb;
       double E1;
     };
@@ -256,29 +377,27 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
       v.x = Vp[n * hP];
       v.hy = __ldg(hy + n * hP);
       v.hp = HV[n * hP];
-      if ((int)n + 1 <= N) {
-        v.hx = __ldg(hx + (n + 1) * hP);
-        v.hz = __ldg(hz + (n + 1) * hP);
-      } else {
-        v.hx = v.hz = (RN)0;
-      }
-      if (i + 1 < M) {
-        v.tb = tab_row(T, MP, (size_t)(i + 1) * P);
-        v.E1 = __ldg(T + 6 * MP + (size_t)(i + 1) * P);
-      }
+      if constexpr (sizeof(RN) == 8) v.fac = __ldg(t.tau.n1 + n);
+      else v.fac = (RN)(2 * ((int)n + 1));
+      const size_t no = min((int)n + 1, N), o = (size_t)min(i + 1, M - 1) * P;
+      v.hx = __ldg(hx + no * hP);
+      v.hz = __ldg(hz + no * hP);
+      v.tb = tab_row(T, MP, o);
+      v.E1 = __ldg(T + 6 * MP + o);
       return v;
     };
     double S0 = 0.0, sum = 0.0, r1 = 0.0, r2 = 0.0, x1 = 0.0, an = 0.0;
     RN dtt = 0;  // D(i kx H_x + i kz H_z), from the top down
     auto step = [&](int i, const In& v) {
       const int n = 2 * i + sig;
-      const RN t2 = (RN)(2 * (n + 1)) * (sgn * (kx * v.hx + kz * v.hz)) + dtt;
+      const RN tt = n + 1 <= N ? kx * v.hx + kz * v.hz : (RN)0;
+      const RN t2 = v.fac * tt + dtt;
       dtt = n == 0 ? (RN)0.5 * t2 : t2;
       const RN hv = -k2n * v.hy - dtt;
       HV[(size_t)n * hP] = hv;
-      const RN q = dtn * (gan * hv + zen * v.hp);
+      const RN q = nc.dga * hv + nc.dze * v.hp;
       S0 += v.x;
-      const double r0 = fma(ck2, v.x, (double)q);
+      const double r0 = fma(ck2, v.x, widen(q));
       if (i + 1 < M) {
         const double a =
             fma(-v.tb.h, an, fma(v.E1, x1, fma(v.tb.eC, r2, fma(-v.tb.eB, r1, v.tb.eA * r0))));
@@ -290,59 +409,30 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
       r1 = r0;
       x1 = v.x;
     };
-    In u = load(M - 1), v = load(M - 2);
-    int i = M - 1;
-    for (; i >= 3; i -= 2) {
-      const In u1 = load(i - 2);
-      step(i, u);
-      const In v1 = load(i - 3);
-      step(i - 1, v);
-      u = u1;
-      v = v1;
-    }
-    if (i == 2) {
-      const In w = load(0);
-      step(2, u);
-      step(1, v);
-      step(0, w);
-    } else {
-      step(1, u);
-      step(0, v);
-    }
+    sweep_down<D>(M - 1, 0, load, step);
     // phi, with zero wall sum
     double fp = t.tau.helm_isq[(size_t)(sc.k * 2 + sig) * P + p] * -sum;
     f[0] = fp;
-    for (int i = 1; i < M; i += 4) {
-      double bb[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (i + k < M) bb[k] = __ldg(T + 4 * MP + (size_t)(i + k) * P);
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (i + k < M) {
-          fp = fma(bb[k], fp, f[(i + k) * NT]);
-          f[(i + k) * NT] = fp;
-        }
-    }
+    sweep_up<2 * D>(
+        1, M, [&](int i) { return __ldg(T + 4 * MP + (size_t)i * P); },
+        [&](int i, double bi) {
+          fp = fma(bi, fp, f[i * NT]);
+          f[i * NT] = fp;
+        });
     // (D^2 - k^2) v_p = phi, the array read at i and written at i + 1
     sum = an = r2 = 0.0;
     r1 = fp;
-    for (int j = M - 1; j >= 1; j -= 2) {
-      const TabRow ta = tab_row(TP, MP, (size_t)j * P);
-      TabRow tb;
-      if (j >= 2) tb = tab_row(TP, MP, (size_t)(j - 1) * P);
-      auto row_j = [&](int jj, const TabRow& tr) {
-        const double r0 = f[(jj - 1) * NT];
-        const double a = fma(-tr.h, an, fma(tr.eC, r2, fma(-tr.eB, r1, tr.eA * r0)));
-        f[jj * NT] = a;
-        sum = fma(tr.W, a, sum);
-        an = a;
-        r2 = r1;
-        r1 = r0;
-      };
-      row_j(j, ta);
-      if (j >= 2) row_j(j - 1, tb);
-    }
+    sweep_down<D>(
+        M - 1, 1, [&](int j) { return tab_row(TP, MP, (size_t)j * P); },
+        [&](int j, const TabRow& tr) {
+          const double r0 = f[(j - 1) * NT];
+          const double a = fma(-tr.h, an, fma(tr.eC, r2, fma(-tr.eB, r1, tr.eA * r0)));
+          f[j * NT] = a;
+          sum = fma(tr.W, a, sum);
+          an = a;
+          r2 = r1;
+          r1 = r0;
+        });
     const size_t vo = (size_t)b * P + p;
     const double* vwn = reinterpret_cast<const double*>(pb.vw_new + vo) + r;
     const double* vwo = reinterpret_cast<const double*>(pb.vw_old + vo) + r;
@@ -350,28 +440,25 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
     const double s = fma(cc, S0, (sig == 0 ? 0.5 : -0.5) * vw);
     // w = v_p - c v_old and its wall sums
     fp = t.tau.pois_isq[(size_t)sig * P + p] * (s - sum);
-    auto wall = [&](int i, double fi, double x) {
-      const double w = fma(-cc, x, fi), nn = __ldg(n2 + 2 * i + sig);
+    auto wall = [&](int i, double fi, double x, double nn) {
+      const double w = fma(-cc, x, fi);
       f[i * NT] = w;
       Bw = fma(nn, w, Bw);
       if (TOP) Aw = fma(nn * (nn - 1.0), w, Aw);  // 3 D^2 at the wall
     };
-    wall(0, fp, Vp[(size_t)sig * hP]);
-    for (int i = 1; i < M; i += 4) {
-      double bb[4], x[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (i + k < M) {
-          bb[k] = __ldg(TP + 4 * MP + (size_t)(i + k) * P);
-          x[k] = Vp[(size_t)(2 * (i + k) + sig) * hP];
-        }
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (i + k < M) {
-          fp = fma(bb[k], fp, f[(i + k) * NT]);
-          wall(i + k, fp, x[k]);
-        }
-    }
+    wall(0, fp, Vp[(size_t)sig * hP], __ldg(n2 + sig));
+    struct Up {
+      double b, x, nn;
+    };
+    sweep_up<D>(
+        1, M,
+        [&](int i) {
+          return Up{__ldg(TP + 4 * MP + (size_t)i * P), Vp[(size_t)(2 * i + sig) * hP], __ldg(n2 + 2 * i + sig)};
+        },
+        [&](int i, const Up& u) {
+          fp = fma(u.b, fp, f[i * NT]);
+          wall(i, fp, u.x, u.nn);
+        });
   }
   // influence coefficient: D v(+-1) = 0 per parity, or D^2 v(+1) = Dv(-1) = 0
   double cI;
@@ -393,41 +480,36 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
     cI = sig == 0 ? ce : co;
   }
   const double* __restrict__ vh = t.tau.vh + (size_t)(sc.k * 2 + sig) * MP + p;
-  for (int i = 0; i < M; i += 4) {
-    double h[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (i + k < M) h[k] = __ldg(vh + (size_t)(i + k) * P);
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (i + k < M) Vp[(size_t)(2 * (i + k) + sig) * hP] = fma(cI, h[k], f[(i + k) * NT]);
-  }
+  sweep_up<2 * D>(
+      0, M, [&](int i) { return __ldg(vh + (size_t)i * P); },
+      [&](int i, double h) { Vp[(size_t)(2 * i + sig) * hP] = fma(cI, h, f[i * NT]); });
 }
 
-// CTA: 16 modes x 2 components (lanes) x 2 classes (warps) of one equation;
-// v (twice the work) in the first half of the grid
+// CTA: 16 modes x 2 components (lanes) x 2 classes (warps) of one equation:
+// the mean flow, then v (twice the work of omega_y), then omega_y.  Five rows
+// are loaded ahead on up to 255 registers: with DRAM or L2 latency covered by
+// the thread itself, four CTAs per SM saturate the FP64 pipe.
+constexpr int kSolveAhead = 5;
 template <typename RN, int TOP>
-__global__ void __launch_bounds__(64, 8) stage_solve_kernel(Grid g, PencilBufs pb, DevTables t,
-                                                             const typename cpx<RN>::T* __restrict__ hc, StageCoef sc) {
+__global__ void __launch_bounds__(64, 4) stage_solve_kernel(Grid g, PencilBufs pb, DevTables t,
+                                                            const typename cpx<RN>::T* __restrict__ hc, StageCoef sc) {
   extern __shared__ __align__(16) double sarr[];  // [Mh][64], then the exchange slots [6][64] of a free-slip top
-  const int b = blockIdx.y;
+  const int b = blockIdx.y, tiles = (g.P + 15) / 16;
   if (pb.active && !pb.active[b]) return;
   pdl_wait_then_release();  // the coefficients of H come from the analysis
   const int lane = threadIdx.x & 31, c = threadIdx.x / 32, r = lane & 1;
-  const int pr = blockIdx.x * 16 + (lane >> 1), p = min(pr, g.P - 1);
+  const int z = (blockIdx.x + tiles - 1) / tiles;  // 0: mean, 1: v, 2: omega_y
+  const int pr = z == 0 ? lane >> 1 : ((int)(blockIdx.x - 1) % tiles) * 16 + (lane >> 1), p = min(pr, g.P - 1);
+  // the mean flow is mode 0; the Nyquist row stays zero
+  const bool live = z == 0 ? lane < 2 : pr > 0 && pr < g.P && p / g.nxh != g.nz / 2;
   // a free-slip top needs every thread at the exchange
-  bool live = pr < g.P && p / g.nxh != g.nz / 2;  // the Nyquist row stays zero
+  if (TOP == 0 && !live) return;
   double* f = sarr + threadIdx.x;
   double* xch = sarr + (size_t)t.tau.Mh * 64;
   const RN* h = reinterpret_cast<const RN*>(hc);
-  if (blockIdx.z == 0) {
-    if (p == 0) live = false;  // the mean flow is the other equation's
-    if (TOP == 0 && !live) return;
-    solve_v<RN, TOP>(f, xch, g, pb, t, sc, b, p, r, c, live, h);
-  } else {
-    if (TOP == 0 && !live) return;
-    solve_omega<RN, TOP>(f, xch, g, pb, t, sc, b, p, r, 1 - c, live, h);
-  }
+  if (z == 0) solve_omega<RN, TOP, kSolveAhead, true>(f, xch, g, pb, t, sc, b, p, r, c, live, h);
+  else if (z == 1) solve_v<RN, TOP, kSolveAhead>(f, xch, g, pb, t, sc, b, p, r, c, live, h);
+  else solve_omega<RN, TOP, kSolveAhead, false>(f, xch, g, pb, t, sc, b, p, r, 1 - c, live, h);
 }
 
 template <typename RN, int TOP>
@@ -437,8 +519,8 @@ cudaError_t solve_top(const Grid& g, int B, const PencilBufs& pb, const DevTable
   static SmemLimit lim;
   const cudaError_t e = raise_smem_limit(stage_solve_kernel<RN, TOP>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(RN) == 4>(stage_solve_kernel<RN, TOP>, dim3((g.P + 15) / 16, B, 2), dim3(64), smem, st, g, pb,
-                                        t, h, sc);
+  return launch_pdl_if<sizeof(RN) == 4>(stage_solve_kernel<RN, TOP>, dim3(1 + 2 * ((g.P + 15) / 16), B), dim3(64), smem, st,
+                                        g, pb, t, h, sc);
 }
 
 }  // namespace chdns
