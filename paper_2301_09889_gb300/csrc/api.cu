@@ -779,7 +779,9 @@ static void set_launch_count(ch_env* env) {
   const ch_params_t* p = &env->prm;
   const bool passes = p->precision == 1 ? env->plane_f.passes : env->plane.passes;
   const int stage = 1 + (passes ? 3 : 1) + stage_post_launches(p->top_bc, env->post_batched);
-  env->launches_per_step = (p->control == 0 ? 2 : p->control == 1 ? 1 : 5) + p->steps_per_action * (3 * stage + 1) + 3;
+  const int obs = io_by_lines(env->g, env->B) ? 2 : 1;
+  env->launches_per_step =
+      (p->control == 0 ? 2 : p->control == 1 ? 1 : 4 + obs) + p->steps_per_action * (3 * stage + 1) + 2 + obs;
 }
 
 // The kernels of one environment step, in stream order.

@@ -65,10 +65,17 @@ cudaError_t launch_wall_shear(const Grid& g, int B, const double* UM, double nu,
                               const int* active, cudaStream_t st);
 cudaError_t launch_sense(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, int js,
                          double alpha, int opposition, cudaStream_t st);
-cudaError_t launch_obs(const Grid& g, int B, const double2* planes, const DevTables& t, double* out,
+cudaError_t launch_obs(const Grid& g, int B, double2* planes, const DevTables& t, double* out,
                        size_t out_stride, const int* active, cudaStream_t st);
 cudaError_t launch_action(const Grid& g, int B, const double* act, double u_tau, const DevTables& t,
                           const PencilBufs& pb, cudaStream_t st);
+// the unpadded transforms by lines (plane_io.cu), chosen by size in launch_obs
+// and launch_action: two launches each
+bool io_by_lines(const Grid& g, int B);
+cudaError_t launch_obs_lines(const Grid& g, int B, double2* planes, const DevTables& t, double* out, size_t out_stride,
+                             const int* active, cudaStream_t st);
+cudaError_t launch_action_lines(const Grid& g, int B, const double* act, double u_tau, const DevTables& t,
+                                const PencilBufs& pb, cudaStream_t st);
 cudaError_t launch_finalize(int B, const double* acc, double inv_steps, double tau_ref, double* out,
                             size_t out_stride, size_t out_offset, const int* active, cudaStream_t st);
 cudaError_t launch_tau_helmholtz(int ny, int M, const double* lam, const double2* r, const double2* top,

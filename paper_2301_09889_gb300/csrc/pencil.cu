@@ -119,72 +119,74 @@ __global__ void wall_shear_kernel(int ny, int B, const double* UM, double nu, do
 // ---------------------------------------------------------------------------
 // sensing plane: Fourier coefficients of u and v at node js (and, for
 // opposition control, the wall spectrum -alpha v(y_s) with the mean removed,
-// paper Sec. 4.1).  One warp per mode: v(y_s) = sum_n v_n T_n(y_s),
-// Dv(y_s) = sum_n v_n T_n'(y_s), omega_y(y_s) likewise.
+// paper Sec. 4.1).  v(y_s) = sum_n v_n T_n(y_s), Dv(y_s) = sum_n v_n T_n'(y_s),
+// omega_y(y_s) likewise.  L lanes per (mode, component q) share the sums;
+// component q of Dv and omega_y makes component 1 - q of u = (i kx Dv - i kz
+// omega_y) / k^2, so a lane group exchanges nothing with the other component.
+// FP64-bound: three operations per coefficient and component.  One lane per
+// system where the batch fills the SMs that way, eight (shorter chains, seven
+// operations more per system) for few modes.
 // ---------------------------------------------------------------------------
+template <int L>
 __global__ void __launch_bounds__(128) sense_kernel(Grid g, int B, PencilBufs pb, DevTables t, int js, double alpha,
                                                     int opposition) {
-  // 8 lanes per mode (4 modes per warp): the sums over the ny coefficients are
-  // split over the lanes and combined by shuffles within the 8-lane group
-  constexpr int L = 8;
   const int P = g.P, ny = g.ny;
   const int lane = threadIdx.x & (L - 1);
-  const long wid = (blockIdx.x * (long)blockDim.x + threadIdx.x) / L;
-  const bool live = wid < (long)P * B;
-  const int p = live ? (int)(wid % P) : 0;
-  const int b = live ? (int)(wid / P) : 0;
-  const bool act = live && !(pb.active && !pb.active[b]);
-  auto gsum = [](double v) {
-#pragma unroll
-    for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, L);
-    return v;
-  };
-  auto gsum2 = [&](double2 v) { return mk(gsum(v.x), gsum(v.y)); };
+  const long sys = (blockIdx.x * (long)blockDim.x + threadIdx.x) / L;  // (b, p, q), q fastest
+  const bool inside = sys < 2L * P * B;
+  const int q = (int)(sys & 1);
+  const int p = inside ? (int)(sys / 2 % P) : 0;
+  const int b = inside ? (int)(sys / 2 / P) : 0;
+  const bool act = inside && !(pb.active && !pb.active[b]);
   const int row = p / g.nxh, ix = p % g.nxh;
   const double* cj = t.cheb + (size_t)js * ny;
+  const bool gen = act && p > 0 && row != g.nz / 2, mean = act && p == 0 && q == 0;
   // partial sums (only the loads are conditional; every lane of the warp then
   // takes part in the same shuffles)
-  double su = 0.0;
-  double2 vs = mk(0.0, 0.0), gs = mk(0.0, 0.0), dvs = mk(0.0, 0.0);
-  if (act && row != g.nz / 2) {
-    if (p == 0) {
-      for (int n = lane; n < ny; n += L) su += cj[n] * pb.UM[(size_t)b * ny + n];
-    } else {
-      const size_t fo = (size_t)b * ny * P + p;
+  double vs = 0.0, gs = 0.0, ds = 0.0;
+  if (gen) {
+    const size_t o = 2 * ((size_t)b * ny * P + p) + q;
+    const double* V = reinterpret_cast<const double*>(pb.V) + o;
+    const double* G = reinterpret_cast<const double*>(pb.G) + o;
 #pragma unroll 8
-      for (int n = lane; n < ny; n += L) {
-        const double2 vn = pb.V[fo + (size_t)n * P];
-        const double2 gn = pb.G[fo + (size_t)n * P];
-        vs = vs + cj[n] * vn;
-        gs = gs + cj[n] * gn;
-        dvs = dvs + t.dts[n] * vn;
-      }
+    for (int n = lane; n < ny; n += L) {
+      const double vn = V[(size_t)n * 2 * P], gn = G[(size_t)n * 2 * P], c = __ldg(cj + n);
+      vs = fma(c, vn, vs);
+      gs = fma(c, gn, gs);
+      ds = fma(__ldg(t.dts + n), vn, ds);
     }
+  } else if (mean) {
+#pragma unroll 8
+    for (int n = lane; n < ny; n += L) gs = fma(__ldg(cj + n), pb.UM[(size_t)b * ny + n], gs);
   }
-  su = gsum(su);
-  vs = gsum2(vs);
-  gs = gsum2(gs);
-  dvs = gsum2(dvs);
-  double2 us = mk(0.0, 0.0);
-  if (p == 0) {
-    us = mk(su, 0.0);
-  } else if (row != g.nz / 2) {
-    const double kx = t.kx[ix], kz = t.kz[row];
-    const double ik2 = 1.0 / (kx * kx + kz * kz);
-    us = ik2 * (imul(kx, dvs) - imul(kz, gs));
+#pragma unroll
+  for (int o = L / 2; o > 0; o >>= 1) {
+    vs += __shfl_xor_sync(0xffffffffu, vs, o, L);
+    gs += __shfl_xor_sync(0xffffffffu, gs, o, L);
+    ds += __shfl_xor_sync(0xffffffffu, ds, o, L);
   }
-  if (!act) return;
-  if (lane != 0) return;
+  if (!act || lane != 0) return;
+  const size_t o = (size_t)b * P + p;
   if (opposition) {
     // new action: the previous one becomes the start of the ramp, the wall
     // shear average restarts
-    const size_t o = (size_t)b * P + p;
-    pb.vw_old[o] = pb.vw_new[o];
-    pb.vw_new[o] = (p == 0) ? mk(0.0, 0.0) : (-alpha) * vs;
-    if (p == 0) pb.tau_acc[b] = 0.0;
+    double* old = reinterpret_cast<double*>(pb.vw_old + o) + q;
+    double* now = reinterpret_cast<double*>(pb.vw_new + o) + q;
+    *old = *now;
+    *now = p == 0 ? 0.0 : -alpha * vs;
+    if (p == 0 && q == 0) pb.tau_acc[b] = 0.0;
   } else {
-    pb.planes[((size_t)b * 2 + 0) * P + p] = us;
-    pb.planes[((size_t)b * 2 + 1) * P + p] = vs;
+    double us = 0.0;
+    int ru = 1 - q;  // component of u this thread makes
+    if (gen) {
+      const double kx = t.kx[ix], kz = t.kz[row];
+      us = (q == 0 ? 1.0 : -1.0) * (kx * ds - kz * gs) / (kx * kx + kz * kz);
+    } else if (p == 0) {
+      us = gs;  // U in the real part, zero in the imaginary one
+      ru = q;
+    }
+    reinterpret_cast<double*>(pb.planes + ((size_t)b * 2 + 0) * P + p)[ru] = us;
+    reinterpret_cast<double*>(pb.planes + ((size_t)b * 2 + 1) * P + p)[q] = vs;
   }
 }
 
@@ -327,21 +329,81 @@ __global__ void finalize_kernel(int B, const double* acc, double inv_steps, doub
   out[(size_t)b * out_stride + out_offset + 1] = 1.0 - tau / tau_ref;
 }
 
-// stateless tau problems: one thread per (problem, parity)
-__global__ void tau_helmholtz_kernel(int ny, int M, const double* lam, const double2* r, const double2* top,
-                                     const double2* bot, double2* f) {
-  const long tid = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (tid >= 2L * M) return;
-  const int m = (int)(tid / 2), sig = (int)(tid % 2);
-  const int N = ny - 1;
-  double e[kMaxHalf], h[kMaxHalf], bb[kMaxHalf], Q[kMaxHalf], isq;
-  tau_factor(N, sig, lam[m], e, h, bb, Q, &isq);
+// ---------------------------------------------------------------------------
+// stateless tau problems, one thread per (problem, parity, component): the
+// elimination factors and the particular solution in one sweep down, the back
+// substitution in one sweep up, a_i and b_i in columns of shared memory.  With
+// W_{M-1} = 1, W_i = 1 + b_{i+1} W_{i+1} the sweep down also gives
+// sum_i P_i = sum_i W_i a_i and sum_i Q_i = W_0, so f_0 = (s - sum P) / W_0.
+// Lanes (component, parity) of a problem read whole 32-byte sectors of r.
+//
+// What bounds it: the FP64 pipe and, below 4864 problems, the chain of one
+// warp per sub-partition (64 cycles per FP64 operation).  The row constants
+// come from a table and each row divides once; the former one thread per
+// (problem, parity) recomputed the constants with six more divisions per row
+// and kept its vectors in local memory.
+// ---------------------------------------------------------------------------
+struct TauRows {
+  double a[kMaxNy + 1] = {}, b[kMaxNy + 1] = {}, c[kMaxNy + 1] = {};  // cA_n, and cB_n, cC_n away from the cut
+  constexpr TauRows() {
+    for (int n = 2; n <= kMaxNy; ++n) {
+      a[n] = (n == 2 ? 2.0 : 1.0) / (4.0 * n * (n - 1));
+      b[n] = 1.0 / (2.0 * ((double)n * n - 1.0));
+      c[n] = 1.0 / (4.0 * n * (n + 1));
+    }
+  }
+};
+static __device__ const TauRows g_tau_rows{};
+
+constexpr int kTauNT = 32;
+
+__global__ void __launch_bounds__(kTauNT) tau_helmholtz_kernel(int ny, int M, const double* __restrict__ lam,
+                                                               const double2* r, const double2* __restrict__ top,
+                                                               const double2* __restrict__ bot, double2* f) {
+  extern __shared__ __align__(16) double tausm[];  // [2][rows][kTauNT]
+  const int N = ny - 1, rows = N / 2 + 1;
+  const long tid = blockIdx.x * (long)kTauNT + threadIdx.x;
+  if (tid >= 4L * M) return;
+  const int q = (int)(tid & 1), sig = (int)(tid >> 1 & 1);
+  const long m = tid >> 2;
   const int Mp = (N - sig) / 2 + 1;
-  double2 rr[kMaxHalf], ff[kMaxHalf];
-  for (int i = 0; i < Mp; ++i) rr[i] = r[(size_t)m * ny + 2 * i + sig];
-  const double2 s = sig == 0 ? 0.5 * (top[m] + bot[m]) : 0.5 * (top[m] - bot[m]);
-  tau_solve(N, sig, rr, ff, TabLocal{e, h, bb, Q}, isq, s);
-  for (int i = 0; i < Mp; ++i) f[(size_t)m * ny + 2 * i + sig] = ff[i];
+  const double l = lam[m];
+  const double* rr = reinterpret_cast<const double*>(r + m * ny + sig) + q;  // element i at 4 i
+  double* ca = tausm + threadIdx.x;
+  double* cb = ca + rows * kTauNT;
+  double r1 = rr[4 * (Mp - 1)], r2 = 0.0, an = 0.0, bn = 0.0, W = 1.0, sum = 0.0;
+#pragma unroll 4
+  for (int i = Mp - 1; i >= 1; --i) {
+    const int n = 2 * i + sig;
+    const double cA = __ldg(&g_tau_rows.a[n]);
+    const double cB = n <= N - 2 ? __ldg(&g_tau_rows.b[n]) : 0.0;
+    const double cC = n + 2 <= N - 2 ? __ldg(&g_tau_rows.c[n]) : 0.0;
+    const double r0 = rr[4 * (i - 1)];
+    if (i < Mp - 1) W = fma(bn, W, 1.0);
+    const double U = -l * cC;  // zero in the last row
+    const double e = 1.0 / fma(U, bn, fma(l, cB, 1.0));
+    double R = fma(cA, r0, -(cB * r1));
+    if (i + 1 < Mp) R = fma(cC, r2, R);
+    const double a = e * fma(-U, an, R);
+    const double b = e * (l * cA);
+    ca[i * kTauNT] = a;
+    cb[i * kTauNT] = b;
+    sum = fma(W, a, sum);
+    an = a;
+    bn = b;
+    r2 = r1;
+    r1 = r0;
+  }
+  if (Mp > 1) W = fma(bn, W, 1.0);  // sum Q
+  const double t = reinterpret_cast<const double*>(top + m)[q], u = reinterpret_cast<const double*>(bot + m)[q];
+  double fp = (0.5 * (sig == 0 ? t + u : t - u) - sum) / W;
+  double* out = reinterpret_cast<double*>(f + m * ny + sig) + q;
+  out[0] = fp;
+#pragma unroll 4
+  for (int i = 1; i < Mp; ++i) {
+    fp = fma(cb[i * kTauNT], fp, ca[i * kTauNT]);
+    out[4 * i] = fp;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -355,13 +417,17 @@ cudaError_t launch_wall_shear(const Grid& g, int B, const double* UM, double nu,
 
 cudaError_t launch_sense(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, int js, double alpha,
                          int opposition, cudaStream_t st) {
-  const long threads = (long)g.P * B * 8;  // 8 lanes per mode
-  sense_kernel<<<(unsigned)((threads + 127) / 128), 128, 0, st>>>(g, B, pb, t, js, alpha, opposition);
+  const long sys = 2L * g.P * B;
+  if (sys >= 16384)
+    sense_kernel<1><<<(unsigned)((sys + 127) / 128), 128, 0, st>>>(g, B, pb, t, js, alpha, opposition);
+  else
+    sense_kernel<8><<<(unsigned)((8 * sys + 127) / 128), 128, 0, st>>>(g, B, pb, t, js, alpha, opposition);
   return cudaGetLastError();
 }
 
-cudaError_t launch_obs(const Grid& g, int B, const double2* planes, const DevTables& t, double* out,
-                       size_t out_stride, const int* active, cudaStream_t st) {
+cudaError_t launch_obs(const Grid& g, int B, double2* planes, const DevTables& t, double* out, size_t out_stride,
+                       const int* active, cudaStream_t st) {
+  if (io_by_lines(g, B)) return launch_obs_lines(g, B, planes, t, out, out_stride, active, st);
   // several output rows per CTA once the batch alone gives 128 or more
   // (environment, field) CTAs; otherwise one row per CTA, its sums split over
   // the CTA's threads
@@ -376,6 +442,7 @@ cudaError_t launch_obs(const Grid& g, int B, const double2* planes, const DevTab
 
 cudaError_t launch_action(const Grid& g, int B, const double* act, double u_tau, const DevTables& t,
                           const PencilBufs& pb, cudaStream_t st) {
+  if (io_by_lines(g, B)) return launch_action_lines(g, B, act, u_tau, t, pb, st);
   // the sensing-plane buffer is free at this point of the step: it is the scratch plane
   double2* tx = pb.planes;
   const long n = (long)B * g.nz * g.nxh;
@@ -396,17 +463,20 @@ cudaError_t launch_finalize(int B, const double* acc, double inv_steps, double t
 
 cudaError_t launch_tau_helmholtz(int ny, int M, const double* lam, const double2* r, const double2* top,
                                  const double2* bot, double2* f, cudaStream_t st) {
-  const long n = 2L * M;
-  tau_helmholtz_kernel<<<(unsigned)((n + 63) / 64), 64, 0, st>>>(ny, M, lam, r, top, bot, f);
+  const size_t smem = (size_t)2 * ((ny - 1) / 2 + 1) * kTauNT * sizeof(double);
+  static SmemLimit lim;
+  const cudaError_t e = raise_smem_limit(tau_helmholtz_kernel, &lim, smem);
+  if (e != cudaSuccess) return e;
+  tau_helmholtz_kernel<<<(unsigned)((4L * M + kTauNT - 1) / kTauNT), kTauNT, smem, st>>>(ny, M, lam, r, top, bot, f);
   return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
 // Allocation-free variant of the stateless tau entry point.
 //
-// tau_helmholtz_kernel above keeps each problem's factorisation and work
-// vectors (about 6.5 KB per thread) in local memory, which the CUDA driver
-// allocates and may have to grow at launch time.  Some callers cannot let
+// Kernels that spill work vectors (6.5 KB per problem and parity at 201 nodes)
+// to local memory rely on an allocation of the CUDA driver, which may have to
+// grow at launch time.  Some callers cannot let
 // anything allocate device memory: a control loop with a fixed real-time
 // budget (cudaMalloc and a driver-side resize can block for milliseconds and
 // synchronise the device), a process whose device memory is already fully

@@ -67,14 +67,30 @@ __global__ void __launch_bounds__(64 * NF, ctas_of(pre_dct_regs<RN, N>(), 64 * N
   if (pb.active && !pb.active[b]) return;
   pdl_wait_then_release();  // v, omega_y come from the previous stage
   if constexpr (kTile) {
+    // a column per warp and step, every load in flight before the first store
+    constexpr int KL = (2 * (N + 1) + 2 * NF - 1) / (2 * NF);
     const size_t c0 = 2 * ((size_t)b * ny * P + blockIdx.x * 16) + lane;
-#pragma unroll 4
-    for (int n = threadIdx.x / 32; n < 2 * ny; n += 2 * NF) {
-      const int m = n < ny ? n : n - ny;
-      const double* src = reinterpret_cast<const double*>(n < ny ? pb.V : pb.G) + 2 * (size_t)P * m + c0;
-      // the columns of mode 0 hold W and U instead of omega_y
-      if (p == 0 && n >= ny) src = (r == 0 ? pb.WM : pb.UM) + (size_t)b * ny + m;
-      tile[n * 32 + lane] = p < P ? (RN)*src : (RN)0;
+    const double* v0 = reinterpret_cast<const double*>(pb.V) + c0;
+    const double* g0 = reinterpret_cast<const double*>(pb.G) + c0;
+    size_t gs = 2 * (size_t)P;
+    if (p == 0) {  // the columns of mode 0 hold W and U instead of omega_y
+      g0 = (r == 0 ? pb.WM : pb.UM) + (size_t)b * ny;
+      gs = 1;
+    }
+    constexpr int KC = KL <= 12 ? KL : (KL + (KL + 11) / 12 - 1) / ((KL + 11) / 12);  // at most 12 at a time
+    for (int k0 = 0; k0 < KL; k0 += KC) {
+      double d[KC];
+#pragma unroll
+      for (int k = 0; k < KC; ++k) {
+        const int n = threadIdx.x / 32 + 2 * NF * (k0 + k);
+        d[k] = 0.0;
+        if (p < P && n < 2 * ny) d[k] = n < ny ? v0[(size_t)n * 2 * P] : g0[(size_t)(n - ny) * gs];
+      }
+#pragma unroll
+      for (int k = 0; k < KC; ++k) {
+        const int n = threadIdx.x / 32 + 2 * NF * (k0 + k);
+        if (n < 2 * ny) tile[n * 32 + lane] = (RN)d[k];
+      }
     }
     __syncthreads();
   }
@@ -158,7 +174,7 @@ __global__ void __launch_bounds__(64 * NF, ctas_of(pre_dct_regs<RN, N>(), 64 * N
   if (p >= P) return;
   RN* dst = reinterpret_cast<RN*>(q) + 2 * (((size_t)b * 6 + f) * ny * P + p) + r;
   const size_t qs = 2 * (size_t)P;
-#pragma unroll 8
+#pragma unroll 16
   for (int j = half; j < H; j += 2) {
     const RN e = part[j * 32 + lane], o = part[(H + 1 + j) * 32 + lane];
     dst[(size_t)j * qs] = e + o;
