@@ -73,6 +73,20 @@ __device__ __forceinline__ double widen(float f) {
 }
 __device__ __forceinline__ double widen(double f) { return f; }
 
+// double -> float, round to nearest even, by integer operations (as widen).
+// Magnitudes below the smallest normal float become zero.
+__device__ __forceinline__ float narrow(double d) {
+  const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d), a = h & 0x7fffffffu;
+  unsigned u = __funnelshift_l(l, a - 0x38000000u, 3);             // exponent rebiased, 23 fraction bits
+  u += ((l & 0x1fffffffu) + 0x0fffffffu + (u & 1u)) >> 29;          // the 29 bits dropped
+  if (a < 0x38100000u) u = 0u;
+  if (a >= 0x47f00000u) u = a > 0x7ff00000u || (a == 0x7ff00000u && l) ? 0x7fffffffu : 0x7f800000u;  // NaN, else infinity
+  return __uint_as_float(u | (h & 0x80000000u));
+}
+template <typename RN> __device__ __forceinline__ RN to_rn(double d);
+template <> __device__ __forceinline__ double to_rn<double>(double d) { return d; }
+template <> __device__ __forceinline__ float to_rn<float>(double d) { return narrow(d); }
+
 #define CH_CPX_OPS(C, R)                                                                   \
   __host__ __device__ __forceinline__ C operator+(C a, C b) { return mk(a.x + b.x, a.y + b.y); } \
   __host__ __device__ __forceinline__ C operator-(C a, C b) { return mk(a.x - b.x, a.y - b.y); } \

@@ -187,9 +187,11 @@ __device__ __forceinline__ void dft_reg(C (&x)[N]) {
 //   forward: x = ka + A kb -> B-point DFTs over kb, twiddle, A-point DFTs over
 //            ka -> k = B p + s (kept: p outside the middle third).
 // B = 4 leaves the fewest operations (twiddles on 3/4 of the points, one
-// radix-4 butterfly) and enough independent lines per plane; A <= 48 points
-// fit the register file in FP64.
-__host__ __device__ constexpr int line_b(int m) { return m == 6 || m == 18 ? 2 : m >= 288 ? 8 : 4; }
+// radix-4 butterfly) and enough independent lines per plane; longer lines take
+// B = 8 and 16, so that A stays at 24 points or fewer and a step needs little
+// more than 100 registers in FP64 (with A = 48 the passes over 192 and 384
+// points held 6 warps per SM).
+__host__ __device__ constexpr int line_b(int m) { return m == 6 || m == 18 ? 2 : m <= 96 ? 4 : m <= 192 ? 8 : 16; }
 __host__ __device__ constexpr int line_a(int m) { return m / line_b(m); }
 // padded lengths built: 3/2 of 8, 12, 16, 24, 32, 48, 64, 96, 128, 192 and 256 modes
 #define CH_LINE_LENGTHS(X) X(12) X(18) X(24) X(36) X(48) X(72) X(96) X(144) X(192) X(288) X(384)

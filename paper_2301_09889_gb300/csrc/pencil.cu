@@ -124,8 +124,8 @@ __global__ void wall_shear_kernel(int ny, int B, const double* UM, double nu, do
 // component q of Dv and omega_y makes component 1 - q of u = (i kx Dv - i kz
 // omega_y) / k^2, so a lane group exchanges nothing with the other component.
 // FP64-bound: three operations per coefficient and component.  One lane per
-// system where the batch fills the SMs that way, eight (shorter chains, seven
-// operations more per system) for few modes.
+// system where the batch fills the SMs that way; four or eight (shorter chains
+// of loads, a few operations more) for fewer systems or longer columns.
 // ---------------------------------------------------------------------------
 template <int L>
 __global__ void __launch_bounds__(128) sense_kernel(Grid g, int B, PencilBufs pb, DevTables t, int js, double alpha,
@@ -418,8 +418,10 @@ cudaError_t launch_wall_shear(const Grid& g, int B, const double* UM, double nu,
 cudaError_t launch_sense(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, int js, double alpha,
                          int opposition, cudaStream_t st) {
   const long sys = 2L * g.P * B;
-  if (sys >= 16384)
+  if (sys >= 65536 && g.ny <= 97)
     sense_kernel<1><<<(unsigned)((sys + 127) / 128), 128, 0, st>>>(g, B, pb, t, js, alpha, opposition);
+  else if (sys >= 16384)
+    sense_kernel<4><<<(unsigned)((4 * sys + 127) / 128), 128, 0, st>>>(g, B, pb, t, js, alpha, opposition);
   else
     sense_kernel<8><<<(unsigned)((8 * sys + 127) / 128), 128, 0, st>>>(g, B, pb, t, js, alpha, opposition);
   return cudaGetLastError();

@@ -20,14 +20,15 @@ __host__ __device__ constexpr int io_a(int n) { return n / io_b(n); }
 // line lengths built
 #define CH_IO_LENGTHS(X) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(192) X(256)
 
-constexpr int kIoCols = 8;   // columns per single-warp CTA of a z pass
-constexpr int kIoPairs = 8;  // row pairs per CTA of an x pass
+// columns per single-warp CTA of a z pass and row pairs per CTA of an x pass:
+// eight where the batch has CTAs to spare, two for single large planes, whose
+// few lines spread over more SMs (the chain of a warp is what their passes take)
 constexpr int kIoNT = 64;
 
 // z inverse of the sensing spectra in place: planes [B][2][nz][nxh]
-template <int NZ>
+template <int NZ, int CT>
 __global__ void __launch_bounds__(32) obs_z_kernel(int nxh, double2* planes, const double2* __restrict__ tw, const int* active) {
-  constexpr int A = io_a(NZ), B = io_b(NZ), CT = kIoCols;
+  constexpr int A = io_a(NZ), B = io_b(NZ);
   __shared__ double2 T[NZ * CT];
   const int b = blockIdx.y, c0 = blockIdx.x * CT;
   if (active && !active[b]) return;
@@ -59,16 +60,16 @@ __global__ void __launch_bounds__(32) obs_z_kernel(int nxh, double2* planes, con
 }
 
 // x inverse of row pairs of both fields to the observation planes
-template <int NX>
+template <int NX, int NPR>
 __global__ void __launch_bounds__(kIoNT) obs_x_kernel(int nz, const double2* __restrict__ planes,
                                                       const double2* __restrict__ tw, double* out, size_t out_stride,
                                                       const int* active) {
   constexpr int A = io_a(NX), B = io_b(NX), A1 = A | 1, LS = B * A1, NXH = NX / 2;
-  extern __shared__ __align__(16) double2 iosm[];  // [kIoPairs][B][A1]
-  const int b = blockIdx.y, g0 = blockIdx.x * kIoPairs;  // row pair (field, m): rows 2 m, 2 m + 1
+  extern __shared__ __align__(16) double2 iosm[];  // [NPR][B][A1]
+  const int b = blockIdx.y, g0 = blockIdx.x * NPR;  // row pair (field, m): rows 2 m, 2 m + 1
   if (active && !active[b]) return;
   const double2* F = planes + (size_t)b * 2 * nz * NXH;
-  for (int w = threadIdx.x; w < kIoPairs * B; w += kIoNT) {
+  for (int w = threadIdx.x; w < NPR * B; w += kIoNT) {
     const int kb = w % B, g = g0 + w / B;
     if (g >= nz) continue;
     const double2* r1 = F + (size_t)2 * g * NXH;  // the rows of both fields follow one another
@@ -94,7 +95,7 @@ __global__ void __launch_bounds__(kIoNT) obs_x_kernel(int nz, const double2* __r
     for (int p = 0; p < A; ++p) iosm[(w / B) * LS + kb * A1 + p] = x[p];
   }
   __syncthreads();
-  for (int w = threadIdx.x; w < kIoPairs * A; w += kIoNT) {
+  for (int w = threadIdx.x; w < NPR * A; w += kIoNT) {
     const int ka = w % A, g = g0 + w / A;
     if (g >= nz) continue;
     const double2* X = iosm + (w / A) * LS + ka;
@@ -114,17 +115,17 @@ __global__ void __launch_bounds__(kIoNT) obs_x_kernel(int nz, const double2* __r
 
 // x forward of the clipped action, row pairs; starts the new action as
 // action_x_kernel (pencil.cu)
-template <int NX>
+template <int NX, int NPR>
 __global__ void __launch_bounds__(kIoNT) act_x_kernel(int nz, const double* __restrict__ act, double u_tau,
                                                       const double2* __restrict__ tw, double2* tx, double2* vw_old,
                                                       const double2* vw, double* acc, const int* active) {
   constexpr int A = io_a(NX), B = io_b(NX), A1 = A | 1, LS = B * A1, NXH = NX / 2;
   extern __shared__ __align__(16) double2 iosm[];
-  const int b = blockIdx.y, g0 = blockIdx.x * kIoPairs, pairs = nz / 2;
+  const int b = blockIdx.y, g0 = blockIdx.x * NPR, pairs = nz / 2;
   if (active && !active[b]) return;
   const double* src = act + (size_t)b * nz * NX;
   auto clip = [u_tau](double v) { return fmin(fmax(v, -u_tau), u_tau); };
-  for (int w = threadIdx.x; w < kIoPairs * A; w += kIoNT) {
+  for (int w = threadIdx.x; w < NPR * A; w += kIoNT) {
     const int ka = w % A, g = g0 + w / A;
     if (g >= pairs) continue;
     const double* r1 = src + (size_t)2 * g * NX;
@@ -138,7 +139,7 @@ __global__ void __launch_bounds__(kIoNT) act_x_kernel(int nz, const double* __re
     for (int s = 1; s < B; ++s) X[s * A1] = cmul(x[s], cconj(tw[s * ka]));
   }
   __syncthreads();
-  for (int w = threadIdx.x; w < kIoPairs * B; w += kIoNT) {
+  for (int w = threadIdx.x; w < NPR * B; w += kIoNT) {
     double2* X = iosm + (w / B) * LS + (w % B) * A1;
     if (g0 + w / B >= pairs) continue;
     double2 x[A];
@@ -149,7 +150,7 @@ __global__ void __launch_bounds__(kIoNT) act_x_kernel(int nz, const double* __re
     for (int p = 0; p < A; ++p) X[p] = x[p];  // k = B p + s
   }
   __syncthreads();
-  for (int w = threadIdx.x; w < kIoPairs * NXH; w += kIoNT) {
+  for (int w = threadIdx.x; w < NPR * NXH; w += kIoNT) {
     const int i = w % NXH, g = g0 + w / NXH;
     if (g >= pairs) continue;
     const int im = i == 0 ? 0 : NX - i;
@@ -164,10 +165,10 @@ __global__ void __launch_bounds__(kIoNT) act_x_kernel(int nz, const double* __re
 }
 
 // z forward of the action to the wall spectrum
-template <int NZ>
+template <int NZ, int CT>
 __global__ void __launch_bounds__(32) act_z_kernel(int nx, const double2* __restrict__ tx, const double2* __restrict__ tw,
                                                    double2* vw, const int* active) {
-  constexpr int A = io_a(NZ), B = io_b(NZ), CT = kIoCols;
+  constexpr int A = io_a(NZ), B = io_b(NZ);
   __shared__ double2 T[NZ * CT];
   const int b = blockIdx.y, c0 = blockIdx.x * CT, nxh = nx / 2;
   if (active && !active[b]) return;

@@ -24,23 +24,24 @@
 
 namespace chdns {
 
-// z passes: CTAs of W warps on 8 W adjacent columns
-constexpr int kZCols = 8;
-template <typename R> constexpr int z_warps() { return sizeof(R) == 4 ? 2 : 1; }
+// z passes: tiles of 16 (FP32) or 8 (FP64) adjacent columns, one task of the
+// first step per thread
+template <typename R> constexpr int z_cols() { return sizeof(R) == 4 ? 16 : 8; }
+template <typename R> constexpr int z_threads(int m) { return line_b(m) * z_cols<R>() < 32 ? 32 : line_b(m) * z_cols<R>(); }
 
 // x pass: row pairs per CTA (multiples of 8 fill every warp of every phase;
-// fewer where six fields of M points outgrow shared memory) and threads
+// fewer where six fields of M points would leave one CTA per SM) and threads
 template <typename R> constexpr int x_pairs(int m) {
-  return (sizeof(R) == 4 ? m <= 192 : m <= 144) ? 8 : (sizeof(R) == 4 || m <= 192) ? 4 : 2;
+  return (sizeof(R) == 4 ? m <= 192 : m <= 96) ? 8 : (sizeof(R) == 4 || m <= 192) ? 4 : 2;
 }
-template <typename R> constexpr int x_threads(int m) { return m <= 24 ? 96 : 192; }
+template <typename R> constexpr int x_threads(int m) { return m <= 24 ? 96 : sizeof(R) == 4 && m >= 144 ? 384 : 192; }
 // odd row stride: the transposing accesses of the exchange meet no bank twice
 __host__ __device__ constexpr int x_stride(int m) { return line_a(m) | 1; }
 
-template <typename R, int MZ, int W>
-__global__ void __launch_bounds__(32 * W) zpass_inverse_kernel(PlaneArgs<R> a) {
+template <typename R, int MZ>
+__global__ void __launch_bounds__(z_threads<R>(MZ)) zpass_inverse_kernel(PlaneArgs<R> a) {
   using C = typename cpx<R>::T;
-  constexpr int A = line_a(MZ), B = line_b(MZ), CT = kZCols * W, NT = 32 * W;
+  constexpr int A = line_a(MZ), B = line_b(MZ), CT = z_cols<R>(), NT = z_threads<R>(MZ);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* T = reinterpret_cast<C*>(smem_raw);  // [B][A][CT]
   const int b = blockIdx.y, nxh = a.nxh;
@@ -73,7 +74,7 @@ __global__ void __launch_bounds__(32 * W) zpass_inverse_kernel(PlaneArgs<R> a) {
     x[0] = T[ka * CT + c];
 #pragma unroll
     for (int s = 1; s < B; ++s) x[s] = cmul(T[(s * A + ka) * CT + c], a.tw_mz[s * ka]);
-    small_dft_ct<+1, B, C, R>(x);
+    dft_pow2<+1, B, R>(x);
     C* dst = yb + (size_t)(g / nxh) * MZ * nxh + g % nxh;
 #pragma unroll
     for (int s = 0; s < B; ++s) dst[(size_t)(ka + A * s) * nxh] = x[s];
@@ -120,39 +121,76 @@ __global__ void __launch_bounds__(NT) xpass_kernel(PlaneArgs<R> a) {
     for (int p = 0; p < A; ++p) X[line * LS + kb * A1 + p] = x[p];
   }
   __syncthreads();
-  // second half of the inverse lines, products and first half of the forward
-  // lines at the points ka + A kb of one row pair (real parts: first row,
-  // imaginary parts: second row); each thread reads and writes its own slots
-  for (int w = threadIdx.x; w < NPR * A; w += NT) {
-    const int ka = w % A, pp = w / A;
-    if (g0 + pp >= npairs) continue;
-    C t[B];
+  if constexpr (B <= 4) {
+    // second half of the inverse lines, products and first half of the forward
+    // lines at the points ka + A kb of one row pair (real parts: first row,
+    // imaginary parts: second row); each thread reads and writes its own slots
+    for (int w = threadIdx.x; w < NPR * A; w += NT) {
+      const int ka = w % A, pp = w / A;
+      if (g0 + pp >= npairs) continue;
+      C t[B];
 #pragma unroll
-    for (int s = 1; s < B; ++s) t[s] = a.tw_x[s * ka];
-    C* slot = X + pp * LS + ka;
+      for (int s = 1; s < B; ++s) t[s] = a.tw_x[s * ka];
+      C* slot = X + pp * LS + ka;
+      constexpr int FS = NPR * LS;
+      C v[6][B];
+#pragma unroll
+      for (int f = 0; f < 6; ++f) {
+        v[f][0] = slot[f * FS];
+#pragma unroll
+        for (int s = 1; s < B; ++s) v[f][s] = cmul(slot[f * FS + s * A1], t[s]);
+        small_dft_ct<+1, B, C, R>(v[f]);
+      }
+      C h[3][B];
+#pragma unroll
+      for (int s = 0; s < B; ++s) {
+        const C u = v[0][s], vv = v[1][s], ww = v[2][s], ox = v[3][s], oy = v[4][s], oz = v[5][s];
+        h[0][s] = mk(vv.x * oz.x - ww.x * oy.x, vv.y * oz.y - ww.y * oy.y);
+        h[1][s] = mk(ww.x * ox.x - u.x * oz.x, ww.y * ox.y - u.y * oz.y);
+        h[2][s] = mk(u.x * oy.x - vv.x * ox.x, u.y * oy.y - vv.y * ox.y);
+      }
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        small_dft_ct<-1, B, C, R>(h[f]);
+        slot[f * FS] = h[f][0];
+#pragma unroll
+        for (int s = 1; s < B; ++s) slot[f * FS + s * A1] = cmul(h[f][s], cconj(t[s]));
+      }
+    }
+  } else {
+    // longer lines: field by field in place, the products point by point (six
+    // lines of B points would take 200 registers in FP64)
     constexpr int FS = NPR * LS;
-    C v[6][B];
+    for (int w = threadIdx.x; w < 6 * NPR * A; w += NT) {
+      const int ka = w % A;
+      C* slot = X + (w / A) * LS + ka;
+      C v[B];
+      v[0] = slot[0];
 #pragma unroll
-    for (int f = 0; f < 6; ++f) {
-      v[f][0] = slot[f * FS];
+      for (int s = 1; s < B; ++s) v[s] = cmul(slot[s * A1], a.tw_x[s * ka]);
+      dft_pow2<+1, B, R>(v);
 #pragma unroll
-      for (int s = 1; s < B; ++s) v[f][s] = cmul(slot[f * FS + s * A1], t[s]);
-      small_dft_ct<+1, B, C, R>(v[f]);
+      for (int s = 0; s < B; ++s) slot[s * A1] = v[s];
     }
-    C h[3][B];
-#pragma unroll
-    for (int s = 0; s < B; ++s) {
-      const C u = v[0][s], vv = v[1][s], ww = v[2][s], ox = v[3][s], oy = v[4][s], oz = v[5][s];
-      h[0][s] = mk(vv.x * oz.x - ww.x * oy.x, vv.y * oz.y - ww.y * oy.y);
-      h[1][s] = mk(ww.x * ox.x - u.x * oz.x, ww.y * ox.y - u.y * oz.y);
-      h[2][s] = mk(u.x * oy.x - vv.x * ox.x, u.y * oy.y - vv.y * ox.y);
+    __syncthreads();
+    for (int w = threadIdx.x; w < NPR * B * A; w += NT) {
+      C* L = X + (w / (A * B)) * LS + (w / A % B) * A1 + w % A;
+      const C u = L[0], vv = L[FS], ww = L[2 * FS], ox = L[3 * FS], oy = L[4 * FS], oz = L[5 * FS];
+      L[0] = mk(vv.x * oz.x - ww.x * oy.x, vv.y * oz.y - ww.y * oy.y);
+      L[FS] = mk(ww.x * ox.x - u.x * oz.x, ww.y * ox.y - u.y * oz.y);
+      L[2 * FS] = mk(u.x * oy.x - vv.x * ox.x, u.y * oy.y - vv.y * ox.y);
     }
+    __syncthreads();
+    for (int w = threadIdx.x; w < 3 * NPR * A; w += NT) {
+      const int ka = w % A;
+      C* slot = X + (w / A) * LS + ka;
+      C v[B];
 #pragma unroll
-    for (int f = 0; f < 3; ++f) {
-      small_dft_ct<-1, B, C, R>(h[f]);
-      slot[f * FS] = h[f][0];
+      for (int s = 0; s < B; ++s) v[s] = slot[s * A1];
+      dft_pow2<-1, B, R>(v);
+      slot[0] = v[0];
 #pragma unroll
-      for (int s = 1; s < B; ++s) slot[f * FS + s * A1] = cmul(h[f][s], cconj(t[s]));
+      for (int s = 1; s < B; ++s) slot[s * A1] = cmul(v[s], cconj(a.tw_x[s * ka]));
     }
   }
   __syncthreads();
@@ -175,15 +213,15 @@ __global__ void __launch_bounds__(NT) xpass_kernel(PlaneArgs<R> a) {
     const C zk = X[line * LS + (i % B) * A1 + i / B];
     const C zm = X[line * LS + (im % B) * A1 + im / B];
     C* dst = rows(g, line / NPR);
-    dst[i] = mk((zk.x + zm.x) * (R)0.5, (zk.y - zm.y) * (R)0.5);
-    dst[NXH + i] = mk((zk.y + zm.y) * (R)0.5, (zm.x - zk.x) * (R)0.5);
+    dst[i] = mk(zk.x + zm.x, zk.y - zm.y);  // twice the rows: the last pass scales by half as much
+    dst[NXH + i] = mk(zk.y + zm.y, zm.x - zk.x);
   }
 }
 
-template <typename R, int MZ, int W>
-__global__ void __launch_bounds__(32 * W) zpass_forward_kernel(PlaneArgs<R> a) {
+template <typename R, int MZ>
+__global__ void __launch_bounds__(z_threads<R>(MZ)) zpass_forward_kernel(PlaneArgs<R> a) {
   using C = typename cpx<R>::T;
-  constexpr int A = line_a(MZ), B = line_b(MZ), CT = kZCols * W, NT = 32 * W;
+  constexpr int A = line_a(MZ), B = line_b(MZ), CT = z_cols<R>(), NT = z_threads<R>(MZ);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* T = reinterpret_cast<C*>(smem_raw);  // [B][A][CT]
   const int b = blockIdx.y, nxh = a.nxh;
@@ -199,7 +237,7 @@ __global__ void __launch_bounds__(32 * W) zpass_forward_kernel(PlaneArgs<R> a) {
     C x[B];
 #pragma unroll
     for (int s = 0; s < B; ++s) x[s] = src[(size_t)(ka + A * s) * nxh];
-    small_dft_ct<-1, B, C, R>(x);
+    dft_pow2<-1, B, R>(x);
     T[ka * CT + c] = x[0];
 #pragma unroll
     for (int s = 1; s < B; ++s) T[(s * A + ka) * CT + c] = cmul(x[s], cconj(a.tw_mz[s * ka]));
@@ -214,35 +252,36 @@ __global__ void __launch_bounds__(32 * W) zpass_forward_kernel(PlaneArgs<R> a) {
     for (int p = 0; p < A; ++p) x[p] = T[(s * A + p) * CT + c];
     dft_reg<-1, false, A, R>(x);
     C* dst = a.h + (((size_t)b * 3 + f) * a.ny + j) * a.P + i;
+    const R sc = (R)0.5 * a.scale;
 #pragma unroll
-    for (int p = 0; p < A / 3; ++p) dst[(size_t)(B * p + s) * nxh] = a.scale * x[p];
+    for (int p = 0; p < A / 3; ++p) dst[(size_t)(B * p + s) * nxh] = sc * x[p];
 #pragma unroll
     for (int p = 2 * A / 3; p < A; ++p) {
       const int row = B * p + s - MZ / 3;
-      dst[(size_t)row * nxh] = (p == 2 * A / 3 && s == 0) ? czero<C>() : a.scale * x[p];
+      dst[(size_t)row * nxh] = (p == 2 * A / 3 && s == 0) ? czero<C>() : sc * x[p];
     }
   }
 }
 
 template <typename R, int MZ>
 cudaError_t zpass_inverse_m(const PlaneArgs<R>& a, int B, cudaStream_t st) {
-  constexpr int W = z_warps<R>(), CT = kZCols * W;
+  constexpr int CT = z_cols<R>(), NT = z_threads<R>(MZ);
   constexpr size_t smem = (size_t)MZ * CT * sizeof(typename cpx<R>::T);
   static SmemLimit lim;
-  const cudaError_t e = raise_smem_limit(zpass_inverse_kernel<R, MZ, W>, &lim, smem);
+  const cudaError_t e = raise_smem_limit(zpass_inverse_kernel<R, MZ>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(R) == 4>(zpass_inverse_kernel<R, MZ, W>, dim3((a.ny * 6 * a.nxh + CT - 1) / CT, B),
-                                       dim3(32 * W), smem, st, a);
+  return launch_pdl_if<sizeof(R) == 4>(zpass_inverse_kernel<R, MZ>, dim3((a.ny * 6 * a.nxh + CT - 1) / CT, B),
+                                       dim3(NT), smem, st, a);
 }
 template <typename R, int MZ>
 cudaError_t zpass_forward_m(const PlaneArgs<R>& a, int B, cudaStream_t st) {
-  constexpr int W = z_warps<R>(), CT = kZCols * W;
+  constexpr int CT = z_cols<R>(), NT = z_threads<R>(MZ);
   constexpr size_t smem = (size_t)MZ * CT * sizeof(typename cpx<R>::T);
   static SmemLimit lim;
-  const cudaError_t e = raise_smem_limit(zpass_forward_kernel<R, MZ, W>, &lim, smem);
+  const cudaError_t e = raise_smem_limit(zpass_forward_kernel<R, MZ>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(R) == 4>(zpass_forward_kernel<R, MZ, W>, dim3((a.ny * 3 * a.nxh + CT - 1) / CT, B),
-                                       dim3(32 * W), smem, st, a);
+  return launch_pdl_if<sizeof(R) == 4>(zpass_forward_kernel<R, MZ>, dim3((a.ny * 3 * a.nxh + CT - 1) / CT, B),
+                                       dim3(NT), smem, st, a);
 }
 template <typename R, int MX>
 cudaError_t xpass_m(const PlaneArgs<R>& a, int B, cudaStream_t st) {

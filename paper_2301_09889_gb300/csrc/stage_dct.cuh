@@ -37,39 +37,42 @@ namespace chdns {
 //   omega_x, omega_z: cD (D^2 v)_n + cS (DS)_n + cV Va_n      S = Ga (mean: W, U)
 // The derivatives are running sums from n = N down (c_m b_m = b_{m+2} +
 // 2 (m+1) a_{m+1}), in the node precision.
+//
+// The coefficients of a parity are formed by rolled loops into the thread's
+// column of the exchange buffer and then read into registers: with the loops
+// unrolled, the kernel's paths (three kinds of field, two parities) outgrew
+// the instruction cache wherever an SM ran several of them.
+//
+// CTA: NF fields of one tile, two warps (even, odd) each.  FP32 lines of up to
+// 65 nodes: all six, which share v and omega_y, rounded once into shared memory
+// (a conversion instruction occupies the FP64 pipe as an FP64 operation does);
+// longer and FP64 lines: one, reading its columns in place.
 // ---------------------------------------------------------------------------
-template <typename RN> constexpr int dct_fields(int nf) { return sizeof(RN) == 4 ? nf : 1; }  // fields per CTA
-// CTAs per SM the registers are held to: one parity's array and the transform
-// around it
+template <typename RN, int N> constexpr int pre_fields() { return sizeof(RN) == 4 && N <= 64 ? 6 : 1; }
 constexpr int ctas_of(int regs, int threads) { return 65536 / (regs * threads) > 0 ? 65536 / (regs * threads) : 1; }
-template <typename RN, int N> constexpr int pre_dct_regs() {
-  return sizeof(RN) == 8 ? (N <= 32 ? 96 : N <= 64 ? 168 : 255) : (N <= 32 ? 56 : N <= 64 ? 80 : N <= 96 ? 112 : 168);
-}
-template <typename RN, int N> constexpr int analysis_dct_regs() {
-  return sizeof(RN) == 8 ? (N <= 32 ? 128 : 255) : (N <= 32 ? 72 : N <= 64 ? 128 : N <= 96 ? 168 : 255);
+// registers a thread is held to: one parity's array and the transform around it
+template <typename RN, int N> constexpr int dct_regs() {
+  return sizeof(RN) == 8 ? (N <= 32 ? 96 : N <= 64 ? 168 : 255) : (N <= 32 ? 56 : N <= 64 ? 80 : N <= 96 ? 96 : N <= 128 ? 128 : 168);
 }
 
 template <typename RN, int N, int NF>
-__global__ void __launch_bounds__(64 * NF, ctas_of(pre_dct_regs<RN, N>(), 64 * NF)) stage_pre_dct_kernel(Grid g, PencilBufs pb, DevTables t,
-                                                                    typename cpx<RN>::T* __restrict__ q) {
-  constexpr int H = N / 2;
-  // FP32 lines: v and omega_y of the tile are rounded to FP32 once, into shared
-  // memory (a conversion costs as much as an FP64 operation, and every line
-  // reads two of the columns); FP64 lines read them in place
-  constexpr bool kTile = sizeof(RN) == 4;
+__global__ void __launch_bounds__(64 * NF, ctas_of(dct_regs<RN, N>(), 64 * NF)) stage_pre_dct_kernel(Grid g, PencilBufs pb,
+                                                                DevTables t, typename cpx<RN>::T* __restrict__ q) {
+  constexpr int H = N / 2, ny = N + 1;
+  constexpr bool kTile = NF > 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int P = g.P, ny = N + 1;
-  const int lane = threadIdx.x & 31, fl = threadIdx.x / 64, half = (threadIdx.x / 32) & 1, f = blockIdx.z * NF + fl;
-  RN* tile = reinterpret_cast<RN*>(smem_raw);  // [v, omega_y][ny][32], until the partial sums take its place
-  RN* part = reinterpret_cast<RN*>(smem_raw) + fl * (N + 1) * 32;  // [E_0 .. E_H, O_0 .. O_{H-1}][32]
-  const int p = blockIdx.x * 16 + (lane >> 1), r = lane & 1;
+  const int P = g.P;
+  const int lane = threadIdx.x & 31, fl = threadIdx.x / 64, half = (threadIdx.x / 32) & 1, f = blockIdx.x % (6 / NF) * NF + fl;
+  RN* part = reinterpret_cast<RN*>(smem_raw) + fl * ny * 32;        // [E_0 .. E_H, O_0 .. O_{H-1}][32]
+  RN* tile = reinterpret_cast<RN*>(smem_raw) + NF * ny * 32;        // [v, omega_y][ny][32]
+  const int p0 = (int)blockIdx.x / (6 / NF) * 16, p = p0 + (lane >> 1), r = lane & 1;
   const int b = blockIdx.y;
   if (pb.active && !pb.active[b]) return;
   pdl_wait_then_release();  // v, omega_y come from the previous stage
   if constexpr (kTile) {
     // a column per warp and step, every load in flight before the first store
-    constexpr int KL = (2 * (N + 1) + 2 * NF - 1) / (2 * NF);
-    const size_t c0 = 2 * ((size_t)b * ny * P + blockIdx.x * 16) + lane;
+    constexpr int KL = (2 * ny + 2 * NF - 1) / (2 * NF);
+    const size_t c0 = 2 * ((size_t)b * ny * P + p0) + lane;
     const double* v0 = reinterpret_cast<const double*>(pb.V) + c0;
     const double* g0 = reinterpret_cast<const double*>(pb.G) + c0;
     size_t gs = 2 * (size_t)P;
@@ -77,104 +80,115 @@ __global__ void __launch_bounds__(64 * NF, ctas_of(pre_dct_regs<RN, N>(), 64 * N
       g0 = (r == 0 ? pb.WM : pb.UM) + (size_t)b * ny;
       gs = 1;
     }
-    constexpr int KC = KL <= 12 ? KL : (KL + (KL + 11) / 12 - 1) / ((KL + 11) / 12);  // at most 12 at a time
-    for (int k0 = 0; k0 < KL; k0 += KC) {
-      double d[KC];
+    double d[KL];
 #pragma unroll
-      for (int k = 0; k < KC; ++k) {
-        const int n = threadIdx.x / 32 + 2 * NF * (k0 + k);
-        d[k] = 0.0;
-        if (p < P && n < 2 * ny) d[k] = n < ny ? v0[(size_t)n * 2 * P] : g0[(size_t)(n - ny) * gs];
-      }
+    for (int k = 0; k < KL; ++k) {
+      const int n = threadIdx.x / 32 + 2 * NF * k;
+      d[k] = 0.0;
+      if (p < P && n < 2 * ny) d[k] = n < ny ? v0[(size_t)n * 2 * P] : g0[(size_t)(n - ny) * gs];
+    }
 #pragma unroll
-      for (int k = 0; k < KC; ++k) {
-        const int n = threadIdx.x / 32 + 2 * NF * (k0 + k);
-        if (n < 2 * ny) tile[n * 32 + lane] = (RN)d[k];
-      }
+    for (int k = 0; k < KL; ++k) {
+      const int n = threadIdx.x / 32 + 2 * NF * k;
+      if (n < 2 * ny) tile[n * 32 + lane] = (RN)d[k];
     }
     __syncthreads();
   }
-  RN x[H + 1];
+  RN* mine = part + half * (H + 1) * 32 + lane;
   if (p < P) {
     const int row = p / g.nxh, ix = p % g.nxh;
     const bool mean = p == 0, gen = !mean && row != g.nz / 2;
+    const bool own = f == 1 || f == 4, deriv = f == 3 || f == 5;
     const RN kx = (RN)t.kx[ix], kz = (RN)t.kz[row];
     const RN sg = r == 0 ? (RN)-1.0 : (RN)1.0;
     const RN ik2 = gen ? sg / (kx * kx + kz * kz) : (RN)0;
-    const bool own = f == 1 || f == 4, deriv = f == 3 || f == 5;
-    const size_t col = 2 * ((size_t)b * ny * P + p);  // component 0 of coefficient 0; 2 P per coefficient
-    const double* Vp = reinterpret_cast<const double*>(pb.V) + col + (1 - r);
-    const double* Sp;
-    size_t ss = 2 * (size_t)P;
     RN cD = 0, cS = 1, cV = 0;
-    if (own) {
-      Sp = reinterpret_cast<const double*>(f == 1 ? pb.V : pb.G) + col + r;
-    } else if (mean) {
-      Sp = (f == 0 || f == 5 ? pb.UM : pb.WM) + (size_t)b * ny;
-      ss = 1;
-      if (f == 5) cS = (RN)-1.0;
-    } else {
-      Sp = reinterpret_cast<const double*>(pb.G) + col + (1 - r);
+    if (gen && !own) {
       if (f == 0) { cD = ik2 * kx; cS = -ik2 * kz; }
       if (f == 2) { cD = ik2 * kz; cS = ik2 * kx; }
       if (f == 3) { cD = ik2 * kz; cS = ik2 * kx; cV = -sg * kz; }
       if (f == 5) { cD = -ik2 * kx; cS = ik2 * kz; cV = sg * kx; }
+    } else if (mean && f == 5) {
+      cS = (RN)-1.0;
     }
     const bool liveS = gen || (mean && !own && r == 0);
+    const size_t col = 2 * ((size_t)b * ny * P + p);  // component 0 of coefficient 0; 2 P per coefficient
+    const double* Vp = reinterpret_cast<const double*>(pb.V) + col + (1 - r);
+    const double* Sp = reinterpret_cast<const double*>(f == 1 ? pb.V : pb.G) + col + (own ? r : 1 - r);
+    const size_t vs = 2 * (size_t)P;
+    size_t ss = vs;
+    if (mean && !own) {
+      Sp = (f == 0 || f == 5 ? pb.UM : pb.WM) + (size_t)b * ny;
+      ss = 1;
+    }
     const RN* Vt = tile + (lane ^ 1);
     const RN* St = tile + (f == 1 ? 0 : ny * 32) + (own ? lane : !mean ? lane ^ 1 : f == 0 || f == 5 ? 1 : 0);
-    auto V = [&](int n) { return !gen ? (RN)0 : kTile ? Vt[n * 32] : (RN)Vp[(size_t)n * ss]; };
-    auto S = [&](int n) { return !liveS ? (RN)0 : kTile ? St[n * 32] : (RN)Sp[(size_t)n * ss]; };
-    // coefficients of one parity, n = 2 i + par, from the top down
-    auto coefs = [&](int par, int count) {
-      if (own) {
-#pragma unroll
-        for (int i = count - 1; i >= 0; --i) x[i] = S(2 * i + par);
-      } else if (!deriv) {
-        RN dv = 0;
-#pragma unroll
-        for (int i = count - 1; i >= 0; --i) {
-          const int n = 2 * i + par;
-          if (n + 1 <= N) dv = dv + (RN)(2 * (n + 1)) * V(n + 1);
-          const RN d = n == 0 ? (RN)0.5 * dv : dv;
-          x[i] = cD * d + cS * S(n);
-        }
-      } else {
-        RN dv = 0, d2 = 0, ds = 0;
-#pragma unroll
-        for (int i = count - 1; i >= 0; --i) {
-          const int n = 2 * i + par, m = n + 1;
-          if (m <= N) {
-            if (m + 1 <= N) dv = dv + (RN)(2 * (m + 1)) * V(m + 1);
-            d2 = d2 + (RN)(2 * m) * dv;
-            ds = ds + (RN)(2 * m) * S(m);
-          }
-          const RN h = n == 0 ? (RN)0.5 : (RN)1.0;
-          x[i] = (cD * d2 + cS * ds) * h + cV * V(n);
-        }
-      }
+    auto V = [&](int n) { return !gen ? (RN)0 : kTile ? Vt[n * 32] : to_rn<RN>(__ldg(Vp + n * vs)); };
+    auto S = [&](int n) { return !liveS ? (RN)0 : kTile ? St[n * 32] : to_rn<RN>(__ldg(Sp + n * ss)); };
+    // 2 k; from a table in FP64, where converting it would cost an operation
+    auto c2 = [&](int k) {
+      if constexpr (sizeof(RN) == 8) return __ldg(t.tau.n1 + k - 1);
+      else return (RN)(2 * k);
     };
-    if (half == 0) coefs(0, H + 1);
-    else coefs(1, H);
+    // coefficients of this warp's parity, n = 2 i + half, from the top down
+    const int top = half == 0 ? H : H - 1;
+    if (own) {
+#pragma unroll 8
+      for (int i = top; i >= 0; --i) mine[i * 32] = S(2 * i + half);
+    } else if (!deriv) {
+      RN dv = half == 0 ? (RN)0 : (RN)(2 * N) * V(N);
+      mine[top * 32] = cD * dv + cS * S(2 * top + half);
+#pragma unroll 8
+      for (int i = top - 1; i >= 1; --i) {
+        const int n = 2 * i + half;
+        dv = dv + c2(n + 1) * V(n + 1);
+        mine[i * 32] = cD * dv + cS * S(n);
+      }
+      dv = dv + c2(half + 1) * V(half + 1);
+      mine[0] = cD * (half == 0 ? (RN)0.5 * dv : dv) + cS * S(half);
+    } else {
+      // the step at i adds m = 2 i + half + 1 to D^2 v and DS and m + 1 to Dv
+      RN dv = 0, d2 = 0, ds = 0;
+      if (half == 1) {
+        d2 = (RN)0;
+        ds = (RN)(2 * N) * S(N);
+      }
+      mine[top * 32] = cD * d2 + cS * ds + cV * V(2 * top + half);
+#pragma unroll 4
+      for (int i = top - 1; i >= 1; --i) {
+        const int m = 2 * i + half + 1;
+        dv = dv + c2(m + 1) * V(m + 1);
+        d2 = d2 + c2(m) * dv;
+        ds = ds + c2(m) * S(m);
+        mine[i * 32] = cD * d2 + cS * ds + cV * V(m - 1);
+      }
+      const int m = half + 1;
+      dv = dv + c2(m + 1) * V(m + 1);
+      d2 = d2 + c2(m) * dv;
+      ds = ds + c2(m) * S(m);
+      mine[0] = (cD * d2 + cS * ds) * (half == 0 ? (RN)0.5 : (RN)1.0) + cV * V(half);
+    }
   }
-  if constexpr (kTile) __syncthreads();
   if (half == 0) {
+    RN x[H + 1];
+#pragma unroll
+    for (int j = 0; j <= H; ++j) x[j] = mine[j * 32];
     dct1<H, RN>(x);
 #pragma unroll
-    for (int j = 0; j <= H; ++j) part[j * 32 + lane] = x[j];
+    for (int j = 0; j <= H; ++j) mine[j * 32] = x[j];
   } else {
-    RN o[H];
+    RN x[H];
 #pragma unroll
-    for (int j = 0; j < H; ++j) o[j] = x[j];
-    dct2<H, RN>(o);
+    for (int j = 0; j < H; ++j) x[j] = mine[j * 32];
+    dct2<H, RN>(x);
 #pragma unroll
-    for (int j = 0; j < H; ++j) part[(H + 1 + j) * 32 + lane] = o[j];
+    for (int j = 0; j < H; ++j) mine[j * 32] = x[j];
   }
   __syncthreads();
   if (p >= P) return;
   RN* dst = reinterpret_cast<RN*>(q) + 2 * (((size_t)b * 6 + f) * ny * P + p) + r;
   const size_t qs = 2 * (size_t)P;
-#pragma unroll 16
+#pragma unroll 8
   for (int j = half; j < H; j += 2) {
     const RN e = part[j * 32 + lane], o = part[(H + 1 + j) * 32 + lane];
     dst[(size_t)j * qs] = e + o;
@@ -184,61 +198,66 @@ __global__ void __launch_bounds__(64 * NF, ctas_of(pre_dct_regs<RN, N>(), 64 * N
 }
 
 // a_n = 2/(N cb_n) sum_j f_j cos(pi n j / N) / cb_j (cb_0 = cb_N = 2): even n
-// from f_j + f_{N-j}, odd n from f_j - f_{N-j}.  Both warps of a line have read
-// their columns before either writes coefficients over them.
-template <typename RN, int N, int NF>
-__global__ void __launch_bounds__(64 * NF, ctas_of(analysis_dct_regs<RN, N>(), 64 * NF)) analysis_dct_kernel(Grid g, PencilBufs pb,
+// from f_j + f_{N-j}, odd n from f_j - f_{N-j}.  The columns are staged in
+// shared memory, so both warps have all nodes before either writes
+// coefficients over them.
+template <typename RN, int N>
+__global__ void __launch_bounds__(64, ctas_of(dct_regs<RN, N>(), 64)) analysis_dct_kernel(Grid g, PencilBufs pb,
                                                                     typename cpx<RN>::T* __restrict__ hn) {
-  constexpr int H = N / 2;
-  const int P = g.P, ny = N + 1;
-  const int lane = threadIdx.x & 31, half = (threadIdx.x / 32) & 1, f = blockIdx.z * NF + threadIdx.x / 64;
+  constexpr int H = N / 2, ny = N + 1;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int P = g.P;
+  const int lane = threadIdx.x & 31, half = threadIdx.x / 32, f = blockIdx.z;
   const int p = blockIdx.x * 16 + (lane >> 1), r = lane & 1;
   const int b = blockIdx.y;
   if (pb.active && !pb.active[b]) return;
   pdl_wait_then_release();  // H comes from the nonlinear term
   RN* col = reinterpret_cast<RN*>(hn) + 2 * (((size_t)b * 3 + f) * ny * P + min(p, P - 1)) + r;
+  RN* sm = reinterpret_cast<RN*>(smem_raw) + lane;
   const size_t hs = 2 * (size_t)P;
-  const RN s0 = (RN)2.0 / (RN)N;
-  RN x[H + 1];
-#pragma unroll
-  for (int j = 0; j < H; ++j) {
-    const RN a = col[(size_t)j * hs], c = col[(size_t)(N - j) * hs];
-    x[j] = half == 0 ? a + c : a - c;
-  }
-  x[0] = (RN)0.5 * x[0];
-  x[H] = col[(size_t)H * hs];
+#pragma unroll 16
+  for (int j = half; j <= N; j += 2) sm[j * 32] = col[(size_t)j * hs];
   __syncthreads();
-  if (p >= P) return;
+  const RN s0 = (RN)2.0 / (RN)N;
   if (half == 0) {
+    RN x[H + 1];
+#pragma unroll
+    for (int j = 0; j < H; ++j) x[j] = sm[j * 32] + sm[(N - j) * 32];
+    x[0] = (RN)0.5 * x[0];
+    x[H] = sm[H * 32];
     dct1<H, RN>(x);
+    if (p >= P) return;
 #pragma unroll
     for (int i = 0; i <= H; ++i) col[(size_t)(2 * i) * hs] = ((i == 0 || i == H) ? (RN)0.5 * s0 : s0) * x[i];
   } else {
-    RN o[H];
+    RN x[H];
 #pragma unroll
-    for (int i = 0; i < H; ++i) o[i] = x[i];
-    dct3<H, RN>(o);
+    for (int j = 0; j < H; ++j) x[j] = sm[j * 32] - sm[(N - j) * 32];
+    x[0] = (RN)0.5 * x[0];
+    dct3<H, RN>(x);
+    if (p >= P) return;
 #pragma unroll
-    for (int i = 0; i < H; ++i) col[(size_t)(2 * i + 1) * hs] = s0 * o[i];
+    for (int i = 0; i < H; ++i) col[(size_t)(2 * i + 1) * hs] = s0 * x[i];
   }
 }
 
-// FP32 lines: all fields of a mode tile in one CTA, so that v and omega_y
-// are shared through L1; FP64 lines: one field per
-// CTA, which evens the FP64 work out over the SMs.
 template <typename RN, int N>
 cudaError_t pre_dct_n(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, typename cpx<RN>::T* q, cudaStream_t st) {
-  constexpr int NF = dct_fields<RN>(6);
-  constexpr size_t smem = (size_t)NF * (N + 1) * 32 * sizeof(RN);
+  constexpr int NF = pre_fields<RN, N>();
+  constexpr size_t smem = (size_t)(NF + (NF > 1 ? 2 : 0)) * (N + 1) * 32 * sizeof(RN);
   static SmemLimit lim;
   const cudaError_t e = raise_smem_limit(stage_pre_dct_kernel<RN, N, NF>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(RN) == 4>(stage_pre_dct_kernel<RN, N, NF>, dim3((g.P + 15) / 16, B, 6 / NF), dim3(64 * NF),
+  return launch_pdl_if<sizeof(RN) == 4>(stage_pre_dct_kernel<RN, N, NF>, dim3((g.P + 15) / 16 * (6 / NF), B), dim3(64 * NF),
                                         smem, st, g, pb, t, q);
 }
 template <typename RN, int N>
 cudaError_t analysis_dct_n(const Grid& g, int B, const PencilBufs& pb, typename cpx<RN>::T* h, cudaStream_t st) {
-  return launch_pdl_if<sizeof(RN) == 4>(analysis_dct_kernel<RN, N, 1>, dim3((g.P + 15) / 16, B, 3), dim3(64), 0, st, g, pb, h);
+  constexpr size_t smem = (size_t)(N + 1) * 32 * sizeof(RN);
+  static SmemLimit lim;
+  const cudaError_t e = raise_smem_limit(analysis_dct_kernel<RN, N>, &lim, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl_if<sizeof(RN) == 4>(analysis_dct_kernel<RN, N>, dim3((g.P + 15) / 16, B, 3), dim3(64), smem, st, g, pb, h);
 }
 
 }  // namespace chdns
