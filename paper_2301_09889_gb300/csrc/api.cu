@@ -684,6 +684,7 @@ int set_state_dev(ch_env* env, int e, const double* buf) {
   CK(cudaMemcpyAsync(env->pb.UM + (size_t)e * ny, U, ny * sizeof(double), cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(env->pb.WM + (size_t)e * ny, W, ny * sizeof(double), cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(env->pb.vw_new + (size_t)e * P, vw, P * sizeof(double2), cudaMemcpyHostToDevice, st));
+  if (env->prm.precision == 1) CK(launch_round_state(g, e, env->pb, st));
   // previous right-hand sides: complex values in the node precision, [B][ny][P]
   const size_t hsz = env->prm.precision == 1 ? sizeof(float2) : sizeof(double2);
   CK(cudaMemsetAsync(reinterpret_cast<char*>(env->pb.HVP) + (size_t)e * ny * P * hsz, 0, ny * P * hsz, st));
@@ -1108,6 +1109,12 @@ int env_create(const ch_params_t* p, ch_env_t** out) {
       (rc = dalloc(env, &pb.vw_old, B * P)) || (rc = dalloc(env, &pb.vw_new, B * P)) ||
       (rc = dalloc(env, &pb.planes, B * 2 * P)) || (rc = dalloc(env, &pb.tau_acc, B)))
     return fail(rc);
+  if (p->precision == 1) {
+    // the previous right-hand sides are FP32 pairs: the other half of their
+    // buffers holds the FP32 copies of the state
+    pb.V32 = reinterpret_cast<float2*>(pb.HVP) + B * ny * P;
+    pb.G32 = reinterpret_cast<float2*>(pb.HGP) + B * ny * P;
+  }
   env->out_stride = (size_t)2 * g.nz * g.nx + 2;
   if ((rc = dalloc(env, &env->d_act, B * g.nz * g.nx)) || (rc = dalloc(env, &env->d_out, B * env->out_stride)))
     return fail(rc);

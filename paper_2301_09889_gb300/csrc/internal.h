@@ -23,6 +23,8 @@ cudaError_t launch_plane_passes(const PlaneArgs<R>& a, int B, cudaStream_t st);
 struct PencilBufs {
   double2 *V, *G;               // [B][ny][P]
   double2 *HVP, *HGP;           // [B][ny][P] complex in the node precision (FP32 pairs in mixed mode)
+  float2 *V32, *G32;            // [B][ny][P] V and G rounded to FP32 (mixed precision): what stage_pre reads;
+                                // mode 0 of G32 holds the mean flow (W, U)
   double *UM, *WM, *HXP, *HZP;  // [B][ny]
   double2* Q;                   // [B][6][ny][P] node values of u, v, w, ox, oy, oz (nonlinear input)
   double2* R;                   // [B][3][ny][P] node values of H
@@ -61,6 +63,8 @@ template <typename RN>
 cudaError_t launch_stage_post(const Grid& g, int B, const PencilBufs& pb, const DevTables& t,
                               typename cpx<RN>::T* h, const StageCoef& sc, int ppc, bool batched,
                               cudaStream_t st);
+// V32, G32 of one environment from V, G (after its state has been set)
+cudaError_t launch_round_state(const Grid& g, int b, const PencilBufs& pb, cudaStream_t st);
 cudaError_t launch_wall_shear(const Grid& g, int B, const double* UM, double nu, double* acc,
                               const int* active, cudaStream_t st);
 cudaError_t launch_sense(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, int js,

@@ -409,6 +409,21 @@ __global__ void __launch_bounds__(kTauNT) tau_helmholtz_kernel(int ny, int M, co
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
+// the FP32 copies of a state that came from the host
+__global__ void round_state_kernel(Grid g, int b, PencilBufs pb) {
+  const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  if (i >= (long)g.ny * g.P) return;
+  const int n = (int)(i / g.P), p = (int)(i % g.P);
+  const size_t o = (size_t)b * g.ny * g.P + i;
+  const double2 v = pb.V[o], w = p == 0 ? mk(pb.WM[(size_t)b * g.ny + n], pb.UM[(size_t)b * g.ny + n]) : pb.G[o];
+  pb.V32[o] = make_float2((float)v.x, (float)v.y);
+  pb.G32[o] = make_float2((float)w.x, (float)w.y);
+}
+cudaError_t launch_round_state(const Grid& g, int b, const PencilBufs& pb, cudaStream_t st) {
+  round_state_kernel<<<(unsigned)(((long)g.ny * g.P + 255) / 256), 256, 0, st>>>(g, b, pb);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_wall_shear(const Grid& g, int B, const double* UM, double nu, double* acc, const int* active,
                               cudaStream_t st) {
   wall_shear_kernel<<<B, 32, 0, st>>>(g.ny, B, UM, nu, acc, active);

@@ -43,57 +43,30 @@ namespace chdns {
 // unrolled, the kernel's paths (three kinds of field, two parities) outgrew
 // the instruction cache wherever an SM ran several of them.
 //
-// CTA: NF fields of one tile, two warps (even, odd) each.  FP32 lines of up to
-// 65 nodes: all six, which share v and omega_y, rounded once into shared memory
-// (a conversion instruction occupies the FP64 pipe as an FP64 operation does);
-// longer and FP64 lines: one, reading its columns in place.
+// CTA: one field of a tile, two warps; the fields of a tile are neighbouring
+// CTAs.  FP32 lines read the copies of v and omega_y that the implicit half
+// rounded to FP32: a conversion instruction occupies the FP64 pipe as an FP64
+// operation does, and the lines read every column four to five times.
 // ---------------------------------------------------------------------------
-template <typename RN, int N> constexpr int pre_fields() { return sizeof(RN) == 4 && N <= 64 ? 6 : 1; }
 constexpr int ctas_of(int regs, int threads) { return 65536 / (regs * threads) > 0 ? 65536 / (regs * threads) : 1; }
 // registers a thread is held to: one parity's array and the transform around it
 template <typename RN, int N> constexpr int dct_regs() {
   return sizeof(RN) == 8 ? (N <= 32 ? 96 : N <= 64 ? 168 : 255) : (N <= 32 ? 56 : N <= 64 ? 80 : N <= 96 ? 96 : N <= 128 ? 128 : 168);
 }
 
-template <typename RN, int N, int NF>
-__global__ void __launch_bounds__(64 * NF, ctas_of(dct_regs<RN, N>(), 64 * NF)) stage_pre_dct_kernel(Grid g, PencilBufs pb,
-                                                                DevTables t, typename cpx<RN>::T* __restrict__ q) {
+template <typename RN, int N>
+__global__ void __launch_bounds__(64, ctas_of(dct_regs<RN, N>(), 64)) stage_pre_dct_kernel(Grid g, PencilBufs pb, DevTables t,
+                                                                typename cpx<RN>::T* __restrict__ q) {
   constexpr int H = N / 2, ny = N + 1;
-  constexpr bool kTile = NF > 1;
+  constexpr bool kF32 = sizeof(RN) == 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  RN* part = reinterpret_cast<RN*>(smem_raw);  // [E_0 .. E_H, O_0 .. O_{H-1}][32]
   const int P = g.P;
-  const int lane = threadIdx.x & 31, fl = threadIdx.x / 64, half = (threadIdx.x / 32) & 1, f = blockIdx.x % (6 / NF) * NF + fl;
-  RN* part = reinterpret_cast<RN*>(smem_raw) + fl * ny * 32;        // [E_0 .. E_H, O_0 .. O_{H-1}][32]
-  RN* tile = reinterpret_cast<RN*>(smem_raw) + NF * ny * 32;        // [v, omega_y][ny][32]
-  const int p0 = (int)blockIdx.x / (6 / NF) * 16, p = p0 + (lane >> 1), r = lane & 1;
+  const int lane = threadIdx.x & 31, half = threadIdx.x / 32, f = blockIdx.x % 6;
+  const int p = (int)blockIdx.x / 6 * 16 + (lane >> 1), r = lane & 1;
   const int b = blockIdx.y;
   if (pb.active && !pb.active[b]) return;
   pdl_wait_then_release();  // v, omega_y come from the previous stage
-  if constexpr (kTile) {
-    // a column per warp and step, every load in flight before the first store
-    constexpr int KL = (2 * ny + 2 * NF - 1) / (2 * NF);
-    const size_t c0 = 2 * ((size_t)b * ny * P + p0) + lane;
-    const double* v0 = reinterpret_cast<const double*>(pb.V) + c0;
-    const double* g0 = reinterpret_cast<const double*>(pb.G) + c0;
-    size_t gs = 2 * (size_t)P;
-    if (p == 0) {  // the columns of mode 0 hold W and U instead of omega_y
-      g0 = (r == 0 ? pb.WM : pb.UM) + (size_t)b * ny;
-      gs = 1;
-    }
-    double d[KL];
-#pragma unroll
-    for (int k = 0; k < KL; ++k) {
-      const int n = threadIdx.x / 32 + 2 * NF * k;
-      d[k] = 0.0;
-      if (p < P && n < 2 * ny) d[k] = n < ny ? v0[(size_t)n * 2 * P] : g0[(size_t)(n - ny) * gs];
-    }
-#pragma unroll
-    for (int k = 0; k < KL; ++k) {
-      const int n = threadIdx.x / 32 + 2 * NF * k;
-      if (n < 2 * ny) tile[n * 32 + lane] = (RN)d[k];
-    }
-    __syncthreads();
-  }
   RN* mine = part + half * (H + 1) * 32 + lane;
   if (p < P) {
     const int row = p / g.nxh, ix = p % g.nxh;
@@ -111,20 +84,27 @@ __global__ void __launch_bounds__(64 * NF, ctas_of(dct_regs<RN, N>(), 64 * NF)) 
     } else if (mean && f == 5) {
       cS = (RN)-1.0;
     }
-    const bool liveS = gen || (mean && !own && r == 0);
+    const bool liveM = mean && !own && r == 0;  // the columns of the mean flow
     const size_t col = 2 * ((size_t)b * ny * P + p);  // component 0 of coefficient 0; 2 P per coefficient
-    const double* Vp = reinterpret_cast<const double*>(pb.V) + col + (1 - r);
-    const double* Sp = reinterpret_cast<const double*>(f == 1 ? pb.V : pb.G) + col + (own ? r : 1 - r);
+    const RN* v0 = reinterpret_cast<const RN*>(kF32 ? (const void*)pb.V32 : pb.V) + col;
+    const RN* g0 = reinterpret_cast<const RN*>(kF32 ? (const void*)pb.G32 : pb.G) + col;
+    const RN* Vp = v0 + (1 - r);
+    const RN* Sp = (f == 1 ? v0 : g0) + (own ? r : 1 - r);
     const size_t vs = 2 * (size_t)P;
     size_t ss = vs;
-    if (mean && !own) {
-      Sp = (f == 0 || f == 5 ? pb.UM : pb.WM) + (size_t)b * ny;
-      ss = 1;
+    if (liveM) {
+      // the mean flow: its own columns, or the FP32 copies (W, U) in mode 0's column
+      if constexpr (kF32) {
+        Sp = g0 + (f == 0 || f == 5 ? 1 : 0);
+      } else {
+        Sp = (f == 0 || f == 5 ? pb.UM : pb.WM) + (size_t)b * ny;
+        ss = 1;
+      }
     }
-    const RN* Vt = tile + (lane ^ 1);
-    const RN* St = tile + (f == 1 ? 0 : ny * 32) + (own ? lane : !mean ? lane ^ 1 : f == 0 || f == 5 ? 1 : 0);
-    auto V = [&](int n) { return !gen ? (RN)0 : kTile ? Vt[n * 32] : to_rn<RN>(__ldg(Vp + n * vs)); };
-    auto S = [&](int n) { return !liveS ? (RN)0 : kTile ? St[n * 32] : to_rn<RN>(__ldg(Sp + n * ss)); };
+    const bool liveS = gen || liveM;
+    // every load is unconditional (the loops batch them), dead lanes drop theirs
+    auto V = [&](int n) { const RN x = __ldg(Vp + n * vs); return gen ? x : (RN)0; };
+    auto S = [&](int n) { const RN x = __ldg(Sp + n * ss); return liveS ? x : (RN)0; };
     // 2 k; from a table in FP64, where converting it would cost an operation
     auto c2 = [&](int k) {
       if constexpr (sizeof(RN) == 8) return __ldg(t.tau.n1 + k - 1);
@@ -243,13 +223,12 @@ __global__ void __launch_bounds__(64, ctas_of(dct_regs<RN, N>(), 64)) analysis_d
 
 template <typename RN, int N>
 cudaError_t pre_dct_n(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, typename cpx<RN>::T* q, cudaStream_t st) {
-  constexpr int NF = pre_fields<RN, N>();
-  constexpr size_t smem = (size_t)(NF + (NF > 1 ? 2 : 0)) * (N + 1) * 32 * sizeof(RN);
+  constexpr size_t smem = (size_t)(N + 1) * 32 * sizeof(RN);
   static SmemLimit lim;
-  const cudaError_t e = raise_smem_limit(stage_pre_dct_kernel<RN, N, NF>, &lim, smem);
+  const cudaError_t e = raise_smem_limit(stage_pre_dct_kernel<RN, N>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(RN) == 4>(stage_pre_dct_kernel<RN, N, NF>, dim3((g.P + 15) / 16 * (6 / NF), B), dim3(64 * NF),
-                                        smem, st, g, pb, t, q);
+  return launch_pdl_if<sizeof(RN) == 4>(stage_pre_dct_kernel<RN, N>, dim3((g.P + 15) / 16 * 6, B), dim3(64), smem, st, g, pb,
+                                        t, q);
 }
 template <typename RN, int N>
 cudaError_t analysis_dct_n(const Grid& g, int B, const PencilBufs& pb, typename cpx<RN>::T* h, cudaStream_t st) {

@@ -98,10 +98,6 @@ __device__ __forceinline__ void analysis_sums(const typename cpx<RN>::T* col, in
   }
 }
 
-template <typename C> __device__ __forceinline__ C to_node(double2 v);
-template <> __device__ __forceinline__ double2 to_node<double2>(double2 v) { return v; }
-template <> __device__ __forceinline__ float2 to_node<float2>(double2 v) { return make_float2((float)v.x, (float)v.y); }
-
 // ---------------------------------------------------------------------------
 // Fast Chebyshev synthesis (DCT-I) of complex lines through an N-point FFT,
 // N even:  F_j = sum_{n=0}^{N} x_n cos(pi j n / N), j = 0..N.
@@ -260,8 +256,7 @@ __global__ void __launch_bounds__(128) stage_pre_kernel(Grid g, int B, PencilBuf
   using CN = typename cpx<RN>::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int P = g.P, ny = g.ny, N = g.N;
-  // v, omega_y coefficients rounded once to the node precision (every use
-  // below is in that precision), then the six fields
+  // v, omega_y coefficients in the node precision, then the six fields
   CN* sV = reinterpret_cast<CN*>(smem_raw);  // [ny][ppc]
   CN* sG = sV + ny * ppc;                    // [ny][ppc]
   CN* sC = sG + ny * ppc;                    // [6][ny][ppc]
@@ -274,8 +269,13 @@ __global__ void __launch_bounds__(128) stage_pre_kernel(Grid g, int B, PencilBuf
     const int pl = w % ppc, n = w / ppc;
     const int p = p0 + pl;
     const size_t o = ((size_t)b * ny + n) * P + p;
-    sV[w] = to_node<CN>((p < P) ? pb.V[o] : mk(0.0, 0.0));
-    sG[w] = to_node<CN>((p < P) ? pb.G[o] : mk(0.0, 0.0));
+    if constexpr (sizeof(RN) == 4) {
+      sV[w] = (p < P) ? pb.V32[o] : czero<CN>();
+      sG[w] = (p < P) ? pb.G32[o] : czero<CN>();
+    } else {
+      sV[w] = (p < P) ? pb.V[o] : czero<CN>();
+      sG[w] = (p < P) ? pb.G[o] : czero<CN>();
+    }
   }
   __syncthreads();
 
@@ -697,6 +697,11 @@ __global__ void __launch_bounds__(64 * kPostTileLanes) stage_post_kernel(Grid g,
     const size_t o = ((size_t)b * ny + n) * P + p2;
     pb.V[o] = sV[w];
     pb.G[o] = sG[w];
+    if constexpr (sizeof(RN) == 4) {
+      pb.V32[o] = make_float2((float)sV[w].x, (float)sV[w].y);
+      const double2 gv = p2 == 0 ? mk(pb.WM[(size_t)b * ny + n], pb.UM[(size_t)b * ny + n]) : sG[w];
+      pb.G32[o] = make_float2((float)gv.x, (float)gv.y);
+    }
     reinterpret_cast<CN*>(pb.HVP)[o] = sHV[w];
     reinterpret_cast<CN*>(pb.HGP)[o] = sHG[w];
   }

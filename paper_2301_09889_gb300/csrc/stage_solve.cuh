@@ -249,8 +249,8 @@ __device__ __forceinline__ Wall mean_down(double* f, const DevTables& t, const S
 // up: X <- X + d (+ the response u1 to the forcing of U)
 template <int TOP>
 __device__ __forceinline__ void mean_up(double* f, const DevTables& t, const StageCoef& sc, int N, size_t P, int sig,
-                                     bool forced, const double* __restrict__ T, double* X, double f0, double fc,
-                                     double wx) {
+                                     bool forced, const double* __restrict__ T, double* X, float* X32, double f0,
+                                     double fc, double wx) {
   constexpr int NT = 64;
   const size_t MP = (size_t)t.tau.Mh * P;
   const int M = (N - sig) / 2 + 1;
@@ -268,7 +268,11 @@ __device__ __forceinline__ void mean_up(double* f, const DevTables& t, const Sta
   const double* u1 = t.tau.u1 + (size_t)sc.k * t.tau.Mh;
   sweep_up<4>(
       0, M, [&](int i) { return Bw{X[2 * i + sig], __ldg(u1 + i)}; },
-      [&](int i, const Bw& v) { X[2 * i + sig] = fma(fc, v.w, v.b + f[i * NT]); });
+      [&](int i, const Bw& v) {
+        const double x = fma(fc, v.w, v.b + f[i * NT]);
+        X[2 * i + sig] = x;
+        if (X32) X32[2 * P * (2 * i + sig)] = narrow(x);
+      });
 }
 
 // Solve omega_y of parity sig of one (mode, component), or (MEAN) the mean flow
@@ -321,15 +325,23 @@ __device__ __forceinline__ void solve_omega(double* f, double* xch, const Grid& 
     f0 = sig == 0 ? xe : xo;
   }
   if constexpr (MEAN) {
-    mean_up<TOP>(f, t, sc, g.N, P, sig, r == 0, T, X, f0, fc, w.wx);
+    // the FP32 copies go to mode 0's column: (W, U)
+    float* X32 = sizeof(RN) == 4 ? reinterpret_cast<float*>(pb.G32) + 2 * (size_t)b * ny * P + (1 - r) : nullptr;
+    mean_up<TOP>(f, t, sc, g.N, P, sig, r == 0, T, X, X32, f0, fc, w.wx);
     return;
   }
   // up: f_i = a_i + b_i f_{i-1}; g <- f - c g
   const size_t hP = 2 * P;
-  double* G = reinterpret_cast<double*>(pb.G) + 2 * ((size_t)b * ny * P + p) + r + (size_t)sig * hP;
+  const size_t base = 2 * ((size_t)b * ny * P + p) + r + (size_t)sig * hP;
+  double* G = reinterpret_cast<double*>(pb.G) + base;
+  float* G32 = reinterpret_cast<float*>(pb.G32) + base;
   const double cc = sc.cc;
   double fp = f0;
-  G[0] = fma(-cc, G[0], fp);
+  auto put = [&](int i, double v) {
+    G[(size_t)i * 2 * hP] = v;
+    if constexpr (sizeof(RN) == 4) G32[(size_t)i * 2 * hP] = narrow(v);
+  };
+  put(0, fma(-cc, G[0], fp));
   struct Up {
     double b, x;
   };
@@ -337,7 +349,7 @@ __device__ __forceinline__ void solve_omega(double* f, double* xch, const Grid& 
       1, M, [&](int i) { return Up{__ldg(T + 4 * MP + (size_t)i * P), G[(size_t)i * 2 * hP]}; },
       [&](int i, const Up& u) {
         fp = fma(u.b, fp, f[i * NT]);
-        G[(size_t)i * 2 * hP] = fma(-cc, u.x, fp);
+        put(i, fma(-cc, u.x, fp));
       });
 }
 
@@ -356,6 +368,7 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
   const size_t hP = 2 * P, base = 2 * ((size_t)b * ny * P + p) + r;
   double* Vp = reinterpret_cast<double*>(pb.V) + base;
   RN* HV = reinterpret_cast<RN*>(pb.HVP) + base;
+  float* V32 = reinterpret_cast<float*>(pb.V32) + base;
   const RN* H0 = hc + 2 * ((size_t)b * 3 * ny * P + p);
   const RN* hx = H0 + 1 - r;
   const RN* hy = H0 + (size_t)ny * hP + r;
@@ -482,16 +495,23 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
   const double* __restrict__ vh = t.tau.vh + (size_t)(sc.k * 2 + sig) * MP + p;
   sweep_up<2 * D>(
       0, M, [&](int i) { return __ldg(vh + (size_t)i * P); },
-      [&](int i, double h) { Vp[(size_t)(2 * i + sig) * hP] = fma(cI, h, f[i * NT]); });
+      [&](int i, double h) {
+        const size_t o = (size_t)(2 * i + sig) * hP;
+        const double v = fma(cI, h, f[i * NT]);
+        Vp[o] = v;
+        if constexpr (sizeof(RN) == 4) V32[o] = narrow(v);
+      });
 }
 
 // CTA: 16 modes x 2 components (lanes) x 2 classes (warps) of one equation:
-// the mean flow, then v (twice the work of omega_y), then omega_y.  Five rows
-// are loaded ahead on up to 255 registers: with DRAM or L2 latency covered by
-// the thread itself, four CTAs per SM saturate the FP64 pipe.
-constexpr int kSolveAhead = 5;
-template <typename RN, int TOP>
-__global__ void __launch_bounds__(64, 4) stage_solve_kernel(Grid g, PencilBufs pb, DevTables t,
+// the mean flow, then v (twice the work of omega_y), then omega_y.  D rows are
+// loaded ahead: three on 168 registers where six CTAs per SM are there to be
+// resident, five on 255 where the grid or the shared memory of the columns
+// leaves four or fewer (us per RK step with 3 and 5: 256 minimal mixed 840 and
+// 951, 128x129x128 mixed 418 and 460; 24x50x48 x 8 mixed 219 and 168,
+// 256x193x256 mixed 2546 and 2368).
+template <typename RN, int TOP, int D>
+__global__ void __launch_bounds__(64, D == 3 ? 6 : 4) stage_solve_kernel(Grid g, PencilBufs pb, DevTables t,
                                                             const typename cpx<RN>::T* __restrict__ hc, StageCoef sc) {
   extern __shared__ __align__(16) double sarr[];  // [Mh][64], then the exchange slots [6][64] of a free-slip top
   const int b = blockIdx.y, tiles = (g.P + 15) / 16;
@@ -507,20 +527,28 @@ __global__ void __launch_bounds__(64, 4) stage_solve_kernel(Grid g, PencilBufs p
   double* f = sarr + threadIdx.x;
   double* xch = sarr + (size_t)t.tau.Mh * 64;
   const RN* h = reinterpret_cast<const RN*>(hc);
-  if (z == 0) solve_omega<RN, TOP, kSolveAhead, true>(f, xch, g, pb, t, sc, b, p, r, c, live, h);
-  else if (z == 1) solve_v<RN, TOP, kSolveAhead>(f, xch, g, pb, t, sc, b, p, r, c, live, h);
-  else solve_omega<RN, TOP, kSolveAhead, false>(f, xch, g, pb, t, sc, b, p, r, 1 - c, live, h);
+  if (z == 0) solve_omega<RN, TOP, D, true>(f, xch, g, pb, t, sc, b, p, r, c, live, h);
+  else if (z == 1) solve_v<RN, TOP, D>(f, xch, g, pb, t, sc, b, p, r, c, live, h);
+  else solve_omega<RN, TOP, D, false>(f, xch, g, pb, t, sc, b, p, r, 1 - c, live, h);
+}
+
+template <typename RN, int TOP, int D>
+cudaError_t solve_ahead(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, const typename cpx<RN>::T* h,
+                        const StageCoef& sc, dim3 grid, size_t smem, cudaStream_t st) {
+  static SmemLimit lim;
+  const cudaError_t e = raise_smem_limit(stage_solve_kernel<RN, TOP, D>, &lim, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl_if<sizeof(RN) == 4>(stage_solve_kernel<RN, TOP, D>, grid, dim3(64), smem, st, g, pb, t, h, sc);
 }
 
 template <typename RN, int TOP>
 cudaError_t solve_top(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, const typename cpx<RN>::T* h,
                       const StageCoef& sc, cudaStream_t st) {
   const size_t smem = ((size_t)t.tau.Mh + (TOP ? 6 : 0)) * 64 * sizeof(double);
-  static SmemLimit lim;
-  const cudaError_t e = raise_smem_limit(stage_solve_kernel<RN, TOP>, &lim, smem);
-  if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(RN) == 4>(stage_solve_kernel<RN, TOP>, dim3(1 + 2 * ((g.P + 15) / 16), B), dim3(64), smem, st,
-                                        g, pb, t, h, sc);
+  const dim3 grid(1 + 2 * ((g.P + 15) / 16), B);
+  if ((long)grid.x * grid.y > 4 * 152 && smem <= (size_t)44 * 1024)
+    return solve_ahead<RN, TOP, 3>(g, B, pb, t, h, sc, grid, smem, st);
+  return solve_ahead<RN, TOP, 5>(g, B, pb, t, h, sc, grid, smem, st);
 }
 
 }  // namespace chdns
