@@ -99,144 +99,6 @@ __device__ __forceinline__ void analysis_sums(const typename cpx<RN>::T* col, in
 }
 
 // ---------------------------------------------------------------------------
-// Fast Chebyshev synthesis (DCT-I) of complex lines through an N-point FFT,
-// N even:  F_j = sum_{n=0}^{N} x_n cos(pi j n / N), j = 0..N.
-// With y_n = (x_n + x_{N-n})/2 - sin(pi n / N) (x_n - x_{N-n}), n = 0..N-1,
-// and Z_k = sum_n y_n e^{2 pi i k n / N}: the cosine sums pick out the part
-// of y symmetric under n -> N - n, which reproduces the even outputs, and the
-// sine sums the antisymmetric part, which gives differences of odd outputs:
-//   F_{2k} = (Z_k + Z_{N-k}) / 2 + (x_0 + x_N) / 2,          k = 0..N/2,
-//   F_{2k+1} = F_{2k-1} - i (Z_k - Z_{N-k}) / 2,             k = 1..N/2-1,
-//   F_1 = sum_n x_n cos(pi n / N).
-// O(N log N) FP64 operations per line instead of the (N/2)(N+1) of the sums.
-// Lines: line l = f G + pl at buf + f LS + pl, element stride G.
-// ---------------------------------------------------------------------------
-template <int N, int ST>
-__device__ __forceinline__ void lines_dif(double2* buf, const double2* tw, int nlines, int G, int LS) {
-  if constexpr (ST < ct_nst(N)) {
-    constexpr int r = ct_radix(N, ST);
-    constexpr int L = ct_len_before(N, ST);
-    constexpr int m = L / r;
-    constexpr int nb = N / r;
-    constexpr int tstep = N / L;
-    for (int w = threadIdx.x; w < nlines * nb; w += blockDim.x) {
-      const int l = w % nlines, bf = w / nlines;
-      double2* base = buf + (l / G) * LS + (l % G);
-      const int blk = bf / m, q = bf % m;
-      const int i0 = blk * L + q;
-      double2 x[r];
-#pragma unroll
-      for (int t = 0; t < r; ++t) x[t] = base[(i0 + t * m) * G];
-      small_dft_ct<+1, r, double2, double>(x);
-#pragma unroll
-      for (int u = 0; u < r; ++u) {
-        double2 y = x[u];
-        if (u > 0 && q > 0) y = cmul_rn(y, tw[q * u * tstep]);
-        base[(i0 + u * m) * G] = y;
-      }
-    }
-    __syncthreads();
-    lines_dif<N, ST + 1>(buf, tw, nlines, G, LS);
-  }
-}
-
-// position of frequency k in the digit-reversed output of the DIF passes:
-// sum over passes of (digit of k in that pass's radix) x (sub-block length)
-template <int N>
-__device__ __forceinline__ int dif_pos(int k) {
-  int p = 0, L = N;
-#pragma unroll
-  for (int st = 0; st < ct_nst(N); ++st) {
-    const int r = ct_radix(N, st);
-    const int m = L / r;
-    p += (k % r) * m;
-    k /= r;
-    L = m;
-  }
-  return p;
-}
-
-// Chebyshev analysis of the three fields of a tile in FP64 through the same
-// FFT form of the DCT-I: a_n = (2 / (N cb_n)) F_n, F the DCT-I of
-// g_j = f_j / cb_j (cb_0 = cb_N = 2).  X: tile [3][ny][ppc], nodal values in,
-// coefficients out.  The FFT leaves Z in digit-reversed order in the tile's
-// own storage: each even output is stored in Z_k's slot and each odd-output
-// difference in Z_{N-k}'s slot (every slot read and written by one item
-// only), and the natural-order coefficients pass through this tile's columns
-// of the global node array Rt (modes of this CTA, read by no other CTA) before
-// they are copied back.  hf: shared scratch of 6 ppc values.
-template <int NF>
-__device__ __forceinline__ void analysis_fft(double2* X, int ppc, int ny, int P, int p0, double2* hf,
-                                             const double* cheb, const double2* tw, double2* Rt) {
-  constexpr int N = NF;
-  const int nl = 3 * ppc, LS = ny * ppc;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  double2* sHalf = hf;       // (g_0 + g_N) / 2
-  double2* sF1 = hf + nl;    // F_1
-  for (int l = tid; l < nl; l += nt) {
-    double2* x = X + (l / ppc) * LS + (l % ppc);
-    x[0] = 0.5 * x[0];
-    x[N * ppc] = 0.5 * x[N * ppc];
-    double2 s1 = mk(0.0, 0.0);
-    for (int n = 0; n <= N; ++n) s1 = s1 + cheb[ny + n] * x[n * ppc];
-    sF1[l] = s1;
-    sHalf[l] = 0.5 * (x[0] + x[N * ppc]);
-  }
-  __syncthreads();
-  for (int w = tid; w < nl * (N / 2); w += nt) {
-    const int l = w % nl, n = w / nl;
-    double2* x = X + (l / ppc) * LS + (l % ppc);
-    if (n == 0) {
-      x[0] = sHalf[l];
-      continue;
-    }
-    const double2 xa = x[n * ppc], xb = x[(N - n) * ppc];
-    const double sn = cheb[ny + N / 2 - n];  // sin(pi n / N)
-    const double2 sm = 0.5 * (xa + xb), d = xa - xb;
-    x[n * ppc] = sm - sn * d;
-    x[(N - n) * ppc] = sm + sn * d;
-  }
-  __syncthreads();
-  lines_dif<NF, 0>(X, tw, nl, ppc, LS);
-  for (int w = tid; w < nl * (N / 2 + 1); w += nt) {
-    const int l = w % nl, k = w / nl;
-    double2* Z = X + (l / ppc) * LS + (l % ppc);
-    const int ik = dif_pos<NF>(k) * ppc, in = dif_pos<NF>((N - k) % N) * ppc;
-    const double2 zk = Z[ik], zn = Z[in];
-    Z[ik] = 0.5 * (zk + zn) + sHalf[l];
-    if (k >= 1 && k < N / 2) {
-      const double2 dd = zk - zn;
-      Z[in] = mk(0.5 * dd.y, -0.5 * dd.x);
-    }
-  }
-  __syncthreads();
-  const double s0 = 2.0 / N;
-  for (int l = tid; l < nl; l += nt) {
-    const int f = l / ppc, pl = l % ppc;
-    if (p0 + pl >= P) continue;
-    const double2* Z = X + f * LS + pl;
-    double2* dst = Rt + (size_t)f * ny * P + pl;
-    double2 fo = sF1[l];
-    dst[0] = (0.5 * s0) * Z[0];
-    dst[P] = s0 * fo;
-#pragma unroll 4
-    for (int k = 1; k <= N / 2; ++k) {
-      dst[(size_t)(2 * k) * P] = (2 * k == N ? 0.5 * s0 : s0) * Z[dif_pos<NF>(k) * ppc];
-      if (k < N / 2) {
-        fo = fo + Z[dif_pos<NF>(N - k) * ppc];
-        dst[(size_t)(2 * k + 1) * P] = s0 * fo;
-      }
-    }
-  }
-  __syncthreads();
-  for (int w = tid; w < 3 * ny * ppc; w += nt) {
-    const int pl = w % ppc, fn = w / ppc;
-    if (p0 + pl < P) X[w] = Rt[(size_t)fn * P + pl];
-  }
-  __syncthreads();
-}
-
-// ---------------------------------------------------------------------------
 // stage_pre
 //   u = (i kx Dv - i kz g)/k^2, w = (i kz Dv + i kx g)/k^2,
 //   omega_x = Dw - i kz v, omega_z = i kx v - Du;  mean mode: u = U, w = W,
@@ -507,11 +369,11 @@ __global__ void __launch_bounds__(128) stage_pre_kernel(Grid g, int B, PencilBuf
 // 1-c, e = 1 v on parity c.  The mean mode solves U at constant flow rate
 // (e = 0) and W (e = 1) on parity c, real component only.
 // ---------------------------------------------------------------------------
-// Lanes per system of the per-tile form (the scan solves of stage_scan.cuh)
-constexpr int kPostTileLanes = 4;
+// Per-tile form: 8 systems of kLanes lanes (stage_scan.cuh), four warps, per mode
+constexpr int kModeThreads = 8 * kLanes;
 
 template <typename RN, int MH>
-__global__ void __launch_bounds__(64 * kPostTileLanes) stage_post_kernel(Grid g, int B, PencilBufs pb, DevTables t,
+__global__ void __launch_bounds__(8 * kModeThreads) stage_post_kernel(Grid g, int B, PencilBufs pb, DevTables t,
                                                         const typename cpx<RN>::T* __restrict__ hn, StageCoef sc,
                                                         int ppc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -574,84 +436,66 @@ __global__ void __launch_bounds__(64 * kPostTileLanes) stage_post_kernel(Grid g,
   cp_async_wait_all();
   __syncthreads();
 
-  // ---- Chebyshev analysis of H_x, H_y, H_z (in place after a barrier)
-  constexpr int NF = 2 * (MH - 1);
-  bool analysed = false;
-  if constexpr (std::is_same<RN, double>::value && ct_plan_ok(NF)) {
-    if (N == NF) {
-      analysis_fft<NF>(sH, ppc, ny, P, p0, reinterpret_cast<double2*>(ss + 6 * ppc), t.cheb, t.tw_cheb,
-                       pb.R + (size_t)b * 3 * ny * P + p0);
-      analysed = true;
-    }
+  // ---- Chebyshev analysis of H_x, H_y, H_z by direct sums over the node pairs
+  // (j, N - j), folded in place: f_j + f_{N-j} at j, f_j - f_{N-j} at N - j; j = 0
+  // and N weigh 1/2.  Thread t of a mode's threads forms the values (field,
+  // component, n) t, t + kModeThreads, ...; with so few modes the sums spread over
+  // four warps finish before a transform in one.
+  const int ml = tid / kModeThreads, mt = tid % kModeThreads;  // mode of the tile, thread of the mode
+  RN* sR = reinterpret_cast<RN*>(sN);  // component r of (field, n, mode) at 2 ((f ny + n) ppc + mode) + r
+  for (int w = mt; w < 6 * ((N + 1) / 2); w += kModeThreads) {
+    const int j = w / 6, f = w % 6 / 2, r = w & 1;
+    RN* a = sR + 2 * ((size_t)(f * ny + j) * ppc + ml) + r;
+    RN* c = sR + 2 * ((size_t)(f * ny + N - j) * ppc + ml) + r;
+    const RN x = j == 0 ? (RN)0.5 * *a : *a, y = j == 0 ? (RN)0.5 * *c : *c;
+    *a = x + y;
+    *c = x - y;
   }
-  if (!analysed) {
-    // Thread (mode pl, group g of GA) computes the coefficients n = g, g+GA, ...
-    // of the three fields of its mode: every pair f_j, f_{N-j} it loads feeds
-    // all of its outputs, and the outputs are independent accumulation chains.
-    // n and g share their parity, so the folding sign is fixed per thread.
-    constexpr int GA = 8 * kPostTileLanes;
-    constexpr int KN = (2 * MH + GA - 1) / GA;  // n values per thread
-    const int pl = tid % ppc, gq = tid / ppc;  // blockDim = GA ppc
+  __syncthreads();
+  {
+    constexpr int KN = (12 * MH + kModeThreads - 1) / kModeThreads;  // values per thread, 6 (N + 1) <= 12 MH - 6
     const RN* cheb = cheb_table<RN>(t);
-    const RN sg = (gq & 1) ? (RN)-1.0 : (RN)1.0;
-    CN a[3][KN];
-    const CN* colf[3];
-#pragma unroll
-    for (int f = 0; f < 3; ++f) {
-      colf[f] = sN + (size_t)f * ny * ppc + pl;
-      const CN w0 = (RN)0.5 * (colf[f][0] + sg * colf[f][N * ppc]);  // j = 0 and j = N weigh 1/2
-#pragma unroll
-      for (int k = 0; k < KN; ++k) a[f][k] = w0;
-    }
-    for (int j = 1; 2 * j < N; ++j) {
-      CN fold[3];
-#pragma unroll
-      for (int f = 0; f < 3; ++f) fold[f] = colf[f][j * ppc] + sg * colf[f][(N - j) * ppc];
-#pragma unroll
-      for (int k = 0; k < KN; ++k) {
-        const int n = gq + GA * k;
-        const RN c = cheb[(size_t)min(n, N) * ny + j];
-#pragma unroll
-        for (int f = 0; f < 3; ++f) a[f][k] = a[f][k] + c * fold[f];
-      }
-    }
-    CN acc[3][KN];
     const RN s0 = (RN)2.0 / (RN)N;
+    RN acc[KN];
 #pragma unroll
     for (int k = 0; k < KN; ++k) {
-      const int n = gq + GA * k;
-      const RN cbn = (n == 0 || n == N) ? (RN)2.0 : (RN)1.0;
-      const RN cH = ((N & 1) == 0) ? cheb[(size_t)min(n, N) * ny + N / 2] : (RN)0.0;
-#pragma unroll
-      for (int f = 0; f < 3; ++f) {
-        CN v = a[f][k];
-        if ((N & 1) == 0) v = v + cH * colf[f][(N / 2) * ppc];
-        acc[f][k] = (s0 / cbn) * v;
+      const int w = mt + kModeThreads * k;
+      acc[k] = (RN)0;
+      if (w < 6 * ny) {
+        // even n first, so that the lanes of a warp mostly share the folded values
+        const int fr = w / ny, m = w % ny, ne = N / 2 + 1;
+        const int n = m < ne ? 2 * m : 2 * (m - ne) + 1;
+        const int st = m < ne ? 2 * ppc : -2 * ppc;
+        const RN* x = sR + 2 * ((size_t)((fr / 2) * ny + (m < ne ? 0 : N)) * ppc + ml) + (fr & 1);
+        RN a = 0;
+#pragma unroll 8
+        for (int j = 0; 2 * j < N; ++j) a = fma_rn(cheb[(size_t)j * ny + n], x[j * st], a);
+        if (m < ne && (N & 1) == 0) a = fma_rn((n & 2) ? (RN)-1.0 : (RN)1.0, x[(N / 2) * st], a);
+        acc[k] = ((n == 0 || n == N) ? (RN)0.5 * s0 : s0) * a;
       }
     }
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < KN; ++k) {
-      const int n = gq + GA * k;
-      if (n <= N) {
-#pragma unroll
-        for (int f = 0; f < 3; ++f) sN[((size_t)f * ny + n) * ppc + pl] = acc[f][k];
+      const int w = mt + kModeThreads * k;
+      if (w < 6 * ny) {
+        const int fr = w / ny, m = w % ny, ne = N / 2 + 1;
+        const int n = m < ne ? 2 * m : 2 * (m - ne) + 1;
+        sR[2 * ((size_t)((fr / 2) * ny + n) * ppc + ml) + (fr & 1)] = acc[k];
       }
     }
-    __syncthreads();
   }
+  __syncthreads();
 
-  // ---- implicit solves, system (mode pl, class c, component r, equation
-  // e) on the four lanes q of a group
-  const int q = tid & 3, sys = tid >> 2;
-  const int pl = sys % ppc;
-  const int combo = sys / ppc;
+  // ---- implicit solves, system (mode, class c, component r, equation e) on
+  // the lanes q of a group; e is uniform over each warp
+  const int q = mt & (kLanes - 1), combo = mt / kLanes, pl = ml;
   const int p = p0 + pl;
   const int c = combo & 1, r = (combo >> 1) & 1, e = combo >> 2;
   const int row = p / g.nxh, ix = p % g.nxh;
   // a whole group is live or idle together
   if (p < P && row != g.nz / 2 && (p != 0 || r == 0)) {
-    const double cc = sc.alpha / sc.beta;
+    const double cc = sc.cc;
     const double* rowc = t.tau.rowc;
     const CN* Hx = reinterpret_cast<const CN*>(sH) + pl;
     const CN* Hy = Hx + ny * ppc;
@@ -661,7 +505,8 @@ __global__ void __launch_bounds__(64 * kPostTileLanes) stage_post_kernel(Grid g,
     if (p == 0) {
       mean_scan<MH, RN>(N, ny, ppc, c, e, (e == 0 ? pb.UM : pb.WM) + (size_t)b * ny,
                         (e == 0 ? pb.HXP : pb.HZP) + (size_t)b * ny, (e == 0) ? Hx : Hz, cc, sc, helm(c),
-                        ss[(0 * 2 + c) * ppc + pl], rowc, t.tau.u1 + (size_t)sc.k * Mh, t.tau.u1_iflux[sc.k], q);
+                        ss[(0 * 2 + c) * ppc + pl], rowc, t.tau.u1 + (size_t)sc.k * Mh, t.tau.u1_iflux[sc.k],
+                        t.tau.wint, q);
     } else {
       const double kx = t.kx[ix], kz = t.kz[row], k2 = kx * kx + kz * kz;
       const double sgn = (r == 0) ? -1.0 : 1.0;
@@ -775,7 +620,7 @@ cudaError_t post_mh(const Grid& g, int B, const PencilBufs& pb, const DevTables&
   const cudaError_t e = raise_smem_limit(stage_post_kernel<RN, MH>, &lim, smem);
   if (e != cudaSuccess) return e;
   return launch_pdl_if<sizeof(RN) == 4>(stage_post_kernel<RN, MH>, dim3((g.P + ppc - 1) / ppc, B),
-                                        dim3(8 * kPostTileLanes * ppc), smem, st, g, B, pb, t, h, sc, ppc);
+                                        dim3(kModeThreads * ppc), smem, st, g, B, pb, t, h, sc, ppc);
 }
 
 template <typename RN, int MH>
