@@ -364,17 +364,16 @@ int setup_plane(ch_env* env, PlaneArgs<R>* a, size_t* smem) {
     *smem = zb + (size_t)6 * np * g.mx * csz;
   }
   if (!a->S) return CH_ERR_UNSUPPORTED;
-  // planes of 16 x 16 modes run one plane per team of threads with the line
-  // transforms in registers once the batch supplies enough planes to fill
-  // the SMs (four per SM, two per CTA); fewer planes keep the cluster split,
-  // which spreads each plane over S CTAs
-  a->team16 = 0;
-  if (plane16_shape(g.mx, g.mz, g.nxh, g.nz) && (long)g.ny * env->B >= 4L * nsm) {
-    a->team16 = 1;
+  a->cluster = a->S;
+  // planes of 16 x 16 modes have kernels of their own (in the precision of the
+  // handle's steps and for ch_nonlinear alike): pooled register lines once the
+  // batch supplies four planes per SM, two-CTA clusters below
+  if (plane16_shape(g.mx, g.mz, g.nxh, g.nz)) {
+    a->team16 = (long)g.ny * env->B >= 4L * nsm ? 1 : 2;
+    if (a->team16 == 1) a->cluster = 1;
     a->S = 1;
     a->Lz = g.mz;
   }
-  a->cluster = a->S;
   if (!fft_plan(g.mx, &a->px) || !fft_plan(a->Lz, &a->pz)) return CH_ERR_UNSUPPORTED;
   if (a->S > 8) {
     int clusters = 0;
@@ -581,7 +580,20 @@ int build_tables(ch_env* env) {
   env->tab.tau.top_bc = top ? 1 : 0;
   RC(dupload(env, &env->tab.tw_nx, twiddles(g.nx)));
   RC(dupload(env, &env->tab.tw_nz, twiddles(g.nz)));
-  RC(dupload(env, &env->tab.tw_cheb, twiddles(g.N)));
+  if (stage_direct(g)) {
+    const int Jp = direct_pre_pitch(N), Ip = direct_ana_pitch(N), J = N / 2 + 1;
+    std::vector<double> cp((size_t)ny * Jp, 0.0), ca((size_t)J * 2 * Ip, 0.0);
+    for (int j = 0; j < J; ++j)
+      for (int n = 0; n < ny; ++n) {
+        const double c = cheb[(size_t)j * ny + n];
+        cp[(size_t)n * Jp + j] = c;
+        ca[((size_t)j * 2 + n % 2) * Ip + n / 2] = c;
+      }
+    RC(dupload(env, &env->tab.cos_pre, cp));
+    RC(dupload(env, &env->tab.cos_ana, ca));
+    RC(dupload(env, &env->tab.cos_pre_f, std::vector<float>(cp.begin(), cp.end())));
+    RC(dupload(env, &env->tab.cos_ana_f, std::vector<float>(ca.begin(), ca.end())));
+  }
 
   // the plane of the handle's precision is required; the other one serves
   // ch_nonlinear (FP64) and is skipped where its slab does not fit
@@ -750,13 +762,13 @@ int run_stage(ch_env* env, int k, double theta) {
   const bool mixed = env->prm.precision == 1;
   if (mixed) {
     float2* q = reinterpret_cast<float2*>(env->pb.Q);
-    LAUNCH(0, launch_stage_pre<float>(g, B, env->pb, env->tab, q, env->ppc_pre, st));
+    LAUNCH(0, launch_stage_pre<float>(g, B, env->pb, env->tab, q, st));
     PlaneArgs<float> a = env->plane_f;
     a.q = q;
     a.h = reinterpret_cast<float2*>(env->pb.R);
     LAUNCH(1, launch_plane<float>(a, B, env->plane_f_smem, st));
   } else {
-    LAUNCH(0, launch_stage_pre<double>(g, B, env->pb, env->tab, env->pb.Q, env->ppc_pre, st));
+    LAUNCH(0, launch_stage_pre<double>(g, B, env->pb, env->tab, env->pb.Q, st));
     PlaneArgs<double> a = env->plane;
     a.q = env->pb.Q;
     a.h = env->pb.R;
@@ -850,11 +862,16 @@ int capture_step(ch_env* env, int gi, const int* d_active) {
 // modes per CTA), so the widths change speed only, never results.  The
 // autotuner keeps the form the size rule chose.
 // ---------------------------------------------------------------------------
+// (the explicit half runs in one shape; its widths are accepted and refused as
+// when it worked on tiles of ppc_pre modes in shared memory)
+size_t pre_tile_bytes(const Grid& g, int ppc, size_t node_bytes) {
+  return (size_t)8 * g.ny * ppc * node_bytes + (size_t)12 * ppc * sizeof(double2);
+}
 bool tiles_valid(const ch_env* env, int smem_max, int ppc_pre, int ppc_post, int post_batched) {
   const Grid& g = env->g;
   const size_t node = env->prm.precision == 1 ? sizeof(float2) : sizeof(double2);
   auto pow2 = [](int v, int hi) { return v >= 1 && v <= hi && (v & (v - 1)) == 0; };
-  if (!pow2(ppc_pre, 8) || stage_pre_smem(g, ppc_pre, node) > (size_t)smem_max) return false;
+  if (!pow2(ppc_pre, 8) || pre_tile_bytes(g, ppc_pre, node) > (size_t)smem_max) return false;
   if (post_batched == 1) return pow2(ppc_post, 16);
   if (post_batched != 0) return false;
   // the per-tile form runs 8 ppc threads and any tile width up to 8 (widths
@@ -921,11 +938,6 @@ int autotune_tiles(ch_env* env, int smem_max) {
   for (double* x : {pb.UM, pb.WM, pb.HXP, pb.HZP}) CK(cudaMemsetAsync(x, 0, Bs * ny * sizeof(double), st));
   const bool mixed = env->prm.precision == 1;
   const StageCoef sc = stage_coef(env, 0, 1.0);
-  auto pre = [&](int ppc) {
-    const cudaError_t e = mixed ? launch_stage_pre<float>(g, B, pb, env->tab, reinterpret_cast<float2*>(pb.Q), ppc, st)
-                                : launch_stage_pre<double>(g, B, pb, env->tab, pb.Q, ppc, st);
-    return e == cudaSuccess ? CH_OK : CH_ERR_CUDA;
-  };
   auto post = [&](int ppc, bool batched) {
     const cudaError_t e =
         mixed ? launch_stage_post<float>(g, B, pb, env->tab, reinterpret_cast<float2*>(pb.R), sc, ppc, batched, st)
@@ -935,18 +947,6 @@ int autotune_tiles(ch_env* env, int smem_max) {
   constexpr int kReps = 3;
   float best = 0.f;
   bool have = false;
-  for (int ppc : {8, 4, 2}) {
-    if (!stage_pre_tiled(g)) break;  // register transforms: one shape
-    if (!tiles_valid(env, smem_max, ppc, env->ppc_post, env->post_batched ? 1 : 0)) continue;
-    float ms = 0.f;
-    RC(time_launches(st, kReps, [&] { return pre(ppc); }, &ms));
-    if (!have || ms < best) {
-      best = ms;
-      env->ppc_pre = ppc;
-      have = true;
-    }
-  }
-  have = false;
   // widths of the form the size rule chose: the per-tile and batched forms of
   // the no-slip solves sum in different orders (four-lane scans against one
   // thread per system), so timing never switches between them
@@ -1138,12 +1138,13 @@ int env_create(const ch_params_t* p, ch_env_t** out) {
     while (env->ppc_post > 1 && stage_post_smem(g, env->tab.tau.Mh, env->ppc_post) > (size_t)smem_max)
       env->ppc_post /= 2;
     env->ppc_pre = 8;
-    while (env->ppc_pre > 1 && stage_pre_smem(g, env->ppc_pre, sizeof(double2)) > (size_t)smem_max) env->ppc_pre /= 2;
+    while (env->ppc_pre > 1 && pre_tile_bytes(g, env->ppc_pre, sizeof(double2)) > (size_t)smem_max) env->ppc_pre /= 2;
     if (stage_post_smem(g, env->tab.tau.Mh, env->ppc_post) > (size_t)smem_max) return fail(CH_ERR_UNSUPPORTED);
-    // The two-launch form runs eight threads per mode; from 256 modes on it
-    // beats the four-lane scans (64x65x64 FP64: 226 against 338 us per RK step,
-    // 32x65x32 FP64: 192 against 197, 128x129x128 mixed: 463 against 1330).
-    if ((size_t)B * P >= (size_t)256) {
+    // The two-launch form runs eight threads per mode; from 768 modes on it
+    // beats the scans, which spread every system over sixteen lanes (us per
+    // launch, scans and two launches: 65 nodes FP64 48 and 62 at 512 modes, 80
+    // and 64 at 1024; mixed 33 and 41, 50 and 41).
+    if ((size_t)B * P >= (size_t)768) {
       env->post_batched = true;
       env->ppc_post = 16;
     }
@@ -1290,7 +1291,7 @@ int env_info(const ch_env_t* env, ch_info_t* info) {
   info->ppc_post = env->ppc_post;
   info->tuned = env->tuned ? 1 : 0;
   info->tune_ms = env->tune_ms;
-  info->plane_team = env->prm.precision == 1 ? env->plane_f.team16 : env->plane.team16;
+  info->plane_team = (env->prm.precision == 1 ? env->plane_f.team16 : env->plane.team16) == 1 ? 1 : 0;
   return CH_OK;
 }
 

@@ -503,8 +503,8 @@ struct PlaneArgs {
   FftPlan px, pz;
   R scale;             // 1 / (mx mz)
   const int* active;   // [B] slots to process (nullptr: all)
-  // planes of 16 x 16 modes in batches that fill the GPU: one plane per team
-  // of threads, line transforms in registers (plane_small.cu)
+  // planes of 16 x 16 modes (plane_small.cu): 1 in batches that fill the GPU, 2
+  // on two-CTA clusters
   int team16;
   // three passes through global memory (z inverse, x transforms and products,
   // z forward; plane_pass.cuh)

@@ -40,22 +40,27 @@ struct DevTables {
   const double* cheb;  // [ny][ny] cos(pi j n / N)
   const float* cheb_f; // the same table in FP32 (mixed precision)
   const double* dts;   // [ny] T_n'(y_js) at the sensing node
+  // direct sums (orders without a register transform): cos(pi j n / N) as
+  // [n][j <= N/2, padded] and as [j <= N/2][parity of n][i, padded], n = 2 i + parity
+  const double *cos_pre, *cos_ana;
+  const float *cos_pre_f, *cos_ana_f;
   TauTables tau;
   const double2* tw_nx;  // [nx]
   const double2* tw_nz;  // [nz]
-  const double2* tw_cheb;  // [N] e^{2 pi i k / N}: fast Chebyshev synthesis
 };
 
-// fused wall-normal halves of a stage (stage.cu); ppc = modes per CTA
-size_t stage_pre_smem(const Grid& g, int ppc, size_t node_bytes);  // node_bytes: one complex node value
-size_t stage_post_smem(const Grid& g, int Mh, int ppc);
-// the explicit half works on tiles of ppc modes (false: register cosine transforms)
-bool stage_pre_tiled(const Grid& g);
+// wall-normal halves of a stage (stage.cu)
+size_t stage_post_smem(const Grid& g, int Mh, int ppc);  // per-tile implicit half, ppc modes per CTA
+// direct Chebyshev sums (no register cosine transform for this order): the
+// handle needs their tables, of these pitches
+bool stage_direct(const Grid& g);
+int direct_pre_pitch(int N);
+int direct_ana_pitch(int N);
 // kernels one launch_stage_post issues
 int stage_post_launches(int top, bool batched);
 template <typename RN>
 cudaError_t launch_stage_pre(const Grid& g, int B, const PencilBufs& pb, const DevTables& t,
-                             typename cpx<RN>::T* q, int ppc, cudaStream_t st);
+                             typename cpx<RN>::T* q, cudaStream_t st);
 // batched (and every handle under a free-slip top): the analysis of H over its
 // nodal values h in place, then one thread per (mode, class, component,
 // equation); otherwise four lanes per system on a shared-memory tile of ppc modes

@@ -185,145 +185,6 @@ __global__ void __launch_bounds__(256) plane_kernel(PlaneArgs<R> a) {
 }
 
 
-// The same kernel with the transform lengths, the kept kx count, the row
-// pairs per batch and the CTA size fixed at compile time (index arithmetic by
-// constants, FFT passes unrolled).  Instantiated for the grids of the
-// configurations in use; planes whose shared memory allows one CTA per SM run
-// more threads per CTA to hide shared-memory latency.
-template <typename R, int MX, int LZ, int NXH, int NP, int NT>
-__global__ void __launch_bounds__(NT, (sizeof(R) == 4 && NT == 256 && MX == LZ) ? 8 : 0) plane_kernel_ct(PlaneArgs<R> a) {
-  using C = typename cpx<R>::T;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* Z = reinterpret_cast<C*>(smem_raw);  // [6][LZ][NXH]
-  C* X = Z + 6 * LZ * NXH;                // [6][NP][MX]
-  // launched only when the cluster size a.S equals MX / LZ (mz = mx)
-  constexpr int S = MX / LZ;
-  const int nz = a.nz, mz = a.mz;
-  const int tid = threadIdx.x;
-  int rank = 0;
-  if constexpr (S > 1) rank = (int)cg::this_cluster().block_rank();
-  const int j = blockIdx.y;
-  const int b = blockIdx.z;
-  if (a.active && !a.active[b]) return;  // whole cluster (same b) returns together
-  pdl_wait_then_release();               // the node values come from stage_pre
-  const size_t plane = (size_t)a.P;
-  const C* qb = a.q + (size_t)b * 6 * a.ny * plane + (size_t)j * plane;
-  C* hb = a.h + (size_t)b * 3 * a.ny * plane + (size_t)j * plane;
-
-  // 1. gather + fold + pre-twiddle
-  for (int w = tid; w < 6 * LZ * NXH; w += NT) {
-    const int i = w % NXH;
-    const int t = w / NXH;
-    const int m = t % LZ;
-    const int f = t / LZ;
-    const C* qf = qb + (size_t)f * a.ny * plane;
-    C acc = czero<C>();
-    for (int qq = 0; qq < S; ++qq) {
-      const int u = m + qq * LZ;
-      int kz;
-      if (u < nz / 2) kz = u;
-      else if (u > mz - nz / 2) kz = u - mz;
-      else continue;
-      const int row = kz >= 0 ? kz : nz + kz;
-      C val = qf[row * NXH + i];
-      if (rank > 0) val = turn(val, (qq * rank) % S, S, LZ, a.tw_mz);
-      acc = acc + val;
-    }
-    if (rank > 0) acc = cmul(acc, a.tw_mz[m * rank]);
-    Z[(f * LZ + m) * NXH + i] = acc;
-  }
-  __syncthreads();
-  fft_dif_ct<+1, R, LZ, 6 * NXH, NXH, false, NT>(Z, a.tw_z);
-
-  // 2. rows in pairs: x transforms and products
-  constexpr int NPAIRS = LZ / 2;
-  for (int pb = 0; pb < NPAIRS; pb += NP) {
-    for (int w = tid; w < 6 * NP * MX; w += NT) {
-      const int k = w % MX;
-      const int t = w / MX;
-      const int pp = t % NP;
-      const int f = t / NP;
-      const int r1 = 2 * (pb + pp);
-      const C* A = Z + (f * LZ + r1) * NXH;
-      const C* Bv = A + NXH;
-      C val;
-      if (k == 0) {
-        val = mk(A[0].x, Bv[0].x);
-      } else if (k < NXH) {
-        const C av = A[k], bv = Bv[k];
-        val = mk(av.x - bv.y, av.y + bv.x);
-      } else if (k > MX - NXH) {
-        const int kk = MX - k;
-        const C av = A[kk], bv = Bv[kk];
-        val = mk(av.x + bv.y, bv.x - av.y);
-      } else {
-        val = czero<C>();
-      }
-      X[(f * NP + pp) * MX + k] = val;
-    }
-    __syncthreads();
-    fft_dif_ct<+1, R, MX, 6 * NP, 1, true, NT>(X, a.tw_x);
-    for (int w = tid; w < NP * MX; w += NT) {
-      const int x = w % MX;
-      const int pp = w / MX;
-      C* L0 = X + pp * MX;
-      constexpr int fs = NP * MX;
-      const C u = L0[x], v = L0[fs + x], ww = L0[2 * fs + x];
-      const C ox = L0[3 * fs + x], oy = L0[4 * fs + x], oz = L0[5 * fs + x];
-      L0[x] = mk(v.x * oz.x - ww.x * oy.x, v.y * oz.y - ww.y * oy.y);
-      L0[fs + x] = mk(ww.x * ox.x - u.x * oz.x, ww.y * ox.y - u.y * oz.y);
-      L0[2 * fs + x] = mk(u.x * oy.x - v.x * ox.x, u.y * oy.y - v.y * ox.y);
-    }
-    __syncthreads();
-    fft_dit_ct<-1, R, MX, 3 * NP, 1, true, NT>(X, a.tw_x);
-    for (int w = tid; w < 3 * NP * NXH; w += NT) {
-      const int i = w % NXH;
-      const int t = w / NXH;
-      const int pp = t % NP;
-      const int f = t / NP;
-      const C* line = X + (f * NP + pp) * MX;
-      const C zk = line[i];
-      const C zm = line[(MX - i) % MX];
-      const int r1 = 2 * (pb + pp);
-      Z[(f * LZ + r1) * NXH + i] = mk((zk.x + zm.x) * (R)0.5, (zk.y - zm.y) * (R)0.5);
-      Z[(f * LZ + r1 + 1) * NXH + i] = mk((zk.y + zm.y) * (R)0.5, (zm.x - zk.x) * (R)0.5);
-    }
-    __syncthreads();
-  }
-
-  // 3. forward z transform of H_x, H_y, H_z and cluster combination
-  fft_dit_ct<-1, R, LZ, 3 * NXH, NXH, false, NT>(Z, a.tw_z);
-  if (rank > 0) {
-    for (int w = tid; w < 3 * LZ * NXH; w += NT) Z[w] = cmul(Z[w], cconj(a.tw_mz[((w / NXH) % LZ) * rank]));
-  }
-  if (S > 1) cg::this_cluster().sync();
-  for (int w = tid; w < 3 * nz * NXH; w += NT) {
-    const int i = w % NXH;
-    const int t = w / NXH;
-    const int row = t % nz;
-    const int f = t / nz;
-    if (S > 1 && (row % S) != rank) continue;
-    C out = czero<C>();
-    if (row != nz / 2) {
-      const int kz = row < nz / 2 ? row : row - nz;
-      int u = kz % LZ;
-      if (u < 0) u += LZ;
-      int q = ((kz - u) / LZ) % S;
-      if (q < 0) q += S;
-      for (int rr = 0; rr < S; ++rr) {
-        const C* Zr = Z;
-        if (S > 1 && rr != rank) Zr = cg::this_cluster().map_shared_rank(Z, rr);
-        C gval = Zr[(f * LZ + u) * NXH + i];
-        if (rr > 0) gval = turn(gval, (S - (q * rr) % S) % S, S, LZ, a.tw_mz);
-        out = out + gval;
-      }
-      out = a.scale * out;
-    }
-    hb[(size_t)f * a.ny * plane + row * NXH + i] = out;
-  }
-  if (S > 1) cg::this_cluster().sync();
-}
-
 template <typename K, typename R>
 static cudaError_t launch_with(K kernel, const PlaneArgs<R>& a, int B, size_t smem, cudaStream_t st,
                                SmemLimit* lim, int nt = 256) {
@@ -361,20 +222,10 @@ static SmemLimit& generic_limit() {
   return lim;
 }
 
-// compile-time instantiations: (MX, LZ, NXH, NP) of the grids in use
-#define CH_PLANE_CT_NT(MX_, LZ_, NXH_, NP_, NT_)                                                      \
-  if (a.mx == MX_ && a.Lz == LZ_ && a.nxh == NXH_ && a.NP == NP_ && a.S == MX_ / LZ_) {             \
-    static SmemLimit lim_;                                                                            \
-    return launch_with(plane_kernel_ct<R, MX_, LZ_, NXH_, NP_, NT_>, a, B, smem, st, &lim_, NT_);     \
-  }
-#define CH_PLANE_CT(MX_, LZ_, NXH_, NP_) CH_PLANE_CT_NT(MX_, LZ_, NXH_, NP_, 256)
-
 template <typename R>
 cudaError_t launch_plane(const PlaneArgs<R>& a, int B, size_t smem, cudaStream_t st) {
   if (a.team16) return launch_plane16<R>(a, B, st);
   if (a.passes) return launch_plane_passes<R>(a, B, st);
-  CH_PLANE_CT(24, 6, 8, 3)
-  CH_PLANE_CT(24, 24, 8, 12)
   return launch_with(plane_kernel<R>, a, B, smem, st, &generic_limit<R>());
 }
 

@@ -28,33 +28,22 @@ static bool dct_order(int N) {
   }
 }
 
-size_t stage_pre_smem(const Grid& g, int ppc, size_t node_bytes) {
-  return (size_t)8 * g.ny * ppc * node_bytes + (size_t)12 * ppc * sizeof(double2);
-}
-// (with six complex values per mode for the FP64 fast analysis; the
-// coefficient tile is smaller in FP32 node precision, the FP64 size bounds both)
+bool stage_direct(const Grid& g) { return !dct_order(g.N); }
+// (three fields of H, the state and the previous right-hand sides of a tile of
+// modes, their tables, and six complex values per mode)
 size_t stage_post_smem(const Grid& g, int Mh, int ppc) {
   return ((size_t)7 * g.ny + 6) * ppc * sizeof(double2) + ((size_t)18 * Mh * ppc + 6 * ppc) * sizeof(double);
 }
-bool stage_pre_tiled(const Grid& g) { return !dct_order(g.N); }
 int stage_post_launches(int top, bool batched) { return (batched || top) ? 2 : 1; }
 
 template <typename RN>
 cudaError_t launch_stage_pre(const Grid& g, int B, const PencilBufs& pb, const DevTables& t,
-                             typename cpx<RN>::T* q, int ppc, cudaStream_t st) {
+                             typename cpx<RN>::T* q, cudaStream_t st) {
   switch (g.N) {
 #define X(n) case n: return pre_dct_n<RN, n>(g, B, pb, t, q, st);
     CH_DCT_ORDERS(X)
 #undef X
-    default: break;
-  }
-  const size_t smem = stage_pre_smem(g, ppc, sizeof(typename cpx<RN>::T));
-  // 16 (MH - 1) / 16 >= (N + 1) / 2 node pairs per mode
-  switch (mh_bucket((g.N + 1) / 2 + 1)) {
-#define X(m) case m: return pre_mh<RN, m>(g, B, pb, t, q, ppc, smem, st);
-    CH_MH_BUCKETS(X)
-#undef X
-    default: return cudaErrorInvalidValue;
+    default: return launch_pre_direct<RN>(g, B, pb, t, q, st);
   }
 }
 
@@ -64,39 +53,36 @@ cudaError_t launch_stage_pre(const Grid& g, int B, const PencilBufs& pb, const D
 template <typename RN>
 cudaError_t launch_stage_post(const Grid& g, int B, const PencilBufs& pb, const DevTables& t,
                               typename cpx<RN>::T* h, const StageCoef& sc, int ppc, bool batched, cudaStream_t st) {
-  const int mh = mh_bucket(g.N / 2 + 1);
   if (!batched && !t.tau.top_bc) {
     const size_t smem = stage_post_smem(g, t.tau.Mh, ppc);
-    switch (mh) {
+    switch (mh_bucket(g.N / 2 + 1)) {
 #define X(m) case m: return post_mh<RN, m>(g, B, pb, t, h, sc, ppc, smem, st);
       CH_MH_BUCKETS(X)
 #undef X
       default: return cudaErrorInvalidValue;
     }
   }
-  cudaError_t e = cudaErrorInvalidValue;
-  if (dct_order(g.N)) {
-    switch (g.N) {
+  // the coefficients of H: over its nodal values, or (direct sums) over the node
+  // values of the velocity and vorticity, which no kernel reads any more
+  typename cpx<RN>::T* hc = h;
+  cudaError_t e;
+  switch (g.N) {
 #define X(n) case n: e = analysis_dct_n<RN, n>(g, B, pb, h, st); break;
-      CH_DCT_ORDERS(X)
+    CH_DCT_ORDERS(X)
 #undef X
-    }
-  } else {
-    switch (mh) {
-#define X(m) case m: e = analysis_mh<RN, m>(g, B, pb, t, h, st); break;
-      CH_MH_BUCKETS(X)
-#undef X
-    }
+    default:
+      hc = reinterpret_cast<typename cpx<RN>::T*>(pb.Q);
+      e = launch_analysis_direct<RN>(g, B, pb, t, h, hc, st);
   }
   if (e != cudaSuccess) return e;
-  return launch_stage_solve<RN>(g, B, pb, t, h, sc, st);
+  return launch_stage_solve<RN>(g, B, pb, t, hc, sc, st);
 }
 
-template cudaError_t launch_stage_pre<double>(const Grid&, int, const PencilBufs&, const DevTables&, double2*, int,
+template cudaError_t launch_stage_pre<double>(const Grid&, int, const PencilBufs&, const DevTables&, double2*,
                                               cudaStream_t);
 template cudaError_t launch_stage_post<double>(const Grid&, int, const PencilBufs&, const DevTables&, double2*,
                                                const StageCoef&, int, bool, cudaStream_t);
-template cudaError_t launch_stage_pre<float>(const Grid&, int, const PencilBufs&, const DevTables&, float2*, int,
+template cudaError_t launch_stage_pre<float>(const Grid&, int, const PencilBufs&, const DevTables&, float2*,
                                              cudaStream_t);
 template cudaError_t launch_stage_post<float>(const Grid&, int, const PencilBufs&, const DevTables&, float2*,
                                               const StageCoef&, int, bool, cudaStream_t);

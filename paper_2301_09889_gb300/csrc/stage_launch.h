@@ -12,14 +12,15 @@
 namespace chdns {
 
 template <typename RN, int MH>
-cudaError_t pre_mh(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, typename cpx<RN>::T* q, int ppc,
-                   size_t smem, cudaStream_t st);
-template <typename RN, int MH>
 cudaError_t post_mh(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, const typename cpx<RN>::T* h,
                     const StageCoef& sc, int ppc, size_t smem, cudaStream_t st);
-template <typename RN, int MH>
-cudaError_t analysis_mh(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, typename cpx<RN>::T* h,
-                        cudaStream_t st);
+// direct sums (stage_direct.cu); pitches of their cosine tables
+template <typename RN>
+cudaError_t launch_pre_direct(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, typename cpx<RN>::T* q,
+                              cudaStream_t st);
+template <typename RN>
+cudaError_t launch_analysis_direct(const Grid& g, int B, const PencilBufs& pb, const DevTables& t,
+                                   const typename cpx<RN>::T* hn, typename cpx<RN>::T* hc, cudaStream_t st);
 // register cosine transforms (stage_dct.cuh)
 template <typename RN, int N>
 cudaError_t pre_dct_n(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, typename cpx<RN>::T* q,

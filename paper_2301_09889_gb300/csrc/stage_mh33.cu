@@ -1,4 +1,4 @@
-// Fused stage kernels instantiated for MH = 33.
+// Per-tile implicit half instantiated for MH = 33.
 #include "stage_kernels.cuh"
 
-CH_STAGE_INSTANTIATE(33)
+CH_STAGE_POST(33)

@@ -1,4 +1,4 @@
-// Fused stage kernels instantiated for MH = 49.
+// Per-tile implicit half instantiated for MH = 49.
 #include "stage_kernels.cuh"
 
-CH_STAGE_INSTANTIATE(49)
+CH_STAGE_POST(49)

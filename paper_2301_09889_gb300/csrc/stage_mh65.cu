@@ -1,5 +1,4 @@
-// Fused stage kernels instantiated for MH = 65, per-tile forms.
+// Per-tile implicit half instantiated for MH = 65.
 #include "stage_kernels.cuh"
 
-CH_STAGE_PRE(65)
 CH_STAGE_POST(65)
