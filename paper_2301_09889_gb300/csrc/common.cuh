@@ -111,20 +111,6 @@ template <typename C> __device__ __forceinline__ C czero();
 template <> __device__ __forceinline__ double2 czero<double2>() { return make_double2(0.0, 0.0); }
 template <> __device__ __forceinline__ float2 czero<float2>() { return make_float2(0.f, 0.f); }
 
-// Programmatic dependent launch.  The step's stage and plane kernels may be
-// launched with the programmatic-serialisation attribute, so a kernel may start while its
-// predecessor in the stream drains.  Each kernel reads its predecessor's
-// output only after griddepcontrol.wait (predecessor complete, its writes
-// visible), and lets its successor launch only after that wait: a kernel
-// that starts early therefore finds every grid before its predecessor
-// complete, and may read their outputs (the state, the tables) in its
-// prologue.  Both instructions are no-ops in a kernel launched without the
-// attribute.
-__device__ __forceinline__ void pdl_wait_then_release() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 // Asynchronous copy of one 4-, 8- or 16-byte element from global to shared
 // memory (cp.async): no register holds the value, so a thread issues all its
 // copies of a tile before any completes.  cp_async_wait_all() waits for the
@@ -165,40 +151,21 @@ inline cudaError_t raise_smem_limit(K kernel, SmemLimit* lim, size_t smem, bool 
   return cudaSuccess;
 }
 
-// launch with the programmatic-serialisation attribute (see above)
+// Plain stream-ordered launch.  Programmatic dependent launch was measured and
+// left out: a dependent that starts early takes shared memory and registers
+// from the CTAs that its predecessor still has to place.  With the trigger
+// after the wait a 64x65x64 FP64 step took 25 % longer; mixed-precision steps
+// took with / without it (us): 388 / 366 at 24x50x48 x 8, 402 / 391 at
+// 64x65x64 x 2 (forced), 878 / 875 at 128x129x128, 1084 / 1086 at 16x65x16 x 256.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                              Args&&... args) {
+inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                 Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-
-// The attribute is given to the kernels of FP32-node handles only: measured on
-// GB300 it shortens the mixed-precision steps (64x65x64 by 1-4 %, 256 minimal
-// channels by 1.2 %) and lengthens the all-FP64 64x65x64 step by 2-3.5 %, also
-// when the FP64 plane kernel alone is launched without it.
-template <bool PDL, typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl_if(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                                 Args&&... args) {
-  if constexpr (PDL) {
-    return launch_pdl(kernel, grid, block, smem, st, std::forward<Args>(args)...);
-  } else {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-  }
 }
 
 // ---------------------------------------------------------------------------

@@ -64,7 +64,6 @@ __global__ void __launch_bounds__(256) plane_kernel(PlaneArgs<R> a) {
   const int j = blockIdx.y;
   const int b = blockIdx.z;
   if (a.active && !a.active[b]) return;  // whole cluster (same b) returns together
-  pdl_wait_then_release();               // the node values come from stage_pre
   const size_t plane = (size_t)a.P;
   const C* qb = a.q + (size_t)b * 6 * a.ny * plane + (size_t)j * plane;
   C* hb = a.h + (size_t)b * 3 * a.ny * plane + (size_t)j * plane;
@@ -196,13 +195,8 @@ static cudaError_t launch_with(K kernel, const PlaneArgs<R>& a, int B, size_t sm
   cfg.blockDim = dim3(nt, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[1];
   int na = 0;
-  if (sizeof(R) == 4) {  // programmatic launch for the FP32 plane only (see launch_pdl_if)
-    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[na].val.programmaticStreamSerializationAllowed = 1;
-    ++na;
-  }
   if (a.S > 1) {
     attr[na].id = cudaLaunchAttributeClusterDimension;
     attr[na].val.clusterDim.x = a.S;

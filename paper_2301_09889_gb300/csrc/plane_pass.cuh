@@ -47,7 +47,6 @@ __global__ void __launch_bounds__(z_threads<R>(MZ)) zpass_inverse_kernel(PlaneAr
   const int b = blockIdx.y, nxh = a.nxh;
   if (a.active && !a.active[b]) return;
   const int cols = a.ny * 6 * nxh, c0 = blockIdx.x * CT;  // column (j, f, i), i fastest
-  pdl_wait_then_release();  // the node values come from stage_pre
   for (int w = threadIdx.x; w < B * CT; w += NT) {
     const int c = w % CT, kb = w / CT, g = c0 + c;
     if (g >= cols) continue;
@@ -90,7 +89,6 @@ __global__ void __launch_bounds__(NT) xpass_kernel(PlaneArgs<R> a) {
   const int b = blockIdx.y, hz = a.mz / 2;
   if (a.active && !a.active[b]) return;
   const int npairs = a.ny * hz, g0 = blockIdx.x * NPR;  // row pair (j, m), m fastest
-  pdl_wait_then_release();
   C* yb = a.y + (size_t)b * a.ny * 6 * a.mz * NXH;
   auto rows = [&](int g, int f) { return yb + ((size_t)(g / hz * 6 + f) * a.mz + 2 * (g % hz)) * NXH; };
   // every read of this CTA's rows happens before the first barrier; the rows
@@ -227,7 +225,6 @@ __global__ void __launch_bounds__(z_threads<R>(MZ)) zpass_forward_kernel(PlaneAr
   const int b = blockIdx.y, nxh = a.nxh;
   if (a.active && !a.active[b]) return;
   const int cols = a.ny * 3 * nxh, c0 = blockIdx.x * CT;  // column (j, f, i), i fastest
-  pdl_wait_then_release();
   const C* yb = a.y + (size_t)b * a.ny * 6 * MZ * nxh;
   for (int w = threadIdx.x; w < A * CT; w += NT) {
     const int c = w % CT, ka = w / CT, g = c0 + c;
@@ -270,7 +267,7 @@ cudaError_t zpass_inverse_m(const PlaneArgs<R>& a, int B, cudaStream_t st) {
   static SmemLimit lim;
   const cudaError_t e = raise_smem_limit(zpass_inverse_kernel<R, MZ>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(R) == 4>(zpass_inverse_kernel<R, MZ>, dim3((a.ny * 6 * a.nxh + CT - 1) / CT, B),
+  return launch_kernel(zpass_inverse_kernel<R, MZ>, dim3((a.ny * 6 * a.nxh + CT - 1) / CT, B),
                                        dim3(NT), smem, st, a);
 }
 template <typename R, int MZ>
@@ -280,7 +277,7 @@ cudaError_t zpass_forward_m(const PlaneArgs<R>& a, int B, cudaStream_t st) {
   static SmemLimit lim;
   const cudaError_t e = raise_smem_limit(zpass_forward_kernel<R, MZ>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(R) == 4>(zpass_forward_kernel<R, MZ>, dim3((a.ny * 3 * a.nxh + CT - 1) / CT, B),
+  return launch_kernel(zpass_forward_kernel<R, MZ>, dim3((a.ny * 3 * a.nxh + CT - 1) / CT, B),
                                        dim3(NT), smem, st, a);
 }
 template <typename R, int MX>
@@ -290,7 +287,7 @@ cudaError_t xpass_m(const PlaneArgs<R>& a, int B, cudaStream_t st) {
   static SmemLimit lim;
   const cudaError_t e = raise_smem_limit(xpass_kernel<R, MX, NPR, NT>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(R) == 4>(xpass_kernel<R, MX, NPR, NT>, dim3((a.ny * (a.mz / 2) + NPR - 1) / NPR, B),
+  return launch_kernel(xpass_kernel<R, MX, NPR, NT>, dim3((a.ny * (a.mz / 2) + NPR - 1) / NPR, B),
                                        dim3(NT), smem, st, a);
 }
 

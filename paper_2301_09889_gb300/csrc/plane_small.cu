@@ -47,7 +47,6 @@ __global__ void __launch_bounds__(kNT, sizeof(R) == 4 ? 6 : 3) plane16_kernel(Pl
   C* S = reinterpret_cast<C*>(smem_raw);  // [planes][kX], at first with the columns of step 1
   const int tid = threadIdx.x, b = blockIdx.y, j0 = blockIdx.x * kPPB;
   if (a.active && !a.active[b]) return;  // whole CTA (same b) returns together
-  pdl_wait_then_release();               // the node values come from stage_pre
   const size_t P = a.P;
 
   // 1. z inverse
@@ -178,7 +177,6 @@ __global__ void __launch_bounds__(kPairNT) plane16_pair_kernel(PlaneArgs<R> a) {
   auto cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank(), tid = threadIdx.x, j = blockIdx.y, b = blockIdx.z;
   if (a.active && !a.active[b]) return;  // whole cluster (same b) returns together
-  pdl_wait_then_release();               // the node values come from stage_pre
   const C* __restrict__ tw = a.tw_x;     // e^{2 pi i k / 24}
   const size_t P = a.P;
   C* Zr = cluster.map_shared_rank(Z, rank ^ 1);
@@ -331,15 +329,13 @@ static cudaError_t launch_plane16_pair(const PlaneArgs<R>& a, int B, cudaStream_
   cfg.blockDim = dim3(kPairNT);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // FP32 nodes only (see launch_pdl_if)
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = sizeof(R) == 4 ? 2 : 1;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, plane16_pair_kernel<R>, a);
 }
 
@@ -352,7 +348,7 @@ cudaError_t launch_plane16(const PlaneArgs<R>& a, int B, cudaStream_t st) {
   static SmemLimit lim;
   const cudaError_t e = raise_smem_limit(plane16_kernel<R>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(R) == 4>(plane16_kernel<R>, dim3((a.ny + kPPB - 1) / kPPB, B), dim3(kNT), smem, st, a);
+  return launch_kernel(plane16_kernel<R>, dim3((a.ny + kPPB - 1) / kPPB, B), dim3(kNT), smem, st, a);
 }
 
 template cudaError_t launch_plane16<double>(const PlaneArgs<double>&, int, cudaStream_t);

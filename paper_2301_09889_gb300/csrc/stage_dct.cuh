@@ -66,7 +66,6 @@ __global__ void __launch_bounds__(64, ctas_of(dct_regs<RN, N>(), 64)) stage_pre_
   const int p = (int)blockIdx.x / 6 * 16 + (lane >> 1), r = lane & 1;
   const int b = blockIdx.y;
   if (pb.active && !pb.active[b]) return;
-  pdl_wait_then_release();  // v, omega_y come from the previous stage
   RN* mine = part + half * (H + 1) * 32 + lane;
   if (p < P) {
     const int row = p / g.nxh, ix = p % g.nxh;
@@ -191,7 +190,6 @@ __global__ void __launch_bounds__(64, ctas_of(dct_regs<RN, N>(), 64)) analysis_d
   const int p = blockIdx.x * 16 + (lane >> 1), r = lane & 1;
   const int b = blockIdx.y;
   if (pb.active && !pb.active[b]) return;
-  pdl_wait_then_release();  // H comes from the nonlinear term
   RN* col = reinterpret_cast<RN*>(hn) + 2 * (((size_t)b * 3 + f) * ny * P + min(p, P - 1)) + r;
   RN* sm = reinterpret_cast<RN*>(smem_raw) + lane;
   const size_t hs = 2 * (size_t)P;
@@ -227,7 +225,7 @@ cudaError_t pre_dct_n(const Grid& g, int B, const PencilBufs& pb, const DevTable
   static SmemLimit lim;
   const cudaError_t e = raise_smem_limit(stage_pre_dct_kernel<RN, N>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(RN) == 4>(stage_pre_dct_kernel<RN, N>, dim3((g.P + 15) / 16 * 6, B), dim3(64), smem, st, g, pb,
+  return launch_kernel(stage_pre_dct_kernel<RN, N>, dim3((g.P + 15) / 16 * 6, B), dim3(64), smem, st, g, pb,
                                         t, q);
 }
 template <typename RN, int N>
@@ -236,7 +234,7 @@ cudaError_t analysis_dct_n(const Grid& g, int B, const PencilBufs& pb, typename 
   static SmemLimit lim;
   const cudaError_t e = raise_smem_limit(analysis_dct_kernel<RN, N>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(RN) == 4>(analysis_dct_kernel<RN, N>, dim3((g.P + 15) / 16, B, 3), dim3(64), smem, st, g, pb, h);
+  return launch_kernel(analysis_dct_kernel<RN, N>, dim3((g.P + 15) / 16, B, 3), dim3(64), smem, st, g, pb, h);
 }
 
 }  // namespace chdns

@@ -25,7 +25,7 @@ static cudaError_t pre_k(const Grid& g, int B, const PencilBufs& pb, const DevTa
   static SmemLimit lim;
   const cudaError_t e = raise_smem_limit(stage_pre_direct_kernel<RN, K>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(RN) == 4>(stage_pre_direct_kernel<RN, K>, dim3((g.P + 15) / 16 * 6, B, z), dim3(32 * nw), smem,
+  return launch_kernel(stage_pre_direct_kernel<RN, K>, dim3((g.P + 15) / 16 * 6, B, z), dim3(32 * nw), smem,
                                         st, g, pb, t, q);
 }
 template <typename RN, int K>
@@ -36,7 +36,7 @@ static cudaError_t analysis_k(const Grid& g, int B, const PencilBufs& pb, const 
   static SmemLimit lim;
   const cudaError_t e = raise_smem_limit(analysis_direct_kernel<RN, K>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(RN) == 4>(analysis_direct_kernel<RN, K>, dim3((g.P + 15) / 16, B, 6 * groups),
+  return launch_kernel(analysis_direct_kernel<RN, K>, dim3((g.P + 15) / 16, B, 6 * groups),
                                         dim3(32 * kAnaWarps), smem, st, g, pb, t, hn, hc, direct_ana_pitch(g.N));
 }
 

@@ -53,7 +53,6 @@ __global__ void __launch_bounds__(192) stage_pre_direct_kernel(Grid g, PencilBuf
   const int p = (int)blockIdx.x / 6 * 16 + (lane >> 1), r = lane & 1;
   const int b = blockIdx.y;
   if (pb.active && !pb.active[b]) return;
-  pdl_wait_then_release();  // v, omega_y come from the previous stage
   if (p < P) {
     const int row = p / g.nxh, ix = p % g.nxh;
     const bool mean = p == 0, gen = !mean && row != g.nz / 2;
@@ -184,7 +183,6 @@ __global__ void __launch_bounds__(32 * kAnaWarps) analysis_direct_kernel(Grid g,
   const int p = blockIdx.x * 16 + (lane >> 1), r = lane & 1;
   const int b = blockIdx.y;
   if (pb.active && !pb.active[b]) return;
-  pdl_wait_then_release();  // H comes from the nonlinear term
   const size_t base = 2 * (((size_t)b * 3 + f) * ny * P + min(p, P - 1)) + r, hs = 2 * (size_t)P;
   const RN* col = reinterpret_cast<const RN*>(hn) + base;
 #pragma unroll 4

@@ -136,7 +136,6 @@ __global__ void __launch_bounds__(8 * kModeThreads) stage_post_kernel(Grid g, in
   }
   // everything above is independent of the nonlinear term; H comes from the
   // preceding kernel
-  pdl_wait_then_release();
   // nodal values in the node precision, in the first bytes of the sH region
   CN* sN = reinterpret_cast<CN*>(sH);
   for (int w = tid; w < 3 * ny * ppc; w += nt) {
@@ -273,7 +272,7 @@ cudaError_t post_mh(const Grid& g, int B, const PencilBufs& pb, const DevTables&
   static SmemLimit lim;
   const cudaError_t e = raise_smem_limit(stage_post_kernel<RN, MH>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(RN) == 4>(stage_post_kernel<RN, MH>, dim3((g.P + ppc - 1) / ppc, B),
+  return launch_kernel(stage_post_kernel<RN, MH>, dim3((g.P + ppc - 1) / ppc, B),
                                         dim3(kModeThreads * ppc), smem, st, g, B, pb, t, h, sc, ppc);
 }
 

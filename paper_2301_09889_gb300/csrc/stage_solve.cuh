@@ -516,7 +516,6 @@ __global__ void __launch_bounds__(64, D == 3 ? 6 : 4) stage_solve_kernel(Grid g,
   extern __shared__ __align__(16) double sarr[];  // [Mh][64], then the exchange slots [6][64] of a free-slip top
   const int b = blockIdx.y, tiles = (g.P + 15) / 16;
   if (pb.active && !pb.active[b]) return;
-  pdl_wait_then_release();  // the coefficients of H come from the analysis
   const int lane = threadIdx.x & 31, c = threadIdx.x / 32, r = lane & 1;
   const int z = (blockIdx.x + tiles - 1) / tiles;  // 0: mean, 1: v, 2: omega_y
   const int pr = z == 0 ? lane >> 1 : ((int)(blockIdx.x - 1) % tiles) * 16 + (lane >> 1), p = min(pr, g.P - 1);
@@ -538,7 +537,7 @@ cudaError_t solve_ahead(const Grid& g, int B, const PencilBufs& pb, const DevTab
   static SmemLimit lim;
   const cudaError_t e = raise_smem_limit(stage_solve_kernel<RN, TOP, D>, &lim, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl_if<sizeof(RN) == 4>(stage_solve_kernel<RN, TOP, D>, grid, dim3(64), smem, st, g, pb, t, h, sc);
+  return launch_kernel(stage_solve_kernel<RN, TOP, D>, grid, dim3(64), smem, st, g, pb, t, h, sc);
 }
 
 template <typename RN, int TOP>
