@@ -287,12 +287,22 @@ void free_env(ch_env* env) {
     if (r_ != CH_OK) return r_;  \
   } while (0)
 
+// layout of the node values: a node's fields in padded planes for the passes
+// (both precisions run the passes of the lengths that are built), dense otherwise
+void node_strides(Grid* g) {
+  const bool passes = passes_built(g->mx, g->mz);
+  g->qf = passes ? (size_t)g->mz * g->nxh : (size_t)g->ny * g->P;
+  g->qj = passes ? 6 * g->qf : (size_t)g->P;
+  g->qb = passes ? g->ny * g->qj : 6 * g->qf;
+}
+
 // nonlinear plane kernel: smallest cluster whose z-slab fits shared memory
 template <typename R>
 int setup_plane(ch_env* env, PlaneArgs<R>* a, size_t* smem) {
   using C = typename cpx<R>::T;
   const Grid& g = env->g;
   a->nxh = g.nxh; a->nz = g.nz; a->ny = g.ny; a->mx = g.mx; a->mz = g.mz; a->P = g.P;
+  a->qf = (size_t)g.ny * g.P; a->qj = g.P; a->qb = 6 * a->qf; a->hb = 3 * a->qf;
   a->S = 0;
   const size_t csz = sizeof(C);
   // cluster size: the smallest feasible S whose ny * B * S CTAs fill the SMs
@@ -314,8 +324,8 @@ int setup_plane(ch_env* env, PlaneArgs<R>* a, size_t* smem) {
   // a 16-CTA cluster (non-portable opt-in) only where no portable size fits
   if (!nf && g.mz % 16 == 0 && (g.mz / 16) % 2 == 0 && (size_t)6 * (g.mz / 16) * g.nxh * csz <= 160 * 1024)
     feasible[nf++] = 16;
-  // Three passes through a global scratch array where the padded lengths are
-  // built (plane_pass.cu), in the precision the handle steps in; the other
+  // Three passes through global memory (in place in a step) where the padded
+  // lengths are built (plane_pass.cu), in the precision the handle steps in; the other
   // plane keeps a cluster, for ch_nonlinear, where one fits.  Planes of
   // 256 x 256 modes fit no portable cluster.
   const bool stepping = (sizeof(R) == 8) == (env->prm.precision == 0);
@@ -332,9 +342,7 @@ int setup_plane(ch_env* env, PlaneArgs<R>* a, size_t* smem) {
     a->cluster = large || fp64_square ? 0 : feasible[nf - 1];
     for (int k = 0; k < nf && a->cluster; ++k)
       if ((long)g.ny * env->B * feasible[k] >= nsm) { a->cluster = feasible[k]; break; }
-    C* y = nullptr;
-    RC(dalloc(env, &y, (size_t)env->B * g.ny * 6 * g.mz * g.nxh));
-    a->y = y;
+    a->y = reinterpret_cast<C*>(env->pb.Q);
     auto cast2 = [](const std::vector<double2>& v) {
       std::vector<C> o(v.size());
       for (size_t i = 0; i < v.size(); ++i) o[i] = mk((R)v[i].x, (R)v[i].y);
@@ -755,33 +763,26 @@ StageCoef stage_coef(const ch_env* env, int k, double theta) {
   return sc;
 }
 
-int run_stage(ch_env* env, int k, double theta) {
+// node values, nonlinear term and implicit half of one stage, R: the node precision
+template <typename R>
+int run_stage_in(ch_env* env, const PlaneArgs<R>& plane, size_t smem, const StageCoef& sc) {
   const Grid& g = env->g;
   const int B = env->B;
   cudaStream_t st = env->stream;
-  const bool mixed = env->prm.precision == 1;
-  if (mixed) {
-    float2* q = reinterpret_cast<float2*>(env->pb.Q);
-    LAUNCH(0, launch_stage_pre<float>(g, B, env->pb, env->tab, q, st));
-    PlaneArgs<float> a = env->plane_f;
-    a.q = q;
-    a.h = reinterpret_cast<float2*>(env->pb.R);
-    LAUNCH(1, launch_plane<float>(a, B, env->plane_f_smem, st));
-  } else {
-    LAUNCH(0, launch_stage_pre<double>(g, B, env->pb, env->tab, env->pb.Q, st));
-    PlaneArgs<double> a = env->plane;
-    a.q = env->pb.Q;
-    a.h = env->pb.R;
-    LAUNCH(1, launch_plane<double>(a, B, env->plane_smem, st));
-  }
-  const StageCoef sc = stage_coef(env, k, theta);
-  if (mixed)
-    LAUNCH(2, launch_stage_post<float>(g, B, env->pb, env->tab, reinterpret_cast<float2*>(env->pb.R), sc,
-                                       env->ppc_post, env->post_batched, st));
-  else
-    LAUNCH(2, launch_stage_post<double>(g, B, env->pb, env->tab, env->pb.R, sc, env->ppc_post, env->post_batched,
-                                        st));
+  auto* q = reinterpret_cast<typename cpx<R>::T*>(env->pb.Q);
+  LAUNCH(0, launch_stage_pre<R>(g, B, env->pb, env->tab, q, st));
+  PlaneArgs<R> a = plane;
+  a.q = a.h = q;
+  a.qf = g.qf; a.qj = g.qj; a.qb = a.hb = g.qb;
+  LAUNCH(1, launch_plane<R>(a, B, smem, st));
+  LAUNCH(2, launch_stage_post<R>(g, B, env->pb, env->tab, q, sc, env->ppc_post, env->post_batched, st));
   return CH_OK;
+}
+
+int run_stage(ch_env* env, int k, double theta) {
+  const StageCoef sc = stage_coef(env, k, theta);
+  return env->prm.precision == 1 ? run_stage_in(env, env->plane_f, env->plane_f_smem, sc)
+                                 : run_stage_in(env, env->plane, env->plane_smem, sc);
 }
 
 // kernels of one env_step: the action or control kernels, per RK step three
@@ -930,7 +931,7 @@ int autotune_tiles(ch_env* env, int smem_max) {
   CK(cudaMemsetAsync(pb.G, 0, Bs * ny * P * sizeof(double2), st));
   CK(cudaMemsetAsync(pb.HVP, 0, Bs * ny * P * sizeof(double2), st));
   CK(cudaMemsetAsync(pb.HGP, 0, Bs * ny * P * sizeof(double2), st));
-  CK(cudaMemsetAsync(pb.R, 0, Bs * 3 * ny * P * sizeof(double2), st));
+  CK(cudaMemsetAsync(pb.Q, 0, Bs * g.qb * (env->prm.precision == 1 ? sizeof(float2) : sizeof(double2)), st));
   CK(cudaMemsetAsync(pb.vw_old, 0, Bs * P * sizeof(double2), st));
   CK(cudaMemsetAsync(pb.vw_new, 0, Bs * P * sizeof(double2), st));
   for (double* x : {pb.UM, pb.WM, pb.HXP, pb.HZP}) CK(cudaMemsetAsync(x, 0, Bs * ny * sizeof(double), st));
@@ -938,8 +939,8 @@ int autotune_tiles(ch_env* env, int smem_max) {
   const StageCoef sc = stage_coef(env, 0, 1.0);
   auto post = [&](int ppc, bool batched) {
     const cudaError_t e =
-        mixed ? launch_stage_post<float>(g, B, pb, env->tab, reinterpret_cast<float2*>(pb.R), sc, ppc, batched, st)
-              : launch_stage_post<double>(g, B, pb, env->tab, pb.R, sc, ppc, batched, st);
+        mixed ? launch_stage_post<float>(g, B, pb, env->tab, reinterpret_cast<float2*>(pb.Q), sc, ppc, batched, st)
+              : launch_stage_post<double>(g, B, pb, env->tab, pb.Q, sc, ppc, batched, st);
     return e == cudaSuccess ? CH_OK : CH_ERR_CUDA;
   };
   constexpr int kReps = 3;
@@ -1022,18 +1023,17 @@ int env_slot_seed(ch_env* env, int e, uint64_t seed, double amplitude, int kmax)
 size_t env_footprint(const ch_params_t* p) {
   const size_t B = p->batch > 0 ? p->batch : 1;
   const size_t nxh = p->nx / 2, P = nxh * p->nz, ny = p->ny, Mh = (ny - 1) / 2 + 1;
-  const size_t state = B * (4 * ny * P * 16 + 4 * ny * 8 + 9 * ny * P * 16 + 3 * P * 16 + 8 +
+  Grid g{};
+  g.ny = (int)ny; g.nxh = (int)nxh; g.P = (int)P; g.mx = 3 * p->nx / 2; g.mz = 3 * p->nz / 2;
+  node_strides(&g);
+  const size_t state = B * (4 * ny * P * 16 + 4 * ny * 8 + g.qb * (p->precision == 1 ? 8 : 16) + 3 * P * 16 + 8 +
                             (size_t)p->nz * p->nx * 8 + (2 * (size_t)p->nz * p->nx + 2) * 8);
   const size_t folded = (3 * 2 * (p->top_bc ? 8 : 7) * Mh * P + 2 * 6 * Mh * P) * 8;
   const size_t scan = p->top_bc ? 0 : (3 * 2 * 4 + 2 * 4) * Mh * P;
   const size_t tables = (scan + 3 * 2 * P + 2 * P + 3 * 2 * Mh * P + 3 * 2 * P +
                          3 * Mh + 3 + 3 * ny + ny + 2 * 3 * 2 * 2 * P) * 8 + ny * ny * 12 + (nxh + p->nz) * 8 +
                         folded;
-  // the scratch of the three-pass nonlinear term, where it runs in passes
-  // (complex values of the plane's precision)
-  const size_t mx = 3 * (size_t)p->nx / 2, mz = 3 * (size_t)p->nz / 2;
-  const size_t passes = passes_built((int)mx, (int)mz) ? B * ny * 6 * mz * nxh * (p->precision == 0 ? 16 : 8) : 0;
-  return state + tables + passes + ((size_t)4 << 20);  // plus twiddles and rounding slack
+  return state + tables + ((size_t)4 << 20);  // plus twiddles and rounding slack
 }
 }  // namespace chdns
 
@@ -1087,6 +1087,7 @@ int env_create(const ch_params_t* p, ch_env_t** out) {
   Grid& g = env->g;
   g.nx = p->nx; g.ny = p->ny; g.nz = p->nz; g.nxh = p->nx / 2; g.P = g.nz * g.nxh; g.N = p->ny - 1;
   g.mx = 3 * p->nx / 2; g.mz = 3 * p->nz / 2;
+  node_strides(&g);
   env->nu = channel_height(p) / p->re_bulk;
   env->u_tau = p->re_tau / p->re_bulk;
   env->tau_ref = p->tau_ref > 0 ? p->tau_ref : env->u_tau * env->u_tau;
@@ -1103,7 +1104,7 @@ int env_create(const ch_params_t* p, ch_env_t** out) {
       (rc = dalloc(env, &pb.HVP, B * ny * P)) || (rc = dalloc(env, &pb.HGP, B * ny * P)) ||
       (rc = dalloc(env, &pb.UM, B * ny)) || (rc = dalloc(env, &pb.WM, B * ny)) ||
       (rc = dalloc(env, &pb.HXP, B * ny)) || (rc = dalloc(env, &pb.HZP, B * ny)) ||
-      (rc = dalloc(env, &pb.Q, B * 6 * ny * P)) || (rc = dalloc(env, &pb.R, B * 3 * ny * P)) ||
+      (rc = dalloc(env, &pb.Q, p->precision == 1 ? B * g.qb / 2 : B * g.qb)) ||
       (rc = dalloc(env, &pb.vw_old, B * P)) || (rc = dalloc(env, &pb.vw_new, B * P)) ||
       (rc = dalloc(env, &pb.planes, B * 2 * P)) || (rc = dalloc(env, &pb.tau_acc, B)))
     return fail(rc);

@@ -455,13 +455,20 @@ __device__ __forceinline__ void fft_dit_ct(typename cpx<R>::T* buf, const typena
 // ---------------------------------------------------------------------------
 struct Grid {
   int nx, ny, nz, nxh, P, N, mx, mz;
+  // strides (complex values) of PencilBufs.Q between fields, nodes and environments
+  size_t qf, qj, qb;
 };
 
 template <typename R>
 struct PlaneArgs {
   using C = typename cpx<R>::T;
-  const C* q;          // [B][6][ny][P]
-  C* h;                // [B][3][ny][P]
+  // q [B][6][ny][P] and h [B][3][ny][P] in ch_nonlinear.  In a step both are
+  // PencilBufs.Q, H over the first three fields: every kernel reads the part of
+  // q that its writes of h cover (the columns of a pass, the plane of a CTA or a
+  // cluster) before a barrier in front of them
+  const C* q;
+  C* h;
+  size_t qf, qj, qb, hb;  // strides of fields and nodes (both), of environments (q, h)
   int nxh, nz, ny, mx, mz, P;
   int S, Lz, NP;
   const C* tw_x;       // [mx]  e^{2 pi i k / mx}
@@ -476,7 +483,7 @@ struct PlaneArgs {
   // three passes through global memory (z inverse, x transforms and products,
   // z forward; plane_pass.cuh)
   int passes;
-  C* y;                // [B][ny][6][mz][nxh] scratch: z-transformed columns, then H in fields 0..2
+  C* y;                // [B][ny][6][mz][nxh]: z-transformed columns, then H in fields 0..2 (PencilBufs.Q)
   int cluster;         // ch_info_t.plane_cluster
 };
 

@@ -26,8 +26,13 @@ struct PencilBufs {
   float2 *V32, *G32;            // [B][ny][P] V and G rounded to FP32 (mixed precision): what stage_pre reads;
                                 // mode 0 of G32 holds the mean flow (W, U)
   double *UM, *WM, *HXP, *HZP;  // [B][ny]
-  double2* Q;                   // [B][6][ny][P] node values of u, v, w, ox, oy, oz (nonlinear input)
-  double2* R;                   // [B][3][ny][P] node values of H
+  // node values of u, v, w, ox, oy, oz in the node precision, then those of H (or
+  // its coefficients) over the first three: strides Grid.qf, qj, qb.  Where the
+  // nonlinear term runs in passes a node's fields are [6][mz][nxh], the
+  // first nz rows of each in use, so that the z transforms run in place;
+  // otherwise [6][ny][P].  (A step so holds no array beside the six fields:
+  // 9 ny P values with passes, 6 ny P without)
+  double2* Q;
   double2 *vw_old, *vw_new;     // [B][P] wall-velocity spectra
   double2* planes;              // [B][2][P] u, v spectra at the sensing node
   double* tau_acc;              // [B]

@@ -64,9 +64,8 @@ __global__ void __launch_bounds__(256) plane_kernel(PlaneArgs<R> a) {
   const int j = blockIdx.y;
   const int b = blockIdx.z;
   if (a.active && !a.active[b]) return;  // whole cluster (same b) returns together
-  const size_t plane = (size_t)a.P;
-  const C* qb = a.q + (size_t)b * 6 * a.ny * plane + (size_t)j * plane;
-  C* hb = a.h + (size_t)b * 3 * a.ny * plane + (size_t)j * plane;
+  const C* qb = a.q + b * a.qb + j * a.qj;
+  C* hb = a.h + b * a.hb + j * a.qj;
 
   // 1. gather + fold + pre-twiddle
   for (int w = tid; w < 6 * Lz * nxh; w += nt) {
@@ -74,7 +73,7 @@ __global__ void __launch_bounds__(256) plane_kernel(PlaneArgs<R> a) {
     const int t = w / nxh;
     const int m = t % Lz;
     const int f = t / Lz;
-    const C* qf = qb + (size_t)f * a.ny * plane;
+    const C* qf = qb + f * a.qf;
     C acc = czero<C>();
     for (int qq = 0; qq < S; ++qq) {
       const int u = m + qq * Lz;
@@ -178,7 +177,7 @@ __global__ void __launch_bounds__(256) plane_kernel(PlaneArgs<R> a) {
       }
       out = a.scale * out;
     }
-    hb[(size_t)f * a.ny * plane + row * nxh + i] = out;
+    hb[f * a.qf + row * nxh + i] = out;
   }
   if (S > 1) cg::this_cluster().sync();
 }

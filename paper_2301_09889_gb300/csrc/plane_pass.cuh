@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(z_threads<R>(MZ)) zpass_inverse_kernel(PlaneAr
     const int c = w % CT, kb = w / CT, g = c0 + c;
     if (g >= cols) continue;
     const int i = g % nxh, jf = g / nxh, f = jf % 6, j = jf / 6;
-    const C* src = a.q + (((size_t)b * 6 + f) * a.ny + j) * a.P + i;
+    const C* src = a.q + b * a.qb + f * a.qf + j * a.qj + i;
     C x[A];
 #pragma unroll
     for (int p = 0; p < A / 3; ++p) x[p] = src[(size_t)(B * p + kb) * nxh];
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(z_threads<R>(MZ)) zpass_forward_kernel(PlaneAr
 #pragma unroll
     for (int p = 0; p < A; ++p) x[p] = T[(s * A + p) * CT + c];
     dft_reg<-1, false, A, R>(x);
-    C* dst = a.h + (((size_t)b * 3 + f) * a.ny + j) * a.P + i;
+    C* dst = a.h + b * a.hb + f * a.qf + j * a.qj + i;
     const R sc = (R)0.5 * a.scale;
 #pragma unroll
     for (int p = 0; p < A / 3; ++p) dst[(size_t)(B * p + s) * nxh] = sc * x[p];

@@ -47,13 +47,12 @@ __global__ void __launch_bounds__(kNT, sizeof(R) == 4 ? 6 : 3) plane16_kernel(Pl
   C* S = reinterpret_cast<C*>(smem_raw);  // [planes][kX], at first with the columns of step 1
   const int tid = threadIdx.x, b = blockIdx.y, j0 = blockIdx.x * kPPB;
   if (a.active && !a.active[b]) return;  // whole CTA (same b) returns together
-  const size_t P = a.P;
 
   // 1. z inverse
   if (tid < kPPB * 6 * kNxh) {
     const int i = tid % kNxh, f = tid / kNxh % 6, pl = tid / (6 * kNxh);
     if (j0 + pl < a.ny) {
-      const C* q = a.q + (((size_t)b * 6 + f) * a.ny + j0 + pl) * P + i;
+      const C* q = a.q + b * a.qb + f * a.qf + (j0 + pl) * a.qj + i;
       C x[kM];
 #pragma unroll
       for (int u = 0; u < kNz / 2; ++u) x[u] = q[u * kNxh];
@@ -138,7 +137,7 @@ __global__ void __launch_bounds__(kNT, sizeof(R) == 4 ? 6 : 3) plane16_kernel(Pl
       }
       dft_reg<-1, false, kM, R>(x);
       const R sc = (R)0.5 * a.scale;
-      C* h = a.h + (((size_t)b * 3 + f) * a.ny + j0 + pl) * P + i;
+      C* h = a.h + b * a.hb + f * a.qf + (j0 + pl) * a.qj + i;
 #pragma unroll
       for (int row = 0; row < kNz; ++row)
         h[row * kNxh] = row == kNz / 2 ? czero<C>() : sc * x[row < kNz / 2 ? row : row + kM - kNz];
@@ -178,14 +177,13 @@ __global__ void __launch_bounds__(kPairNT) plane16_pair_kernel(PlaneArgs<R> a) {
   const int rank = (int)cluster.block_rank(), tid = threadIdx.x, j = blockIdx.y, b = blockIdx.z;
   if (a.active && !a.active[b]) return;  // whole cluster (same b) returns together
   const C* __restrict__ tw = a.tw_x;     // e^{2 pi i k / 24}
-  const size_t P = a.P;
   C* Zr = cluster.map_shared_rank(Z, rank ^ 1);
   C* Hr = cluster.map_shared_rank(H, rank ^ 1);
 
   // z inverse of this CTA's three fields
   if (tid < 96) {
     const int c = tid % 24, kb = tid / 24;
-    const C* q = a.q + (((size_t)b * 6 + 3 * rank + c / 8) * a.ny + j) * P + c % 8;
+    const C* q = a.q + b * a.qb + (3 * rank + c / 8) * a.qf + j * a.qj + c % 8;
     C x[6];
 #pragma unroll
     for (int p = 0; p < 2; ++p) x[p] = q[(4 * p + kb) * kNxh];
@@ -310,7 +308,7 @@ __global__ void __launch_bounds__(kPairNT) plane16_pair_kernel(PlaneArgs<R> a) {
     for (int p = 0; p < 6; ++p) x[p] = T[c * kT6 + s * kA1 + p];
     dft_reg<-1, false, 6, R>(x);
     const R sc = (R)0.5 * a.scale;
-    C* h = a.h + (((size_t)b * 3 + c / 4) * a.ny + j) * P + rank * 4 + c % 4;
+    C* h = a.h + b * a.hb + c / 4 * a.qf + j * a.qj + rank * 4 + c % 4;
 #pragma unroll
     for (int p = 0; p < 2; ++p) h[(4 * p + s) * kNxh] = sc * x[p];
 #pragma unroll

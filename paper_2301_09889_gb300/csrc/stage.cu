@@ -63,7 +63,7 @@ cudaError_t launch_stage_post(const Grid& g, int B, const PencilBufs& pb, const 
     }
   }
   // the coefficients of H: over its nodal values, or (direct sums) over the node
-  // values of the velocity and vorticity, which no kernel reads any more
+  // values of the vorticity, which no kernel reads any more
   typename cpx<RN>::T* hc = h;
   cudaError_t e;
   switch (g.N) {
@@ -71,7 +71,7 @@ cudaError_t launch_stage_post(const Grid& g, int B, const PencilBufs& pb, const 
     CH_DCT_ORDERS(X)
 #undef X
     default:
-      hc = reinterpret_cast<typename cpx<RN>::T*>(pb.Q);
+      hc = h + 3 * g.qf;
       e = launch_analysis_direct<RN>(g, B, pb, t, h, hc, st);
   }
   if (e != cudaSuccess) return e;

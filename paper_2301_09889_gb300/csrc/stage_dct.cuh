@@ -165,8 +165,8 @@ __global__ void __launch_bounds__(64, ctas_of(dct_regs<RN, N>(), 64)) stage_pre_
   }
   __syncthreads();
   if (p >= P) return;
-  RN* dst = reinterpret_cast<RN*>(q) + 2 * (((size_t)b * 6 + f) * ny * P + p) + r;
-  const size_t qs = 2 * (size_t)P;
+  RN* dst = reinterpret_cast<RN*>(q) + 2 * (b * g.qb + f * g.qf + p) + r;
+  const size_t qs = 2 * g.qj;
 #pragma unroll 8
   for (int j = half; j < H; j += 2) {
     const RN e = part[j * 32 + lane], o = part[(H + 1 + j) * 32 + lane];
@@ -183,16 +183,16 @@ __global__ void __launch_bounds__(64, ctas_of(dct_regs<RN, N>(), 64)) stage_pre_
 template <typename RN, int N>
 __global__ void __launch_bounds__(64, ctas_of(dct_regs<RN, N>(), 64)) analysis_dct_kernel(Grid g, PencilBufs pb,
                                                                     typename cpx<RN>::T* __restrict__ hn) {
-  constexpr int H = N / 2, ny = N + 1;
+  constexpr int H = N / 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int P = g.P;
   const int lane = threadIdx.x & 31, half = threadIdx.x / 32, f = blockIdx.z;
   const int p = blockIdx.x * 16 + (lane >> 1), r = lane & 1;
   const int b = blockIdx.y;
   if (pb.active && !pb.active[b]) return;
-  RN* col = reinterpret_cast<RN*>(hn) + 2 * (((size_t)b * 3 + f) * ny * P + min(p, P - 1)) + r;
+  RN* col = reinterpret_cast<RN*>(hn) + 2 * (b * g.qb + f * g.qf + min(p, P - 1)) + r;
   RN* sm = reinterpret_cast<RN*>(smem_raw) + lane;
-  const size_t hs = 2 * (size_t)P;
+  const size_t hs = 2 * g.qj;
 #pragma unroll 16
   for (int j = half; j <= N; j += 2) sm[j * 32] = col[(size_t)j * hs];
   __syncthreads();

@@ -152,8 +152,8 @@ __global__ void __launch_bounds__(192) stage_pre_direct_kernel(Grid g, PencilBuf
 #pragma unroll
     for (int k = 0; k < K; ++k) E[k] = E[k] + c[k] * x;
   }
-  RN* dst = reinterpret_cast<RN*>(q) + 2 * (((size_t)b * 6 + f) * ny * P + p) + r;
-  const size_t qs = 2 * (size_t)P;
+  RN* dst = reinterpret_cast<RN*>(q) + 2 * (b * g.qb + f * g.qf + p) + r;
+  const size_t qs = 2 * g.qj;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     const int j = j0 + k;
@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(192) stage_pre_direct_kernel(Grid g, PencilBuf
 
 // a_n = 2/(N cb_n) sum_j f_j cos(pi n j / N) / cb_j (cb_0 = cb_N = 2) of one
 // parity of one field of 16 modes, from the nodal values hn to the coefficients
-// hc (another array: the CTAs of a field share its nodes).
+// hc (other fields of the array: the CTAs of a field share its nodes).
 // grid (tiles, B, 3 fields x 2 parities x groups of 4 K)
 constexpr int kAnaWarps = 4;
 template <typename RN, int K>
@@ -177,13 +177,13 @@ __global__ void __launch_bounds__(32 * kAnaWarps) analysis_direct_kernel(Grid g,
                                                                          typename cpx<RN>::T* __restrict__ hc, int Ip) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   RN* sm = reinterpret_cast<RN*>(smem_raw);  // [N/2 + 1][32] folded nodes
-  const int P = g.P, N = g.N, ny = g.ny;
+  const int P = g.P, N = g.N;
   const int lane = threadIdx.x & 31, warp = threadIdx.x / 32;
   const int f = blockIdx.z % 3, par = blockIdx.z / 3 % 2, i0 = (blockIdx.z / 6 * kAnaWarps + warp) * K;
   const int p = blockIdx.x * 16 + (lane >> 1), r = lane & 1;
   const int b = blockIdx.y;
   if (pb.active && !pb.active[b]) return;
-  const size_t base = 2 * (((size_t)b * 3 + f) * ny * P + min(p, P - 1)) + r, hs = 2 * (size_t)P;
+  const size_t base = 2 * (b * g.qb + f * g.qf + min(p, P - 1)) + r, hs = 2 * g.qj;
   const RN* col = reinterpret_cast<const RN*>(hn) + base;
 #pragma unroll 4
   for (int j = warp; 2 * j < N; j += kAnaWarps) {

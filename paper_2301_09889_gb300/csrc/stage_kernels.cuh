@@ -134,14 +134,12 @@ __global__ void __launch_bounds__(8 * kModeThreads) stage_post_kernel(Grid g, in
     cp_async_elem(ss + (1 * 2 + sig) * ppc + pl, t.tau.pois_isq + (size_t)sig * P + p);
     cp_async_elem(ss + (2 * 2 + sig) * ppc + pl, t.tau.vh_idv + (size_t)(sc.k * 2 + sig) * P + p);
   }
-  // everything above is independent of the nonlinear term; H comes from the
-  // preceding kernel
   // nodal values in the node precision, in the first bytes of the sH region
   CN* sN = reinterpret_cast<CN*>(sH);
   for (int w = tid; w < 3 * ny * ppc; w += nt) {
     const int pl = w % ppc, fn = w / ppc;  // fn = f * ny + n
     const int p = min(p0 + pl, P - 1);
-    cp_async_elem(sN + w, hn + ((size_t)b * 3 * ny + fn) * P + p);
+    cp_async_elem(sN + w, hn + b * g.qb + fn / ny * g.qf + fn % ny * g.qj + p);
   }
   cp_async_wait_all();
   __syncthreads();

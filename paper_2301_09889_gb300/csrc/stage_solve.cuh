@@ -134,8 +134,9 @@ __device__ __forceinline__ Wall omega_down(double* f, const Grid& g, const Penci
   const size_t hP = 2 * P, base = 2 * ((size_t)b * ny * P + p) + r;
   const double* G = reinterpret_cast<const double*>(pb.G) + base;
   RN* HG = reinterpret_cast<RN*>(pb.HGP) + base;
-  const RN* hx = hc + 2 * ((size_t)b * 3 * ny * P + p) + 1 - r;
-  const RN* hz = hx + 2 * (size_t)ny * hP;
+  const RN* hx = hc + 2 * (b * g.qb + p) + 1 - r;
+  const RN* hz = hx + 4 * g.qf;
+  const size_t hS = 2 * g.qj;
   const RN sgn = r == 0 ? (RN)-1 : (RN)1, kx = sgn * (RN)t.kx[ix], kz = sgn * (RN)t.kz[row];
   const Coef3<RN> nc = node_coef<RN>(sc);
   struct In {
@@ -152,8 +153,8 @@ __device__ __forceinline__ Wall omega_down(double* f, const Grid& g, const Penci
         In v;
         const size_t n = 2 * i + sig, o = (size_t)min(i + 1, M - 1) * P;  // row i + 1 of the elimination
         v.x = G[n * hP];
-        v.hx = __ldg(hx + n * hP);
-        v.hz = __ldg(hz + n * hP);
+        v.hx = __ldg(hx + n * hS);
+        v.hz = __ldg(hz + n * hS);
         v.hp = HG[n * hP];
         v.tb = tab_row(T, MP, o);
         if (TOP) v.W2 = __ldg(T + 7 * MP + o);
@@ -181,9 +182,9 @@ __device__ __forceinline__ Wall omega_down(double* f, const Grid& g, const Penci
 
 // The mean flow (component 0: U, 1: W) of parity sig, in the lanes of mode 0:
 // down, for the increment.  X: coefficients, XP: previous plane means of H,
-// hm: its new ones (2 P apart).
+// hm: its new ones (2 qj apart).
 template <typename RN, int TOP>
-__device__ __forceinline__ Wall mean_down(double* f, const DevTables& t, const StageCoef& sc, int N, size_t P, int sig,
+__device__ __forceinline__ Wall mean_down(double* f, const DevTables& t, const StageCoef& sc, int N, size_t P, size_t qj, int sig,
                                        const double* __restrict__ T, const double* X, double* XP,
                                        const RN* __restrict__ hm) {
   constexpr int NT = 64;
@@ -206,7 +207,7 @@ __device__ __forceinline__ Wall mean_down(double* f, const DevTables& t, const S
         const size_t o = (size_t)min(i + 1, M - 1) * P;
         v.x = X[n];
         v.hp = XP[n];
-        v.h = __ldg(hm + 2 * P * n);
+        v.h = __ldg(hm + 2 * qj * n);
         v.wi = __ldg(t.tau.wint + n);
         v.tb = tab_row(T, MP, o);
         v.E1 = __ldg(T + 6 * MP + o);
@@ -289,8 +290,8 @@ __device__ __forceinline__ void solve_omega(double* f, double* xch, const Grid& 
   Wall w;
   if (live) {
     if constexpr (MEAN) {
-      const RN* hm = hc + 2 * (size_t)b * 3 * ny * P + (r == 0 ? 0 : 2 * (size_t)ny * 2 * P);
-      w = mean_down<RN, TOP>(f, t, sc, g.N, P, sig, T, X, (r == 0 ? pb.HXP : pb.HZP) + (size_t)b * ny, hm);
+      const RN* hm = hc + 2 * b * g.qb + (r == 0 ? 0 : 4 * g.qf);
+      w = mean_down<RN, TOP>(f, t, sc, g.N, P, g.qj, sig, T, X, (r == 0 ? pb.HXP : pb.HZP) + (size_t)b * ny, hm);
     } else {
       w = omega_down<RN, TOP, D>(f, g, pb, t, sc, b, p, r, sig, T, hc);
     }
@@ -369,10 +370,11 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
   double* Vp = reinterpret_cast<double*>(pb.V) + base;
   RN* HV = reinterpret_cast<RN*>(pb.HVP) + base;
   float* V32 = reinterpret_cast<float*>(pb.V32) + base;
-  const RN* H0 = hc + 2 * ((size_t)b * 3 * ny * P + p);
+  const RN* H0 = hc + 2 * (b * g.qb + p);
   const RN* hx = H0 + 1 - r;
-  const RN* hy = H0 + (size_t)ny * hP + r;
-  const RN* hz = H0 + 2 * (size_t)ny * hP + 1 - r;
+  const RN* hy = H0 + 2 * g.qf + r;
+  const RN* hz = H0 + 4 * g.qf + 1 - r;
+  const size_t hS = 2 * g.qj;
   const double kxd = t.kx[ix], kzd = t.kz[row], k2 = fma(kxd, kxd, kzd * kzd), ck2 = -(1.0 + cc) * k2;
   const RN sgn = r == 0 ? (RN)-1 : (RN)1, kx = sgn * (RN)kxd, kz = sgn * (RN)kzd, k2n = (RN)k2;
   const Coef3<RN> nc = node_coef<RN>(sc);
@@ -388,13 +390,13 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
       In v;
       const size_t n = 2 * i + sig;
       v.x = Vp[n * hP];
-      v.hy = __ldg(hy + n * hP);
+      v.hy = __ldg(hy + n * hS);
       v.hp = HV[n * hP];
       if constexpr (sizeof(RN) == 8) v.fac = __ldg(t.tau.n1 + n);
       else v.fac = (RN)(2 * ((int)n + 1));
       const size_t no = min((int)n + 1, N), o = (size_t)min(i + 1, M - 1) * P;
-      v.hx = __ldg(hx + no * hP);
-      v.hz = __ldg(hz + no * hP);
+      v.hx = __ldg(hx + no * hS);
+      v.hz = __ldg(hz + no * hS);
       v.tb = tab_row(T, MP, o);
       v.E1 = __ldg(T + 6 * MP + o);
       return v;
