@@ -439,7 +439,7 @@ int build_tables(ch_env* env) {
     for (int i = M - 1; i >= 1; --i) {
       const int n = 2 * i + sig;
       if (i < M - 1) w = 1.0 + F.b[i + 1] * w;
-      w2 = (double)n * n + (i < M - 1 ? F.b[i + 1] * w2 : 0.0);
+      if (top) w2 = (double)n * n + (i < M - 1 ? F.b[i + 1] * w2 : 0.0);
       tab[base + ((size_t)0 * Mh + i) * P + pp] = F.e[i] * cA(n);
       tab[base + ((size_t)1 * Mh + i) * P + pp] = F.e[i] * cB(n, N);
       tab[base + ((size_t)2 * Mh + i) * P + pp] = F.e[i] * cC(n, N);
@@ -588,7 +588,7 @@ int build_tables(ch_env* env) {
   env->tab.tau.top_bc = top ? 1 : 0;
   RC(dupload(env, &env->tab.tw_nx, twiddles(g.nx)));
   RC(dupload(env, &env->tab.tw_nz, twiddles(g.nz)));
-  if (stage_direct(g)) {
+  if (stage_direct(g) || (p.precision == 0 && pre_few(g, env->B))) {
     const int Jp = direct_pre_pitch(N), Ip = direct_ana_pitch(N), J = N / 2 + 1;
     std::vector<double> cp((size_t)ny * Jp, 0.0), ca((size_t)J * 2 * Ip, 0.0);
     for (int j = 0; j < J; ++j)

@@ -59,6 +59,8 @@ size_t stage_post_smem(const Grid& g, int Mh, int ppc);  // per-tile implicit ha
 // direct Chebyshev sums (no register cosine transform for this order): the
 // handle needs their tables, of these pitches
 bool stage_direct(const Grid& g);
+// FP64 handles whose explicit half runs as direct sums spread over the GPU
+bool pre_few(const Grid& g, int B);
 int direct_pre_pitch(int N);
 int direct_ana_pitch(int N);
 // kernels one launch_stage_post issues

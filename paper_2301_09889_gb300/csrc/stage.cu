@@ -39,6 +39,9 @@ int stage_post_launches(int top, bool batched) { return (batched || top) ? 2 : 1
 template <typename RN>
 cudaError_t launch_stage_pre(const Grid& g, int B, const PencilBufs& pb, const DevTables& t,
                              typename cpx<RN>::T* q, cudaStream_t st) {
+  if constexpr (sizeof(RN) == 8) {
+    if (pre_few(g, B)) return launch_pre_few(g, B, pb, t, q, st);
+  }
   switch (g.N) {
 #define X(n) case n: return pre_dct_n<RN, n>(g, B, pb, t, q, st);
     CH_DCT_ORDERS(X)

@@ -28,6 +28,24 @@ static cudaError_t pre_k(const Grid& g, int B, const PencilBufs& pb, const DevTa
   return launch_kernel(stage_pre_direct_kernel<RN, K>, dim3((g.P + 15) / 16 * 6, B, z), dim3(32 * nw), smem,
                                         st, g, pb, t, q);
 }
+// The few-mode form, in FP64 where its CTAs find an SM each.  Us per launch, it /
+// the transforms or direct sums above: 128 modes N = 32 15.2 / 16.7, N = 48 18.9 /
+// 22.5, N = 49 19.1 / 33.2, N = 64 21.1 / 28.1; 32 modes N = 128 33.5 / 49.6.  With
+// twice the modes a CTA of four pairs per warp no longer gains (28.6 / 27.0 at
+// 256 modes, N = 64).  Its shared memory bounds N.
+static unsigned few_groups(const Grid& g) { return (g.N / 2 + kFewPairs) / kFewPairs; }
+bool pre_few(const Grid& g, int B) {
+  return g.N <= 128 && (long)((g.P + 15) / 16) * 6 * B * few_groups(g) <= 152;
+}
+cudaError_t launch_pre_few(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, double2* q, cudaStream_t st) {
+  const size_t smem = (size_t)g.ny * (4 * 32 + kFewPairs + 1) * sizeof(double);
+  static SmemLimit lim;
+  const cudaError_t e = raise_smem_limit(stage_pre_few_kernel, &lim, smem);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(stage_pre_few_kernel, dim3((g.P + 15) / 16 * 6, B, few_groups(g)), dim3(32 * kFewWarps),
+                       smem, st, g, pb, t, q);
+}
+
 template <typename RN, int K>
 static cudaError_t analysis_k(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, const typename cpx<RN>::T* hn,
                               typename cpx<RN>::T* hc, cudaStream_t st) {

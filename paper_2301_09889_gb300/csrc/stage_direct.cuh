@@ -166,6 +166,154 @@ __global__ void __launch_bounds__(192) stage_pre_direct_kernel(Grid g, PencilBuf
   }
 }
 
+// The explicit half of handles with so few modes that a transform per line
+// leaves most SMs idle (FP64; an operation holds its sub-partition 64 cycles, so
+// one warp's line is a chain of its operations; 28 us per launch of 128 modes
+// at N = 64, 21 here).  A CTA forms 12 node pairs of a field of 16 modes.
+// Everything it reads arrives in one round of loads; the recurrences of the
+// derivatives run on four warps (parity x the terms of d2 v or D v, and of the
+// others), every CTA its own copy; then each warp sums two node pairs.
+// grid (6 tiles, B, groups of 12 pairs)
+constexpr int kFewWarps = 6, kFewPairs = 2 * kFewWarps;
+__global__ void __launch_bounds__(32 * kFewWarps) stage_pre_few_kernel(Grid g, PencilBufs pb, DevTables t,
+                                                                       double2* __restrict__ q) {
+  constexpr int K = 2, KC = kFewPairs;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int P = g.P, N = g.N, ny = g.ny, J = N / 2 + 1, Jp = (J + 15) / 8 * 8;
+  double* co = reinterpret_cast<double*>(smem_raw);  // [ny][32] coefficients of the field
+  double* sv = co + 32 * ny;                         // [ny][32] v
+  double* so = sv + 32 * ny;                         // [ny][32] omega_y, the mean flow, or the field itself
+  double* pd = so + 32 * ny;                         // [ny][32] terms of d2 v or D v
+  double* tb = pd + 32 * ny;                         // [ny][KC] cos(pi j n / N) of the CTA's pairs
+  double* c2 = tb + KC * ny;                         // [ny] 2 (n + 1)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x / 32, f = blockIdx.x % 6;
+  const int p = (int)blockIdx.x / 6 * 16 + (lane >> 1), r = lane & 1;
+  const int b = blockIdx.y, jc = blockIdx.z * KC;
+  if (pb.active && !pb.active[b]) return;
+  const int pc = min(p, P - 1), row = pc / g.nxh, ix = pc % g.nxh;
+  const bool mean = p == 0, gen = p > 0 && p < P && row != g.nz / 2;
+  const bool own = f == 1 || f == 4, deriv = f == 3 || f == 5;
+  const double kx = t.kx[ix], kz = t.kz[row];
+  const double sg = r == 0 ? -1.0 : 1.0;
+  const double ik2 = gen ? sg / (kx * kx + kz * kz) : 0.0;
+  double cD = 0.0, cS = 1.0, cV = 0.0;
+  if (gen && !own) {
+    if (f == 0) { cD = ik2 * kx; cS = -ik2 * kz; }
+    if (f == 2) { cD = ik2 * kz; cS = ik2 * kx; }
+    if (f == 3) { cD = ik2 * kz; cS = ik2 * kx; cV = -sg * kz; }
+    if (f == 5) { cD = -ik2 * kx; cS = ik2 * kz; cV = sg * kx; }
+  } else if (mean && f == 5) {
+    cS = -1.0;
+  }
+  {
+    const bool liveM = mean && !own && r == 0, liveS = gen || liveM;
+    const size_t col = 2 * ((size_t)b * ny * P + pc), vs = 2 * (size_t)P;
+    const double* v0 = reinterpret_cast<const double*>(pb.V) + col;
+    const double* Vp = v0 + (1 - r);
+    const double* Sp = (f == 1 ? v0 : reinterpret_cast<const double*>(pb.G) + col) + (own ? r : 1 - r);
+    size_t ss = vs;
+    if (liveM) {
+      Sp = (f == 0 || f == 5 ? pb.UM : pb.WM) + (size_t)b * ny;
+      ss = 1;
+    }
+#pragma unroll 11
+    for (int n = warp; n < ny; n += kFewWarps) {
+      const double x = __ldg(Vp + n * vs), y = __ldg(Sp + n * ss);
+      sv[n * 32 + lane] = gen ? x : 0.0;
+      so[n * 32 + lane] = liveS ? y : 0.0;
+    }
+#pragma unroll 4
+    for (int w = threadIdx.x; w < ny * KC; w += 32 * kFewWarps) {
+      const int n = w / KC, j = jc + w % KC;
+      tb[w] = j < J ? __ldg(t.cos_pre + (size_t)n * Jp + j) : 0.0;
+    }
+    for (int n = threadIdx.x; n < ny; n += 32 * kFewWarps) c2[n] = t.tau.n1[n];
+  }
+  __syncthreads();
+  const double* src = own ? so : co;
+  if (!own) {
+    if (warp < 4) {
+      const int par = warp & 1, top = (N - par) / 2;
+      const double* V = sv + lane;
+      const double* S = so + lane;
+      auto two = [&](int k) { return c2[k - 1]; };  // 2 k
+      if (warp < 2) {
+        // cD D v, or cD D^2 v: the step at i adds m = 2 i + par + 1 (and m + 1 to D v)
+        double* o = pd + par * 32 + lane;
+        double dv = 0.0, d2 = 0.0;
+        if (!deriv) {
+          if (2 * top + par < N) dv = two(N) * V[32 * N];
+          o[64 * top] = cD * dv;
+#pragma unroll 4
+          for (int i = top - 1; i >= 0; --i) {
+            const int m = 2 * i + par + 1;
+            dv = dv + two(m) * V[32 * m];
+            o[64 * i] = (i == 0 && par == 0 ? 0.5 * cD : cD) * dv;
+          }
+        } else {
+          o[64 * top] = 0.0;
+#pragma unroll 4
+          for (int i = top - 1; i >= 0; --i) {
+            const int m = 2 * i + par + 1;
+            dv = dv + two(m + 1) * V[32 * (m + 1)];
+            d2 = d2 + two(m) * dv;
+            o[64 * i] = (i == 0 && par == 0 ? 0.5 * cD : cD) * d2;
+          }
+        }
+      } else {
+        double* o = co + par * 32 + lane;
+        if (!deriv) {
+#pragma unroll 4
+          for (int i = top; i >= 0; --i) o[64 * i] = cS * S[32 * (2 * i + par)];
+        } else {
+          double ds = 2 * top + par < N ? two(N) * S[32 * N] : 0.0;
+          o[64 * top] = cS * ds + cV * V[32 * (2 * top + par)];
+#pragma unroll 4
+          for (int i = top - 1; i >= 0; --i) {
+            const int m = 2 * i + par + 1;
+            ds = ds + two(m) * S[32 * m];
+            o[64 * i] = (i == 0 && par == 0 ? 0.5 * cS : cS) * ds + cV * V[32 * (m - 1)];
+          }
+        }
+      }
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int w = threadIdx.x; w < 32 * ny; w += 32 * kFewWarps) co[w] = co[w] + pd[w];
+    __syncthreads();
+  }
+  const int j0 = jc + warp * K;
+  if (p >= P || j0 >= J) return;
+  double E[K] = {}, O[K] = {};
+  const double* c = tb + warp * K;
+  int n = 0;
+#pragma unroll 4
+  for (; n + 1 <= N; n += 2) {
+    const double x = src[n * 32 + lane], y = src[(n + 1) * 32 + lane];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      E[k] = E[k] + c[n * KC + k] * x;
+      O[k] = O[k] + c[(n + 1) * KC + k] * y;
+    }
+  }
+  if (n == N) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) E[k] = E[k] + c[n * KC + k] * src[n * 32 + lane];
+  }
+  double* dst = reinterpret_cast<double*>(q) + 2 * (b * g.qb + f * g.qf + p) + r;
+  const size_t qs = 2 * g.qj;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int j = j0 + k;
+    if (2 * j < N) {
+      dst[(size_t)j * qs] = E[k] + O[k];
+      dst[(size_t)(N - j) * qs] = E[k] - O[k];
+    } else if (2 * j == N) {
+      dst[(size_t)j * qs] = E[k];
+    }
+  }
+}
+
 // a_n = 2/(N cb_n) sum_j f_j cos(pi n j / N) / cb_j (cb_0 = cb_N = 2) of one
 // parity of one field of 16 modes, from the nodal values hn to the coefficients
 // hc (other fields of the array: the CTAs of a field share its nodes).

@@ -18,6 +18,7 @@ cudaError_t post_mh(const Grid& g, int B, const PencilBufs& pb, const DevTables&
 template <typename RN>
 cudaError_t launch_pre_direct(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, typename cpx<RN>::T* q,
                               cudaStream_t st);
+cudaError_t launch_pre_few(const Grid& g, int B, const PencilBufs& pb, const DevTables& t, double2* q, cudaStream_t st);
 template <typename RN>
 cudaError_t launch_analysis_direct(const Grid& g, int B, const PencilBufs& pb, const DevTables& t,
                                    const typename cpx<RN>::T* hn, typename cpx<RN>::T* hc, cudaStream_t st);
