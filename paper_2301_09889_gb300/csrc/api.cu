@@ -14,6 +14,7 @@
 
 #include "../../include/channel_dns.h"
 #include "common.cuh"
+#include "fft_reg.cuh"
 #include "internal.h"
 
 using namespace chdns;
@@ -343,13 +344,18 @@ int setup_plane(ch_env* env, PlaneArgs<R>* a, size_t* smem) {
     for (int k = 0; k < nf && a->cluster; ++k)
       if ((long)g.ny * env->B * feasible[k] >= nsm) { a->cluster = feasible[k]; break; }
     a->y = reinterpret_cast<C*>(env->pb.Q);
-    auto cast2 = [](const std::vector<double2>& v) {
-      std::vector<C> o(v.size());
-      for (size_t i = 0; i < v.size(); ++i) o[i] = mk((R)v[i].x, (R)v[i].y);
+    auto line_twiddles = [](int m) {  // [line_b][line_a] e^{2 pi i s k / m}
+      const std::vector<double2> w = twiddles(m);
+      const int A = line_a(m);
+      std::vector<C> o(m);
+      for (int i = 0; i < m; ++i) {
+        const double2 v = w[(i / A) * (i % A)];
+        o[i] = mk((R)v.x, (R)v.y);
+      }
       return o;
     };
-    RC(dupload(env, &a->tw_x, cast2(twiddles(g.mx))));
-    RC(dupload(env, &a->tw_mz, cast2(twiddles(g.mz))));
+    RC(dupload(env, &a->tw_x, line_twiddles(g.mx)));
+    RC(dupload(env, &a->tw_mz, line_twiddles(g.mz)));
     a->scale = (R)(1.0 / ((double)g.mx * g.mz));
     return CH_OK;
   }

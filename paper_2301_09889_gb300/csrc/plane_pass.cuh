@@ -15,7 +15,10 @@
 // sub-partitions busy: 1.06 TFLOP/s per GPU), whatever its active lanes, so
 // the passes are shaped for the fewest operations with every lane at work:
 // tiles whose task counts are multiples of a warp, small CTAs that even out
-// over the SMs.  FP32 planes by L2 and instruction issue.
+// over the SMs.  FP32 planes by L2 and instruction issue.  The twiddles of a
+// line of A x B points stand as [B][A], in the order in which the lanes of a
+// warp take them (as gathers from one table of roots they took more L1 cycles
+// than the exchange: __TW__).
 #pragma once
 
 #include "common.cuh"
@@ -37,6 +40,12 @@ template <typename R> constexpr int x_pairs(int m) {
 template <typename R> constexpr int x_threads(int m) { return m <= 24 ? 96 : sizeof(R) == 4 && m >= 144 ? 384 : 192; }
 // odd row stride: the transposing accesses of the exchange meet no bank twice
 __host__ __device__ constexpr int x_stride(int m) { return line_a(m) | 1; }
+// elements between lines: with sixteen lines of A points the second step's
+// lanes run on into the next line, which continues the banks of the first
+template <typename R> __host__ __device__ constexpr int x_line(int m) {
+  const int banks = sizeof(R) == 4 ? 16 : 8, l = line_b(m) * x_stride(m);
+  return line_b(m) == 16 ? l + ((line_a(m) - l) % banks + banks) % banks : l;
+}
 
 template <typename R, int MZ>
 __global__ void __launch_bounds__(z_threads<R>(MZ)) zpass_inverse_kernel(PlaneArgs<R> a) {
@@ -72,7 +81,7 @@ __global__ void __launch_bounds__(z_threads<R>(MZ)) zpass_inverse_kernel(PlaneAr
     C x[B];
     x[0] = T[ka * CT + c];
 #pragma unroll
-    for (int s = 1; s < B; ++s) x[s] = cmul(T[(s * A + ka) * CT + c], a.tw_mz[s * ka]);
+    for (int s = 1; s < B; ++s) x[s] = cmul(T[(s * A + ka) * CT + c], a.tw_mz[s * A + ka]);
     dft_pow2<+1, B, R>(x);
     C* dst = yb + (size_t)(g / nxh) * MZ * nxh + g % nxh;
 #pragma unroll
@@ -83,9 +92,9 @@ __global__ void __launch_bounds__(z_threads<R>(MZ)) zpass_inverse_kernel(PlaneAr
 template <typename R, int MX, int NPR, int NT>
 __global__ void __launch_bounds__(NT) xpass_kernel(PlaneArgs<R> a) {
   using C = typename cpx<R>::T;
-  constexpr int A = line_a(MX), B = line_b(MX), A1 = x_stride(MX), LS = B * A1, NXH = MX / 3;
+  constexpr int A = line_a(MX), B = line_b(MX), A1 = x_stride(MX), LS = x_line<R>(MX), NXH = MX / 3;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* X = reinterpret_cast<C*>(smem_raw);  // [6][NPR][B][A1]
+  C* X = reinterpret_cast<C*>(smem_raw);  // [6][NPR][LS]: [B][A1] in use
   const int b = blockIdx.y, hz = a.mz / 2;
   if (a.active && !a.active[b]) return;
   const int npairs = a.ny * hz, g0 = blockIdx.x * NPR;  // row pair (j, m), m fastest
@@ -128,7 +137,7 @@ __global__ void __launch_bounds__(NT) xpass_kernel(PlaneArgs<R> a) {
       if (g0 + pp >= npairs) continue;
       C t[B];
 #pragma unroll
-      for (int s = 1; s < B; ++s) t[s] = a.tw_x[s * ka];
+      for (int s = 1; s < B; ++s) t[s] = a.tw_x[s * A + ka];
       C* slot = X + pp * LS + ka;
       constexpr int FS = NPR * LS;
       C v[6][B];
@@ -165,7 +174,7 @@ __global__ void __launch_bounds__(NT) xpass_kernel(PlaneArgs<R> a) {
       C v[B];
       v[0] = slot[0];
 #pragma unroll
-      for (int s = 1; s < B; ++s) v[s] = cmul(slot[s * A1], a.tw_x[s * ka]);
+      for (int s = 1; s < B; ++s) v[s] = cmul(slot[s * A1], a.tw_x[s * A + ka]);
       dft_pow2<+1, B, R>(v);
 #pragma unroll
       for (int s = 0; s < B; ++s) slot[s * A1] = v[s];
@@ -188,7 +197,7 @@ __global__ void __launch_bounds__(NT) xpass_kernel(PlaneArgs<R> a) {
       dft_pow2<-1, B, R>(v);
       slot[0] = v[0];
 #pragma unroll
-      for (int s = 1; s < B; ++s) slot[s * A1] = cmul(v[s], cconj(a.tw_x[s * ka]));
+      for (int s = 1; s < B; ++s) slot[s * A1] = cmul(v[s], cconj(a.tw_x[s * A + ka]));
     }
   }
   __syncthreads();
@@ -237,7 +246,7 @@ __global__ void __launch_bounds__(z_threads<R>(MZ)) zpass_forward_kernel(PlaneAr
     dft_pow2<-1, B, R>(x);
     T[ka * CT + c] = x[0];
 #pragma unroll
-    for (int s = 1; s < B; ++s) T[(s * A + ka) * CT + c] = cmul(x[s], cconj(a.tw_mz[s * ka]));
+    for (int s = 1; s < B; ++s) T[(s * A + ka) * CT + c] = cmul(x[s], cconj(a.tw_mz[s * A + ka]));
   }
   __syncthreads();
   for (int w = threadIdx.x; w < B * CT; w += NT) {
@@ -283,7 +292,7 @@ cudaError_t zpass_forward_m(const PlaneArgs<R>& a, int B, cudaStream_t st) {
 template <typename R, int MX>
 cudaError_t xpass_m(const PlaneArgs<R>& a, int B, cudaStream_t st) {
   constexpr int NPR = x_pairs<R>(MX), NT = x_threads<R>(MX);
-  constexpr size_t smem = (size_t)6 * NPR * line_b(MX) * x_stride(MX) * sizeof(typename cpx<R>::T);
+  constexpr size_t smem = (size_t)6 * NPR * x_line<R>(MX) * sizeof(typename cpx<R>::T);
   static SmemLimit lim;
   const cudaError_t e = raise_smem_limit(xpass_kernel<R, MX, NPR, NT>, &lim, smem);
   if (e != cudaSuccess) return e;
