@@ -344,9 +344,8 @@ int setup_plane(ch_env* env, PlaneArgs<R>* a, size_t* smem) {
     for (int k = 0; k < nf && a->cluster; ++k)
       if ((long)g.ny * env->B * feasible[k] >= nsm) { a->cluster = feasible[k]; break; }
     a->y = reinterpret_cast<C*>(env->pb.Q);
-    auto line_twiddles = [](int m) {  // [line_b][line_a] e^{2 pi i s k / m}
+    auto line_twiddles = [](int m, int A) {  // [m / A][A] e^{2 pi i s k / m}
       const std::vector<double2> w = twiddles(m);
-      const int A = line_a(m);
       std::vector<C> o(m);
       for (int i = 0; i < m; ++i) {
         const double2 v = w[(i / A) * (i % A)];
@@ -354,8 +353,8 @@ int setup_plane(ch_env* env, PlaneArgs<R>* a, size_t* smem) {
       }
       return o;
     };
-    RC(dupload(env, &a->tw_x, line_twiddles(g.mx)));
-    RC(dupload(env, &a->tw_mz, line_twiddles(g.mz)));
+    RC(dupload(env, &a->tw_x, line_twiddles(g.mx, x_line_a<R>(g.mx))));
+    RC(dupload(env, &a->tw_mz, line_twiddles(g.mz, line_a(g.mz))));
     a->scale = (R)(1.0 / ((double)g.mx * g.mz));
     return CH_OK;
   }

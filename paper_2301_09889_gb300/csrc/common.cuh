@@ -477,7 +477,7 @@ struct PlaneArgs {
   size_t qf, qj, qb, hb;  // strides of fields and nodes (both), of environments (q, h)
   int nxh, nz, ny, mx, mz, P;
   int S, Lz, NP;
-  // (in passes tw_x and tw_mz hold [line_b][line_a] e^{2 pi i s k / length}, see fft_reg.cuh)
+  // (in passes tw_x and tw_mz hold [B][A] e^{2 pi i s k / (A B)} of their line splits, fft_reg.cuh)
   const C* tw_x;       // [mx]  e^{2 pi i k / mx}
   const C* tw_z;       // [Lz]  e^{2 pi i k / Lz}
   const C* tw_mz;      // [mz]  e^{2 pi i k / mz}

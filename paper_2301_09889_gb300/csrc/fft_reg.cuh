@@ -193,6 +193,12 @@ __device__ __forceinline__ void dft_reg(C (&x)[N]) {
 // points held 6 warps per SM).
 __host__ __device__ constexpr int line_b(int m) { return m == 6 || m == 18 ? 2 : m <= 96 ? 4 : m <= 192 ? 8 : 16; }
 __host__ __device__ constexpr int line_a(int m) { return m / line_b(m); }
+// x lines in FP32: up to eight points of all six fields fit a thread, which
+// keeps the products in registers
+template <typename R> __host__ __device__ constexpr int x_line_b(int m) {
+  return sizeof(R) == 4 && m > 192 ? 8 : line_b(m);
+}
+template <typename R> __host__ __device__ constexpr int x_line_a(int m) { return m / x_line_b<R>(m); }
 // padded lengths built: 3/2 of 8, 12, 16, 24, 32, 48, 64, 96, 128, 192 and 256 modes
 #define CH_LINE_LENGTHS(X) X(12) X(18) X(24) X(36) X(48) X(72) X(96) X(144) X(192) X(288) X(384)
 

@@ -18,7 +18,9 @@
 // over the SMs.  FP32 planes by L2 and instruction issue.  The twiddles of a
 // line of A x B points stand as [B][A], in the order in which the lanes of a
 // warp take them (as gathers from one table of roots they took more L1 cycles
-// than the exchange: __TW__).
+// than the exchange: 278 us, 238 in lane order, for the x pass of
+// 256x193x256 in FP32, split 24 x 16; 206 split 48 x 8 with the products in
+// registers; 128x129x128 48 and 38).
 #pragma once
 
 #include "common.cuh"
@@ -32,19 +34,26 @@ namespace chdns {
 template <typename R> constexpr int z_cols() { return sizeof(R) == 4 ? 16 : 8; }
 template <typename R> constexpr int z_threads(int m) { return line_b(m) * z_cols<R>() < 32 ? 32 : line_b(m) * z_cols<R>(); }
 
-// x pass: row pairs per CTA (multiples of 8 fill every warp of every phase;
-// fewer where six fields of M points would leave one CTA per SM) and threads
+// x pass: row pairs per CTA (the task counts of its steps are multiples of the
+// threads, or nearly), threads and CTAs per SM (bounds the registers)
 template <typename R> constexpr int x_pairs(int m) {
-  return (sizeof(R) == 4 ? m <= 192 : m <= 96) ? 8 : (sizeof(R) == 4 || m <= 192) ? 4 : 2;
+  if (sizeof(R) == 4) return m <= 96 ? 8 : m <= 192 ? 4 : 2;
+  return m <= 96 ? 8 : m <= 192 ? 4 : 2;
 }
-template <typename R> constexpr int x_threads(int m) { return m <= 24 ? 96 : sizeof(R) == 4 && m >= 144 ? 384 : 192; }
-// odd row stride: the transposing accesses of the exchange meet no bank twice
-__host__ __device__ constexpr int x_stride(int m) { return line_a(m) | 1; }
-// elements between lines: with sixteen lines of A points the second step's
-// lanes run on into the next line, which continues the banks of the first
+template <typename R> constexpr int x_threads(int m) { return m <= 24 || (sizeof(R) == 4 && m >= 144) ? 96 : 192; }
+template <typename R> constexpr int x_ctas(int m) { return sizeof(R) == 4 && m >= 144 ? 5 : 1; }
+// elements between the sub-lines of a line, odd, and between lines: the
+// exchanges meet (nearly) no bank twice.  FP32 lines of 48 x 8 and 36 x 8: 50,
+// with an odd line, for the unpacking of eight adjacent modes of two sub-lines.
+// Lines of sixteen: the second step's lanes run on into the next line, which
+// continues the banks of the first.
+template <typename R> __host__ __device__ constexpr int x_stride(int m) {
+  return sizeof(R) == 4 && m > 192 ? 50 : x_line_a<R>(m) | 1;
+}
 template <typename R> __host__ __device__ constexpr int x_line(int m) {
-  const int banks = sizeof(R) == 4 ? 16 : 8, l = line_b(m) * x_stride(m);
-  return line_b(m) == 16 ? l + ((line_a(m) - l) % banks + banks) % banks : l;
+  const int b = x_line_b<R>(m), l = b * x_stride<R>(m);
+  if (sizeof(R) == 4 && m > 192) return l + 1;
+  return b == 16 ? l + ((x_line_a<R>(m) - l) % 8 + 8) % 8 : l;
 }
 
 template <typename R, int MZ>
@@ -89,10 +98,15 @@ __global__ void __launch_bounds__(z_threads<R>(MZ)) zpass_inverse_kernel(PlaneAr
   }
 }
 
+template <int SIGN, int B, typename R> __device__ __forceinline__ void x_dft(typename cpx<R>::T* v) {
+  if constexpr (B <= 4) small_dft_ct<SIGN, B, typename cpx<R>::T, R>(v);
+  else dft_pow2<SIGN, B, R>(v);
+}
+
 template <typename R, int MX, int NPR, int NT>
-__global__ void __launch_bounds__(NT) xpass_kernel(PlaneArgs<R> a) {
+__global__ void __launch_bounds__(NT, x_ctas<R>(MX)) xpass_kernel(PlaneArgs<R> a) {
   using C = typename cpx<R>::T;
-  constexpr int A = line_a(MX), B = line_b(MX), A1 = x_stride(MX), LS = x_line<R>(MX), NXH = MX / 3;
+  constexpr int A = x_line_a<R>(MX), B = x_line_b<R>(MX), A1 = x_stride<R>(MX), LS = x_line<R>(MX), NXH = MX / 3;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* X = reinterpret_cast<C*>(smem_raw);  // [6][NPR][LS]: [B][A1] in use
   const int b = blockIdx.y, hz = a.mz / 2;
@@ -128,7 +142,7 @@ __global__ void __launch_bounds__(NT) xpass_kernel(PlaneArgs<R> a) {
     for (int p = 0; p < A; ++p) X[line * LS + kb * A1 + p] = x[p];
   }
   __syncthreads();
-  if constexpr (B <= 4) {
+  if constexpr (B <= 4 || (B == 8 && sizeof(R) == 4)) {
     // second half of the inverse lines, products and first half of the forward
     // lines at the points ka + A kb of one row pair (real parts: first row,
     // imaginary parts: second row); each thread reads and writes its own slots
@@ -146,7 +160,7 @@ __global__ void __launch_bounds__(NT) xpass_kernel(PlaneArgs<R> a) {
         v[f][0] = slot[f * FS];
 #pragma unroll
         for (int s = 1; s < B; ++s) v[f][s] = cmul(slot[f * FS + s * A1], t[s]);
-        small_dft_ct<+1, B, C, R>(v[f]);
+        x_dft<+1, B, R>(v[f]);
       }
       C h[3][B];
 #pragma unroll
@@ -158,7 +172,7 @@ __global__ void __launch_bounds__(NT) xpass_kernel(PlaneArgs<R> a) {
       }
 #pragma unroll
       for (int f = 0; f < 3; ++f) {
-        small_dft_ct<-1, B, C, R>(h[f]);
+        x_dft<-1, B, R>(h[f]);
         slot[f * FS] = h[f][0];
 #pragma unroll
         for (int s = 1; s < B; ++s) slot[f * FS + s * A1] = cmul(h[f][s], cconj(t[s]));
