@@ -41,7 +41,8 @@ namespace chdns {
 // The coefficients of a parity are formed by rolled loops into the thread's
 // column of the exchange buffer and then read into registers: with the loops
 // unrolled, the kernel's paths (three kinds of field, two parities) outgrew
-// the instruction cache wherever an SM ran several of them.
+// the instruction cache wherever an SM ran several of them (FP32, 256x193x256:
+// 232 us by sixteen rows, 176 by eight, 180 by four).
 //
 // CTA: one field of a tile, two warps; the fields of a tile are neighbouring
 // CTAs.  FP32 lines read the copies of v and omega_y that the implicit half
@@ -132,17 +133,19 @@ __global__ void __launch_bounds__(64, ctas_of(dct_regs<RN, N>(), 64)) stage_pre_
         d2 = (RN)0;
         ds = (RN)(2 * N) * S(N);
       }
-      mine[top * 32] = cD * d2 + cS * ds + cV * V(2 * top + half);
-#pragma unroll 4
+      RN vn = V(2 * top + half);
+      mine[top * 32] = cD * d2 + cS * ds + cV * vn;
+#pragma unroll 8
       for (int i = top - 1; i >= 1; --i) {
         const int m = 2 * i + half + 1;
-        dv = dv + c2(m + 1) * V(m + 1);
+        dv = dv + c2(m + 1) * vn;
         d2 = d2 + c2(m) * dv;
         ds = ds + c2(m) * S(m);
-        mine[i * 32] = cD * d2 + cS * ds + cV * V(m - 1);
+        vn = V(m - 1);
+        mine[i * 32] = cD * d2 + cS * ds + cV * vn;
       }
       const int m = half + 1;
-      dv = dv + c2(m + 1) * V(m + 1);
+      dv = dv + c2(m + 1) * vn;
       d2 = d2 + c2(m) * dv;
       ds = ds + c2(m) * S(m);
       mine[0] = (cD * d2 + cS * ds) * (half == 0 ? (RN)0.5 : (RN)1.0) + cV * V(half);

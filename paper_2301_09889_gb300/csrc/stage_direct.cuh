@@ -109,17 +109,19 @@ __global__ void __launch_bounds__(192) stage_pre_direct_kernel(Grid g, PencilBuf
         mine[0] = cD * (par == 0 ? (RN)0.5 * dv : dv) + cS * S(par);
       } else {
         RN dv = 0, d2 = 0, ds = nt < N ? c2(N) * S(N) : (RN)0;
-        mine[64 * top] = cS * ds + cV * V(nt);
-#pragma unroll 4
+        RN vn = V(nt);
+        mine[64 * top] = cS * ds + cV * vn;
+#pragma unroll 8
         for (int i = top - 1; i >= 1; --i) {
           const int m = 2 * i + par + 1;
-          dv = dv + c2(m + 1) * V(m + 1);
+          dv = dv + c2(m + 1) * vn;
           d2 = d2 + c2(m) * dv;
           ds = ds + c2(m) * S(m);
-          mine[64 * i] = cD * d2 + cS * ds + cV * V(m - 1);
+          vn = V(m - 1);
+          mine[64 * i] = cD * d2 + cS * ds + cV * vn;
         }
         const int m = par + 1;
-        dv = dv + c2(m + 1) * V(m + 1);
+        dv = dv + c2(m + 1) * vn;
         d2 = d2 + c2(m) * dv;
         ds = ds + c2(m) * S(m);
         mine[0] = (cD * d2 + cS * ds) * (par == 0 ? (RN)0.5 : (RN)1.0) + cV * V(par);
