@@ -225,7 +225,7 @@ struct ch_env {
   int ev_used[4] = {0, 0, 0, 0};
   // The step's launch sequence is fixed for a handle: it is captured once into
   // a CUDA graph on the internal action/output buffers and replayed (one
-  // launch instead of 14-15).  [0]: every slot; [1]: slots masked by
+  // launch instead of 15 or more).  [0]: every slot; [1]: slots masked by
   // graph_mask (serving ticks).  Profiling launches the same kernels directly.
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   const int* graph_mask = nullptr;

@@ -14,7 +14,6 @@
 namespace chdns {
 
 constexpr int kMaxNy = 201;                    // largest Chebyshev node count built
-constexpr int kMaxHalf = (kMaxNy + 1) / 2 + 1; // unknowns of one parity, upper bound
 constexpr int kMaxRadixStages = 16;
 
 // ---------------------------------------------------------------------------
@@ -99,11 +98,6 @@ template <> __device__ __forceinline__ float to_rn<float>(double d) { return nar
   __host__ __device__ __forceinline__ C operator*(R s, C a) { return mk(s * a.x, s * a.y); }     \
   __host__ __device__ __forceinline__ C cmul(C a, C b) {                                  \
     return mk(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);                              \
-  }                                                                                       \
-  /* the same product with its fused multiply-adds pinned (code shared by several     */ \
-  /* kernel forms whose results must agree bit for bit)                                */ \
-  __host__ __device__ __forceinline__ C cmul_rn(C a, C b) {                               \
-    return mk(fma_rn(a.x, b.x, -mul_rn(a.y, b.y)), fma_rn(a.x, b.y, mul_rn(a.y, b.x)));    \
   }                                                                                       \
   __host__ __device__ __forceinline__ C cconj(C a) { return mk(a.x, -a.y); }                \
   /* i * s * a */                                                                         \
@@ -191,15 +185,14 @@ __device__ __forceinline__ C twiddle(const C* tw, int k) {
   return w;
 }
 
-// Small DFT y_u = sum_t x_t e^{SIGN 2 pi i t u / r}, r in {2, 3, 4}.
-template <int SIGN, typename C, typename R>
-__device__ __forceinline__ void small_dft(C* x, int r) {
-  if (r == 2) {
+// Small DFT y_u = sum_t x_t e^{SIGN 2 pi i t u / r}, r in {2, 3, 4, 8}; {2, 3, 4} at run time.
+template <int SIGN, int RADIX, typename C, typename R>
+__device__ __forceinline__ void small_dft_ct(C* x) {
+  if constexpr (RADIX == 2) {
     C a = x[0], b = x[1];
     x[0] = a + b;
     x[1] = a - b;
-  } else if (r == 3) {
-    // sin(2 pi / 3) = sqrt(3) / 2
+  } else if constexpr (RADIX == 3) {
     const R k = (R)SIGN * (R)0.86602540378443864676372317075293618;
     C s = x[1] + x[2];
     C d = x[1] - x[2];
@@ -208,7 +201,7 @@ __device__ __forceinline__ void small_dft(C* x, int r) {
     x[0] = x[0] + s;
     x[1] = t1 + rot;
     x[2] = t1 - rot;
-  } else {
+  } else if constexpr (RADIX == 4) {
     C a0 = x[0] + x[2], a1 = x[0] - x[2];
     C b0 = x[1] + x[3], b1 = x[1] - x[3];
     C wb1 = imul((R)SIGN, b1);
@@ -216,7 +209,35 @@ __device__ __forceinline__ void small_dft(C* x, int r) {
     x[1] = a1 + wb1;
     x[2] = a0 - b0;
     x[3] = a1 - wb1;
+  } else {
+    // radix 8: length-4 DFTs of the even and the odd samples, combined with
+    // w^u, w = e^{SIGN 2 pi i / 8} = (1 + SIGN i) / sqrt 2
+    const C a0 = x[0] + x[4], a1 = x[0] - x[4], a2 = x[2] + x[6], a3 = x[2] - x[6];
+    const C e0 = a0 + a2, e2 = a0 - a2;
+    const C e1 = a1 + imul((R)SIGN, a3), e3 = a1 - imul((R)SIGN, a3);
+    const C b0 = x[1] + x[5], b1 = x[1] - x[5], b2 = x[3] + x[7], b3 = x[3] - x[7];
+    const C o0 = b0 + b2;
+    const C p2 = b0 - b2;
+    const C p1 = b1 + imul((R)SIGN, b3), p3 = b1 - imul((R)SIGN, b3);
+    const R h = (R)0.70710678118654752440084436210484904;
+    const C o1 = mk(h * (p1.x - (R)SIGN * p1.y), h * (p1.y + (R)SIGN * p1.x));    // p1 w
+    const C o2 = imul((R)SIGN, p2);                                               // p2 w^2
+    const C o3 = mk(h * (-p3.x - (R)SIGN * p3.y), h * (-p3.y + (R)SIGN * p3.x));  // p3 w^3
+    x[0] = e0 + o0;
+    x[4] = e0 - o0;
+    x[1] = e1 + o1;
+    x[5] = e1 - o1;
+    x[2] = e2 + o2;
+    x[6] = e2 - o2;
+    x[3] = e3 + o3;
+    x[7] = e3 - o3;
   }
+}
+template <int SIGN, typename C, typename R>
+__device__ __forceinline__ void small_dft(C* x, int r) {
+  if (r == 2) small_dft_ct<SIGN, 2, C, R>(x);
+  else if (r == 3) small_dft_ct<SIGN, 3, C, R>(x);
+  else small_dft_ct<SIGN, 4, C, R>(x);
 }
 
 // Line l of a batch starts at (l / g) * (n g) + (l % g) with element stride g
@@ -288,171 +309,6 @@ __device__ void fft_dit(typename cpx<R>::T* buf, int nlines, int g, const FftPla
       for (int u = 0; u < r; ++u) base[(i0 + u * m) * g] = x[u];
     }
     __syncthreads();
-  }
-}
-
-
-// ---------------------------------------------------------------------------
-// Compile-time FFT plans and stages: the same in-place DIF/DIT passes with
-// the length, the radix of every pass and the line layout fixed at compile
-// time, so that index arithmetic reduces to constant multiplies and shifts.
-// Plan of n = 8^a 4^b 2^c 3^d: radices 8, ..., 8, 4, ..., 4, 2, ..., 2, 3, ..., 3
-// (radix 8 first: fewest passes, hence fewest barriers and shared-memory
-// round trips per transform).
-// ---------------------------------------------------------------------------
-__host__ __device__ constexpr int ct_nst(int n) {
-  int s = 0;
-  while (n % 8 == 0) { n /= 8; ++s; }
-  while (n % 4 == 0) { n /= 4; ++s; }
-  while (n % 2 == 0) { n /= 2; ++s; }
-  while (n % 3 == 0) { n /= 3; ++s; }
-  return s;
-}
-__host__ __device__ constexpr int ct_radix(int n, int st) {
-  int s = 0;
-  while (n % 8 == 0) { if (s == st) return 8; n /= 8; ++s; }
-  while (n % 4 == 0) { if (s == st) return 4; n /= 4; ++s; }
-  while (n % 2 == 0) { if (s == st) return 2; n /= 2; ++s; }
-  while (n % 3 == 0) { if (s == st) return 3; n /= 3; ++s; }
-  return 1;
-}
-// true when the radix-8/4/2/3 plan factors n completely
-__host__ __device__ constexpr bool ct_plan_ok(int n) {
-  if (n < 2) return false;
-  while (n % 8 == 0) n /= 8;
-  while (n % 4 == 0) n /= 4;
-  while (n % 2 == 0) n /= 2;
-  while (n % 3 == 0) n /= 3;
-  return n == 1;
-}
-// sub-length L before pass st of the DIF order
-__host__ __device__ constexpr int ct_len_before(int n, int st) {
-  int L = n;
-  for (int s = 0; s < st; ++s) L /= ct_radix(n, s);
-  return L;
-}
-
-template <int SIGN, int RADIX, typename C, typename R>
-__device__ __forceinline__ void small_dft_ct(C* x) {
-  if constexpr (RADIX == 2) {
-    C a = x[0], b = x[1];
-    x[0] = a + b;
-    x[1] = a - b;
-  } else if constexpr (RADIX == 3) {
-    const R k = (R)SIGN * (R)0.86602540378443864676372317075293618;
-    C s = x[1] + x[2];
-    C d = x[1] - x[2];
-    C t1 = x[0] - (R)0.5 * s;
-    C rot = imul(k, d);
-    x[0] = x[0] + s;
-    x[1] = t1 + rot;
-    x[2] = t1 - rot;
-  } else if constexpr (RADIX == 4) {
-    C a0 = x[0] + x[2], a1 = x[0] - x[2];
-    C b0 = x[1] + x[3], b1 = x[1] - x[3];
-    C wb1 = imul((R)SIGN, b1);
-    x[0] = a0 + b0;
-    x[1] = a1 + wb1;
-    x[2] = a0 - b0;
-    x[3] = a1 - wb1;
-  } else {
-    // radix 8: length-4 DFTs of the even and the odd samples, combined with
-    // w^u, w = e^{SIGN 2 pi i / 8} = (1 + SIGN i) / sqrt 2
-    const C a0 = x[0] + x[4], a1 = x[0] - x[4], a2 = x[2] + x[6], a3 = x[2] - x[6];
-    const C e0 = a0 + a2, e2 = a0 - a2;
-    const C e1 = a1 + imul((R)SIGN, a3), e3 = a1 - imul((R)SIGN, a3);
-    const C b0 = x[1] + x[5], b1 = x[1] - x[5], b2 = x[3] + x[7], b3 = x[3] - x[7];
-    const C o0 = b0 + b2;
-    const C p2 = b0 - b2;
-    const C p1 = b1 + imul((R)SIGN, b3), p3 = b1 - imul((R)SIGN, b3);
-    const R h = (R)0.70710678118654752440084436210484904;
-    const C o1 = mk(h * (p1.x - (R)SIGN * p1.y), h * (p1.y + (R)SIGN * p1.x));    // p1 w
-    const C o2 = imul((R)SIGN, p2);                                               // p2 w^2
-    const C o3 = mk(h * (-p3.x - (R)SIGN * p3.y), h * (-p3.y + (R)SIGN * p3.x));  // p3 w^3
-    x[0] = e0 + o0;
-    x[4] = e0 - o0;
-    x[1] = e1 + o1;
-    x[5] = e1 - o1;
-    x[2] = e2 + o2;
-    x[6] = e2 - o2;
-    x[3] = e3 + o3;
-    x[7] = e3 - o3;
-  }
-}
-
-// one DIF pass (natural order in, digit-reversed out after all passes)
-template <int SIGN, typename R, int N, int ST, int NLINES, int G, bool BF_FASTEST, int NT>
-__device__ __forceinline__ void dif_pass(typename cpx<R>::T* buf, const typename cpx<R>::T* tw) {
-  using C = typename cpx<R>::T;
-  constexpr int r = ct_radix(N, ST);
-  constexpr int L = ct_len_before(N, ST);
-  constexpr int m = L / r;
-  constexpr int nb = N / r;
-  constexpr int tstep = N / L;
-  constexpr int total = NLINES * nb;
-  for (int w = threadIdx.x; w < total; w += NT) {
-    int l, bf;
-    if (BF_FASTEST) { bf = w % nb; l = w / nb; } else { l = w % NLINES; bf = w / NLINES; }
-    C* base = buf + (l / G) * (N * G) + (l % G);
-    const int blk = bf / m, q = bf % m;
-    const int i0 = blk * L + q;
-    C x[r];
-#pragma unroll
-    for (int t = 0; t < r; ++t) x[t] = base[(i0 + t * m) * G];
-    small_dft_ct<SIGN, r, C, R>(x);
-#pragma unroll
-    for (int u = 0; u < r; ++u) {
-      C y = x[u];
-      if (u > 0 && q > 0) y = cmul(y, twiddle<SIGN>(tw, q * u * tstep));
-      base[(i0 + u * m) * G] = y;
-    }
-  }
-  __syncthreads();
-}
-
-// one DIT pass, passes applied in reverse plan order (digit-reversed in, natural out)
-template <int SIGN, typename R, int N, int ST, int NLINES, int G, bool BF_FASTEST, int NT>
-__device__ __forceinline__ void dit_pass(typename cpx<R>::T* buf, const typename cpx<R>::T* tw) {
-  using C = typename cpx<R>::T;
-  constexpr int r = ct_radix(N, ST);
-  constexpr int m = ct_len_before(N, ST + 1);  // sub-length before this pass in DIT order
-  constexpr int L = m * r;
-  constexpr int nb = N / r;
-  constexpr int tstep = N / L;
-  constexpr int total = NLINES * nb;
-  for (int w = threadIdx.x; w < total; w += NT) {
-    int l, bf;
-    if (BF_FASTEST) { bf = w % nb; l = w / nb; } else { l = w % NLINES; bf = w / NLINES; }
-    C* base = buf + (l / G) * (N * G) + (l % G);
-    const int blk = bf / m, q = bf % m;
-    const int i0 = blk * L + q;
-    C x[r];
-#pragma unroll
-    for (int t = 0; t < r; ++t) {
-      C v = base[(i0 + t * m) * G];
-      if (t > 0 && q > 0) v = cmul(v, twiddle<SIGN>(tw, q * t * tstep));
-      x[t] = v;
-    }
-    small_dft_ct<SIGN, r, C, R>(x);
-#pragma unroll
-    for (int u = 0; u < r; ++u) base[(i0 + u * m) * G] = x[u];
-  }
-  __syncthreads();
-}
-
-template <int SIGN, typename R, int N, int NLINES, int G, bool BF_FASTEST, int NT, int ST = 0>
-__device__ __forceinline__ void fft_dif_ct(typename cpx<R>::T* buf, const typename cpx<R>::T* tw) {
-  if constexpr (ST < ct_nst(N)) {
-    dif_pass<SIGN, R, N, ST, NLINES, G, BF_FASTEST, NT>(buf, tw);
-    fft_dif_ct<SIGN, R, N, NLINES, G, BF_FASTEST, NT, ST + 1>(buf, tw);
-  }
-}
-
-template <int SIGN, typename R, int N, int NLINES, int G, bool BF_FASTEST, int NT, int ST = ct_nst(N) - 1>
-__device__ __forceinline__ void fft_dit_ct(typename cpx<R>::T* buf, const typename cpx<R>::T* tw) {
-  if constexpr (ST >= 0) {
-    dit_pass<SIGN, R, N, ST, NLINES, G, BF_FASTEST, NT>(buf, tw);
-    fft_dit_ct<SIGN, R, N, NLINES, G, BF_FASTEST, NT, ST - 1>(buf, tw);
   }
 }
 

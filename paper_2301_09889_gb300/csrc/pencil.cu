@@ -33,15 +33,6 @@ __device__ __forceinline__ double tau_cA(int n) { return (n == 2 ? 2.0 : 1.0) / 
 __device__ __forceinline__ double tau_cB(int n, int N) { return n <= N - 2 ? 1.0 / (2.0 * ((double)n * n - 1.0)) : 0.0; }
 __device__ __forceinline__ double tau_cC(int n, int N) { return n + 2 <= N - 2 ? 1.0 / (4.0 * n * (n + 1)) : 0.0; }
 
-struct TabGlobal {
-  const double* base;  // element (field f, index i) at base[(f * Mh + i) * P]
-  int Mh, P;
-  __device__ double e(int i) const { return base[(size_t)(0 * Mh + i) * P]; }
-  __device__ double h(int i) const { return base[(size_t)(1 * Mh + i) * P]; }
-  __device__ double b(int i) const { return base[(size_t)(2 * Mh + i) * P]; }
-  __device__ double Q(int i) const { return base[(size_t)(3 * Mh + i) * P]; }
-};
-
 struct TabLocal {
   const double *pe, *ph, *pb, *pQ;
   __device__ double e(int i) const { return pe[i]; }
