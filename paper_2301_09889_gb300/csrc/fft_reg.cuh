@@ -89,6 +89,61 @@ __device__ __forceinline__ void dft_pow2(C* x) {
   }
 }
 
+// (a, b) <- (a + w b, a - w b) in six fused operations: a - w b = 2 a - (a + w b)
+template <typename R, typename C>
+__device__ __forceinline__ void bfly(C& a, C& b, C w) {
+  const C s = mk(fma_rn(-w.y, b.y, fma_rn(w.x, b.x, a.x)), fma_rn(w.y, b.x, fma_rn(w.x, b.y, a.y)));
+  b = mk(fma_rn((R)2.0, a.x, -s.x), fma_rn((R)2.0, a.y, -s.y));
+  a = s;
+}
+
+// Length N of x_b w^b, the second half of an inverse line with its twiddles,
+// natural order out; w[i] = w^(2^i).  24, 76 and 208 operations at N = 4, 8
+// and 16, where the products w^b x_b and dft_pow2 take 28, 80 and 228; two,
+// three and four twiddles to load instead of N - 1.
+template <int N, typename R, typename C>
+__device__ __forceinline__ void dft_tw(C* x, const C* w) {
+  if constexpr (N == 2) {
+    bfly<R>(x[0], x[1], w[0]);
+  } else {
+    constexpr int H = N / 2;
+    C e[H], o[H];
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      e[i] = x[2 * i];
+      o[i] = x[2 * i + 1];
+    }
+    dft_tw<H, R>(e, w + 1);
+    dft_tw<H, R>(o, w + 1);
+    // X_k, X_{k+H} = E_k +- w e^{2 pi i k / N} O_k
+    C v = w[0];
+#pragma unroll
+    for (int k = 0; k < (H + 1) / 2; ++k) {
+      if constexpr (N == 8) {
+        if (k == 1) v = rot<+1, R>(w[0], 0.70710678118654752440, 0.70710678118654752440);
+      } else if constexpr (N == 16) {
+        if (k == 1) v = rot<+1, R>(w[0], 0.92387953251128675613, 0.38268343236508977173);
+        if (k == 2) v = rot<+1, R>(w[0], 0.70710678118654752440, 0.70710678118654752440);
+        if (k == 3) v = rot<+1, R>(w[0], 0.38268343236508977173, 0.92387953251128675613);
+      }
+      bfly<R>(e[k], o[k], v);
+      if (H > 1) bfly<R>(e[k + H / 2], o[k + H / 2], imul((R)1.0, v));
+    }
+#pragma unroll
+    for (int k = 0; k < H; ++k) {
+      x[k] = e[k];
+      x[k + H] = o[k];
+    }
+  }
+}
+// the twiddles of dft_tw: entries 1, 2, 4, ... of a table column
+template <int N, int A, typename C>
+__device__ __forceinline__ void load_tw(C* w, const C* tab) {
+#pragma unroll
+  for (int i = 0; (1 << i) < N; ++i) w[i] = tab[(1 << i) * A];
+}
+constexpr int log2i(int n) { return n <= 1 ? 0 : 1 + log2i(n / 2); }
+
 // length 1, 3 or 9; z(n) says which of its inputs are known to be zero
 template <int SIGN, int N, typename R, typename C, class Z>
 __device__ __forceinline__ void dft_pow3(C* x, Z&& zero) {

@@ -88,10 +88,11 @@ __global__ void __launch_bounds__(z_threads<R>(MZ)) zpass_inverse_kernel(PlaneAr
     const int c = w % CT, ka = w / CT, g = c0 + c;
     if (g >= cols) continue;
     C x[B];
-    x[0] = T[ka * CT + c];
+    C tw[log2i(B)];
+    load_tw<B, A>(tw, a.tw_mz + ka);
 #pragma unroll
-    for (int s = 1; s < B; ++s) x[s] = cmul(T[(s * A + ka) * CT + c], a.tw_mz[s * A + ka]);
-    dft_pow2<+1, B, R>(x);
+    for (int s = 0; s < B; ++s) x[s] = T[(s * A + ka) * CT + c];
+    dft_tw<B, R>(x, tw);
     C* dst = yb + (size_t)(g / nxh) * MZ * nxh + g % nxh;
 #pragma unroll
     for (int s = 0; s < B; ++s) dst[(size_t)(ka + A * s) * nxh] = x[s];
@@ -149,18 +150,16 @@ __global__ void __launch_bounds__(NT, x_ctas<R>(MX)) xpass_kernel(PlaneArgs<R> a
     for (int w = threadIdx.x; w < NPR * A; w += NT) {
       const int ka = w % A, pp = w / A;
       if (g0 + pp >= npairs) continue;
-      C t[B];
-#pragma unroll
-      for (int s = 1; s < B; ++s) t[s] = a.tw_x[s * A + ka];
+      C tw[log2i(B)];
+      load_tw<B, A>(tw, a.tw_x + ka);
       C* slot = X + pp * LS + ka;
       constexpr int FS = NPR * LS;
       C v[6][B];
 #pragma unroll
       for (int f = 0; f < 6; ++f) {
-        v[f][0] = slot[f * FS];
 #pragma unroll
-        for (int s = 1; s < B; ++s) v[f][s] = cmul(slot[f * FS + s * A1], t[s]);
-        x_dft<+1, B, R>(v[f]);
+        for (int s = 0; s < B; ++s) v[f][s] = slot[f * FS + s * A1];
+        dft_tw<B, R>(v[f], tw);
       }
       C h[3][B];
 #pragma unroll
@@ -175,7 +174,7 @@ __global__ void __launch_bounds__(NT, x_ctas<R>(MX)) xpass_kernel(PlaneArgs<R> a
         x_dft<-1, B, R>(h[f]);
         slot[f * FS] = h[f][0];
 #pragma unroll
-        for (int s = 1; s < B; ++s) slot[f * FS + s * A1] = cmul(h[f][s], cconj(t[s]));
+        for (int s = 1; s < B; ++s) slot[f * FS + s * A1] = cmul(h[f][s], cconj(a.tw_x[s * A + ka]));
       }
     }
   } else {
@@ -185,11 +184,11 @@ __global__ void __launch_bounds__(NT, x_ctas<R>(MX)) xpass_kernel(PlaneArgs<R> a
     for (int w = threadIdx.x; w < 6 * NPR * A; w += NT) {
       const int ka = w % A;
       C* slot = X + (w / A) * LS + ka;
-      C v[B];
-      v[0] = slot[0];
+      C v[B], tw[log2i(B)];
+      load_tw<B, A>(tw, a.tw_x + ka);
 #pragma unroll
-      for (int s = 1; s < B; ++s) v[s] = cmul(slot[s * A1], a.tw_x[s * A + ka]);
-      dft_pow2<+1, B, R>(v);
+      for (int s = 0; s < B; ++s) v[s] = slot[s * A1];
+      dft_tw<B, R>(v, tw);
 #pragma unroll
       for (int s = 0; s < B; ++s) slot[s * A1] = v[s];
     }

@@ -196,11 +196,11 @@ __global__ void __launch_bounds__(kPairNT) plane16_pair_kernel(PlaneArgs<R> a) {
   cluster.sync();  // also: both CTAs are running before either writes to the other
   if (tid < 144) {
     const int c = tid % 24, ka = tid / 24;
+    const C w[2] = {tw[ka], tw[2 * ka]};
     C x[4];
-    x[0] = T[c * kT6 + ka];
 #pragma unroll
-    for (int s = 1; s < 4; ++s) x[s] = cmul(T[c * kT6 + s * kA1 + ka], tw[s * ka]);
-    small_dft_ct<+1, 4, C, R>(x);
+    for (int s = 0; s < 4; ++s) x[s] = T[c * kT6 + s * kA1 + ka];
+    dft_tw<4, R>(x, w);
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
       const int z = ka + 6 * s, m = z / 2;
@@ -238,11 +238,11 @@ __global__ void __launch_bounds__(kPairNT) plane16_pair_kernel(PlaneArgs<R> a) {
   if (tid < 216) {
     const int ka = tid % 6;
     C* L = X + (tid / 6) * kT6 + ka;
+    const C w[2] = {tw[ka], tw[2 * ka]};
     C x[4];
-    x[0] = L[0];
 #pragma unroll
-    for (int s = 1; s < 4; ++s) x[s] = cmul(L[s * kA1], tw[s * ka]);
-    small_dft_ct<+1, 4, C, R>(x);
+    for (int s = 0; s < 4; ++s) x[s] = L[s * kA1];
+    dft_tw<4, R>(x, w);
 #pragma unroll
     for (int s = 0; s < 4; ++s) L[s * kA1] = x[s];
   }

@@ -1,6 +1,6 @@
 // The no-slip implicit solves of one (mode, class, component, equation) spread
 // over a group of kLanes lanes, for handles with too few modes to fill the GPU
-// with one thread per system (one environment of up to 255 modes).
+// with one thread per system (fewer than 768 in a batch).
 //
 // Lane q of the group holds the block of coefficient indices
 //   i = MH - 1 - q K - k,  k = 0 .. K - 1,  K = ceil(MH / kLanes),

@@ -36,13 +36,13 @@
 // are the two warps of a CTA: each publishes the sums of its parity and both
 // solve the same closure.
 //
-// What bounds it: the FP64 pipe, 29 operations per coefficient and (mode,
-// component), of which two convert FP32 right-hand sides.  A warp-wide FP64
+// What bounds it: the FP64 pipe, 27 operations per coefficient and (mode,
+// component), FP32 right-hand sides apart.  A warp-wide FP64
 // operation takes the same 64 to 76 cycles of its sub-partition whatever the
 // dependences, so what counts is that every sub-partition always has a warp
 // whose operands are there: the coefficient array of a thread lives in a
 // column of shared memory (M doubles; up to 24 warps per SM at 65 nodes,
-// where arrays in registers left ten), loads run two rows ahead, the loops
+// where arrays in registers left ten), loads run three or five rows ahead, the loops
 // stay rolled, and the two equations are CTAs of their own.
 #pragma once
 
