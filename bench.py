@@ -163,19 +163,19 @@ def kernel_bytes(nx: int, ny: int, nz: int, batch: int, node_bytes: int) -> dict
 
 
 def implicit_half_fp64_flops(nx: int, ny: int, nz: int, batch: int, mixed: bool = False) -> float:
-    """Algorithmic FP64 FLOPs of one launch of the implicit half of a stage
-    (right-hand sides, tau solves, influence correction), counting a fused
-    multiply-add as 2.  Per Chebyshev coefficient of one class and real
-    component: omega_y right-hand side 12, tau solve 13, update 2; v wall sums
-    4, derivative walk and right-hand side 21, two tau solves 26, influence
-    sum 3, update 4: 85 per coefficient, (N+1) coefficients of both parities
-    over the two classes and 2 components: 170 (N+1) per mode, for every mode
-    but the Nyquist row.  In the mixed path the nonlinear-term part of the
-    right-hand sides (h_g, t, Dt, h_v and dt (gamma h + zeta h')) is FP32:
-    8 of the omega_y and 12 of the v FLOPs, leaving 65 FP64 per coefficient,
-    130 (N+1) per mode."""
+    """FP64 FLOPs of the implicit half of one stage (right-hand sides, tau
+    solves, influence correction) in the library's folded form, counting a
+    fused multiply-add as 2.  Per Chebyshev coefficient of one class and real
+    component, omega_y: wall sum 1, right-hand side 2, elimination 7, weighted
+    sum 2, back substitution 2, update 2; v: wall sum 1, right-hand side 2, phi
+    elimination 9, sum 2, back substitution 2, v elimination 7, sum 2, back
+    substitution 2, shift 2, influence sum 2, update 2: 49 per coefficient,
+    (N+1) coefficients of both parities over 2 components: 98 (N+1) per mode,
+    for every mode but the Nyquist row.  In all-FP64 handles the nonlinear part
+    of the right-hand sides (h_g, t, Dt, h_v and dt (gamma h + zeta h')) adds 16
+    per coefficient, 130 (N+1) per mode."""
     modes = batch * (nx // 2) * (nz - 1)
-    return (130.0 if mixed else 170.0) * ny * modes
+    return (98.0 if mixed else 130.0) * ny * modes
 
 
 def slowest_rank_ms(total_ms: float, dist, device: str = "cuda") -> float:
@@ -209,12 +209,10 @@ def measured_peaks() -> dict:
 # the roofline kernel, from one ncu capture of the same workload (summaries
 # under profiles/); absent where no capture of the current kernel exists
 TRAFFIC_BYTES = {
-    ("minimal_batch256_mixed", "stage_post"): (152.163072 + 42.973952) * 1e6,
-    # the three passes of one FP64 64x64-mode stage (the scratch stays in L2)
-    ("larger_fp64", "nonlinear_plane"): (12.597248 + 19.201792 + 9.604352) * 1e6,
-    # the three passes of one FP64 256x256-mode stage (z inverse + x pass + z forward)
-    ("large550_fp64", "nonlinear_plane"): (604.911872 + 852.392448 + 910.863872 + 413.775360 + 455.520000
-                                           + 259.116544) * 1e6,
+    # analysis and solves of one stage
+    ("minimal_batch256_mixed", "stage_post"): (52.6 + 222.3) * 1e6,
+    # the three passes of one FP64 64x64-mode stage (the node values stay in L2)
+    ("larger_fp64", "nonlinear_plane"): (12.6 + 19.2 + 9.6) * 1e6,
 }
 
 # FP64 FMA rate: 152 SMs x 2 FP64 FMA/clk/SM x 2 FLOP x 2.07 GHz; an FMA-chain probe

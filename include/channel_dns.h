@@ -101,21 +101,25 @@ typedef struct ch_info {
     double nu, u_tau, tau_ref;
     size_t state_bytes;      /* bytes of one environment's serialised state                */
     size_t device_bytes;     /* device memory held by the handle                           */
-    int plane_cluster;       /* CTAs of a thread-block cluster cooperating on one y-plane of
-                                the nonlinear term; 0: no portable cluster holds the plane
-                                (planes of 256 x 256 modes), the term runs in three passes
-                                through a global scratch array (z inverse, x transforms and
-                                products, z forward)                                     */
+    int plane_cluster;       /* CTAs of a thread-block cluster that hold one y-plane of the
+                                nonlinear term where it runs on clusters; where it runs in
+                                three passes (z inverse, x transforms and products, z
+                                forward) the size such a cluster would have; 0 for planes
+                                of 256 x 256 modes and FP64 planes of 64 x 64 and
+                                128 x 128                                                */
     int launches_per_step;   /* kernels launched by one env_step                            */
     int post_batched;        /* 1: the implicit half of a stage runs one thread per (mode,
-                                class, component); 0: eight threads per mode on a tile  */
-    int ppc_pre, ppc_post;   /* Fourier modes per CTA of the explicit and implicit halves */
+                                class, component, equation); 0: 128 threads per mode on a
+                                tile (no-slip top; a free-slip top has the first form)   */
+    int ppc_pre, ppc_post;   /* tile widths: ppc_post Fourier modes per CTA of the implicit
+                                half where post_batched is 0; the other forms have one
+                                shape, and the values set are only reported              */
     int tuned;               /* 1 if the tile shapes were chosen by timing (autotune)    */
     double tune_ms;          /* host time env_create spent timing candidates            */
     int plane_team;          /* 1: planes of 16 x 16 modes in a batch of at least four
-                                planes per SM; each padded 24 x 24 plane is owned by a team
-                                of 96 threads that transforms its 24-point lines in
-                                registers (plane_cluster is then 1); 0 otherwise          */
+                                planes per SM: two padded 24 x 24 planes per CTA, one line
+                                per thread in registers (plane_cluster is then 1);
+                                0 otherwise                                               */
 } ch_info_t;
 
 typedef struct ch_env ch_env_t;
@@ -210,12 +214,14 @@ int env_profile_read(ch_env_t* env, int cls, double* total_ms, int* launches);
 
 int env_info(const ch_env_t* env, ch_info_t* info);
 
-/* Pin the tile shapes of the two stage kernels (overriding the autotuner):
- * ppc_pre in {1, 2, 4, 8} modes per 128-thread CTA of the explicit half;
- * post_batched 0 with ppc_post in 1..8 (8 threads per mode) or 1 with
- * ppc_post in {1, 2, 4, 8, 16} (4 threads per mode).  Every shape gives
- * bit-identical results.  Waits for the handle's stream.  No counterpart in
- * the paper (a tuning control of this implementation).
+/* Pin the form and the tile shape of the implicit half (overriding the size
+ * rule and the autotuner): post_batched 0 with ppc_post in 1..8 modes per CTA
+ * or 1 with ppc_post in {1, 2, 4, 8, 16}; ppc_pre in {1, 2, 4, 8}.  ppc_pre,
+ * and ppc_post of form 1, are checked and reported but name one shape each;
+ * under a free-slip top both forms are one.  Every width of a form gives
+ * bit-identical results, the two forms agree to rounding.  Waits for the
+ * handle's stream.  No counterpart in the paper (a tuning control of this
+ * implementation).
  * Errors: CH_ERR_ARG (bad handle or shape, or a shape whose shared memory
  * exceeds the device limit), CH_ERR_CUDA. */
 int env_set_tiles(ch_env_t* env, int ppc_pre, int ppc_post, int post_batched);
@@ -370,8 +376,8 @@ int srv_destroy(ch_server_t* s);
  *       at each node, of u, v, w, omega_x, omega_y, omega_z;
  *   d_h [B][3][ny][nz][nx/2] complex: Fourier coefficients of the kept modes
  *       of H = u x omega evaluated on the 3nx/2 x 3nz/2 grid.
- * Uses the handle's twiddle tables (and, for FP64 handles of 256 x 256
- * modes, their three-pass scratch array); allocates nothing.
+ * Uses the handle's twiddle tables (and, in FP64 handles whose nonlinear term
+ * runs in passes, their array of node values as scratch); allocates nothing.
  * CH_ERR_UNSUPPORTED for mixed-precision handles whose FP64 padded plane
  * does not fit a cluster's shared memory (256 x 256 modes). */
 int ch_nonlinear(ch_env_t* env, const double* d_q, double* d_h);
