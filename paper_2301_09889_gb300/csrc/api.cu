@@ -433,26 +433,28 @@ int build_tables(ch_env* env) {
   // free-slip top: sum Q, sum n^2 Q per parity; A, B of vh per parity
   std::vector<double> helm_top((size_t)3 * 2 * 2 * P, 0.0), vh_top((size_t)3 * 2 * 2 * P, 0.0);
   std::vector<double> mean_top((size_t)3 * 4, 0.0);
-  // the folded tables of the per-thread solves, [..][eA, eB, eC, h, b, W (, E1 (, W2))][Mh][P];
+  // the folded tables of the per-thread solves, [..][tile][Mh + 1][eA, eB, eC, h, b, W (, E1 (, W2))][16];
   // e1 > 0 adds E1 = e1 e (the Helmholtz tables, e1 = 1 + alpha/beta of the
   // stage) and under a free-slip top the weights W2 of sum n^2 P
   const int htabs = top ? 8 : 7;
-  std::vector<double> helm_f((size_t)3 * 2 * htabs * Mh * P, 0.0);
-  std::vector<double> pois_f((size_t)2 * 6 * Mh * P, 0.0);
-  auto put_f = [&](std::vector<double>& tab, size_t base, const Factor& F, int M, int pp, int sig, double e1) {
+  const size_t rows = (size_t)((P + 15) / 16) * (Mh + 1) * 16;
+  std::vector<double> helm_f((size_t)3 * 2 * htabs * rows, 0.0);
+  std::vector<double> pois_f((size_t)2 * 6 * rows, 0.0);
+  auto put_f = [&](std::vector<double>& tab, size_t block, int tabs, const Factor& F, int M, int pp, int sig, double e1) {
     double w = 1.0, w2 = 0.0;  // W_{M-1}
     for (int i = M - 1; i >= 1; --i) {
       const int n = 2 * i + sig;
+      double* row = tab.data() + block * tabs * rows + ((size_t)(pp / 16) * (Mh + 1) + i) * tabs * 16 + pp % 16;
       if (i < M - 1) w = 1.0 + F.b[i + 1] * w;
       if (top) w2 = (double)n * n + (i < M - 1 ? F.b[i + 1] * w2 : 0.0);
-      tab[base + ((size_t)0 * Mh + i) * P + pp] = F.e[i] * cA(n);
-      tab[base + ((size_t)1 * Mh + i) * P + pp] = F.e[i] * cB(n, N);
-      tab[base + ((size_t)2 * Mh + i) * P + pp] = F.e[i] * cC(n, N);
-      tab[base + ((size_t)3 * Mh + i) * P + pp] = F.h[i];
-      tab[base + ((size_t)4 * Mh + i) * P + pp] = F.b[i];
-      tab[base + ((size_t)5 * Mh + i) * P + pp] = w;
-      if (e1 > 0.0) tab[base + ((size_t)6 * Mh + i) * P + pp] = e1 * F.e[i];
-      if (e1 > 0.0 && top) tab[base + ((size_t)7 * Mh + i) * P + pp] = w2;
+      row[0 * 16] = F.e[i] * cA(n);
+      row[1 * 16] = F.e[i] * cB(n, N);
+      row[2 * 16] = F.e[i] * cC(n, N);
+      row[3 * 16] = F.h[i];
+      row[4 * 16] = F.b[i];
+      row[5 * 16] = w;
+      if (e1 > 0.0) row[6 * 16] = e1 * F.e[i];
+      if (e1 > 0.0 && top) row[7 * 16] = w2;
     }
   };
   auto put = [&](std::vector<double>& tab, size_t base, const Factor& F, int M, int pp) {
@@ -470,7 +472,7 @@ int build_tables(ch_env* env) {
       const int M = (N - sig) / 2 + 1;
       const Factor Fp = host_factor(N, sig, k2);
       if (!top) put(pois, (size_t)sig * 4 * Mh * P, Fp, M, pp);
-      put_f(pois_f, (size_t)sig * 6 * Mh * P, Fp, M, pp, sig, 0.0);
+      put_f(pois_f, sig, 6, Fp, M, pp, sig, 0.0);
       pois_isq[(size_t)sig * P + pp] = Fp.isq;
       for (int k = 0; k < 3; ++k) {
         const double ibdn = 1.0 / (rk_beta(k) * p.dt * env->nu);
@@ -482,7 +484,7 @@ int build_tables(ch_env* env) {
         Factor Fs = Fh;
         for (double& e : Fs.e) e *= -ibdn;
         if (!top) put(helm, slot * 4 * Mh * P, Fs, M, pp);
-        put_f(helm_f, slot * htabs * Mh * P, Fs, M, pp, sig, 1.0 + rk_alpha(k) / rk_beta(k));
+        put_f(helm_f, slot, htabs, Fs, M, pp, sig, 1.0 + rk_alpha(k) / rk_beta(k));
         helm_isq[slot * P + pp] = Fh.isq;
         {
           double sq = 0.0, sq2 = 0.0;
@@ -1033,7 +1035,7 @@ size_t env_footprint(const ch_params_t* p) {
   node_strides(&g);
   const size_t state = B * (4 * ny * P * 16 + 4 * ny * 8 + g.qb * (p->precision == 1 ? 8 : 16) + 3 * P * 16 + 8 +
                             (size_t)p->nz * p->nx * 8 + (2 * (size_t)p->nz * p->nx + 2) * 8);
-  const size_t folded = (3 * 2 * (p->top_bc ? 8 : 7) * Mh * P + 2 * 6 * Mh * P) * 8;
+  const size_t folded = (3 * 2 * (p->top_bc ? 8 : 7) + 2 * 6) * (Mh + 1) * ((P + 15) / 16 * 16) * 8;
   const size_t scan = p->top_bc ? 0 : (3 * 2 * 4 + 2 * 4) * Mh * P;
   const size_t tables = (scan + 3 * 2 * P + 2 * P + 3 * 2 * Mh * P + 3 * 2 * P +
                          3 * Mh + 3 + 3 * ny + ny + 2 * 3 * 2 * 2 * P) * 8 + ny * ny * 12 + (nxh + p->nz) * 8 +

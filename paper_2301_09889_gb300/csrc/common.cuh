@@ -367,8 +367,10 @@ struct TauTables {
   // W_i = 1 + b_{i+1} W_{i+1}: sum_i P_i = sum_i W_i a_i) and, for the stage's
   // Helmholtz operator, E1 = (1 + alpha/beta) e and under a free-slip top W2
   // (W2_{M-1} = n^2, W2_i = n_i^2 + b_{i+1} W2_{i+1}: sum n^2 P = sum W2_i a_i)
-  const double* helm_f;    // [3][2][7 or 8][Mh][P] eA, eB, eC, h, b, W, E1 (, W2) per stage, parity
-  const double* pois_f;    // [2][6][Mh][P]     eA, eB, eC, h, b, W
+  // eA, eB, eC, h, b, W, E1 (, W2) per stage, parity and eA, eB, eC, h, b, W per parity, the entries of a
+  // row side by side for a tile of sixteen modes: [3][2] and [2] of [tile][Mh + 1][7 or 8, 6][16]
+  const double* helm_f;
+  const double* pois_f;
   const double* n2;        // [ny] n^2
   const double* n1;        // [ny] 2 (n + 1)
   const double* wint;      // [ny] int T_n dy = 2 / (1 - n^2) of the even n, 0 of the odd

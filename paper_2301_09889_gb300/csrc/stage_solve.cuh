@@ -101,12 +101,22 @@ __device__ __forceinline__ void sweep_up(int first, int M, Load&& load, Step&& s
                 [&](int i, const auto& v) { step(M - 1 + first - i, v); });
 }
 
-// one row's table entries
+// one row's table entries, from tables of TABS entries a row: one address serves
+// all of them and, with the row stride fixed, the rows of an unrolled block (the
+// solves issue three other instructions per FP64 operation: as [entry][row][mode]
+// arrays the tables took six addresses a row; 256 minimal mixed channels 1090
+// us per step then and 1064 so)
+template <int TABS> __device__ __forceinline__ const double* tab_of(const double* T, int block, const Grid& g, int Mh, int p) {
+  return T + ((size_t)(block * ((g.P + 15) / 16) + p / 16) * (Mh + 1)) * (TABS * 16) + p % 16;
+}
+template <int TABS> __device__ __forceinline__ double tab(const double* __restrict__ T, int row, int entry) {
+  return __ldg(T + (ptrdiff_t)row * (TABS * 16) + entry * 16);
+}
 struct TabRow {
   double eA, eB, eC, h, W;
 };
-__device__ __forceinline__ TabRow tab_row(const double* __restrict__ T, size_t MP, size_t o) {
-  return TabRow{__ldg(T + o), __ldg(T + MP + o), __ldg(T + 2 * MP + o), __ldg(T + 3 * MP + o), __ldg(T + 5 * MP + o)};
+template <int TABS> __device__ __forceinline__ TabRow tab_row(const double* __restrict__ T, int row) {
+  return TabRow{tab<TABS>(T, row, 0), tab<TABS>(T, row, 1), tab<TABS>(T, row, 2), tab<TABS>(T, row, 3), tab<TABS>(T, row, 5)};
 }
 
 // what a thread's sweep down leaves for the closure
@@ -126,7 +136,8 @@ __device__ __forceinline__ Wall omega_down(double* f, const Grid& g, const Penci
                                            const StageCoef& sc, int b, int p, int r, int sig, const double* __restrict__ T,
                                            const RN* __restrict__ hc) {
   constexpr int NT = 64;
-  const size_t P = g.P, MP = (size_t)t.tau.Mh * P;
+  constexpr int TABS = solve_tabs<TOP>();
+  const size_t P = g.P;
   const int ny = g.ny, M = (g.N - sig) / 2 + 1, row = p / g.nxh, ix = p % g.nxh;
   const double cc1 = 1.0 + sc.cc;
   const double* __restrict__ n2 = t.tau.n2;
@@ -151,13 +162,13 @@ __device__ __forceinline__ Wall omega_down(double* f, const Grid& g, const Penci
       M - 1, 0,
       [&](int i) {
         In v;
-        const size_t n = 2 * i + sig, o = (size_t)min(i + 1, M - 1) * P;  // row i + 1 of the elimination
+        const size_t n = 2 * i + sig;
         v.x = G[n * hP];
         v.hx = __ldg(hx + n * hS);
         v.hz = __ldg(hz + n * hS);
         v.hp = HG[n * hP];
-        v.tb = tab_row(T, MP, o);
-        if (TOP) v.W2 = __ldg(T + 7 * MP + o);
+        v.tb = tab_row<TABS>(T, i + 1);  // row i + 1 of the elimination (row M is not used)
+        if (TOP) v.W2 = tab<TABS>(T, i + 1, 7);
         return v;
       },
       [&](int i, const In& v) {
@@ -184,11 +195,11 @@ __device__ __forceinline__ Wall omega_down(double* f, const Grid& g, const Penci
 // down, for the increment.  X: coefficients, XP: previous plane means of H,
 // hm: its new ones (2 qj apart).
 template <typename RN, int TOP>
-__device__ __forceinline__ Wall mean_down(double* f, const DevTables& t, const StageCoef& sc, int N, size_t P, size_t qj, int sig,
+__device__ __forceinline__ Wall mean_down(double* f, const DevTables& t, const StageCoef& sc, int N, size_t qj, int sig,
                                        const double* __restrict__ T, const double* X, double* XP,
                                        const RN* __restrict__ hm) {
   constexpr int NT = 64;
-  const size_t MP = (size_t)t.tau.Mh * P;
+  constexpr int TABS = solve_tabs<TOP>();
   const int M = (N - sig) / 2 + 1;
   const double bdn = sc.beta * sc.dt * sc.nu;
   Wall w;
@@ -204,16 +215,15 @@ __device__ __forceinline__ Wall mean_down(double* f, const DevTables& t, const S
       [&](int i) {
         In v;
         const int n = 2 * i + sig;
-        const size_t o = (size_t)min(i + 1, M - 1) * P;
         v.x = X[n];
         v.hp = XP[n];
         v.h = __ldg(hm + 2 * qj * n);
         v.wi = __ldg(t.tau.wint + n);
-        v.tb = tab_row(T, MP, o);
-        v.E1 = __ldg(T + 6 * MP + o);
+        v.tb = tab_row<TABS>(T, i + 1);
+        v.E1 = tab<TABS>(T, i + 1, 6);
         if (TOP) {
           v.n2 = __ldg(t.tau.n2 + n);
-          v.W2 = __ldg(T + 7 * MP + o);
+          v.W2 = tab<TABS>(T, i + 1, 7);
         }
         return v;
       },
@@ -238,7 +248,7 @@ __device__ __forceinline__ Wall mean_down(double* f, const DevTables& t, const S
   if (TOP && sig == 0) {
     double fp = 0.0;
     sweep_up<4>(
-        1, M, [&](int i) { return Bw{__ldg(T + 4 * MP + (size_t)i * P), __ldg(t.tau.wint + 2 * i)}; },
+        1, M, [&](int i) { return Bw{tab<TABS>(T, i, 4), __ldg(t.tau.wint + 2 * i)}; },
         [&](int i, const Bw& v) {
           fp = fma(v.b, fp, f[i * NT]);
           w.wp = fma(v.w, fp, w.wp);
@@ -253,12 +263,12 @@ __device__ __forceinline__ void mean_up(double* f, const DevTables& t, const Sta
                                      bool forced, const double* __restrict__ T, double* X, float* X32, double f0,
                                      double fc, double wx) {
   constexpr int NT = 64;
-  const size_t MP = (size_t)t.tau.Mh * P;
+  constexpr int TABS = solve_tabs<TOP>();
   const int M = (N - sig) / 2 + 1;
   double fp = f0, flux = t.tau.wint[0] * f0;
   f[0] = f0;
   sweep_up<4>(
-      1, M, [&](int i) { return Bw{__ldg(T + 4 * MP + (size_t)i * P), __ldg(t.tau.wint + 2 * i)}; },
+      1, M, [&](int i) { return Bw{tab<TABS>(T, i, 4), __ldg(t.tau.wint + 2 * i)}; },
       [&](int i, const Bw& v) {
         fp = fma(v.b, fp, f[i * NT]);
         f[i * NT] = fp;
@@ -283,15 +293,16 @@ __device__ __forceinline__ void solve_omega(double* f, double* xch, const Grid& 
                                             const DevTables& t, const StageCoef& sc, int b, int p, int r, int sig,
                                             bool live, const RN* __restrict__ hc) {
   constexpr int NT = 64;
-  const size_t P = g.P, MP = (size_t)t.tau.Mh * P;
+  constexpr int TABS = solve_tabs<TOP>();
+  const size_t P = g.P;
   const int ny = g.ny, M = (g.N - sig) / 2 + 1;
-  const double* __restrict__ T = t.tau.helm_f + (size_t)(sc.k * 2 + sig) * solve_tabs<TOP>() * MP + p;
+  const double* __restrict__ T = tab_of<TABS>(t.tau.helm_f, sc.k * 2 + sig, g, t.tau.Mh, p);
   double* X = (r == 0 ? pb.UM : pb.WM) + (size_t)b * ny;
   Wall w;
   if (live) {
     if constexpr (MEAN) {
       const RN* hm = hc + 2 * b * g.qb + (r == 0 ? 0 : 4 * g.qf);
-      w = mean_down<RN, TOP>(f, t, sc, g.N, P, g.qj, sig, T, X, (r == 0 ? pb.HXP : pb.HZP) + (size_t)b * ny, hm);
+      w = mean_down<RN, TOP>(f, t, sc, g.N, g.qj, sig, T, X, (r == 0 ? pb.HXP : pb.HZP) + (size_t)b * ny, hm);
     } else {
       w = omega_down<RN, TOP, D>(f, g, pb, t, sc, b, p, r, sig, T, hc);
     }
@@ -347,7 +358,7 @@ __device__ __forceinline__ void solve_omega(double* f, double* xch, const Grid& 
     double b, x;
   };
   sweep_up<2 * D>(
-      1, M, [&](int i) { return Up{__ldg(T + 4 * MP + (size_t)i * P), G[(size_t)i * 2 * hP]}; },
+      1, M, [&](int i) { return Up{tab<TABS>(T, i, 4), G[(size_t)i * 2 * hP]}; },
       [&](int i, const Up& u) {
         fp = fma(u.b, fp, f[i * NT]);
         put(i, fma(-cc, u.x, fp));
@@ -363,8 +374,9 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
   const size_t P = g.P, MP = (size_t)t.tau.Mh * P;
   const int ny = g.ny, N = g.N, M = (N - sig) / 2 + 1, row = p / g.nxh, ix = p % g.nxh;
   const double cc = sc.cc;
-  const double* __restrict__ T = t.tau.helm_f + (size_t)(sc.k * 2 + sig) * solve_tabs<TOP>() * MP + p;
-  const double* __restrict__ TP = t.tau.pois_f + (size_t)sig * kPoisTabs * MP + p;
+  constexpr int TABS = solve_tabs<TOP>();
+  const double* __restrict__ T = tab_of<TABS>(t.tau.helm_f, sc.k * 2 + sig, g, t.tau.Mh, p);
+  const double* __restrict__ TP = tab_of<kPoisTabs>(t.tau.pois_f, sig, g, t.tau.Mh, p);
   const double* __restrict__ n2 = t.tau.n2;
   const size_t hP = 2 * P, base = 2 * ((size_t)b * ny * P + p) + r;
   double* Vp = reinterpret_cast<double*>(pb.V) + base;
@@ -394,11 +406,11 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
       v.hp = HV[n * hP];
       if constexpr (sizeof(RN) == 8) v.fac = __ldg(t.tau.n1 + n);
       else v.fac = (RN)(2 * ((int)n + 1));
-      const size_t no = min((int)n + 1, N), o = (size_t)min(i + 1, M - 1) * P;
+      const size_t no = min((int)n + 1, N);
       v.hx = __ldg(hx + no * hS);
       v.hz = __ldg(hz + no * hS);
-      v.tb = tab_row(T, MP, o);
-      v.E1 = __ldg(T + 6 * MP + o);
+      v.tb = tab_row<TABS>(T, i + 1);
+      v.E1 = tab<TABS>(T, i + 1, 6);
       return v;
     };
     double S0 = 0.0, sum = 0.0, r1 = 0.0, r2 = 0.0, x1 = 0.0, an = 0.0;
@@ -429,7 +441,7 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
     double fp = t.tau.helm_isq[(size_t)(sc.k * 2 + sig) * P + p] * -sum;
     f[0] = fp;
     sweep_up<2 * D>(
-        1, M, [&](int i) { return __ldg(T + 4 * MP + (size_t)i * P); },
+        1, M, [&](int i) { return tab<TABS>(T, i, 4); },
         [&](int i, double bi) {
           fp = fma(bi, fp, f[i * NT]);
           f[i * NT] = fp;
@@ -438,7 +450,7 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
     sum = an = r2 = 0.0;
     r1 = fp;
     sweep_down<D>(
-        M - 1, 1, [&](int j) { return tab_row(TP, MP, (size_t)j * P); },
+        M - 1, 1, [&](int j) { return tab_row<kPoisTabs>(TP, j); },
         [&](int j, const TabRow& tr) {
           const double r0 = f[(j - 1) * NT];
           const double a = fma(-tr.h, an, fma(tr.eC, r2, fma(-tr.eB, r1, tr.eA * r0)));
@@ -468,7 +480,7 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
     sweep_up<D>(
         1, M,
         [&](int i) {
-          return Up{__ldg(TP + 4 * MP + (size_t)i * P), Vp[(size_t)(2 * i + sig) * hP], __ldg(n2 + 2 * i + sig)};
+          return Up{tab<kPoisTabs>(TP, i, 4), Vp[(size_t)(2 * i + sig) * hP], __ldg(n2 + 2 * i + sig)};
         },
         [&](int i, const Up& u) {
           fp = fma(u.b, fp, f[i * NT]);
