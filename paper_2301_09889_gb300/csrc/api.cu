@@ -433,18 +433,18 @@ int build_tables(ch_env* env) {
   // free-slip top: sum Q, sum n^2 Q per parity; A, B of vh per parity
   std::vector<double> helm_top((size_t)3 * 2 * 2 * P, 0.0), vh_top((size_t)3 * 2 * 2 * P, 0.0);
   std::vector<double> mean_top((size_t)3 * 4, 0.0);
-  // the folded tables of the per-thread solves, [..][tile][Mh + 1][eA, eB, eC, h, b, W (, E1 (, W2))][16];
+  // the folded tables of the per-thread solves, [..][tile][rows 1 .. Mh][eA, eB, eC, h, b, W (, E1 (, W2))][16];
   // e1 > 0 adds E1 = e1 e (the Helmholtz tables, e1 = 1 + alpha/beta of the
   // stage) and under a free-slip top the weights W2 of sum n^2 P
   const int htabs = top ? 8 : 7;
-  const size_t rows = (size_t)((P + 15) / 16) * (Mh + 1) * 16;
+  const size_t rows = (size_t)((P + 15) / 16) * Mh * 16;
   std::vector<double> helm_f((size_t)3 * 2 * htabs * rows, 0.0);
   std::vector<double> pois_f((size_t)2 * 6 * rows, 0.0);
   auto put_f = [&](std::vector<double>& tab, size_t block, int tabs, const Factor& F, int M, int pp, int sig, double e1) {
     double w = 1.0, w2 = 0.0;  // W_{M-1}
     for (int i = M - 1; i >= 1; --i) {
       const int n = 2 * i + sig;
-      double* row = tab.data() + block * tabs * rows + ((size_t)(pp / 16) * (Mh + 1) + i) * tabs * 16 + pp % 16;
+      double* row = tab.data() + block * tabs * rows + ((size_t)(pp / 16) * Mh + i - 1) * tabs * 16 + pp % 16;
       if (i < M - 1) w = 1.0 + F.b[i + 1] * w;
       if (top) w2 = (double)n * n + (i < M - 1 ? F.b[i + 1] * w2 : 0.0);
       row[0 * 16] = F.e[i] * cA(n);
@@ -1035,7 +1035,7 @@ size_t env_footprint(const ch_params_t* p) {
   node_strides(&g);
   const size_t state = B * (4 * ny * P * 16 + 4 * ny * 8 + g.qb * (p->precision == 1 ? 8 : 16) + 3 * P * 16 + 8 +
                             (size_t)p->nz * p->nx * 8 + (2 * (size_t)p->nz * p->nx + 2) * 8);
-  const size_t folded = (3 * 2 * (p->top_bc ? 8 : 7) + 2 * 6) * (Mh + 1) * ((P + 15) / 16 * 16) * 8;
+  const size_t folded = (3 * 2 * (p->top_bc ? 8 : 7) + 2 * 6) * Mh * ((P + 15) / 16 * 16) * 8;
   const size_t scan = p->top_bc ? 0 : (3 * 2 * 4 + 2 * 4) * Mh * P;
   const size_t tables = (scan + 3 * 2 * P + 2 * P + 3 * 2 * Mh * P + 3 * 2 * P +
                          3 * Mh + 3 + 3 * ny + ny + 2 * 3 * 2 * 2 * P) * 8 + ny * ny * 12 + (nxh + p->nz) * 8 +

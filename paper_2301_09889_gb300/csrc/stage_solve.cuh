@@ -107,10 +107,10 @@ __device__ __forceinline__ void sweep_up(int first, int M, Load&& load, Step&& s
 // arrays the tables took six addresses a row; 256 minimal mixed channels 1090
 // us per step then and 1064 so)
 template <int TABS> __device__ __forceinline__ const double* tab_of(const double* T, int block, const Grid& g, int Mh, int p) {
-  return T + ((size_t)(block * ((g.P + 15) / 16) + p / 16) * (Mh + 1)) * (TABS * 16) + p % 16;
+  return T + ((size_t)(block * ((g.P + 15) / 16) + p / 16) * Mh) * (TABS * 16) + p % 16;
 }
 template <int TABS> __device__ __forceinline__ double tab(const double* __restrict__ T, int row, int entry) {
-  return __ldg(T + (ptrdiff_t)row * (TABS * 16) + entry * 16);
+  return __ldg(T + (ptrdiff_t)(row - 1) * (TABS * 16) + entry * 16);  // rows 1 .. Mh
 }
 struct TabRow {
   double eA, eB, eC, h, W;
