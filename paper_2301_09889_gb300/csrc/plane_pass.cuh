@@ -99,11 +99,6 @@ __global__ void __launch_bounds__(z_threads<R>(MZ)) zpass_inverse_kernel(PlaneAr
   }
 }
 
-template <int SIGN, int B, typename R> __device__ __forceinline__ void x_dft(typename cpx<R>::T* v) {
-  if constexpr (B <= 4) small_dft_ct<SIGN, B, typename cpx<R>::T, R>(v);
-  else dft_pow2<SIGN, B, R>(v);
-}
-
 template <typename R, int MX, int NPR, int NT>
 __global__ void __launch_bounds__(NT, x_ctas<R>(MX)) xpass_kernel(PlaneArgs<R> a) {
   using C = typename cpx<R>::T;
@@ -171,7 +166,7 @@ __global__ void __launch_bounds__(NT, x_ctas<R>(MX)) xpass_kernel(PlaneArgs<R> a
       }
 #pragma unroll
       for (int f = 0; f < 3; ++f) {
-        x_dft<-1, B, R>(h[f]);
+        dft_pow2<-1, B, R>(h[f]);
         slot[f * FS] = h[f][0];
 #pragma unroll
         for (int s = 1; s < B; ++s) slot[f * FS + s * A1] = cmul(h[f][s], cconj(a.tw_x[s * A + ka]));
