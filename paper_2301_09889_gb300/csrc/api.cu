@@ -954,7 +954,7 @@ int autotune_tiles(ch_env* env, int smem_max) {
   float best = 0.f;
   bool have = false;
   // widths of the form the size rule chose: the per-tile and batched forms of
-  // the no-slip solves sum in different orders (four-lane scans against one
+  // the no-slip solves sum in different orders (sixteen-lane scans against one
   // thread per system), so timing never switches between them
   for (int ppc = 8; ppc >= 1; --ppc) {
     if (env->post_batched || env->prm.top_bc) break;  // the two-launch form has one shape

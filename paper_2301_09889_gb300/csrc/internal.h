@@ -70,7 +70,7 @@ cudaError_t launch_stage_pre(const Grid& g, int B, const PencilBufs& pb, const D
                              typename cpx<RN>::T* q, cudaStream_t st);
 // batched (and every handle under a free-slip top): the analysis of H over its
 // nodal values h in place, then one thread per (mode, class, component,
-// equation); otherwise four lanes per system on a shared-memory tile of ppc modes
+// equation); otherwise sixteen lanes per system on a shared-memory tile of ppc modes
 template <typename RN>
 cudaError_t launch_stage_post(const Grid& g, int B, const PencilBufs& pb, const DevTables& t,
                               typename cpx<RN>::T* h, const StageCoef& sc, int ppc, bool batched,
