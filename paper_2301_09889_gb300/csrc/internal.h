@@ -24,7 +24,7 @@ struct PencilBufs {
   double2 *V, *G;               // [B][ny][P]
   double2 *HVP, *HGP;           // [B][ny][P] complex in the node precision (FP32 pairs in mixed mode)
   float2 *V32, *G32;            // [B][ny][P] V and G rounded to FP32 (mixed precision): what stage_pre reads;
-                                // mode 0 of G32 holds the mean flow (W, U)
+                                // mode 0 of G32 holds the mean flow (W, U), that of V32 (DW, DU)
   double *UM, *WM, *HXP, *HZP;  // [B][ny]
   // node values of u, v, w, ox, oy, oz in the node precision, then those of H (or
   // its coefficients) over the first three: strides Grid.qf, qj, qb.  Where the

@@ -400,13 +400,21 @@ __global__ void __launch_bounds__(kTauNT) tau_helmholtz_kernel(int ny, int M, co
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-// the FP32 copies of a state that came from the host
+// the FP32 copies of a state that came from the host; mode 0: the mean flow
+// (W, U) and its derivatives, summed in FP64 and rounded once
 __global__ void round_state_kernel(Grid g, int b, PencilBufs pb) {
   const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (i >= (long)g.ny * g.P) return;
   const int n = (int)(i / g.P), p = (int)(i % g.P);
   const size_t o = (size_t)b * g.ny * g.P + i;
-  const double2 v = pb.V[o], w = p == 0 ? mk(pb.WM[(size_t)b * g.ny + n], pb.UM[(size_t)b * g.ny + n]) : pb.G[o];
+  double2 v = pb.V[o], w = pb.G[o];
+  if (p == 0) {
+    const double *U = pb.UM + (size_t)b * g.ny, *W = pb.WM + (size_t)b * g.ny;
+    w = mk(W[n], U[n]);
+    v = mk(0.0, 0.0);
+    for (int m = g.N - ((g.N - n - 1) & 1); m > n; m -= 2) v = mk(fma(2.0 * m, W[m], v.x), fma(2.0 * m, U[m], v.y));
+    if (n == 0) v = 0.5 * v;
+  }
   pb.V32[o] = make_float2((float)v.x, (float)v.y);
   pb.G32[o] = make_float2((float)w.x, (float)w.y);
 }

@@ -93,17 +93,24 @@ __global__ void __launch_bounds__(64, ctas_of(dct_regs<RN, N>(), 64)) stage_pre_
     const size_t vs = 2 * (size_t)P;
     size_t ss = vs;
     if (liveM) {
-      // the mean flow: its own columns, or the FP32 copies (W, U) in mode 0's column
+      // the mean flow: its own columns, or the FP32 copies in mode 0's: (W, U),
+      // and (DW, DU), which the implicit half sums in FP64 (an FP32 sum loses up to
+      // N / 2 roundings of the mean shear)
       if constexpr (kF32) {
-        Sp = g0 + (f == 0 || f == 5 ? 1 : 0);
+        Sp = g0 + (f == 0 ? 1 : 0);
+        if (deriv) {
+          Vp = v0 + (f == 5 ? 1 : 0);
+          cS = 0;
+          cV = f == 5 ? (RN)-1.0 : (RN)1.0;
+        }
       } else {
         Sp = (f == 0 || f == 5 ? pb.UM : pb.WM) + (size_t)b * ny;
         ss = 1;
       }
     }
-    const bool liveS = gen || liveM;
+    const bool liveV = gen || (kF32 && liveM && deriv), liveS = gen || (liveM && !(kF32 && deriv));
     // every load is unconditional (the loops batch them), dead lanes drop theirs
-    auto V = [&](int n) { const RN x = __ldg(Vp + n * vs); return gen ? x : (RN)0; };
+    auto V = [&](int n) { const RN x = __ldg(Vp + n * vs); return liveV ? x : (RN)0; };
     auto S = [&](int n) { const RN x = __ldg(Sp + n * ss); return liveS ? x : (RN)0; };
     // 2 k; from a table in FP64, where converting it would cost an operation
     auto c2 = [&](int k) {

@@ -69,7 +69,8 @@ __global__ void __launch_bounds__(192) stage_pre_direct_kernel(Grid g, PencilBuf
     } else if (mean && f == 5) {
       cS = (RN)-1.0;
     }
-    const bool liveM = mean && !own && r == 0, liveS = gen || liveM;
+    const bool liveM = mean && !own && r == 0;
+    const bool liveV = gen || (kF32 && liveM && deriv), liveS = gen || (liveM && !(kF32 && deriv));
     const size_t col = 2 * ((size_t)b * ny * P + p), vs = 2 * (size_t)P;
     const RN* v0 = reinterpret_cast<const RN*>(kF32 ? (const void*)pb.V32 : pb.V) + col;
     const RN* g0 = reinterpret_cast<const RN*>(kF32 ? (const void*)pb.G32 : pb.G) + col;
@@ -78,13 +79,19 @@ __global__ void __launch_bounds__(192) stage_pre_direct_kernel(Grid g, PencilBuf
     size_t ss = vs;
     if (liveM) {
       if constexpr (kF32) {
-        Sp = g0 + (f == 0 || f == 5 ? 1 : 0);  // the FP32 copies (W, U) in mode 0's column
+        // the FP32 copies in mode 0's columns: (W, U) and (DW, DU)
+        Sp = g0 + (f == 0 ? 1 : 0);
+        if (deriv) {
+          Vp = v0 + (f == 5 ? 1 : 0);
+          cS = 0;
+          cV = f == 5 ? (RN)-1.0 : (RN)1.0;
+        }
       } else {
         Sp = (f == 0 || f == 5 ? pb.UM : pb.WM) + (size_t)b * ny;
         ss = 1;
       }
     }
-    auto V = [&](int n) { const RN x = __ldg(Vp + n * vs); return gen ? x : (RN)0; };
+    auto V = [&](int n) { const RN x = __ldg(Vp + n * vs); return liveV ? x : (RN)0; };
     auto S = [&](int n) { const RN x = __ldg(Sp + n * ss); return liveS ? x : (RN)0; };
     auto c2 = [&](int k) {  // 2 k
       if constexpr (sizeof(RN) == 8) return __ldg(t.tau.n1 + k - 1);

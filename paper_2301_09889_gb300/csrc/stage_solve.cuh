@@ -257,11 +257,13 @@ __device__ __forceinline__ Wall mean_down(double* f, const DevTables& t, const S
   return w;
 }
 
-// up: X <- X + d (+ the response u1 to the forcing of U)
+// up: X <- X + d (+ the response u1 to the forcing of U).  X32, D32 (mixed
+// precision): FP32 copies of X and of its derivative, 2 P apart; the derivative
+// is summed in FP64 from X and rounded once.
 template <int TOP>
 __device__ __forceinline__ void mean_up(double* f, const DevTables& t, const StageCoef& sc, int N, size_t P, int sig,
-                                     bool forced, const double* __restrict__ T, double* X, float* X32, double f0,
-                                     double fc, double wx) {
+                                     bool forced, const double* __restrict__ T, double* X, float* X32, float* D32,
+                                     double f0, double fc, double wx) {
   constexpr int NT = 64;
   constexpr int TABS = solve_tabs<TOP>();
   const int M = (N - sig) / 2 + 1;
@@ -282,8 +284,19 @@ __device__ __forceinline__ void mean_up(double* f, const DevTables& t, const Sta
       [&](int i, const Bw& v) {
         const double x = fma(fc, v.w, v.b + f[i * NT]);
         X[2 * i + sig] = x;
-        if (X32) X32[2 * P * (2 * i + sig)] = narrow(x);
+        if (X32) {
+          X32[2 * P * (2 * i + sig)] = narrow(x);
+          f[i * NT] = x;
+        }
       });
+  if (!X32) return;
+  if ((N - sig) & 1) D32[2 * P * N] = 0.0f;
+  double d = 0.0;
+  for (int i = M - 1; 2 * i + sig >= 1; --i) {
+    const int n = 2 * i + sig;
+    d = fma((double)(2 * n), f[i * NT], d);
+    D32[2 * P * (n - 1)] = narrow(n == 1 ? 0.5 * d : d);
+  }
 }
 
 // Solve omega_y of parity sig of one (mode, component), or (MEAN) the mean flow
@@ -337,9 +350,11 @@ __device__ __forceinline__ void solve_omega(double* f, double* xch, const Grid& 
     f0 = sig == 0 ? xe : xo;
   }
   if constexpr (MEAN) {
-    // the FP32 copies go to mode 0's column: (W, U)
-    float* X32 = sizeof(RN) == 4 ? reinterpret_cast<float*>(pb.G32) + 2 * (size_t)b * ny * P + (1 - r) : nullptr;
-    mean_up<TOP>(f, t, sc, g.N, P, sig, r == 0, T, X, X32, f0, fc, w.wx);
+    // the FP32 copies go to the columns of mode 0: (W, U) and (DW, DU)
+    const size_t col = 2 * (size_t)b * ny * P + (1 - r);
+    float* X32 = sizeof(RN) == 4 ? reinterpret_cast<float*>(pb.G32) + col : nullptr;
+    float* D32 = sizeof(RN) == 4 ? reinterpret_cast<float*>(pb.V32) + col : nullptr;
+    mean_up<TOP>(f, t, sc, g.N, P, sig, r == 0, T, X, X32, D32, f0, fc, w.wx);
     return;
   }
   // up: f_i = a_i + b_i f_{i-1}; g <- f - c g
