@@ -376,8 +376,9 @@ int srv_destroy(ch_server_t* s);
  *       at each node, of u, v, w, omega_x, omega_y, omega_z;
  *   d_h [B][3][ny][nz][nx/2] complex: Fourier coefficients of the kept modes
  *       of H = u x omega evaluated on the 3nx/2 x 3nz/2 grid.
- * Uses the handle's twiddle tables (and, in FP64 handles whose nonlinear term
- * runs in passes, their array of node values as scratch); allocates nothing.
+ * FP64 in handles of both precisions.  Uses the handle's twiddle tables (and,
+ * where the term runs in passes, the array of node values as scratch, which
+ * every step writes anew); allocates nothing.
  * CH_ERR_UNSUPPORTED for mixed-precision handles whose FP64 padded plane
  * does not fit a cluster's shared memory (256 x 256 modes). */
 int ch_nonlinear(ch_env_t* env, const double* d_q, double* d_h);

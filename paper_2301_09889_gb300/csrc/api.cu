@@ -201,10 +201,13 @@ struct ch_env {
   cudaStream_t own_stream = nullptr;
   PencilBufs pb{};
   DevTables tab{};
+  // the nonlinear term of a step, in the handle's precision, and of ch_nonlinear
   PlaneArgs<double> plane{};
   size_t plane_smem = 0;
-  PlaneArgs<float> plane_f{};   // FP32 nonlinear term (precision 1)
+  PlaneArgs<float> plane_f{};
   size_t plane_f_smem = 0;
+  PlaneArgs<double> plane_nl{};  // S = 0: unsupported
+  size_t plane_nl_smem = 0;
   double* d_act = nullptr;
   double* d_out = nullptr;
   double* h_out = nullptr;
@@ -297,41 +300,78 @@ void node_strides(Grid* g) {
   g->qb = passes ? g->ny * g->qj : 6 * g->qf;
 }
 
-// nonlinear plane kernel: smallest cluster whose z-slab fits shared memory
+// Nodes whose FP64 passes the node array has room for, and its size in FP64
+// complex values.  Mixed handles keep FP32 pairs there; ch_nonlinear, which is
+// FP64 in every handle, then runs its passes on half of the nodes at a time, or
+// on all of them where the whole array takes no more than 16 MB (launches count
+// there: 32x65x32 88 us in two parts, 58 in one, 94 on clusters).
+int node_array_nodes(const Grid& g, size_t B, int precision) {
+  return precision == 0 || B * g.qb * sizeof(double2) <= ((size_t)16 << 20) ? g.ny : (g.ny + 1) / 2;
+}
+size_t node_array_size(const Grid& g, size_t B, int precision) {
+  if (passes_built(g.mx, g.mz)) return B * node_array_nodes(g, B, precision) * g.qj;
+  return precision == 1 ? B * g.qb / 2 : B * g.qb;
+}
+
+int sm_count() {
+  int dev = 0, v = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
+    return v;
+  return 152;
+}
+
+// Cluster size for planes of `csz`-byte values: the smallest S whose ny * B * S
+// CTAs fill the SMs once; without one, the largest whose z-slab fits (0: none).
+// Handles of the same grid and batch capacity give bit-identical results; other
+// capacities may split the planes differently and agree to rounding.
+int cluster_size(const Grid& g, int B, size_t csz) {
+  const int nsm = sm_count();
+  int best = 0;
+  for (int S = 1; S <= 8; S *= 2) {
+    if (g.mz % S || (g.mz / S) % 2) continue;
+    if ((size_t)6 * (g.mz / S) * g.nxh * csz > 160 * 1024) continue;
+    best = S;
+    if ((long)g.ny * B * S >= nsm) return S;
+  }
+  // a 16-CTA cluster (non-portable opt-in) only where no portable size fits
+  if (!best && g.mz % 16 == 0 && (g.mz / 16) % 2 == 0 && (size_t)6 * (g.mz / 16) * g.nxh * csz <= 160 * 1024) best = 16;
+  return best;
+}
+
+// ch_nonlinear alone on clusters, whose single launch wins while small planes
+// leave the GPU in one wave: up to 216 points of a plane per CTA and a CTA per
+// SM, or two for the smallest (us per call on clusters and in passes, FP64:
+// 8x44x8 20.7 / 23.9, 8x65x16 24.7 / 27.8, 8x65x24 29.3 / 34, 24x65x8 30.3 /
+// 30.9; 8x161x16 41 / 31, 24x88x8 39 / 33, 32x9x32 58 / 42).  18-point x lines
+// take three radix passes there: 12x44x8 24.6 / 22.7.  Clusters of eight only
+// half a wave of the shortest x lines: 8x9x64 39 / 51, but 8x18x64 51 / 51 and
+// 16x9x32 39 / 36.
+bool small_on_cluster(const Grid& g, int B) {
+  const int S = cluster_size(g, B, sizeof(double2));
+  const int points = S ? g.mx * (g.mz / S) : 0;
+  const long ctas = (long)g.ny * B * S;
+  if (S == 0 || S > 8 || g.mx % 4 || (S == 8 && (g.mx > 12 || 2 * ctas > sm_count()))) return false;
+  return points <= 216 && ctas <= (points <= 72 || g.mx * g.mz <= 144 ? 2L : 1L) * sm_count();
+}
+
+// nonlinear term in three passes (where the padded lengths are built and
+// `passes`), or the smallest cluster whose z-slab fits shared memory
 template <typename R>
-int setup_plane(ch_env* env, PlaneArgs<R>* a, size_t* smem) {
+int setup_plane(ch_env* env, PlaneArgs<R>* a, size_t* smem, bool passes) {
   using C = typename cpx<R>::T;
   const Grid& g = env->g;
   a->nxh = g.nxh; a->nz = g.nz; a->ny = g.ny; a->mx = g.mx; a->mz = g.mz; a->P = g.P;
   a->qf = (size_t)g.ny * g.P; a->qj = g.P; a->qb = 6 * a->qf; a->hb = 3 * a->qf;
   a->S = 0;
   const size_t csz = sizeof(C);
-  // cluster size: the smallest feasible S whose ny * B * S CTAs fill the SMs
-  // once; without one, the largest feasible S.  Handles of the same grid and
-  // batch capacity give bit-identical results; other capacities may split the
-  // planes differently and agree to rounding.
-  int nsm = 152;
-  {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-      nsm = v;
-  }
-  int feasible[5], nf = 0;
-  for (int S = 1; S <= 8; S *= 2) {
-    if (g.mz % S || (g.mz / S) % 2) continue;
-    if ((size_t)6 * (g.mz / S) * g.nxh * csz > 160 * 1024) continue;
-    feasible[nf++] = S;
-  }
-  // a 16-CTA cluster (non-portable opt-in) only where no portable size fits
-  if (!nf && g.mz % 16 == 0 && (g.mz / 16) % 2 == 0 && (size_t)6 * (g.mz / 16) * g.nxh * csz <= 160 * 1024)
-    feasible[nf++] = 16;
+  const int nsm = sm_count();
+  const int S = cluster_size(g, env->B, csz);
   // Three passes through global memory (in place in a step) where the padded
-  // lengths are built (plane_pass.cu), in the precision the handle steps in; the other
-  // plane keeps a cluster, for ch_nonlinear, where one fits.  Planes of
-  // 256 x 256 modes fit no portable cluster.
+  // lengths are built (plane_pass.cu).  Planes of 256 x 256 modes fit no
+  // portable cluster: passes in the precision the handle steps in.
   const bool stepping = (sizeof(R) == 8) == (env->prm.precision == 0);
-  const bool large = g.mx == 384 && g.mz == 384;
-  if (stepping && passes_built(g.mx, g.mz) && (nf || large)) {
+  const bool large = stepping && g.mx == 384 && g.mz == 384;
+  if (passes && passes_built(g.mx, g.mz) && (S || large)) {
     a->passes = 1;
     a->S = 1;
     a->Lz = g.mz;
@@ -340,9 +380,7 @@ int setup_plane(ch_env* env, PlaneArgs<R>* a, size_t* smem) {
     // reported: the cluster that would hold the plane; 0 where none does, and
     // for FP64 planes of 64 x 64 and 128 x 128 modes (the value is part of the ABI)
     const bool fp64_square = sizeof(R) == 8 && g.mx == g.mz && (g.mx == 96 || g.mx == 192);
-    a->cluster = large || fp64_square ? 0 : feasible[nf - 1];
-    for (int k = 0; k < nf && a->cluster; ++k)
-      if ((long)g.ny * env->B * feasible[k] >= nsm) { a->cluster = feasible[k]; break; }
+    a->cluster = large || fp64_square ? 0 : S;
     a->y = reinterpret_cast<C*>(env->pb.Q);
     auto line_twiddles = [](int m, int A) {  // [m / A][A] e^{2 pi i s k / m}
       const std::vector<double2> w = twiddles(m);
@@ -358,10 +396,7 @@ int setup_plane(ch_env* env, PlaneArgs<R>* a, size_t* smem) {
     a->scale = (R)(1.0 / ((double)g.mx * g.mz));
     return CH_OK;
   }
-  if (!nf) return CH_ERR_UNSUPPORTED;
-  int S = feasible[nf - 1];
-  for (int k = 0; k < nf; ++k)
-    if ((long)g.ny * env->B * feasible[k] >= nsm) { S = feasible[k]; break; }
+  if (!S) return CH_ERR_UNSUPPORTED;
   const int Lz = g.mz / S;
   const size_t zb = (size_t)6 * Lz * g.nxh * csz;
   const int npairs = Lz / 2;
@@ -610,13 +645,18 @@ int build_tables(ch_env* env) {
     RC(dupload(env, &env->tab.cos_ana_f, std::vector<float>(ca.begin(), ca.end())));
   }
 
-  // the plane of the handle's precision is required; the other one serves
-  // ch_nonlinear (FP64) and is skipped where its slab does not fit
-  const int r64 = setup_plane(env, &env->plane, &env->plane_smem);
-  const int r32 = setup_plane(env, &env->plane_f, &env->plane_f_smem);
-  if (env->prm.precision == 1 ? r32 != CH_OK : r64 != CH_OK) return env->prm.precision == 1 ? r32 : r64;
-  if (r64 != CH_OK) env->plane.S = 0;
-  if (r32 != CH_OK) env->plane_f.S = 0;
+  const bool mixed = p.precision == 1;
+  RC(mixed ? setup_plane(env, &env->plane_f, &env->plane_f_smem, true)
+           : setup_plane(env, &env->plane, &env->plane_smem, true));
+  // ch_nonlinear (FP64): the form of the step but for small planes; a mixed handle
+  // whose FP64 slab fits no cluster goes without
+  const bool small = small_on_cluster(g, env->B);
+  if (!mixed && !(small && env->plane.passes)) {
+    env->plane_nl = env->plane;
+    env->plane_nl_smem = env->plane_smem;
+  } else if (setup_plane(env, &env->plane_nl, &env->plane_nl_smem, !small) != CH_OK) {
+    env->plane_nl.S = 0;
+  }
   return CH_OK;
 }
 
@@ -1033,7 +1073,7 @@ size_t env_footprint(const ch_params_t* p) {
   Grid g{};
   g.ny = (int)ny; g.nxh = (int)nxh; g.P = (int)P; g.mx = 3 * p->nx / 2; g.mz = 3 * p->nz / 2;
   node_strides(&g);
-  const size_t state = B * (4 * ny * P * 16 + 4 * ny * 8 + g.qb * (p->precision == 1 ? 8 : 16) + 3 * P * 16 + 8 +
+  const size_t state = B * (4 * ny * P * 16 + 4 * ny * 8 + node_array_size(g, 1, p->precision) * 16 + 3 * P * 16 + 8 +
                             (size_t)p->nz * p->nx * 8 + (2 * (size_t)p->nz * p->nx + 2) * 8);
   const size_t folded = (3 * 2 * (p->top_bc ? 8 : 7) + 2 * 6) * Mh * ((P + 15) / 16 * 16) * 8;
   const size_t scan = p->top_bc ? 0 : (3 * 2 * 4 + 2 * 4) * Mh * P;
@@ -1111,7 +1151,7 @@ int env_create(const ch_params_t* p, ch_env_t** out) {
       (rc = dalloc(env, &pb.HVP, B * ny * P)) || (rc = dalloc(env, &pb.HGP, B * ny * P)) ||
       (rc = dalloc(env, &pb.UM, B * ny)) || (rc = dalloc(env, &pb.WM, B * ny)) ||
       (rc = dalloc(env, &pb.HXP, B * ny)) || (rc = dalloc(env, &pb.HZP, B * ny)) ||
-      (rc = dalloc(env, &pb.Q, p->precision == 1 ? B * g.qb / 2 : B * g.qb)) ||
+      (rc = dalloc(env, &pb.Q, node_array_size(g, B, p->precision))) ||
       (rc = dalloc(env, &pb.vw_old, B * P)) || (rc = dalloc(env, &pb.vw_new, B * P)) ||
       (rc = dalloc(env, &pb.planes, B * 2 * P)) || (rc = dalloc(env, &pb.tau_acc, B)))
     return fail(rc);
@@ -1402,11 +1442,15 @@ int env_destroy(ch_env_t* env) {
 
 int ch_nonlinear(ch_env_t* env, const double* d_q, double* d_h) {
   if (!env || !d_q || !d_h) return CH_ERR_ARG;
-  if (env->plane.S == 0) return CH_ERR_UNSUPPORTED;
-  PlaneArgs<double> a = env->plane;
-  a.q = reinterpret_cast<const double2*>(d_q);
-  a.h = reinterpret_cast<double2*>(d_h);
-  CK(launch_plane<double>(a, env->B, env->plane_smem, env->stream));
+  if (env->plane_nl.S == 0) return CH_ERR_UNSUPPORTED;
+  PlaneArgs<double> a = env->plane_nl;
+  const int ny = a.ny, step = a.passes ? node_array_nodes(env->g, env->B, env->prm.precision) : ny;
+  for (int j = 0; j < ny; j += step) {
+    a.q = reinterpret_cast<const double2*>(d_q) + j * a.qj;
+    a.h = reinterpret_cast<double2*>(d_h) + j * a.qj;
+    a.ny = std::min(step, ny - j);
+    CK(launch_plane<double>(a, env->B, env->plane_nl_smem, env->stream));
+  }
   return CH_OK;
 }
 
