@@ -214,7 +214,8 @@ __global__ void __launch_bounds__(8 * kModeThreads) stage_post_kernel(Grid g, in
       mean_scan<MH, RN>(N, ny, ppc, c, e, (e == 0 ? pb.UM : pb.WM) + (size_t)b * ny,
                         (e == 0 ? pb.HXP : pb.HZP) + (size_t)b * ny, (e == 0) ? Hx : Hz, cc, sc, helm(c),
                         ss[(0 * 2 + c) * ppc + pl], rowc, t.tau.u1 + (size_t)sc.k * Mh, t.tau.u1_iflux[sc.k],
-                        t.tau.wint, q, reinterpret_cast<float*>(pb.V32) + 2 * (size_t)b * ny * P + (e == 0 ? 1 : 0), P);
+                        t.tau.wint, t.tau.n1, q, reinterpret_cast<float*>(pb.V32) + 2 * (size_t)b * ny * P + (e == 0 ? 1 : 0),
+                        P);
     } else {
       const double kx = t.kx[ix], kz = t.kz[row], k2 = kx * kx + kz * kz;
       const double sgn = (r == 0) ? -1.0 : 1.0;

@@ -284,17 +284,44 @@ __device__ __forceinline__ void v_scan(int N, int ny, int ppc, int sv, const VV&
   }
 }
 
+// The FP32 copy of the derivative of the mean flow from the coefficients x[k] of
+// index i0 - k (n = 2 i + s; 0 outside the parity) on the lanes of a group: sums
+// of 2 n X_n from the top in FP64, each rounded once.  Coefficients 2 P apart;
+// n1[n] = 2 (n + 1).
+template <int K>
+__device__ __forceinline__ void mean_shear(double (&x)[K], int N, int s, int i0, const double* __restrict__ n1, int q,
+                                           float* D32, size_t P) {
+  const int M = (N - s) / 2 + 1;
+  double d = 0.0;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int n = 2 * (i0 - k) + s;
+    d = fma_rn(__ldg(n1 + min(max(n - 1, 0), N)), x[k], d);
+    x[k] = d;
+  }
+  const double above = scanl::lanes_above(d, q);
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int i = i0 - k, n = 2 * i + s;
+    if (i < 0 || i >= M || n < 1) continue;
+    double b = x[k] + above;
+    if (n == 1) b = 0.5 * b;
+    D32[2 * P * (n - 1)] = narrow(b);
+  }
+  if (q == 0 && ((N - s) & 1)) D32[2 * P * N] = 0.0f;
+}
+
 // mean flow of parity s over a lane group, solved for its increment
 // d = X^k - X^{k-1} (see stage_solve.cuh): right-hand side dt (...), and
-// (1 + c) beta dt nu X on the diagonal for (1 + c) D^2 X.  D32 (mixed
-// precision): the FP32 copy of the derivative of X, summed in FP64 and rounded
-// once, coefficients 2 P apart
+// (1 + c) beta dt nu X on the diagonal for (1 + c) D^2 X.  D32, mixed precision:
+// mean_shear
 template <int MH, typename RN, class Tab>
 __device__ __forceinline__ void mean_scan(int N, int ny, int ppc, int s, int e, double* X, double* XP,
                                           const typename cpx<RN>::T* Hm, double cc, const StageCoef& sc,
                                           const Tab& T, double isq, const double* __restrict__ rowc,
                                           const double* __restrict__ u1, double u1_iflux,
-                                          const double* __restrict__ wint, int q, float* D32, size_t P) {
+                                          const double* __restrict__ wint, const double* __restrict__ n1, int q,
+                                          float* D32, size_t P) {
   constexpr int K = Blk<MH>::K;
   const int M = (N - s) / 2 + 1;
   double f[K], dg[K];
@@ -340,20 +367,12 @@ __device__ __forceinline__ void mean_scan(int N, int ny, int ppc, int s, int e, 
     }
   }
   if constexpr (sizeof(RN) == 4) {
-    double d = 0.0;  // inclusive prefix of 2 n X_n, the derivative's coefficient n - 1
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       const int i = Blk<MH>::i_of(q, k);
-      if (i >= 0 && i < M) d = fma_rn((double)(2 * (2 * i + s)), f[k], d);
-      f[k] = d;
+      if (i < 0 || i >= M) f[k] = 0.0;
     }
-    const double above = scanl::lanes_above(d, q);
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const int i = Blk<MH>::i_of(q, k), n = 2 * i + s;
-      if (i >= 0 && i < M && n >= 1) D32[2 * P * (n - 1)] = (float)((n == 1 ? 0.5 : 1.0) * (f[k] + above));
-    }
-    if (q == 0 && ((N - s) & 1)) D32[2 * P * N] = 0.0f;
+    mean_shear<K>(f, N, s, MH - 1 - q * K, n1, q, D32, P);
   }
 }
 

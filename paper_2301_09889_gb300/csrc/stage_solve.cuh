@@ -49,6 +49,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "stage_close.cuh"
+#include "stage_scan.cuh"
 
 namespace chdns {
 
@@ -257,13 +258,12 @@ __device__ __forceinline__ Wall mean_down(double* f, const DevTables& t, const S
   return w;
 }
 
-// up: X <- X + d (+ the response u1 to the forcing of U).  X32, D32 (mixed
-// precision): FP32 copies of X and of its derivative, 2 P apart; the derivative
-// is summed in FP64 from X and rounded once.
+// up: X <- X + d (+ the response u1 to the forcing of U).  X32 (mixed precision):
+// FP32 copies of X, 2 P apart; X then also takes its column f.
 template <int TOP>
 __device__ __forceinline__ void mean_up(double* f, const DevTables& t, const StageCoef& sc, int N, size_t P, int sig,
-                                     bool forced, const double* __restrict__ T, double* X, float* X32, float* D32,
-                                     double f0, double fc, double wx) {
+                                     bool forced, const double* __restrict__ T, double* X, float* X32, double f0,
+                                     double fc, double wx) {
   constexpr int NT = 64;
   constexpr int TABS = solve_tabs<TOP>();
   const int M = (N - sig) / 2 + 1;
@@ -289,14 +289,18 @@ __device__ __forceinline__ void mean_up(double* f, const DevTables& t, const Sta
           f[i * NT] = x;
         }
       });
-  if (!X32) return;
-  if ((N - sig) & 1) D32[2 * P * N] = 0.0f;
-  double d = 0.0;
-  for (int i = M - 1; 2 * i + sig >= 1; --i) {
-    const int n = 2 * i + sig;
-    d = fma((double)(2 * n), f[i * NT], d);
-    D32[2 * P * (n - 1)] = narrow(n == 1 ? 0.5 * d : d);
-  }
+}
+
+// mean_shear (stage_scan.cuh) of a column x of up to 16 K coefficients
+template <int K>
+__device__ __forceinline__ void mean_shear_of(const double* x, const DevTables& t, int N, size_t P, int sig, int q, float* D32) {
+  constexpr int NT = 64;
+  static_assert(7 * kLanes > kMaxNy / 2, "a column fits the lanes");
+  const int M = (N - sig) / 2 + 1, i0 = (kLanes - q) * K - 1;
+  double v[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) v[k] = i0 - k < M ? x[(i0 - k) * NT] : 0.0;
+  mean_shear<K>(v, N, sig, i0, t.tau.n1, q, D32, P);
 }
 
 // Solve omega_y of parity sig of one (mode, component), or (MEAN) the mean flow
@@ -330,7 +334,7 @@ __device__ __forceinline__ void solve_omega(double* f, double* xch, const Grid& 
 #pragma unroll
     for (int k = 0; k < 6; ++k) xch[k * NT + me] = mine[k];
     __syncthreads();
-    if (!live) return;
+    if (!live && !(MEAN && sizeof(RN) == 4)) return;
     double se[6], so[6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
@@ -351,10 +355,19 @@ __device__ __forceinline__ void solve_omega(double* f, double* xch, const Grid& 
   }
   if constexpr (MEAN) {
     // the FP32 copies go to the columns of mode 0: (W, U) and (DW, DU)
-    const size_t col = 2 * (size_t)b * ny * P + (1 - r);
-    float* X32 = sizeof(RN) == 4 ? reinterpret_cast<float*>(pb.G32) + col : nullptr;
-    float* D32 = sizeof(RN) == 4 ? reinterpret_cast<float*>(pb.V32) + col : nullptr;
-    mean_up<TOP>(f, t, sc, g.N, P, sig, r == 0, T, X, X32, D32, f0, fc, w.wx);
+    const size_t col = 2 * (size_t)b * ny * P;
+    float* X32 = sizeof(RN) == 4 ? reinterpret_cast<float*>(pb.G32) + col + (1 - r) : nullptr;
+    if (live) mean_up<TOP>(f, t, sc, g.N, P, sig, r == 0, T, X, X32, f0, fc, w.wx);
+    if constexpr (sizeof(RN) == 4) {
+      // sixteen lanes of the warp on each of its two columns (as a loop of the two
+      // threads the mean flow outlasted v: 16x201x16 x 8 557 us a step, 583 so)
+      __syncwarp();
+      const int q = threadIdx.x % kLanes, c = threadIdx.x % 32 / kLanes;
+      const double* x = f - threadIdx.x % 32 + c;
+      float* D32 = reinterpret_cast<float*>(pb.V32) + col + (1 - c);
+      if (M <= 3 * kLanes) mean_shear_of<3>(x, t, g.N, P, sig, q, D32);
+      else mean_shear_of<7>(x, t, g.N, P, sig, q, D32);
+    }
     return;
   }
   // up: f_i = a_i + b_i f_{i-1}; g <- f - c g
@@ -550,8 +563,9 @@ __global__ void __launch_bounds__(64, D == 3 ? 6 : 4) stage_solve_kernel(Grid g,
   const int pr = z == 0 ? lane >> 1 : ((int)(blockIdx.x - 1) % tiles) * 16 + (lane >> 1), p = min(pr, g.P - 1);
   // the mean flow is mode 0; the Nyquist row stays zero
   const bool live = z == 0 ? lane < 2 : pr > 0 && pr < g.P && p / g.nxh != g.nz / 2;
-  // a free-slip top needs every thread at the exchange
-  if (TOP == 0 && !live) return;
+  // a free-slip top needs every thread at the exchange, the FP32 copy of the mean
+  // shear every lane
+  if (TOP == 0 && !live && !(z == 0 && sizeof(RN) == 4)) return;
   double* f = sarr + threadIdx.x;
   double* xch = sarr + (size_t)t.tau.Mh * 64;
   const RN* h = reinterpret_cast<const RN*>(hc);
