@@ -472,10 +472,13 @@ int build_tables(ch_env* env) {
   // e1 > 0 adds E1 = e1 e (the Helmholtz tables, e1 = 1 + alpha/beta of the
   // stage) and under a free-slip top the weights W2 of sum n^2 P
   const int htabs = top ? 8 : 7;
-  const size_t rows = (size_t)((P + 15) / 16) * Mh * 16;
+  // they depend on kz^2 alone: rows kz = 0 .. nz/2 - 1 serve the negative ones too
+  const int Pt = g.nxh * (g.nz / 2);
+  const size_t rows = (size_t)((Pt + 15) / 16) * Mh * 16;
   std::vector<double> helm_f((size_t)3 * 2 * htabs * rows, 0.0);
   std::vector<double> pois_f((size_t)2 * 6 * rows, 0.0);
   auto put_f = [&](std::vector<double>& tab, size_t block, int tabs, const Factor& F, int M, int pp, int sig, double e1) {
+    if (pp >= Pt) return;
     double w = 1.0, w2 = 0.0;  // W_{M-1}
     for (int i = M - 1; i >= 1; --i) {
       const int n = 2 * i + sig;
@@ -630,22 +633,25 @@ int build_tables(ch_env* env) {
   env->tab.tau.top_bc = top ? 1 : 0;
   RC(dupload(env, &env->tab.tw_nx, twiddles(g.nx)));
   RC(dupload(env, &env->tab.tw_nz, twiddles(g.nz)));
-  if (stage_direct(g) || (p.precision == 0 && pre_few(g, env->B))) {
+  const bool mixed = p.precision == 1;
+  if (stage_direct(g) || (!mixed && pre_few(g, env->B))) {
     const int Jp = direct_pre_pitch(N), Ip = direct_ana_pitch(N), J = N / 2 + 1;
-    std::vector<double> cp((size_t)ny * Jp, 0.0), ca((size_t)J * 2 * Ip, 0.0);
+    std::vector<double> cp((size_t)ny * Jp, 0.0), ca(stage_direct(g) ? (size_t)J * 2 * Ip : 0, 0.0);
     for (int j = 0; j < J; ++j)
       for (int n = 0; n < ny; ++n) {
         const double c = cheb[(size_t)j * ny + n];
         cp[(size_t)n * Jp + j] = c;
-        ca[((size_t)j * 2 + n % 2) * Ip + n / 2] = c;
+        if (!ca.empty()) ca[((size_t)j * 2 + n % 2) * Ip + n / 2] = c;
       }
-    RC(dupload(env, &env->tab.cos_pre, cp));
-    RC(dupload(env, &env->tab.cos_ana, ca));
-    RC(dupload(env, &env->tab.cos_pre_f, std::vector<float>(cp.begin(), cp.end())));
-    RC(dupload(env, &env->tab.cos_ana_f, std::vector<float>(ca.begin(), ca.end())));
+    if (mixed) {
+      RC(dupload(env, &env->tab.cos_pre_f, std::vector<float>(cp.begin(), cp.end())));
+      RC(dupload(env, &env->tab.cos_ana_f, std::vector<float>(ca.begin(), ca.end())));
+    } else {
+      RC(dupload(env, &env->tab.cos_pre, cp));
+      RC(dupload(env, &env->tab.cos_ana, ca));
+    }
   }
 
-  const bool mixed = p.precision == 1;
   RC(mixed ? setup_plane(env, &env->plane_f, &env->plane_f_smem, true)
            : setup_plane(env, &env->plane, &env->plane_smem, true));
   // ch_nonlinear (FP64): the form of the step but for small planes; a mixed handle
@@ -1075,7 +1081,7 @@ size_t env_footprint(const ch_params_t* p) {
   node_strides(&g);
   const size_t state = B * (4 * ny * P * 16 + 4 * ny * 8 + node_array_size(g, 1, p->precision) * 16 + 3 * P * 16 + 8 +
                             (size_t)p->nz * p->nx * 8 + (2 * (size_t)p->nz * p->nx + 2) * 8);
-  const size_t folded = (3 * 2 * (p->top_bc ? 8 : 7) + 2 * 6) * Mh * ((P + 15) / 16 * 16) * 8;
+  const size_t folded = (3 * 2 * (p->top_bc ? 8 : 7) + 2 * 6) * Mh * ((P / 2 + 15) / 16 * 16) * 8;
   const size_t scan = p->top_bc ? 0 : (3 * 2 * 4 + 2 * 4) * Mh * P;
   const size_t tables = (scan + 3 * 2 * P + 2 * P + 3 * 2 * Mh * P + 3 * 2 * P +
                          3 * Mh + 3 + 3 * ny + ny + 2 * 3 * 2 * 2 * P) * 8 + ny * ny * 12 + (nxh + p->nz) * 8 +

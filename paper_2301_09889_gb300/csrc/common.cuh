@@ -368,7 +368,7 @@ struct TauTables {
   // Helmholtz operator, E1 = (1 + alpha/beta) e and under a free-slip top W2
   // (W2_{M-1} = n^2, W2_i = n_i^2 + b_{i+1} W2_{i+1}: sum n^2 P = sum W2_i a_i)
   // eA, eB, eC, h, b, W, E1 (, W2) per stage, parity and eA, eB, eC, h, b, W per parity, the entries of a
-  // row side by side for a tile of sixteen modes: [3][2] and [2] of [tile][rows 1 .. Mh][7 or 8, 6][16]
+  // row side by side for a tile of sixteen modes kz >= 0: [3][2] and [2] of [tile][rows 1 .. Mh][7 or 8, 6][16]
   const double* helm_f;
   const double* pois_f;
   const double* n2;        // [ny] n^2

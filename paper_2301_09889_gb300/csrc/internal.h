@@ -45,7 +45,8 @@ struct DevTables {
   const double* cheb;  // [ny][ny] cos(pi j n / N)
   const float* cheb_f; // the same table in FP32 (mixed precision)
   const double* dts;   // [ny] T_n'(y_js) at the sensing node
-  // direct sums (orders without a register transform): cos(pi j n / N) as
+  // direct sums, in the node precision (cos_ana for orders without a register
+  // transform, cos_pre for these and the few-mode form): cos(pi j n / N) as
   // [n][j <= N/2, padded] and as [j <= N/2][parity of n][i, padded], n = 2 i + parity
   const double *cos_pre, *cos_ana;
   const float *cos_pre_f, *cos_ana_f;

@@ -106,9 +106,11 @@ __device__ __forceinline__ void sweep_up(int first, int M, Load&& load, Step&& s
 // all of them and, with the row stride fixed, the rows of an unrolled block (the
 // solves issue three other instructions per FP64 operation: as [entry][row][mode]
 // arrays the tables took six addresses a row; 256 minimal mixed channels 1090
-// us per step then and 1064 so)
+// us per step then and 1064 so).  The tables depend on kz^2 alone and hold the
+// rows kz >= 0: modes kz and -kz share theirs.
 template <int TABS> __device__ __forceinline__ const double* tab_of(const double* T, int block, const Grid& g, int Mh, int p) {
-  return T + ((size_t)(block * ((g.P + 15) / 16) + p / 16) * Mh) * (TABS * 16) + p % 16;
+  const int row = p / g.nxh, hz = g.nz / 2, pt = row > hz ? p + (2 * (hz - row)) * g.nxh : p;
+  return T + ((size_t)(block * ((g.nxh * hz + 15) / 16) + pt / 16) * Mh) * (TABS * 16) + pt % 16;
 }
 template <int TABS> __device__ __forceinline__ double tab(const double* __restrict__ T, int row, int entry) {
   return __ldg(T + (ptrdiff_t)(row - 1) * (TABS * 16) + entry * 16);  // rows 1 .. Mh
