@@ -1075,18 +1075,25 @@ int env_slot_seed(ch_env* env, int e, uint64_t seed, double amplitude, int kmax)
 // device bytes env_create allocates for these parameters (tables and buffers)
 size_t env_footprint(const ch_params_t* p) {
   const size_t B = p->batch > 0 ? p->batch : 1;
-  const size_t nxh = p->nx / 2, P = nxh * p->nz, ny = p->ny, Mh = (ny - 1) / 2 + 1;
+  const size_t nxh = p->nx / 2, P = nxh * p->nz, ny = p->ny, Mh = (ny - 1) / 2 + 1, points = (size_t)p->nz * p->nx;
+  const bool mixed = p->precision == 1, top = p->top_bc == 1;
   Grid g{};
-  g.ny = (int)ny; g.nxh = (int)nxh; g.P = (int)P; g.mx = 3 * p->nx / 2; g.mz = 3 * p->nz / 2;
+  g.nx = p->nx; g.ny = p->ny; g.nz = p->nz; g.nxh = (int)nxh; g.P = (int)P; g.N = p->ny - 1;
+  g.mx = 3 * p->nx / 2; g.mz = 3 * p->nz / 2;
   node_strides(&g);
-  const size_t state = B * (4 * ny * P * 16 + 4 * ny * 8 + node_array_size(g, 1, p->precision) * 16 + 3 * P * 16 + 8 +
-                            (size_t)p->nz * p->nx * 8 + (2 * (size_t)p->nz * p->nx + 2) * 8);
-  const size_t folded = (3 * 2 * (p->top_bc ? 8 : 7) + 2 * 6) * Mh * ((P / 2 + 15) / 16 * 16) * 8;
-  const size_t scan = p->top_bc ? 0 : (3 * 2 * 4 + 2 * 4) * Mh * P;
-  const size_t tables = (scan + 3 * 2 * P + 2 * P + 3 * 2 * Mh * P + 3 * 2 * P +
-                         3 * Mh + 3 + 3 * ny + ny + 2 * 3 * 2 * 2 * P) * 8 + ny * ny * 12 + (nxh + p->nz) * 8 +
-                        folded;
-  return state + tables + ((size_t)4 << 20);  // plus twiddles and rounding slack
+  // fields, mean flow, wall and sensing spectra, the wall shear; action, outputs
+  const size_t state = B * (4 * ny * P * 16 + 4 * ny * 8 + 2 * P * 16 + 2 * P * 16 + 8 + points * 8 + (2 * points + 2) * 8) +
+                       node_array_size(g, B, p->precision) * 16;
+  const size_t policy = p->control == 2 ? B * 2 * points * 8 + kPolicyMaxWeights * sizeof(float) : 0;
+  const size_t folded = (3 * 2 * (top ? 8 : 7) + 2 * 6) * Mh * ((P / 2 + 15) / 16 * 16) * 8;
+  const size_t scan = top ? 0 : (3 * 2 * 4 + 2 * 4) * Mh * P * 8;
+  const size_t modes = (3 * 2 * Mh + 2 * 3 * 2 + 2 + 2 * 3 * 2 * 2) * P * 8;  // vh; isq, vh_idv; the free-slip sums
+  const size_t rows = (3 * Mh + 7 * ny + 3 + 12 + nxh + p->nz) * 8 + ny * ny * 12;
+  const size_t cosines = stage_direct(g) || (!mixed && pre_few(g, (int)B))
+                             ? (ny * direct_pre_pitch(g.N) + (stage_direct(g) ? Mh * 2 * direct_ana_pitch(g.N) : 0)) * (mixed ? 4 : 8)
+                             : 0;
+  const size_t roots = (size_t)(p->nx + p->nz + 2 * (g.mx + 2 * g.mz)) * 16;
+  return state + policy + folded + scan + modes + rows + cosines + roots + ((size_t)4 << 20);  // rounding of the allocations
 }
 }  // namespace chdns
 

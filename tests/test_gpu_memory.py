@@ -1,5 +1,5 @@
 """Device memory of single-environment handles, where the tables of the tau
-solves outweigh the fields.
+solves outweigh the fields, and what the server reserves for a class.
 
 Per mode and environment a handle holds V, G and their previous right-hand
 sides (4 ny complex values) and at most 9 ny node values; per mode and row of
@@ -26,3 +26,26 @@ def test_single_handles_stay_small(native_gpu, nx, ny, nz, precision, top_bc, ro
         native.env_destroy(env)
     P, Mh = nx // 2 * nz, (ny - 1) // 2 + 1
     assert held <= 13 * ny * P * 16 + rows * Mh * P * 8 + ny * ny * 12 + 100 * P * 8 + (32 << 10), held
+
+
+# (nx, ny, nz, slots, precision, control, top_bc): sensing planes that add up
+# beyond the allowance for rounding; direct sums; both sizes of a mixed handle's
+# node array
+@pytest.mark.parametrize("nx,ny,nz,slots,precision,control,top_bc", [
+    (128, 17, 128, 64, 1, 0, 0), (128, 17, 128, 64, 0, 1, 1), (64, 17, 64, 24, 1, 1, 0), (16, 50, 16, 8, 1, 0, 1),
+    (16, 201, 16, 1, 0, 1, 0), (36, 9, 36, 16, 1, 0, 0), (32, 33, 32, 1, 1, 0, 0)])
+def test_admission_covers_what_a_class_holds(native_gpu, nx, ny, nz, slots, precision, control, top_bc):
+    native = native_gpu
+    kw = dict(nx=nx, ny=ny, nz=nz, lx=2.67, lz=0.8, precision=precision, control=control, top_bc=top_bc, autotune=0)
+    env = native.env_create(native.params(**kw, batch=slots))
+    try:
+        held = native.env_info(env).device_bytes
+    finally:
+        native.env_destroy(env)
+    srv = native.srv_create(64 << 30, slots)
+    try:
+        native.srv_admit(srv, native.params(**kw), seed=1)
+        used = native.srv_stats(srv).hbm_used
+    finally:
+        native.srv_destroy(srv)
+    assert held <= used <= held + (8 << 20), (held, used)
