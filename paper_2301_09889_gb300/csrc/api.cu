@@ -418,7 +418,7 @@ int setup_plane(ch_env* env, PlaneArgs<R>* a, size_t* smem, bool passes) {
   // batch supplies four planes per SM, two-CTA clusters below
   if (plane16_shape(g.mx, g.mz, g.nxh, g.nz)) {
     a->team16 = (long)g.ny * env->B >= 4L * nsm ? 1 : 2;
-    if (a->team16 == 1) a->cluster = 1;
+    a->cluster = a->team16;  // CTAs per plane, or one CTA for two planes
     a->S = 1;
     a->Lz = g.mz;
   }

@@ -68,3 +68,17 @@ def test_nonlinear_of_mixed_256_planes_stays_unsupported(native_gpu):
         assert exc.value.code == native.CH_ERR_UNSUPPORTED
     finally:
         native.env_destroy(env)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_single_16x16_planes_report_their_cluster(native_gpu, precision):
+    """Planes of 16 x 16 modes run on two-CTA clusters until a batch has four
+    planes per SM, then two to a CTA."""
+    native = native_gpu
+    for batch, cluster in ((1, 2), (80, 1)):
+        env = native.env_create(native.params(nx=16, ny=65, nz=16, batch=batch, precision=precision, autotune=0))
+        try:
+            info = native.env_info(env)
+        finally:
+            native.env_destroy(env)
+        assert info.plane_cluster == cluster and info.plane_team == (1 if batch == 80 else 0)
