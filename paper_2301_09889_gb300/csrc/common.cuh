@@ -8,8 +8,9 @@
 #include <cuda_runtime.h>
 #include <cstddef>
 #include <cstdint>
-#include <mutex>
 #include <utility>
+
+#include "smem_limit.h"
 
 namespace chdns {
 
@@ -122,34 +123,6 @@ __device__ __forceinline__ void cp_async_elem(T* dst, const T* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(sizeof(T)) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// A kernel's dynamic shared-memory limit (and the non-portable cluster-size
-// opt-in) as configured so far.  raise_smem_limit only ever raises it, under
-// one lock for every kernel, so handles of different sizes driven from
-// several host threads never leave a kernel below a size another one needs.
-struct SmemLimit {
-  size_t bytes = 0;
-  bool nonportable = false;
-};
-inline std::mutex& kernel_attr_mutex() {
-  static std::mutex m;
-  return m;
-}
-template <typename K>
-inline cudaError_t raise_smem_limit(K kernel, SmemLimit* lim, size_t smem, bool nonportable_cluster = false) {
-  std::lock_guard<std::mutex> lock(kernel_attr_mutex());
-  if (smem > lim->bytes) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    lim->bytes = smem;
-  }
-  if (nonportable_cluster && !lim->nonportable) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    lim->nonportable = true;
-  }
-  return cudaSuccess;
-}
 
 // Plain stream-ordered launch.  Programmatic dependent launch was measured and
 // left out: a dependent that starts early takes shared memory and registers

@@ -539,7 +539,7 @@ __global__ void tau_helmholtz_noalloc_kernel(int ny, int M, int mpad, const doub
 namespace {
 
 // Device address of the scratch array, looked up once per device.
-constexpr int kMaxDevices = 64;
+using chdns::kMaxDevices;
 double* g_noalloc_ptr[kMaxDevices] = {nullptr};
 std::mutex g_noalloc_mu;
 
