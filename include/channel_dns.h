@@ -101,12 +101,13 @@ typedef struct ch_info {
     double nu, u_tau, tau_ref;
     size_t state_bytes;      /* bytes of one environment's serialised state                */
     size_t device_bytes;     /* device memory held by the handle                           */
-    int plane_cluster;       /* CTAs of a thread-block cluster that hold one y-plane of the
-                                nonlinear term where it runs on clusters; where it runs in
-                                three passes (z inverse, x transforms and products, z
-                                forward) the size such a cluster would have; 0 for planes
-                                of 256 x 256 modes and FP64 planes of 64 x 64 and
-                                128 x 128                                                */
+    int plane_cluster;       /* CTAs of a thread-block cluster that hold one y-plane of a
+                                step's nonlinear term where it runs on clusters; where it
+                                runs in three passes (z inverse, x transforms and products,
+                                z forward) the size such a cluster would have, kept for
+                                callers that read it; 0 for planes of 256 x 256 modes and
+                                FP64 planes of 64 x 64 and 128 x 128.  Whether a step runs
+                                in passes shows in launches_per_step                     */
     int launches_per_step;   /* kernels launched by one env_step                            */
     int post_batched;        /* 1: the implicit half of a stage runs one thread per (mode,
                                 class, component, equation); 0: 128 threads per mode on a
@@ -114,8 +115,9 @@ typedef struct ch_info {
     int ppc_pre, ppc_post;   /* tile widths: ppc_post Fourier modes per CTA of the implicit
                                 half where post_batched is 0; the other forms have one
                                 shape, and the values set are only reported              */
-    int tuned;               /* 1 if the tile shapes were chosen by timing (autotune)    */
-    double tune_ms;          /* host time env_create spent timing candidates            */
+    int tuned;               /* 1 if env_create ran the autotuner (forms with one shape
+                                leave it nothing to time)                               */
+    double tune_ms;          /* host time the autotuner took                            */
     int plane_team;          /* 1: planes of 16 x 16 modes in a batch of at least four
                                 planes per SM: two padded 24 x 24 planes per CTA, one line
                                 per thread in registers (plane_cluster is then 1);

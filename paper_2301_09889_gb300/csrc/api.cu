@@ -916,19 +916,15 @@ int capture_step(ch_env* env, int gi, const int* d_active) {
 // modes per CTA), so the widths change speed only, never results.  The
 // autotuner keeps the form the size rule chose.
 // ---------------------------------------------------------------------------
-// (the explicit half runs in one shape; its widths are accepted and refused as
-// when it worked on tiles of ppc_pre modes in shared memory)
-size_t pre_tile_bytes(const Grid& g, int ppc, size_t node_bytes) {
-  return (size_t)8 * g.ny * ppc * node_bytes + (size_t)12 * ppc * sizeof(double2);
-}
+// (the explicit half and the two-launch form run in one shape each; their widths
+// are checked and reported only)
 bool tiles_valid(const ch_env* env, int smem_max, int ppc_pre, int ppc_post, int post_batched) {
   const Grid& g = env->g;
-  const size_t node = env->prm.precision == 1 ? sizeof(float2) : sizeof(double2);
   auto pow2 = [](int v, int hi) { return v >= 1 && v <= hi && (v & (v - 1)) == 0; };
-  if (!pow2(ppc_pre, 8) || pre_tile_bytes(g, ppc_pre, node) > (size_t)smem_max) return false;
+  if (!pow2(ppc_pre, 8)) return false;
   if (post_batched == 1) return pow2(ppc_post, 16);
   if (post_batched != 0) return false;
-  // the per-tile form runs 8 ppc threads and any tile width up to 8 (widths
+  // the per-tile form runs 128 ppc threads and any tile width up to 8 (widths
   // that are not powers of two fill the resident CTA slots more evenly)
   return ppc_post >= 1 && ppc_post <= 8 && stage_post_smem(g, env->tab.tau.Mh, ppc_post) <= (size_t)smem_max;
 }
@@ -1197,12 +1193,13 @@ int env_create(const ch_params_t* p, ch_env_t** out) {
     while (env->ppc_post > 1 && stage_post_smem(g, env->tab.tau.Mh, env->ppc_post) > (size_t)smem_max)
       env->ppc_post /= 2;
     env->ppc_pre = 8;
-    while (env->ppc_pre > 1 && pre_tile_bytes(g, env->ppc_pre, sizeof(double2)) > (size_t)smem_max) env->ppc_pre /= 2;
     if (stage_post_smem(g, env->tab.tau.Mh, env->ppc_post) > (size_t)smem_max) return fail(CH_ERR_UNSUPPORTED);
     // The two-launch form runs eight threads per mode; from 768 modes on it
     // beats the scans, which spread every system over sixteen lanes (us per
-    // launch, scans and two launches: 65 nodes FP64 48 and 62 at 512 modes, 80
-    // and 64 at 1024; mixed 33 and 41, 50 and 41).
+    // step, scans / two launches, FP64 at 512 and 768 modes: 17 nodes 154 / 162 and
+    // 197 / 181, 65 nodes 353 / 387 and 463 / 442, 129 nodes 660 / 680 and 909 /
+    // 793; mixed 65 nodes 157 / 183 and 195 / 189, 129 nodes 232 / 279 and 273 /
+    // 267; only FP64 at 193 nodes crosses earlier, 1068 / 1018 at 512).
     if ((size_t)B * P >= (size_t)768) {
       env->post_batched = true;
       env->ppc_post = 16;

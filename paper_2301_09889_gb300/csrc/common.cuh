@@ -89,9 +89,6 @@ __device__ __forceinline__ float narrow(double d) {
   if (a >= 0x47f00000u) u = a > 0x7ff00000u || (a == 0x7ff00000u && l) ? 0x7fffffffu : 0x7f800000u;  // NaN, else infinity
   return __uint_as_float(u | (h & 0x80000000u)) * (sub ? 0x1p-64f : 1.0f);
 }
-template <typename RN> __device__ __forceinline__ RN to_rn(double d);
-template <> __device__ __forceinline__ double to_rn<double>(double d) { return d; }
-template <> __device__ __forceinline__ float to_rn<float>(double d) { return narrow(d); }
 
 #define CH_CPX_OPS(C, R)                                                                   \
   __host__ __device__ __forceinline__ C operator+(C a, C b) { return mk(a.x + b.x, a.y + b.y); } \

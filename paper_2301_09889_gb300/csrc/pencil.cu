@@ -116,7 +116,10 @@ __global__ void wall_shear_kernel(int ny, int B, const double* UM, double nu, do
 // omega_y) / k^2, so a lane group exchanges nothing with the other component.
 // FP64-bound: three operations per coefficient and component.  One lane per
 // system where the batch fills the SMs that way; four or eight (shorter chains
-// of loads, a few operations more) for fewer systems or longer columns.
+// of loads, a few operations more) for fewer systems or longer columns (us of a
+// step's small kernels with 1 / 4 / 8 lanes: 16x65x16 x 16 70 / 54 / 52, x 128 81 /
+// 72 / 81, x 256 92 / 94 / 106, 16x129x16 x 256 137 / 123 / 130, 64x33x64 x 16 91 /
+// 101 / 119).
 // ---------------------------------------------------------------------------
 template <int L>
 __global__ void __launch_bounds__(128) sense_kernel(Grid g, int B, PencilBufs pb, DevTables t, int js, double alpha,

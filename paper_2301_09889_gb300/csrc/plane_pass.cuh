@@ -1,6 +1,7 @@
 // Dealiased nonlinear term H = u x omega (3/2 rule; paper Sec. 3.1
-// pseudo-spectral method) in three passes through a global scratch array
-// y[B][ny][6][mz][nxh] that stays in L2 for all but the largest planes:
+// pseudo-spectral method) in three passes through global memory, over node
+// values y[B][ny][6][mz][nxh] that stay in L2 for all but the largest planes (in
+// a step the handle's node array, in place; ch_nonlinear uses it as scratch):
 //   1. z inverse: the kept kz rows of a (node, field, kx) column -> mz rows;
 //   2. x pass: two physical z rows of a field packed into one complex line,
 //      inverse transform, the three products, forward transform, unpacked over
@@ -36,10 +37,7 @@ template <typename R> constexpr int z_threads(int m) { return line_b(m) * z_cols
 
 // x pass: row pairs per CTA (the task counts of its steps are multiples of the
 // threads, or nearly), threads and CTAs per SM (bounds the registers)
-template <typename R> constexpr int x_pairs(int m) {
-  if (sizeof(R) == 4) return m <= 96 ? 8 : m <= 192 ? 4 : 2;
-  return m <= 96 ? 8 : m <= 192 ? 4 : 2;
-}
+constexpr int x_pairs(int m) { return m <= 96 ? 8 : m <= 192 ? 4 : 2; }
 template <typename R> constexpr int x_threads(int m) { return m <= 24 || (sizeof(R) == 4 && m >= 144) ? 96 : 192; }
 template <typename R> constexpr int x_ctas(int m) { return sizeof(R) == 4 && m >= 144 ? 5 : 1; }
 // elements between the sub-lines of a line, odd, and between lines: the
@@ -299,7 +297,7 @@ cudaError_t zpass_forward_m(const PlaneArgs<R>& a, int B, cudaStream_t st) {
 }
 template <typename R, int MX>
 cudaError_t xpass_m(const PlaneArgs<R>& a, int B, cudaStream_t st) {
-  constexpr int NPR = x_pairs<R>(MX), NT = x_threads<R>(MX);
+  constexpr int NPR = x_pairs(MX), NT = x_threads<R>(MX);
   constexpr size_t smem = (size_t)6 * NPR * x_line<R>(MX) * sizeof(typename cpx<R>::T);
   static SmemLimit lim;
   const cudaError_t e = raise_smem_limit(xpass_kernel<R, MX, NPR, NT>, &lim, smem);

@@ -41,8 +41,8 @@
 // operation takes the same 64 to 76 cycles of its sub-partition whatever the
 // dependences, so what counts is that every sub-partition always has a warp
 // whose operands are there: the coefficient array of a thread lives in a
-// column of shared memory (M doubles; up to 24 warps per SM at 65 nodes,
-// where arrays in registers left ten), loads run three or five rows ahead, the loops
+// column of shared memory (M doubles), so that registers hold the rows in flight
+// only (twelve warps per SM with three rows ahead, eight with five), the loops
 // stay rolled, and the two equations are CTAs of their own.
 #pragma once
 
@@ -549,11 +549,15 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
 
 // CTA: 16 modes x 2 components (lanes) x 2 classes (warps) of one equation:
 // the mean flow, then v (twice the work of omega_y), then omega_y.  D rows are
-// loaded ahead: three on 168 registers where six CTAs per SM are there to be
-// resident, five on 255 where the grid or the shared memory of the columns
-// leaves four or fewer (us per RK step with 3 and 5: 256 minimal mixed 840 and
-// 951, 128x129x128 mixed 418 and 460; 24x50x48 x 8 mixed 219 and 168,
-// 256x193x256 mixed 2546 and 2368).
+// loaded ahead: three on 168 registers (six CTAs per SM up to 147 nodes, five up
+// to 175), five on up to 255 where the grid or the columns leave four or fewer.
+// us per step with 3 / 5, the implicit half and all else: 16x65x16 x 256 mixed
+// 1205 / 1302, 128x129x128 mixed 764 / 807, 16x171x16 x 128 mixed 3584 / 3660,
+// 64x65x64 x 4 FP64 2970 / 3066; 64x148x64 x 2 mixed 963 / 938, 24x50x48 x 8
+// mixed 316 / 314, 64x65x64 FP64 945 / 946.  Under a free-slip top, where three
+// rows spill (344 bytes mixed, 520 FP64): 16x65x16 x 128 mixed 781 / 812,
+// 64x65x64 x 4 mixed 479 / 560 and FP64 3014 / 3104, 16x65x16 x 128 FP64 4732 /
+// 4704.
 template <typename RN, int TOP, int D>
 __global__ void __launch_bounds__(64, D == 3 ? 6 : 4) stage_solve_kernel(Grid g, PencilBufs pb, DevTables t,
                                                             const typename cpx<RN>::T* __restrict__ hc, StageCoef sc) {
