@@ -141,25 +141,56 @@ __global__ void __launch_bounds__(192) stage_pre_direct_kernel(Grid g, PencilBuf
   const int Jp = (J + 15) / 8 * 8;
   const RN* tab = pre_table<RN>(t) + j0;  // cos(pi j n / N) at tab[n Jp + j - j0]
   RN E[K] = {}, O[K] = {};
-  int n = 0;
-#pragma unroll 2
-  for (; n + 1 <= N; n += 2) {
-    RN c[K], d[K];
-    load_k(tab + (size_t)n * Jp, c);
-    load_k(tab + (size_t)(n + 1) * Jp, d);
-    const RN x = co[n * 32 + lane], y = co[(n + 1) * 32 + lane];
+  if constexpr (kF32) {
+    // from the highest coefficient down, the small terms first: summed upwards
+    // every term rounds at the size of the lowest ones (mixed 16x148x16: omega_y
+    // 2.5e-7 off after five steps, 1.6e-7 so)
+    const RN* tp = tab + (size_t)N * Jp;
+    const RN* cp = co + N * 32 + lane;
+    if ((N & 1) == 0) {
+      RN c[K];
+      load_k(tp, c);
+      const RN x = *cp;
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-      E[k] = E[k] + c[k] * x;
-      O[k] = O[k] + d[k] * y;
+      for (int k = 0; k < K; ++k) E[k] = c[k] * x;
+      tp -= Jp;
+      cp -= 32;
     }
-  }
-  if (n == N) {
-    RN c[K];
-    load_k(tab + (size_t)n * Jp, c);
-    const RN x = co[n * 32 + lane];
+#pragma unroll 1
+    for (int i = (N + 1) / 2; i > 0; --i) {
+      RN c[K], d[K];
+      load_k(tp - Jp, c);
+      load_k(tp, d);
+      const RN x = cp[-32], y = *cp;
 #pragma unroll
-    for (int k = 0; k < K; ++k) E[k] = E[k] + c[k] * x;
+      for (int k = 0; k < K; ++k) {
+        E[k] = E[k] + c[k] * x;
+        O[k] = O[k] + d[k] * y;
+      }
+      tp -= 2 * Jp;
+      cp -= 64;
+    }
+  } else {
+    int n = 0;
+#pragma unroll 2
+    for (; n + 1 <= N; n += 2) {
+      RN c[K], d[K];
+      load_k(tab + (size_t)n * Jp, c);
+      load_k(tab + (size_t)(n + 1) * Jp, d);
+      const RN x = co[n * 32 + lane], y = co[(n + 1) * 32 + lane];
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        E[k] = E[k] + c[k] * x;
+        O[k] = O[k] + d[k] * y;
+      }
+    }
+    if (n == N) {
+      RN c[K];
+      load_k(tab + (size_t)n * Jp, c);
+      const RN x = co[n * 32 + lane];
+#pragma unroll
+      for (int k = 0; k < K; ++k) E[k] = E[k] + c[k] * x;
+    }
   }
   RN* dst = reinterpret_cast<RN*>(q) + 2 * (b * g.qb + f * g.qf + p) + r;
   const size_t qs = 2 * g.qj;

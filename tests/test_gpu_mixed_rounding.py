@@ -1,0 +1,38 @@
+"""Rounding of the FP32 part of mixed handles against all-FP64 handles."""
+
+import numpy as np
+import pytest
+
+import seeded_inputs as si
+
+pytestmark = pytest.mark.gpu
+
+
+def _omega_y_error(native, ny, batch=16, steps=5):
+    """rms over the slots of the relative error of omega_y after `steps`."""
+    nx, nz = 16, 16
+    kw = dict(nx=nx, ny=ny, nz=nz, lx=2.67, lz=0.8, re_tau=180.0, re_bulk=2800.0, dt=0.005, batch=batch)
+    acts = np.stack([si.wall_action(nx, nz, 40 + e, 0.05 * 180 / 2800) for e in range(batch)])
+    g = []
+    for precision in (0, 1):
+        env = native.env_create(native.params(**kw, precision=precision))
+        try:
+            for e in range(batch):
+                native.env_set_state(env, e, native.pack_state(si.perturbed_poiseuille(nx, ny, nz, 100 + e, 0.2, 99),
+                                                               nx, ny, nz))
+            obs, tau, rew = np.zeros((batch, 2, nz, nx)), np.zeros(batch), np.zeros(batch)
+            for _ in range(steps):
+                assert native.env_step(env, acts, obs, tau, rew) == 0
+            g.append([native.unpack_state(native.env_get_state(env, e), nx, ny, nz)["g"] for e in range(batch)])
+        finally:
+            native.env_destroy(env)
+    return np.sqrt(np.mean([np.linalg.norm(b - a) ** 2 / np.linalg.norm(a) ** 2 for a, b in zip(*g)]))
+
+
+def test_direct_sums_round_like_transforms(native_gpu):
+    """Chebyshev sums of 148 nodes (no register transform) leave omega_y no
+    further off than the transforms of 129 nodes: the sums start at the highest,
+    smallest coefficients.  Sixteen flows each; a sum of 74 terms that starts at
+    the largest rounds each at the size of the whole."""
+    sums, transforms = _omega_y_error(native_gpu, 148), _omega_y_error(native_gpu, 129)
+    assert sums < 1.3 * transforms, (sums, transforms)
