@@ -812,6 +812,8 @@ StageCoef stage_coef(const ch_env* env, int k, double theta) {
   sc.cc = sc.alpha / sc.beta;
   sc.dgaf = (float)(sc.dt * sc.gamma);
   sc.dzef = (float)(sc.dt * sc.zeta);
+  sc.dgal = (float)(sc.dt * sc.gamma - sc.dgaf);
+  sc.dzel = (float)(sc.dt * sc.zeta - sc.dzef);
   sc.k = k;
   return sc;
 }

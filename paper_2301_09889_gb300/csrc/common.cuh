@@ -355,7 +355,7 @@ struct TauTables {
 struct StageCoef {
   double alpha, beta, gamma, zeta, dt, nu, theta, flux;
   double cc;                  // alpha / beta
-  float dgaf, dzef;           // dt gamma, dt zeta in FP32
+  float dgaf, dzef, dgal, dzel;  // dt gamma, dt zeta as sums of two FP32 values (f + l)
   int k;
 };
 

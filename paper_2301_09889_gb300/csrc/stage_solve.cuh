@@ -56,15 +56,14 @@ namespace chdns {
 template <int TOP> constexpr int solve_tabs() { return TOP ? 8 : 7; }  // eA, eB, eC, h, b, W, E1 (, W2)
 constexpr int kPoisTabs = 6;                                           // eA, eB, eC, h, b, W
 
-// dt gamma and dt zeta in the node precision
+// dt (gamma h + zeta h') in the node precision; in FP32 with the coefficients as
+// sums of two values: one rounding of dt gamma is the same for every mode and
+// step, and such errors do not average out (v of 64x65x64 after five steps
+// 8.8e-8 off with one value, 7.6e-8 with two)
 template <typename RN>
-struct Coef3 {
-  RN dga, dze;
-};
-template <typename RN>
-__device__ __forceinline__ Coef3<RN> node_coef(const StageCoef& sc) {
-  if constexpr (sizeof(RN) == 4) return Coef3<RN>{sc.dgaf, sc.dzef};
-  else return Coef3<RN>{sc.dt * sc.gamma, sc.dt * sc.zeta};
+__device__ __forceinline__ RN explicit_rhs(const StageCoef& sc, RN h, RN hp) {
+  if constexpr (sizeof(RN) == 4) return fmaf(sc.dgaf, h, fmaf(sc.dzef, hp, fmaf(sc.dgal, h, sc.dzel * hp)));
+  else return sc.dt * sc.gamma * h + sc.dt * sc.zeta * hp;
 }
 
 // Rows i = M-1 .. 0 (down) or i0 .. M-1 (up) in order, the loads of a row D
@@ -152,7 +151,6 @@ __device__ __forceinline__ Wall omega_down(double* f, const Grid& g, const Penci
   const RN* hz = hx + 4 * g.qf;
   const size_t hS = 2 * g.qj;
   const RN sgn = r == 0 ? (RN)-1 : (RN)1, kx = sgn * (RN)t.kx[ix], kz = sgn * (RN)t.kz[row];
-  const Coef3<RN> nc = node_coef<RN>(sc);
   struct In {
     double x;
     RN hx, hz, hp;
@@ -180,7 +178,7 @@ __device__ __forceinline__ Wall omega_down(double* f, const Grid& g, const Penci
         HG[n * hP] = hg;
         w.S0 += v.x;
         if (TOP) w.S2 = fma(__ldg(n2 + n), v.x, w.S2);
-        const double r0 = fma(cc1, v.x, widen(nc.dga * hg + nc.dze * v.hp));
+        const double r0 = fma(cc1, v.x, widen(explicit_rhs<RN>(sc, hg, v.hp)));
         if (i + 1 < M) {
           const double a = fma(-v.tb.h, an, fma(v.tb.eC, r2, fma(-v.tb.eB, r1, v.tb.eA * r0)));
           f[(i + 1) * NT] = a;
@@ -419,7 +417,6 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
   const size_t hS = 2 * g.qj;
   const double kxd = t.kx[ix], kzd = t.kz[row], k2 = fma(kxd, kxd, kzd * kzd), ck2 = -(1.0 + cc) * k2;
   const RN sgn = r == 0 ? (RN)-1 : (RN)1, kx = sgn * (RN)kxd, kz = sgn * (RN)kzd, k2n = (RN)k2;
-  const Coef3<RN> nc = node_coef<RN>(sc);
   double Aw = 0.0, Bw = 0.0;
   if (live) {
     struct In {
@@ -452,7 +449,7 @@ __device__ __forceinline__ void solve_v(double* f, double* xch, const Grid& g, c
       dtt = n == 0 ? (RN)0.5 * t2 : t2;
       const RN hv = -k2n * v.hy - dtt;
       HV[(size_t)n * hP] = hv;
-      const RN q = nc.dga * hv + nc.dze * v.hp;
+      const RN q = explicit_rhs<RN>(sc, hv, v.hp);
       S0 += v.x;
       const double r0 = fma(ck2, v.x, widen(q));
       if (i + 1 < M) {
