@@ -210,7 +210,7 @@ def measured_peaks() -> dict:
 # under profiles/); absent where no capture of the current kernel exists
 TRAFFIC_BYTES = {
     # analysis and solves of one stage
-    ("minimal_batch256_mixed", "stage_post"): (52.6 + 222.3) * 1e6,
+    ("minimal_batch256_mixed", "stage_post"): (52.3 + 221.1) * 1e6,
     # the three passes of one FP64 64x64-mode stage (the node values stay in L2)
     ("larger_fp64", "nonlinear_plane"): (12.6 + 19.2 + 9.6) * 1e6,
 }

@@ -101,8 +101,9 @@ __device__ __forceinline__ void bfly(C& a, C& b, C w) {
 // natural order out; w[i] = w^(2^i).  24, 76 and 208 operations at N = 4, 8
 // and 16, where the products w^b x_b and dft_pow2 take 28, 80 and 228; two,
 // three and four twiddles to load instead of N - 1.  64x65x64 FP64: the passes of
-// a step 587 -> 566 us; the error of the term grows by 1 to 2 %, 4.50e-16 to
-// 4.57e-16 at 96x32x16.
+// a step 587 -> 566 us.  The error of the term grows by 1 to 2 % and stays below
+// that of the radix passes it replaced (8x8 to 64x64 modes, extended precision:
+// 2.7e-16 to 4.1e-16 against 3.1e-16 to 6.2e-16).
 template <int N, typename R, typename C>
 __device__ __forceinline__ void dft_tw(C* x, const C* w) {
   if constexpr (N == 2) {
